@@ -17,10 +17,10 @@ CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libfedhe.so")
 BUILD = os.path.join(HERE, "_build")
 
-CUDA_SOURCES = ["fedhe_transform.cu", "fedhe_slots.cu", "fedhe_encrypt.cu", "fedhe_server.cu", "fedhe_decrypt.cu",
+CUDA_SOURCES = ["fedhe_transform.cu", "fedhe_slots.cu", "fedhe_encrypt.cu", "fedhe_fft.cu", "fedhe_server.cu", "fedhe_decrypt.cu",
                 "fedhe_mask.cu", "fedhe_api.cu", "fedhe_noalloc.cu"]
 HOST_SOURCES = ["fedhe_host.cpp"]
-HEADERS = ["fedhe_device.cuh", "fedhe_ntt.cuh", "fedhe_internal.cuh", "fedhe_launch.h", "fedhe_host.h",
+HEADERS = ["fedhe_device.cuh", "fedhe_ntt.cuh", "fedhe_fft.cuh", "fedhe_internal.cuh", "fedhe_launch.h", "fedhe_host.h",
            "fedhe_kernels.cuh", "fedhe_slots.cuh",
            os.path.join("..", "..", "include", "fedhe.h")]
 

@@ -50,6 +50,34 @@ int upload(he_ctx *ctx, const T *host, size_t count, const T **dev) {
     return HE_OK;
 }
 
+// How the exact products cut the residues of prime q: the top pieces `most` bits wide, the lowest
+// with what remains.  narrow_bits: widest low piece whose product fits 32 bits.
+void split_residues(uint64_t q, int most, int narrow_bits, FftSplit &f) {
+    int bits = 0;
+    while (q >> bits) bits++;
+    f.pieces = (uint32_t)((bits + most - 1) / most);
+    for (uint32_t p = 0; p < FFT_MAX_PIECES; p++) f.shift[p] = p && p < f.pieces ? (uint32_t)(bits - most * (int)(f.pieces - p)) : 0;
+    f.narrow = f.pieces == 2 && (int)f.shift[1] <= narrow_bits;
+    f.top_scale = ldexp(1.0, (int)f.shift[f.pieces - 1]) / (double)q;
+}
+
+// The public key's residues.  A limb of two pieces is cut as low as the low piece's product is sure to fit
+// 32 bits (a coefficient is below N 2^(width - 1)) or else as high as the top one may be wide: then the
+// product, a sum of N independent terms u_k p_k with variance 2^(2 width) / 18, stays below 2^31 (a ternary
+// u_k is strictly sub-Gaussian, so the chance of a larger one is at most 2 exp(-2^62 9 / (N 2^(2 width))):
+// under e^-95 for every width let in here).
+void split_limb(const CtxDev &d, uint64_t q, LimbDev &lb, size_t &words) {
+    const int sure = fft_sure_bits((int)d.logN), wide = fft_wide_bits((int)d.logN);
+    int bits = 0;
+    while (q >> bits) bits++;
+    const bool low_fits = bits > wide && bits - sure + (int)d.logN - 1 < 31;
+    int narrow = 0;
+    while (ldexp(9.0, 62 - (int)d.logN - 2 * (narrow + 1)) >= 95.0) narrow++;
+    split_residues(q, low_fits ? sure : wide, narrow, lb.split);
+    lb.fft_key = words;
+    words += 2 * (size_t)lb.split.pieces * (d.N / 2);
+}
+
 size_t work_bytes(const he_ctx *ctx, size_t T) { return 2 * T * (size_t)ctx->dev.N * sizeof(uint64_t); }
 
 }  // namespace
@@ -106,7 +134,13 @@ int he_ctx_create(const he_params *p, he_ctx **out) {
         d.LOGB = d.logN <= 14 ? d.logN : 13;   // longer transforms: 2^13 blocks, two per SM
         d.A = d.logN - d.LOGB;
         const uint64_t ql = p->q[p->L - 1];
+        size_t fft_words = 0;
+        split_residues(p->q[0], fft_sure_bits((int)d.logN), 30 - (int)d.logN + 1, d.dec_split);
+        d.term_limit = INT64_MAX;
         for (uint32_t j = 0; j < p->L && rc == HE_OK; j++) {
+            split_limb(d, p->q[j], d.limb[j], fft_words);
+            d.fft_pieces += d.limb[j].split.pieces;
+            if ((int64_t)(p->q[j] / 4) < d.term_limit) d.term_limit = (int64_t)(p->q[j] / 4);
             HostLimb hl;
             host_build_limb(d.N, p->q[j], hl);
             LimbDev &ld = d.limb[j];
@@ -134,10 +168,15 @@ int he_ctx_create(const he_params *p, he_ctx **out) {
             }
         }
         if (rc != HE_OK) break;
-        std::vector<double> roots, ftw;
+        std::vector<double> roots, ftw, fwd, inv;
+        std::vector<uint32_t> slot_of;
         host_unit_roots(d.N, roots);
         host_slot_twiddles(d.N, roots, ftw);
         rc = upload(ctx, reinterpret_cast<const double2 *>(ftw.data()), ftw.size() / 2, &d.ftw);
+        host_fft_tables(d.N, roots, fwd, inv, slot_of);
+        if (rc == HE_OK) rc = upload(ctx, reinterpret_cast<const root_t *>(fwd.data()), fwd.size() / 2, &d.fft_fwd);
+        if (rc == HE_OK) rc = upload(ctx, reinterpret_cast<const root_t *>(inv.data()), inv.size() / 2, &d.fft_inv);
+        if (rc == HE_OK) rc = upload(ctx, slot_of.data(), slot_of.size(), &d.slot_of);
         if (rc != HE_OK) break;
         rc = upload(ctx, d.limb, HE_MAX_LIMBS, &d.limb_dev);
         if (rc != HE_OK) break;
@@ -190,8 +229,9 @@ int he_ctx_status(he_ctx *ctx, int *status) {
 int he_ctx_reserve(he_ctx *ctx, size_t max_k) {
     if (!good(ctx)) return HE_ERR_INVALID_ARG;
     const size_t T = he_num_ct(ctx, max_k);
-    size_t need = encrypt_work_bytes(ctx->dev, ctx->sm_count, T, true);
-    if (ctx->dev.A > 0 && work_bytes(ctx, T) > need) need = work_bytes(ctx, T);     // decryption on the long rings
+    size_t need = encrypt_ntt_work_bytes(ctx->dev, ctx->sm_count, T);
+    const size_t fft = fft_work_bytes(ctx->dev, ctx->sm_count, T);
+    if (fft > need) need = fft;
     return ensure(&ctx->ws, &ctx->ws_bytes, need);
 }
 
@@ -219,7 +259,8 @@ int he_keygen(he_ctx *ctx, uint64_t seed, he_keys **out, void *stream) {
     k->magic = KEYS_MAGIC;
     k->ctx = ctx;
     k->storage = nullptr;
-    const size_t bytes = 3 * LN * sizeof(tw_t) + d.N;
+    const size_t fft_words = (1 + 2 * (size_t)d.fft_pieces) * (d.N / 2);     // the secret, then the pieces of the public key
+    const size_t bytes = 3 * LN * sizeof(tw_t) + fft_words * sizeof(double2) + d.N;
     void *tmp = nullptr;
     int rc = HE_OK;
     do {
@@ -229,13 +270,18 @@ int he_keygen(he_ctx *ctx, uint64_t seed, he_keys **out, void *stream) {
         }
         tw_t *base = static_cast<tw_t *>(k->storage);
         tw_t *pk0 = base, *pk1 = base + LN, *sh = base + 2 * LN;
-        int8_t *s8 = reinterpret_cast<int8_t *>(base + 3 * LN);
-        k->dev = KeysDev{pk0, pk1, sh, s8};
+        double2 *fft_s = reinterpret_cast<double2 *>(base + 3 * LN), *fft_pk = fft_s + d.N / 2;
+        int8_t *s8 = reinterpret_cast<int8_t *>(fft_s + fft_words);
+        k->dev = KeysDev{pk0, pk1, sh, s8, fft_pk, fft_s};
         cudaStream_t st = as_stream(stream);
         uint64_t *t64 = static_cast<uint64_t *>(tmp);
         if (launch_keygen_sample(d, seed, s8, t64, st) != cudaSuccess ||
             launch_ntt(d, true, t64, 3, LN, 0, d.L, st) != cudaSuccess ||
             launch_keygen_combine(d, t64, pk0, pk1, sh, st) != cudaSuccess ||
+            // the public key's coefficients (pk0^ and pk1^ are adjacent), for the tables of the exact products
+            launch_extract_values(pk0, t64, 2 * LN, st) != cudaSuccess ||
+            launch_ntt(d, false, t64, 2, LN, 0, d.L, st) != cudaSuccess ||
+            launch_fft_keys(d, t64, s8, fft_pk, fft_s, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess) {
             rc = HE_ERR_CUDA;
         }
@@ -461,7 +507,8 @@ static int encrypt_range(he_ctx *ctx, const he_keys *keys, const float *sel_dev,
     if (t_count == 0) return HE_OK;
     if (!sel_dev || !ct_dev || !aligned16(ct_dev)) return HE_ERR_INVALID_ARG;
     const CtxDev &d = ctx->dev;
-    int rc = ensure(&ctx->ws, &ctx->ws_bytes, encrypt_work_bytes(d, ctx->sm_count, t_count, ntt_out));
+    int rc = ensure(&ctx->ws, &ctx->ws_bytes, ntt_out ? encrypt_ntt_work_bytes(d, ctx->sm_count, t_count)
+                                                      : fft_work_bytes(d, ctx->sm_count, t_count));
     if (rc != HE_OK) return rc;
     cudaStream_t st = as_stream(stream);
     if (ntt_out)
@@ -611,17 +658,23 @@ static int decrypt_level(he_ctx *ctx, const he_keys *keys, const uint64_t *ct_de
     if (T == 0) return HE_OK;
     if (!ct_dev || !z_dev || !aligned16(ct_dev)) return HE_ERR_INVALID_ARG;
     const CtxDev &d = ctx->dev;
+    cudaStream_t st = as_stream(stream);
+    if (!ntt_in) {
+        if (T >= (1ull << 32)) return HE_ERR_SIZE;
+        const int rc = ensure(&ctx->ws, &ctx->ws_bytes, fft_work_bytes(d, ctx->sm_count, T));
+        if (rc != HE_OK) return rc;
+        CU(launch_decrypt_fft(d, keys->dev, ct_dev, level, T, ctx->ws, ctx->sm_count, z_dev, st));
+        return HE_OK;
+    }
     if (d.logN <= 14) {                 // one fused kernel, no work buffer
-        CU(launch_decrypt_fused(d, keys->dev, ct_dev, level, T, ntt_in, z_dev, as_stream(stream)));
+        CU(launch_decrypt_ntt_fused(d, keys->dev, ct_dev, level, T, z_dev, st));
         return HE_OK;
     }
     int rc = ensure(&ctx->ws, &ctx->ws_bytes, work_bytes(ctx, T));
     if (rc != HE_OK) return rc;
     uint64_t *scratch = static_cast<uint64_t *>(ctx->ws);
     double2 *cplx = reinterpret_cast<double2 *>(scratch + T * d.N);
-    cudaStream_t st = as_stream(stream);
-    if (ntt_in) CU(launch_decrypt_ntt(d, keys->dev, ct_dev, level, T, scratch, st));
-    else CU(launch_decrypt(d, keys->dev, ct_dev, level, T, scratch, st));
+    CU(launch_decrypt_ntt(d, keys->dev, ct_dev, level, T, scratch, st));
     CU(launch_decode(d, reinterpret_cast<const int64_t *>(scratch), T, cplx, z_dev, st));
     return HE_OK;
 }
@@ -703,7 +756,7 @@ int he_threshold_split(he_ctx *ctx, const he_keys *keys, uint64_t seed, he_keys 
             sh[p]->storage = nullptr;
             if (cudaMalloc(&sh[p]->storage, LN * sizeof(tw_t)) != cudaSuccess) { rc = HE_ERR_ALLOC; break; }
             tw_t *tab = static_cast<tw_t *>(sh[p]->storage);
-            sh[p]->dev = KeysDev{nullptr, nullptr, tab, nullptr};
+            sh[p]->dev = KeysDev{nullptr, nullptr, tab, nullptr, nullptr, nullptr};
             if (launch_share_tables(d, t64 + p * LN, tab, st) != cudaSuccess) rc = HE_ERR_CUDA;
         }
         if (rc == HE_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = HE_ERR_CUDA;
@@ -811,12 +864,7 @@ static int round_host_full(he_ctx *ctx, const he_keys *keys, const float *const 
                  b_agg = align(Tmax * aggw * sizeof(uint64_t)), b_z = align(T * n * sizeof(double));
     int rc = ensure(&ctx->round_buf, &ctx->round_bytes, 2 * C * b_sel + b_cts + b_agg + b_z);
     if (rc != HE_OK) return rc;
-    {
-        size_t need = encrypt_work_bytes(d, ctx->sm_count, Tmax, false);
-        if (d.A > 0 && work_bytes(ctx, Tmax) > need) need = work_bytes(ctx, Tmax);
-        rc = ensure(&ctx->ws, &ctx->ws_bytes, need);
-    }
-    if (rc != HE_OK) return rc;
+    if ((rc = ensure(&ctx->ws, &ctx->ws_bytes, fft_work_bytes(d, ctx->sm_count, Tmax))) != HE_OK) return rc;
     if ((rc = round_host_streams(ctx)) != HE_OK) return rc;
     unsigned char *p = static_cast<unsigned char *>(ctx->round_buf);
     unsigned char *selbuf[2];
@@ -917,12 +965,7 @@ static int round_host_queued(he_ctx *ctx, const he_keys *keys, const he_mask *ma
     const size_t total = 2 * b_x + C * (b_sel + b_rest) + b_cts + b_agg + b_z + b_ravg + b_out;
     int rc = ensure(&ctx->round_buf, &ctx->round_bytes, total);
     if (rc != HE_OK) return rc;
-    {
-        size_t need = encrypt_work_bytes(d, ctx->sm_count, Tc, false);
-        if (d.A > 0 && work_bytes(ctx, Tc) > need) need = work_bytes(ctx, Tc);
-        rc = ensure(&ctx->ws, &ctx->ws_bytes, need);
-    }
-    if (rc != HE_OK) return rc;
+    if ((rc = ensure(&ctx->ws, &ctx->ws_bytes, fft_work_bytes(d, ctx->sm_count, Tc))) != HE_OK) return rc;
     unsigned char *p = static_cast<unsigned char *>(ctx->round_buf);
     float *x[2];
     x[0] = reinterpret_cast<float *>(p); p += b_x;

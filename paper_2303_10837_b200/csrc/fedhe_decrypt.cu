@@ -82,56 +82,38 @@ cudaError_t launch_decrypt_ntt(const CtxDev &c, const KeysDev &k, const uint64_t
     return FEDHE_LAUNCHED();
 }
 
-// Fused path for N <= 2^14: one thread block per ciphertext transforms c1
-// (limb 0), multiplies by the secret key, transforms back, adds c0, centres,
-// and runs the slot transform on the result without leaving the SM; only the
-// two limb-0 polynomials are read and the n decoded values written.
+// Fused path for a transform-domain ciphertext, N <= 2^14: one thread block per
+// ciphertext transforms c0^ + c1^ s^ (limb 0) back, centres, and runs the slot
+// transform on the result without leaving the SM; only the two limb-0
+// polynomials are read and the n decoded values written.
 // L: layout of the length-N integer transform (played by L::NT / V threads),
 // LF: layout of the length-n complex transform with LF::NT == L::NT / V.
-// NTT_IN: the ciphertext is in the transform domain, so the forward transform
-// falls away and c0^ + c1^ s^ feeds the inverse transform directly.
-template <class L, int V, class LF, bool NTT_IN>
+template <class L, int V, class LF>
 __global__ void __launch_bounds__(L::NT / V, (L::NT / V) <= 512 ? 2 : 1)
-decrypt_fused_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const uint64_t *ct, uint32_t level,
-                     double *z) {
+decrypt_ntt_fused_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const uint64_t *ct, uint32_t level,
+                         double *z) {
     static_assert(LF::NT == L::NT / V && LF::LOGB + 1 == L::LOGB, "thread counts and sizes must match");
     extern __shared__ __align__(128) uint64_t sm[];
     constexpr uint32_t B = 1u << L::LOGB, n = B >> 1;
     const uint32_t tid = threadIdx.x;
     const size_t t = blockIdx.x;
-    const LimbDev &lb = c.limb[0];
+    const LimbDev &lb = c.limb[0];                           // limb 0 carries the message
     const uint64_t q = lb.q, q2 = 2 * q;
     const uint64_t *c0 = ct + ((t * 2 + 0) * level) * B, *c1 = ct + ((t * 2 + 1) * level) * B;
-    if constexpr (!NTT_IN) {
-        const NttArgs fa = LimbOf<ModInt>::args(lb, true, 0, 0);   // limb 0 carries the message
-        smem_ntt_forward<L, V>(
-            sm, tid, fa, [&](uint32_t i) { return c1[i]; },
-            [&](uint32_t p, uint64_t a, uint64_t b, uint64_t *wa, uint64_t *wb) {
-                const tw_t s0 = load_tw(k.s_hat + p), s1 = load_tw(k.s_hat + p + 1);
-                *wa = shoup_lazy(a, s0.w, s0.wp, q);         // words wswz(p), wswz(p + 1)
-                *wb = shoup_lazy(b, s1.w, s1.wp, q);
-            });
-    }
     int64_t *d = reinterpret_cast<int64_t *>(sm);
-    {
-        const NttArgs ia = LimbOf<ModInt>::args(lb, false, 0, 0);
-        smem_ntt_inverse<L, V, true>(
-            sm, tid, ia, lb.ninv, lb.wn,
-            [&](uint32_t p, const uint64_t *wa, const uint64_t *wb) {
-                if constexpr (NTT_IN) {
-                    const u64x2 a = *reinterpret_cast<const u64x2 *>(c0 + p), b = *reinterpret_cast<const u64x2 *>(c1 + p);
-                    const tw_t s0 = load_tw(k.s_hat + p), s1 = load_tw(k.s_hat + p + 1);
-                    return u64x2{csub(a.x + shoup_lazy(b.x, s0.w, s0.wp, q), q2),
-                                 csub(a.y + shoup_lazy(b.y, s1.w, s1.wp, q), q2)};
-                } else {
-                    return u64x2{*wa, *wb};
-                }
-            },
-            [&](uint32_t i, uint64_t v, uint64_t *wv) {
-                const uint64_t r = NTT_IN ? csub(v, q) : addmod(csub(v, q), c0[i], q);
-                *reinterpret_cast<int64_t *>(wv) = r > q / 2 ? -(int64_t)(q - r) : (int64_t)r;     // d[wswz(i)]
-            });
-    }
+    const NttArgs ia = LimbOf<ModInt>::args(lb, false, 0, 0);
+    smem_ntt_inverse<L, V, true>(
+        sm, tid, ia, lb.ninv, lb.wn,
+        [&](uint32_t p) {
+            const u64x2 a = *reinterpret_cast<const u64x2 *>(c0 + p), b = *reinterpret_cast<const u64x2 *>(c1 + p);
+            const tw_t s0 = load_tw(k.s_hat + p), s1 = load_tw(k.s_hat + p + 1);
+            return u64x2{csub(a.x + shoup_lazy(b.x, s0.w, s0.wp, q), q2),
+                         csub(a.y + shoup_lazy(b.y, s1.w, s1.wp, q), q2)};
+        },
+        [&](uint32_t, uint64_t v, uint64_t *wv) {
+            const uint64_t r = csub(v, q);
+            *reinterpret_cast<int64_t *>(wv) = r > q / 2 ? -(int64_t)(q - r) : (int64_t)r;     // d[wswz(i)]
+        });
     __syncthreads();
     // slot transform: bit-reversed load of (d_k + i d_{k+n}) / Delta from shared memory
     const double inv_delta = __longlong_as_double((long long)(1023 - c.log2_delta) << 52);
@@ -147,26 +129,22 @@ decrypt_fused_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const ui
     for (int r = 0; r < LF::E; r++) z[t * n + LF::template idx<0>(tid, r)] = x[r].re;
 }
 
-template <class L, int V, class LF, bool NTT_IN>
-static cudaError_t launch_decrypt_fused_t(const CtxDev &c, const KeysDev &k, const uint64_t *ct, uint32_t level,
-                                          size_t T, double *z, cudaStream_t s) {
+template <class L, int V, class LF>
+static cudaError_t launch_decrypt_ntt_fused_t(const CtxDev &c, const KeysDev &k, const uint64_t *ct, uint32_t level,
+                                              size_t T, double *z, cudaStream_t s) {
     const size_t smem = sizeof(uint64_t) << L::LOGB;
-    auto kern = decrypt_fused_kernel<L, V, LF, NTT_IN>;
+    auto kern = decrypt_ntt_fused_kernel<L, V, LF>;
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
     kern<<<(unsigned)T, L::NT / V, smem, s>>>(c, k, ct, level, z);
     return FEDHE_LAUNCHED();
 }
 
-cudaError_t launch_decrypt_fused(const CtxDev &c, const KeysDev &k, const uint64_t *ct, uint32_t level,
-                                 size_t T, bool ntt_in, double *z, cudaStream_t s) {
+cudaError_t launch_decrypt_ntt_fused(const CtxDev &c, const KeysDev &k, const uint64_t *ct, uint32_t level,
+                                     size_t T, double *z, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
-    if (c.logN == 13) {
-        if (ntt_in) return launch_decrypt_fused_t<WLay<13>, 2, Lay<12, 3>, true>(c, k, ct, level, T, z, s);
-        return launch_decrypt_fused_t<WLay<13>, 2, Lay<12, 3>, false>(c, k, ct, level, T, z, s);
-    }
-    if (ntt_in) return launch_decrypt_fused_t<WLay<14>, 2, Lay<13, 3>, true>(c, k, ct, level, T, z, s);
-    return launch_decrypt_fused_t<WLay<14>, 2, Lay<13, 3>, false>(c, k, ct, level, T, z, s);
+    if (c.logN == 13) return launch_decrypt_ntt_fused_t<WLay<13>, 2, Lay<12, 3>>(c, k, ct, level, T, z, s);
+    return launch_decrypt_ntt_fused_t<WLay<14>, 2, Lay<13, 3>>(c, k, ct, level, T, z, s);
 }
 
 // ===========================================================================

@@ -157,4 +157,53 @@ void host_slot_twiddles(uint32_t N, const std::vector<double> &roots, std::vecto
     }
 }
 
+void host_fft_tables(uint32_t N, const std::vector<double> &roots, std::vector<double> &fwd, std::vector<double> &inv,
+                     std::vector<uint32_t> &slot_of) {
+    const uint32_t n = N / 2, M = 2 * N;
+    uint32_t logn = 0;
+    while ((1u << logn) < n) logn++;
+    const uint32_t LB = 12, CL = logn - LB, NT = (1u << LB) / 16;
+    // forward: level l, block b -> angle pi / 2^(l+2) + pi brev(b) / 2^l
+    fwd.assign(2 * (size_t)n, 0.0);
+    for (uint32_t l = 0; l < logn; l++)
+        for (uint32_t b = 0; b < (1u << l); b++) {
+            const uint32_t t = (N >> (l + 2)) + (uint32_t)(((uint64_t)N * bit_reverse(b, (int)l)) >> l);
+            fwd[2 * (((size_t)1 << l) + b)] = roots[2 * (size_t)t];
+            fwd[2 * (((size_t)1 << l) + b) + 1] = roots[2 * (size_t)t + 1];
+        }
+    inv.clear();
+    auto push = [&](uint32_t t) {            // exp(-2 pi i t / 2N)
+        inv.push_back(roots[2 * (size_t)t]);
+        inv.push_back(-roots[2 * (size_t)t + 1]);
+    };
+    auto run = [&](uint32_t len, uint32_t first, uint32_t count) {
+        for (uint32_t j = 0; j < count; j++) push((M / len) * (first + j));
+    };
+    run(32, 0, 16);
+    run(64, 0, 16);
+    run(128, 0, 16);
+    run(128, 16, 16);
+    for (uint32_t m = 0; m < 4; m++) run(256, 16 * m, 16);
+    for (uint32_t j = 0; j < NT; j++) push(j);
+    for (uint32_t s = LB - 3; s <= LB + CL; s++) run(1u << s, 0, NT);
+    // angles in units of pi / 256: of the stages between blocks, then what is left of the untwisting
+    for (uint32_t r = 0; r < 16; r++) {
+        for (uint32_t i = 0; i < CL; i++)
+            for (uint32_t a = 0; a < (i == 0 ? 1u : (1u << i) / 2); a++) push((N / 256) * ((16 * r + 256 * a) >> i));
+        for (uint32_t a = 0; a < (1u << CL); a++) push((N / 256) * ((8 * r + 128 * a) >> CL));
+    }
+    // the value at position p is the one at exp(i pi (1 + 4 brev(p)) / N); slot j belongs to exp(i pi 5^j / N)
+    std::vector<uint32_t> slot(n);
+    uint32_t p5 = 1;
+    for (uint32_t j = 0; j < n; j++) {
+        slot[(p5 - 1) / 4] = j;
+        p5 = (uint32_t)(((uint64_t)p5 * 5u) % M);
+    }
+    slot_of.resize(n);
+    for (uint32_t blk = 0; blk < (1u << CL); blk++)
+        for (uint32_t r = 0; r < 16; r++)
+            for (uint32_t tid = 0; tid < NT; tid++)
+                slot_of[(blk * 16 + r) * NT + tid] = slot[bit_reverse((blk << LB) | (16 * tid + r), (int)logn)];
+}
+
 }  // namespace fedhe

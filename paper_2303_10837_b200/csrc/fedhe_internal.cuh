@@ -7,9 +7,29 @@
 #include <vector>
 
 #include "../../include/fedhe.h"
+#include "fedhe_fft.cuh"
 #include "fedhe_ntt.cuh"
 
 namespace fedhe {
+
+// How a centred residue is cut: v = sum_p piece_p 2^shift_p, p < pieces.
+struct FftSplit {
+    uint32_t pieces, shift[FFT_MAX_PIECES];
+    uint32_t narrow;     // two pieces, and the rounded product of the lower one fits 32 bits
+    double top_scale;    // 2^(shift of the top piece) / q
+};
+
+// Cuts a centred residue (|v| < q/2) into its pieces, lowest first; each but the top one lies in
+// [-2^(w-1), 2^(w-1)) for its width w.
+HD int64_t fft_piece(const FftSplit &f, int64_t v, uint32_t p) {
+    for (uint32_t i = 0; i + 1 < f.pieces; i++) {
+        const uint32_t w = f.shift[i + 1] - f.shift[i];
+        const int64_t up = (v + ((int64_t)1 << (w - 1))) >> w;
+        if (i == p) return v - (int64_t)((uint64_t)up << w);
+        v = up;
+    }
+    return v;
+}
 
 // Per-prime constants and table pointers, passed to kernels by value.
 struct LimbDev {
@@ -26,6 +46,8 @@ struct LimbDev {
     const double *inv_d;
     double qd, qi;       // q and 1/q rounded
     double ninv_d, wn_d; // 1/N and (inverse twiddle of stage 0)/N
+    FftSplit split;      // of the public key's residues for the exact products by complex transforms
+    size_t fft_key;      // first word of the limb's key tables: [2 components][pieces][n]
 };
 
 // the pieces of a limb that a transform in arithmetic M needs
@@ -55,6 +77,11 @@ struct CtxDev {
     LimbDev limb[HE_MAX_LIMBS];
     const LimbDev *limb_dev;   // the same table in device memory, for kernels that loop over limbs
     const double2 *ftw;  // slot-transform twiddles, entry [len/2 + j]
+    const root_t *fft_fwd, *fft_inv;   // complex transforms of the exact products (fedhe_fft.cuh)
+    const uint32_t *slot_of;           // slot of every value that the forward transform leaves
+    FftSplit dec_split;                // of c1 on limb 0, for any c1
+    uint32_t fft_pieces;               // of all limbs of a public-key half
+    int64_t term_limit;                // a quarter of the smallest prime
     int *status;         // sticky anomaly word
 };
 
@@ -63,6 +90,8 @@ struct KeysDev {
     const tw_t *pk1_hat;
     const tw_t *s_hat;   // [L][N] transform-domain secret key
     const int8_t *s;     // [N]
+    const double2 *fft_pk; // transformed pieces of the public key, scaled by 1/n, in the threads' order
+    const double2 *fft_s;  // the transformed secret key in the same order and scale
 };
 
 }  // namespace fedhe

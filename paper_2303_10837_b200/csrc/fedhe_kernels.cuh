@@ -41,36 +41,54 @@ __device__ __forceinline__ int gauss_from_u64(uint64_t r) {
     return v;
 }
 
-// The same map through shared-memory tables: the top byte of r selects the
-// thresholds that are certainly below r (`base`) and the few that share its
-// byte (`nb`, compared one by one).
+// The same map through shared-memory tables, by the high word of r.  An entry belongs to one value of
+// its top byte: in the entry's top byte the number of thresholds certainly not above r, below it the
+// next 24 bits of the one threshold that shares the byte, to be compared with those of r (an entry
+// without such a threshold counts one less and compares with 0).  The bytes 00 and ff share more than one
+// threshold (1 sample in 128) and have a second row each for the next byte; what is still undecided there
+// (1 in 32768, and equal bits, 1 in 2^24) is counted threshold by threshold.
+// One 4-byte load and a comparison per sample: a loop over the thresholds that share the byte cost a warp its longest one.
 struct GaussTables {
-    uint64_t cdf[38];
-    uint8_t base[256];
-    uint8_t nb[256];
+    uint32_t entry[3][256];
 };
 
-__device__ __forceinline__ void gauss_tables_init(GaussTables &g, uint32_t tid) {
-    if (tid < 38) g.cdf[tid] = c_gauss_cdf[tid];
-    if (tid < 256) {
-        const uint64_t lo = (uint64_t)tid << 56, hi = lo | 0x00ffffffffffffffull;
-        int base = 0, nb = 0;
-        for (int x = 0; x < 38; x++) {
-            const uint64_t t = c_gauss_cdf[x];
-            if (t <= lo) base++;
-            else if (t <= hi) nb++;
-        }
-        g.base[tid] = (uint8_t)base;
-        g.nb[tid] = (uint8_t)nb;
+__device__ __forceinline__ uint32_t gauss_entry(uint64_t lo, int width) {        // r in [lo, lo + 2^width)
+    const uint64_t last = lo + ((1ull << width) - 1);
+    uint32_t base = 0, in = 0;
+    uint64_t t_in = 0;
+#pragma unroll 1
+    for (int x = 0; x < 38; x++) {
+        const uint64_t t = c_gauss_cdf[x];
+        if (t <= lo) base++;
+        else if (t <= last) { in++; t_in = t; }
+    }
+    if (in > 1 || (in == 0 && base == 0)) return 0xffu << 24;
+    return in ? (base << 24) | ((uint32_t)(t_in >> (width - 24)) & 0xffffffu) : (base - 1) << 24;
+}
+
+__device__ __forceinline__ void gauss_tables_init(GaussTables &g, uint32_t tid, uint32_t nthreads) {
+    for (uint32_t i = tid; i < 768; i += nthreads) {
+        const uint32_t row = i >> 8;
+        const uint64_t b = i & 255u;
+        g.entry[row][b] = row == 0 ? gauss_entry(b << 56, 56) : gauss_entry((row == 2 ? 0xffull << 56 : 0) | (b << 48), 48);
     }
 }
 
+static __device__ __noinline__ int gauss_counted(uint64_t r) {
+    int v = -19;
+#pragma unroll 1
+    for (int x = 0; x < 38; x++) v += (r >= c_gauss_cdf[x]) ? 1 : 0;
+    return v;
+}
 __device__ __forceinline__ int gauss_from_u64(const GaussTables &g, uint64_t r) {
-    const uint32_t b = (uint32_t)(r >> 56);
-    const int base = g.base[b], nb = g.nb[b];
-    int v = base;
-    for (int i = 0; i < nb; i++) v += (r >= g.cdf[base + i]) ? 1 : 0;
-    return v - 19;
+    const uint32_t hi = (uint32_t)(r >> 32);
+    uint32_t e = g.entry[0][hi >> 24], rest = hi & 0xffffffu;
+    if ((e >> 24) == 0xffu) {
+        e = g.entry[(hi >> 31) + 1u][(hi >> 16) & 255u];
+        rest = (uint32_t)(r >> 24) & 0xffffffu;
+    }
+    if ((e >> 24) == 0xffu || rest == (e & 0xffffffu)) return gauss_counted(r);
+    return (int)(e >> 24) + (rest >= (e & 0xffffffu) ? 1 : 0) - 19;
 }
 
 __device__ __forceinline__ uint64_t addmod(uint64_t a, uint64_t b, uint64_t q) { return csub(a + b, q); }

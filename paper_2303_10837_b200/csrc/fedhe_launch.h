@@ -1,4 +1,4 @@
-// Launch wrappers of the CUDA kernels (implemented in fedhe_transform.cu, fedhe_slots.cu, fedhe_encrypt.cu, fedhe_server.cu, fedhe_decrypt.cu and fedhe_mask.cu),
+// Launch wrappers of the CUDA kernels (implemented in fedhe_transform.cu, fedhe_slots.cu, fedhe_encrypt.cu, fedhe_fft.cu, fedhe_server.cu, fedhe_decrypt.cu and fedhe_mask.cu),
 // called by the C ABI in fedhe_api.cu.  All of them enqueue work on `s` and
 // return the launch status; none synchronises.
 #pragma once
@@ -29,16 +29,23 @@ cudaError_t launch_decode(const CtxDev &c, const int64_t *d, size_t T, double2 *
                           cudaStream_t s);
 
 // Encode + encrypt ciphertexts t0 .. t0+T-1 (sel and ct point at the first of
-// them).  `work` is scratch of encrypt_work_bytes() bytes: for N <= 2^14 N words
-// per thread block of the fused kernel (the block's encoded message), for
-// longer rings the encoded messages of all T ciphertexts and the encoder's
-// complex buffer.  n_sm: the device's SM count.
-size_t encrypt_work_bytes(const CtxDev &c, int n_sm, size_t T, bool ntt_out);
+// them).  `work` is scratch of fft_work_bytes() bytes, what the resident thread
+// blocks keep in L2.  n_sm: the device's SM count.
+size_t fft_work_bytes(const CtxDev &c, int n_sm, size_t T);
 cudaError_t launch_encrypt(const CtxDev &c, const KeysDev &k, const float *sel, void *work, int n_sm,
                            uint32_t t0, size_t T, uint64_t seed, uint32_t client, uint64_t *ct,
                            cudaStream_t s);
+// Decrypt + decode T coefficient-domain ciphertexts; the same scratch.
+cudaError_t launch_decrypt_fft(const CtxDev &c, const KeysDev &k, const uint64_t *ct, uint32_t level, size_t T,
+                               void *work, int n_sm, double *z, cudaStream_t s);
+// Key tables of both from the public key's coefficients ([2][L][N], canonical) and the secret.
+cudaError_t launch_fft_keys(const CtxDev &c, const uint64_t *pk, const int8_t *s8, double2 *fft_pk, double2 *fft_s,
+                            cudaStream_t s);
 
-// the same with every limb polynomial of the result in the transform domain
+// Encryption with every limb polynomial of the result in the transform domain; `work`: for N <= 2^14
+// N words per thread block of the fused kernel (the block's encoded message), for longer rings the
+// encoded messages of all T ciphertexts, the encoder's complex buffer and the transform of u.
+size_t encrypt_ntt_work_bytes(const CtxDev &c, int n_sm, size_t T);
 cudaError_t launch_encrypt_ntt(const CtxDev &c, const KeysDev &k, const float *sel, void *work, int n_sm,
                                uint32_t t0, size_t T, uint64_t seed, uint32_t client, uint64_t *ct,
                                cudaStream_t s);
@@ -66,10 +73,9 @@ cudaError_t launch_decrypt(const CtxDev &c, const KeysDev &k, const uint64_t *ct
 cudaError_t launch_decrypt_ntt(const CtxDev &c, const KeysDev &k, const uint64_t *ct, uint32_t level,
                                size_t T, uint64_t *scratch, cudaStream_t s);
 
-// fused decrypt + decode for N <= 2^14 (no scratch): z double [T][n];
-// ntt_in: the ciphertext is in the transform domain
-cudaError_t launch_decrypt_fused(const CtxDev &c, const KeysDev &k, const uint64_t *ct, uint32_t level,
-                                 size_t T, bool ntt_in, double *z, cudaStream_t s);
+// fused decrypt + decode of a transform-domain ciphertext for N <= 2^14 (no scratch): z double [T][n]
+cudaError_t launch_decrypt_ntt_fused(const CtxDev &c, const KeysDev &k, const uint64_t *ct, uint32_t level,
+                                     size_t T, double *z, cudaStream_t s);
 
 // two-party threshold decryption.  tmp: uint64 [2][L][N] (shares as residues)
 cudaError_t launch_threshold_split(const CtxDev &c, const int8_t *s8, uint64_t seed, uint64_t *tmp,

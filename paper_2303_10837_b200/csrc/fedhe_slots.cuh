@@ -13,8 +13,6 @@ namespace fedhe {
 // multiply-add), because the rounded integers are compared bit for bit.
 // ===========================================================================
 
-struct cpx { double re, im; };
-
 __device__ __forceinline__ cpx cadd_rn(cpx a, cpx b) { return cpx{__dadd_rn(a.re, b.re), __dadd_rn(a.im, b.im)}; }
 __device__ __forceinline__ cpx csub_rn(cpx a, cpx b) { return cpx{__dsub_rn(a.re, b.re), __dsub_rn(a.im, b.im)}; }
 // (a + bi)(c + di) = (ac - bd) + (ad + bc) i, data operand first
@@ -122,17 +120,15 @@ __device__ __forceinline__ uint32_t stage_swz(uint32_t k) { return k ^ (((k >> 8
 // it enters the block's stages (the slot itself when the block is the whole
 // vector, the output of the earlier stages otherwise); `sm` is a buffer of
 // 2^LF::LOGB cpx values, used first for the exchanges between phases and then
-// to put the rounded integers in order; coefficient kk of the block (kk its
-// bit-reversed position) goes to m_out[(kk << A) | rb] and its imaginary
-// partner to m_out[((kk << A) | rb) + n], where the whole vector has
-// n = 2^(LF::LOGB + A) slots and rb is the bit-reversed block number.  Ends with
-// a block barrier after which `sm` is free and m_out may be read by the block.
+// to put the rounded integers in order; out(kk, re, im) receives coefficient kk
+// of the block (kk its bit-reversed position) and its imaginary partner, kk in
+// order over the threads.  The whole vector has 2^(LF::LOGB + A) slots.  Ends with
+// a block barrier after which `sm` is free and the block may read what `out` stored.
 // Returns whether a coefficient left the range (the caller raises the status word).
-template <class LF, class In>
-__device__ __forceinline__ bool encode_block_in_place(const CtxDev &c, const In &in, uint64_t *sm, int64_t *m_out,
-                                                      uint32_t A, uint32_t rb) {
+template <class LF, class In, class Out>
+__device__ __forceinline__ bool encode_block_in_place(const CtxDev &c, const In &in, uint64_t *sm, uint32_t A, const Out &out) {
     constexpr uint32_t NB = 1u << LF::LOGB;
-    const uint32_t tid = threadIdx.x, n = NB << A;
+    const uint32_t tid = threadIdx.x;
     cpx x[LF::E];
 #pragma unroll
     for (int r = 0; r < LF::E; r++) x[r] = in(LF::template idx<0>(tid, r));
@@ -152,11 +148,7 @@ __device__ __forceinline__ bool encode_block_in_place(const CtxDev &c, const In 
         stage[NB + stage_swz(kk)] = __double2ll_rn(im);
     }
     __syncthreads();
-    for (uint32_t kk = tid; kk < NB; kk += LF::NT) {
-        const uint32_t k = (kk << A) | rb;
-        m_out[k] = stage[stage_swz(kk)];
-        m_out[k + n] = stage[NB + stage_swz(kk)];
-    }
+    for (uint32_t kk = tid; kk < NB; kk += LF::NT) out(kk, stage[stage_swz(kk)], stage[NB + stage_swz(kk)]);
     __syncthreads();
     return bad;
 }
@@ -164,7 +156,12 @@ __device__ __forceinline__ bool encode_block_in_place(const CtxDev &c, const In 
 // the whole encoder of one slot vector of 2^LF::LOGB slots
 template <class LF>
 __device__ __forceinline__ bool encode_in_block(const CtxDev &c, const float *slots, uint64_t *sm, int64_t *m_out) {
-    return encode_block_in_place<LF>(c, [&](uint32_t i) { return cpx{(double)__ldg(slots + i), 0.0}; }, sm, m_out, 0, 0);
+    return encode_block_in_place<LF>(
+        c, [&](uint32_t i) { return cpx{(double)__ldg(slots + i), 0.0}; }, sm, 0,
+        [&](uint32_t kk, int64_t re, int64_t im) {
+            m_out[kk] = re;
+            m_out[kk + (1u << LF::LOGB)] = im;
+        });
 }
 
 }  // namespace fedhe
