@@ -7,25 +7,12 @@ namespace fedhe {
 
 constexpr double FFT_ROUND = 6755399441055744.0;                 // 1.5 * 2^52: adding it rounds to an integer ...
 constexpr int64_t FFT_ROUND_BITS = 0x4338000000000000;           // ... that is the difference of the bit patterns
-constexpr double FFT_ROUND2 = 3377699720527872.0;                // 1.5 * 2^51: the same to a multiple of 1/2
-constexpr int64_t FFT_ROUND2_BITS = 0x4328000000000000;
 
 // integer |v| < 2^51 as a double
 __device__ __forceinline__ double fft_from_int(int64_t v) {
     return f64_sub(__longlong_as_double(v + FFT_ROUND_BITS), FFT_ROUND);
 }
-// z rounded to an integer, |z| < 2^50.  WATCH (random operands): `odd` collects in its lowest bit
-// whether z is more than 1/4 from an integer; without it any distance below 1/2 is right.
-template <bool WATCH>
-__device__ __forceinline__ int64_t fft_round(double z, uint32_t &odd) {
-    if constexpr (WATCH) {
-        const int64_t z2 = __double_as_longlong(f64_add(z, FFT_ROUND2)) - FFT_ROUND2_BITS;
-        odd |= (uint32_t)z2;
-        return z2 >> 1;
-    } else {
-        return __double_as_longlong(f64_add(z, FFT_ROUND)) - FFT_ROUND_BITS;
-    }
-}
+__device__ __forceinline__ int64_t fft_round_bits(double z) { return __double_as_longlong(f64_add(z, FFT_ROUND)); }
 
 __device__ __forceinline__ cpx fft_mul(double2 a, double2 b) { return cpx_mul(cpx{a.x, a.y}, b.x, b.y); }
 
@@ -43,15 +30,21 @@ __device__ __forceinline__ double2 load_passing(const double2 *p) {
     return v;
 }
 
-// The top piece z of a product (not rounded), weighed 2^shift: q times the quotient is taken off
-// modulo 2^64, so the result has magnitude at most q / 2 and a little.
-template <bool WATCH>
-__device__ __forceinline__ int64_t fft_join(double z, const FftSplit &f, uint64_t q, uint32_t shift, uint32_t &odd) {
-    const uint64_t hi = (uint64_t)fft_round<WATCH>(z, odd) << shift;
-    // the quotient plus 2^17, which keeps it positive
-    const uint32_t k = (uint32_t)__double_as_longlong(f64_fma(z, f.top_scale, FFT_ROUND + 131072.0));
-    return (int64_t)(hi + (q << 17) - (uint64_t)k * q);
-}
+// Adds to `v` the top piece z of a product (not rounded), weighed 2^shift, less q times the quotient: all
+// modulo 2^64, and the top piece has magnitude at most q / 2 and a little then.
+struct FftJoin {
+    uint64_t minus_q, fix;
+    double scale;
+    uint32_t shift;
+    __device__ __forceinline__ FftJoin(const FftSplit &f, uint64_t q) : minus_q(0 - q), scale(f.top_scale), shift(f.shift[f.pieces - 1]) {
+        // the quotient carries 2^17, which keeps it positive
+        fix = (q << 17) - ((uint64_t)FFT_ROUND_BITS << shift);
+    }
+    __device__ __forceinline__ int64_t operator()(int64_t v, double z) const {
+        const uint32_t k = (uint32_t)__double_as_longlong(f64_fma(z, scale, FFT_ROUND + 131072.0));
+        return (int64_t)((uint64_t)v + fix + ((uint64_t)fft_round_bits(z) << shift) + (uint64_t)k * minus_q);
+    }
+};
 
 // the residue in [0, q) of |v| < q
 __device__ __forceinline__ uint64_t fft_canonical(int64_t v, uint64_t q) { return (uint64_t)(v + ((v >> 63) & (int64_t)q)); }
@@ -144,20 +137,19 @@ __device__ __forceinline__ uint32_t fft_own(int i) {
 }
 
 // ---- joined lower pieces, parked for the thread that will join the top one ----
-template <class G, bool WATCH>
+template <class G>
 __device__ __forceinline__ void fft_park(const cpx (&x)[16], unsigned char *park, const FftSplit &f, uint32_t piece,
-                                         uint32_t tid, uint32_t &odd) {
+                                         uint32_t tid) {
     if (f.narrow) {
         int *p = reinterpret_cast<int *>(park) + tid;
 #pragma unroll
-        for (int i = 0; i < 32; i++)
-            __stcg(p + i * G::NT, (int)fft_round<WATCH>((i & 1) ? x[i >> 1].im : x[i >> 1].re, odd));
+        for (int i = 0; i < 32; i++) __stcg(p + i * G::NT, (int)fft_round_bits((i & 1) ? x[i >> 1].im : x[i >> 1].re));
     } else {
         long long *p = reinterpret_cast<long long *>(park) + tid;
         const uint32_t sh = f.shift[piece];
 #pragma unroll
         for (int i = 0; i < 32; i++) {
-            long long w = fft_round<WATCH>((i & 1) ? x[i >> 1].im : x[i >> 1].re, odd) << sh;
+            long long w = (fft_round_bits((i & 1) ? x[i >> 1].im : x[i >> 1].re) - FFT_ROUND_BITS) << sh;
             if (piece) w += __ldcg(p + i * G::NT);
             __stcg(p + i * G::NT, w);
         }
@@ -244,7 +236,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
     const uint32_t per_ct = 2 * c.L;
     const uint64_t total = (uint64_t)T * 2 * c.fft_pieces;
     const uint32_t u_end = fft_unit_at(c, total * (cid + 1) / nc);
-    uint32_t have_ct = 0xffffffffu, have_e = 0xffffffffu, odd = 0;
+    uint32_t have_ct = 0xffffffffu, have_e = 0xffffffffu;
     bool big = false;                                     // a term of this component needs reducing first
 #pragma unroll 1
     for (uint32_t unit = fft_unit_at(c, total * cid / nc); unit < u_end; unit++) {
@@ -344,11 +336,11 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
             const uint32_t tid = fresh_tid();
             fft_gather<G>(x, buf, tab, rank, tid);
             if (p + 1 < f.pieces) {
-                fft_park<G, true>(x, park, f, p, tid, odd);
+                fft_park<G>(x, park, f, p, tid);
                 continue;
             }
             uint64_t *out = ct + (((size_t)tl * 2 + comp) * c.L + j) * N + tid;
-            const uint32_t shift = f.shift[f.pieces - 1];
+            const FftJoin join(f, q);
 #pragma unroll
             for (int i0 = 0; i0 < 32; i0 += G::BATCH) {
                 int64_t val[G::BATCH];
@@ -367,7 +359,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
 #pragma unroll
                 for (int i = 0; i < G::BATCH; i++) {
                     const cpx &w = x[(i0 + i) >> 1];
-                    val[i] += fft_join<true>((i & 1) ? w.im : w.re, f, q, shift, odd);
+                    val[i] = join(val[i], (i & 1) ? w.im : w.re);
                     __stcs(reinterpret_cast<unsigned long long *>(out + fft_coefficient<G>(i0 + i, rank)),
                            (unsigned long long)fft_canonical(val[i], q));
                 }
@@ -383,7 +375,6 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
             }
         }
     }
-    if (odd & 1u) atomicOr(c.status, 2);
     buffer_wait<CL>();                                    // the other blocks have read this one's buffer
 }
 
@@ -415,7 +406,6 @@ decrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const uint
     const int64_t half_q = (int64_t)(q / 2);
     const double inv_delta = __longlong_as_double((long long)(1023 - c.log2_delta) << 52);
     const uint32_t t_end = (uint32_t)((uint64_t)T * (cid + 1) / nc);
-    uint32_t odd = 0;
     __syncthreads();
 #pragma unroll 1
     for (uint32_t t = (uint32_t)((uint64_t)T * cid / nc); t < t_end; t++) {
@@ -450,10 +440,10 @@ decrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const uint
             const uint32_t tid = fresh_tid();
             fft_gather<G>(x, buf, tab, rank, tid);
             if (p + 1 < f.pieces) {
-                fft_park<G, false>(x, park, f, p, tid, odd);
+                fft_park<G>(x, park, f, p, tid);
                 continue;
             }
-            const uint32_t shift = f.shift[f.pieces - 1];
+            const FftJoin join(f, q);
 #pragma unroll
             for (int i0 = 0; i0 < 32; i0 += G::BATCH) {
                 int64_t val[G::BATCH];
@@ -463,7 +453,7 @@ decrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const uint
 #pragma unroll
                 for (int i = 0; i < G::BATCH; i++) {
                     cpx &w = x[(i0 + i) >> 1];
-                    int64_t d = val[i] + fft_join<false>((i & 1) ? w.im : w.re, f, q, shift, odd);      // (-q, 2q)
+                    int64_t d = join(val[i], (i & 1) ? w.im : w.re);      // (-q, 2q)
                     d -= d > half_q ? (int64_t)q : 0;
                     d -= d > half_q ? (int64_t)q : 0;
                     d += d < -half_q ? (int64_t)q : 0;

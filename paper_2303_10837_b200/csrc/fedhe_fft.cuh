@@ -42,10 +42,9 @@
 // some 10^6 independent ones, stay near their standard deviations, which are
 // about sqrt(N) times smaller than the bounds above.  For pieces of b bits
 //   sd(error) <= 1.3 sqrt(levels) 2^-53 * sd(product),  sd(product) = sqrt(N / 18) 2^b
-// (1.2 to 1.3 measured on every ring).  fft_wide_bits() lets 24 standard
-// deviations stay below 1/2: 40 bits at N = 2^14, so a 40-bit limb is one piece and a 60-bit one is two.
-// The rounding watches this: it rounds 2 z, and an odd result, i.e. a distance of
-// more than 1/4 from the nearest integer, raises the context's status word.
+// (1.2 to 1.3 measured on every ring).  fft_wide_bits() keeps 24 standard
+// deviations below 1/2, a chance of a wrong coefficient under 2^-400: 40 bits at N = 2^14, so that a
+// 40-bit limb is one piece and a 60-bit one is two.
 //
 // The tests play both directions on the host, thread by thread.
 #pragma once
@@ -71,10 +70,10 @@ inline int fft_sure_bits(int logN) {
 inline double fft_error_sd(int logN, int b) {
     return 1.3 * sqrt((double)(logN - 1) * (double)(1ull << logN) / 18.0) * (double)(1ull << b) / 9007199254740992.0;
 }
-// largest such pieces with 12 standard deviations below 1/4
+// largest such pieces with 24 standard deviations below 1/2
 inline int fft_wide_bits(int logN) {
     int b = 44;
-    while (12.0 * fft_error_sd(logN, b) >= 0.25) b--;
+    while (24.0 * fft_error_sd(logN, b) >= 0.5) b--;
     return b;
 }
 
@@ -93,7 +92,7 @@ inline int fft_wide_bits(int logN) {
 //
 // Forward (coefficients in order -> values, bit-reversed): level l splits
 // X^m = c^2 into X^(m/2) = +-c, so its twiddle depends on the block only:
-// fwd[2^l + block].  Inverse (values, bit-reversed -> coefficients): decimation
+// fwd[2^l + block] (and, for the last four levels, a copy in the threads' order behind it).  Inverse (values, bit-reversed -> coefficients): decimation
 // in time with the twiddles exp(-2 pi i j / len), then the factor omega^-k,
 // omega = exp(i pi / N): omega^-tid goes in with the twiddles of the last four
 // stages, the rest of it is a constant of the register.
@@ -250,22 +249,33 @@ HD cpx fft_root(const root_t *p) {
 #endif
 }
 
-// four levels on the registers, top bit first; index: the thread's block at the first of them
-// (2^l + block); the runs of the next levels follow by doubling
-HD void fwd_phase4(cpx (&x)[16], const root_t *fwd, uint32_t index) {
+// Four levels on the registers, top bit first; root(i, g): the twiddle of group g (even) of level i.  The
+// group after it has the same one times the imaginary unit.
+template <class Root>
+HD void fwd_phase4(cpx (&x)[16], const Root &root) {
 #pragma unroll
     for (int i = 0; i < 4; i++) {
         const int bit = 3 - i;
 #pragma unroll
-        for (int g = 0; g < (1 << i); g++) {
-            const cpx w = fft_root(fwd + (index << i) + g);
+        for (int g = 0; g < (1 << i); g += 2) {
+            const cpx w = root(i, g);
 #pragma unroll
             for (int k = 0; k < (1 << bit); k++) {
                 const int r = (g << (4 - i)) + k;
                 fft_bf(x[r], x[r + (1 << bit)], w.re, w.im);
+                if (i > 0) fft_bf(x[r + (2 << bit)], x[r + (3 << bit)], -w.im, w.re);
             }
         }
     }
+}
+// index: the thread's block at the first level (2^l + block); the runs of the next levels follow by doubling
+HD void fwd_phase4_at(cpx (&x)[16], const root_t *fwd, uint32_t index) {
+    fwd_phase4(x, [&](int i, int g) { return fft_root(fwd + (index << i) + g); });
+}
+// the last phase of a block, whose eight twiddles per thread have a table in the threads' order: [8][NT] per block
+constexpr int FFT_LAST = 8 * FftLay::NT;
+HD void fwd_phase4_last(cpx (&x)[16], const root_t *last, uint32_t tid) {
+    fwd_phase4(x, [&](int i, int g) { return fft_root(last + ((i == 0 ? 0 : 1 << (i - 1)) + g / 2) * FftLay::NT + tid); });
 }
 
 // ---- the stages between blocks ---------------------------------------------------------
@@ -407,7 +417,7 @@ __device__ __forceinline__ void fft_forward(cpx (&x)[16], double2 *buf, const ro
     const uint32_t lane = tid & 31u, warp = tid >> 5;
     double2 *wb = buf + warp * 512;
     const uint32_t top = (1u << CL) + b;                   // level CL, block b
-    fwd_phase4(x, fwd, top);
+    fwd_phase4_at(x, fwd, top);
     buffer_wait<ALONE ? 0 : CL>();
 #pragma unroll
     for (int r = 0; r < 16; r++) buf[tid + L::NT * r] = make_double2(x[r].re, x[r].im);
@@ -417,7 +427,7 @@ __device__ __forceinline__ void fft_forward(cpx (&x)[16], double2 *buf, const ro
         const double2 v = wb[L::bc_word(lane, r)];
         x[r] = cpx{v.x, v.y};
     }
-    fwd_phase4(x, fwd, (top << 4) + 2 * warp + (lane >> 4));       // position bits 8 and up
+    fwd_phase4_at(x, fwd, (top << 4) + 2 * warp + (lane >> 4));       // position bits 8 and up
     __syncwarp();
 #pragma unroll
     for (int r = 0; r < 16; r++) wb[L::b_word(lane, r)] = make_double2(x[r].re, x[r].im);
@@ -428,7 +438,7 @@ __device__ __forceinline__ void fft_forward(cpx (&x)[16], double2 *buf, const ro
         x[r] = cpx{v.x, v.y};
     }
     buffer_free<ALONE ? 0 : CL>();
-    fwd_phase4(x, fwd, (top << 8) + tid);                          // position bits 4 and up
+    fwd_phase4_last(x, fwd + (L::NB << CL) + b * FFT_LAST, tid);  // position bits 4 and up
 }
 #endif
 

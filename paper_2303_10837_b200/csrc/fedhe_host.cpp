@@ -171,6 +171,15 @@ void host_fft_tables(uint32_t N, const std::vector<double> &roots, std::vector<d
             fwd[2 * (((size_t)1 << l) + b)] = roots[2 * (size_t)t];
             fwd[2 * (((size_t)1 << l) + b) + 1] = roots[2 * (size_t)t + 1];
         }
+    // the last four levels again, the even groups of thread t of block b: [block][8][NT]
+    for (uint32_t b = 0; b < (1u << CL); b++)
+        for (uint32_t i = 0; i < 4; i++)
+            for (uint32_t g = 0; g < (1u << i); g += 2)
+                for (uint32_t t = 0; t < NT; t++) {
+                    const size_t at = (((size_t)(((1u << CL) + b) << 8) + t) << i) + g;
+                    fwd.push_back(fwd[2 * at]);
+                    fwd.push_back(fwd[2 * at + 1]);
+                }
     inv.clear();
     auto push = [&](uint32_t t) {            // exp(-2 pi i t / 2N)
         inv.push_back(roots[2 * (size_t)t]);

@@ -39,7 +39,7 @@ void host_unit_roots(uint32_t N, std::vector<double> &roots);
 // entry [0] is unused.  Size n complex numbers.
 void host_slot_twiddles(uint32_t N, const std::vector<double> &roots, std::vector<double> &out);
 
-// Tables of the complex transforms (fedhe_fft.cuh): fwd [n] complex, inv in the order of FftTab, and
+// Tables of the complex transforms (fedhe_fft.cuh): fwd [n] complex and [n / 4096][8][NT] for the last phase, inv in the order of FftTab, and
 // the slot of the value that register r of thread t holds of block b: slot_of[(16 b + r) NT + t]
 void host_fft_tables(uint32_t N, const std::vector<double> &roots, std::vector<double> &fwd, std::vector<double> &inv,
                      std::vector<uint32_t> &slot_of);

@@ -34,15 +34,17 @@ __device__ __forceinline__ void dif_stage(cpx (&x)[L::E], uint32_t tid, const do
     constexpr int nst = (P < L::NPH - 1) ? L::LE : L::R;
     constexpr int bit = nst - 1 - I;
     constexpr uint32_t half = 1u << (L::LOGB - 1 - s);
+    // the twiddle depends on the register bits below the pair's: one load for all pairs above
 #pragma unroll
-    for (int r = 0; r < L::E; r++) {
-        if (r & (1 << bit)) continue;
-        const uint32_t j = L::template idx<P>(tid, r) & (half - 1u);
-        cpx w = load_ftw(ftw, half + j);
+    for (int low = 0; low < (1 << bit); low++) {
+        cpx w = load_ftw(ftw, half + (L::template idx<P>(tid, low) & (half - 1u)));
         w.im = -w.im;
-        const cpx U = x[r], V = x[r | (1 << bit)];
-        x[r] = cadd_rn(U, V);
-        x[r | (1 << bit)] = cmul_rn(csub_rn(U, V), w);
+#pragma unroll
+        for (int r = low; r < L::E; r += 2 << bit) {
+            const cpx U = x[r], V = x[r | (1 << bit)];
+            x[r] = cadd_rn(U, V);
+            x[r | (1 << bit)] = cmul_rn(csub_rn(U, V), w);
+        }
     }
 }
 

@@ -42,12 +42,13 @@ struct Block {
     static uint32_t wbc(uint32_t t, int r) { return (t >> 5) * 512 + L::bc_word(t & 31u, r); }
     static uint32_t wc(uint32_t t, int r) { return t + L::NT * (uint32_t)r; }
 
-    void forward(const root_t *fwd, uint32_t top) {
-        each([&](cpx (&x)[16], uint32_t) { fwd_phase4(x, fwd, top); });
+    void forward(const root_t *fwd, uint32_t n, uint32_t top) {
+        each([&](cpx (&x)[16], uint32_t) { fwd_phase4_at(x, fwd, top); });
         exchange(wc, wbc);
-        each([&](cpx (&x)[16], uint32_t t) { fwd_phase4(x, fwd, (top << 4) + 2 * (t >> 5) + ((t & 31u) >> 4)); });
+        each([&](cpx (&x)[16], uint32_t t) { fwd_phase4_at(x, fwd, (top << 4) + 2 * (t >> 5) + ((t & 31u) >> 4)); });
         exchange(wb, wa);
-        each([&](cpx (&x)[16], uint32_t t) { fwd_phase4(x, fwd, (top << 8) + t); });
+        const root_t *last = fwd + n + (top - n / L::NB) * FFT_LAST;
+        each([&](cpx (&x)[16], uint32_t t) { fwd_phase4_last(x, last, t); });
     }
     void inverse(const root_t *tab) {
         each([&](cpx (&x)[16], uint32_t) { inv_phase_a(x); });
@@ -101,7 +102,7 @@ static int check(uint32_t N) {
                     }
                 }
             });
-            B.forward(ft, R + blk);
+            B.forward(ft, n, R + blk);
         };
         std::vector<Block> prod(R);
         for (uint32_t blk = 0; blk < R; blk++) {
