@@ -181,10 +181,11 @@ int he_ctx_create(const he_params *p, he_ctx **out) {
         rc = upload(ctx, d.limb, HE_MAX_LIMBS, &d.limb_dev);
         if (rc != HE_OK) break;
         void *st = nullptr;
-        if (cudaMalloc(&st, sizeof(int)) != cudaSuccess) { rc = HE_ERR_ALLOC; break; }
+        if (cudaMalloc(&st, 4 * sizeof(int)) != cudaSuccess) { rc = HE_ERR_ALLOC; break; }
         ctx->owned.push_back(st);
-        if (cudaMemset(st, 0, sizeof(int)) != cudaSuccess) { rc = HE_ERR_CUDA; break; }
+        if (cudaMemset(st, 0, 4 * sizeof(int)) != cudaSuccess) { rc = HE_ERR_CUDA; break; }
         d.status = static_cast<int *>(st);
+        d.deal = static_cast<uint32_t *>(st) + 2;
         // pointer and weight tables of the aggregation calls
         rc = ensure(&ctx->tab, &ctx->tab_bytes,
                     HE_MAX_CLIENTS * (2 * sizeof(void *) + sizeof(double) + HE_MAX_LIMBS * sizeof(tw_t)));

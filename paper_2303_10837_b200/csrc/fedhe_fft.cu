@@ -47,7 +47,10 @@ struct FftJoin {
 };
 
 // the residue in [0, q) of |v| < q
-__device__ __forceinline__ uint64_t fft_canonical(int64_t v, uint64_t q) { return (uint64_t)(v + ((v >> 63) & (int64_t)q)); }
+__device__ __forceinline__ uint64_t fft_canonical(int64_t v, uint64_t q) {
+    if (v < 0) v += (int64_t)q;
+    return (uint64_t)v;
+}
 
 // geometry of a ring: a cluster of R thread blocks, one per block of the transform
 template <int CL_>
@@ -56,8 +59,7 @@ struct FftRing {
     static constexpr int CL = CL_, R = 1 << CL, NB = FftLay::NB, NT = FftLay::NT, n = R * NB, N = 2 * n;
     static constexpr int PER = 16 / R, COLS = NB / R;     // columns of the R x NB view that a thread, a thread block finishes
     // scratch in global memory (it lives in L2): a thread block's, then a cluster's
-    static constexpr size_t UHAT = (size_t)NB * 16, PARK = (size_t)NB * 16, OWN = UHAT + PARK, TERMS = (size_t)N * 8,
-                            UBITS = (size_t)NB * 4, SCRATCH = R * OWN + TERMS + UBITS;
+    static constexpr size_t PARK = (size_t)NB * 16, SCRATCH = R * PARK;
     static constexpr size_t SMEM = (size_t)NB * 16 + (size_t)Tab::WORDS * 16;
     static constexpr int BATCH = 8;                       // coefficients whose loads are in flight together
 };
@@ -184,198 +186,575 @@ __device__ __forceinline__ cpx encoder_stages(const float *slots, const double2 
     }
 }
 
-// The work of an encryption is dealt out in units (ciphertext, component, limb), weighed by their pieces:
-// first unit that begins at or after `pos` pieces of [ciphertext][component][limb][piece].
-__device__ __forceinline__ uint32_t fft_unit_at(const CtxDev &c, uint64_t pos) {
-    const uint32_t half = c.fft_pieces;
-    const uint32_t hc = (uint32_t)(pos / half);               // (ciphertext, component)
-    uint32_t rest = (uint32_t)(pos % half), j = 0;
+// ===========================================================================
+// encryption:  c0 = pk0 u + e0 + m,  c1 = pk1 u + e1   (mod every q_j), coefficient format
+// ===========================================================================
+
+// ---- tensor memory as a store of the threads' own words ----
+//
+// The kernel has no matrix products, so its 256 KB of tensor memory per SM would lie idle: each of the two
+// thread blocks takes half of it (256 columns), which is 128 words for every thread.  Words kept there
+// cost neither L2 nor shared-memory bandwidth.
+constexpr uint32_t TMEM_COLS = 256, TMEM_WORDS = 128;
+
+__device__ __forceinline__ uint32_t tmem_take(uint32_t *where) {       // by the whole block
+    if (threadIdx.x < 32) {
+        const uint32_t at = (uint32_t)__cvta_generic_to_shared(where);
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(at), "n"(TMEM_COLS) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    __syncthreads();
+    // a warp reaches the 32 lanes of its number modulo 4; the warps 0..3 and 4..7 share them by columns
+    const uint32_t warp = threadIdx.x >> 5;
+    return *where + ((warp & 3u) << 21) + (warp >> 2) * TMEM_WORDS;
+}
+__device__ __forceinline__ void tmem_give(uint32_t base) {             // by the whole block, after its last use
+    __syncthreads();
+    if (threadIdx.x < 32)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "n"(TMEM_COLS));
+}
+__device__ __forceinline__ void tmem_put8(uint32_t at, const uint32_t (&w)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(at), "r"(w[0]), "r"(w[1]),
+                 "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_wait_put() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// A load in two halves: the words count only after tmem_wait_get8().
+__device__ __forceinline__ void tmem_start_get8(uint32_t at, uint32_t (&w)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+                 : "r"(at)
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_wait_get8(uint32_t (&w)[8]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3]), "+r"(w[4]), "+r"(w[5]), "+r"(w[6]), "+r"(w[7])
+                 :
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_get32(uint32_t at, uint32_t (&w)[32]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\ttcgen05.wait::ld.sync.aligned;"
+                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]),
+                 "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]),
+                 "=r"(w[8]), "=r"(w[9]), "=r"(w[10]), "=r"(w[11]),
+                 "=r"(w[12]), "=r"(w[13]), "=r"(w[14]), "=r"(w[15]),
+                 "=r"(w[16]), "=r"(w[17]), "=r"(w[18]), "=r"(w[19]),
+                 "=r"(w[20]), "=r"(w[21]), "=r"(w[22]), "=r"(w[23]),
+                 "=r"(w[24]), "=r"(w[25]), "=r"(w[26]), "=r"(w[27]),
+                 "=r"(w[28]), "=r"(w[29]), "=r"(w[30]), "=r"(w[31])
+                 : "r"(at)
+                 : "memory");
+}
+__device__ __forceinline__ cpx tmem_cpx(const uint32_t *w) {
+    return cpx{__hiloint2double((int)w[1], (int)w[0]), __hiloint2double((int)w[3], (int)w[2])};
+}
+__device__ __forceinline__ void tmem_get8(uint32_t at, uint32_t (&w)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\ttcgen05.wait::ld.sync.aligned;"
+                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+                 : "r"(at)
+                 : "memory");
+}
+// ---- the key's table comes in through the transform buffer, ahead of its use ----
+constexpr uint32_t KEY_BYTES = FftLay::NB * 16;
+
+__device__ __forceinline__ void key_fetch(double2 *buf, const double2 *key, uint64_t *bar) {       // by one thread
+    const uint32_t at = (uint32_t)__cvta_generic_to_shared(buf), b = (uint32_t)__cvta_generic_to_shared(bar);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "n"(KEY_BYTES) : "memory");
+    asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(at), "l"(key),
+                 "n"(KEY_BYTES), "r"(b)
+                 : "memory");
+}
+// false if the copy has not come after many tries, which would be an error of the device
+__device__ __forceinline__ bool key_wait(uint64_t *bar, uint32_t parity) {
+    const uint32_t b = (uint32_t)__cvta_generic_to_shared(bar);
+    uint32_t done = 0;
+    for (int i = 0; i < 256 && !done; i++)
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 0x989680;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done)
+                     : "r"(b), "r"(parity)
+                     : "memory");
+    return done;
+}
+
+// two complex values
+__device__ __forceinline__ void tmem_put(uint32_t at, cpx a, cpx b) {
+    const uint32_t w[8] = {(uint32_t)__double2loint(a.re), (uint32_t)__double2hiint(a.re), (uint32_t)__double2loint(a.im),
+                           (uint32_t)__double2hiint(a.im), (uint32_t)__double2loint(b.re), (uint32_t)__double2hiint(b.re),
+                           (uint32_t)__double2loint(b.im), (uint32_t)__double2hiint(b.im)};
+    tmem_put8(at, w);
+}
+__device__ __forceinline__ void tmem_get(uint32_t at, cpx &a, cpx &b) {
+    uint32_t w[8];
+    tmem_get8(at, w);
+    a = cpx{__hiloint2double((int)w[1], (int)w[0]), __hiloint2double((int)w[3], (int)w[2])};
+    b = cpx{__hiloint2double((int)w[5], (int)w[4]), __hiloint2double((int)w[7], (int)w[6])};
+}
+
+// Scratch in global memory (it lives in L2) and tensor memory of an encryption.
+template <int CL_>
+struct EncRing {
+    using Tab = FftTab<CL_>;
+    static constexpr int CL = CL_, R = 1 << CL, NB = FftLay::NB, NT = FftLay::NT, n = R * NB, N = 2 * n;
+    static constexpr bool E_IN_SMEM = CL < 2;             // e1 (a byte each) fits beside the buffers of two blocks
+    // of the R blocks of a product the last stays in registers or shared memory; so many wait in tensor memory ...
+    static constexpr int WAIT_TMEM = R == 1 ? 0 : R == 2 ? 1 : 2, WAIT_L2 = R - 1 - WAIT_TMEM;
+    // ... and for R <= 2 the 32-bit products of low pieces do, in the words from PARK_AT; for R = 1 the transform of u, from 0
+    static constexpr bool PARK_TMEM = R <= 2;
+    static constexpr uint32_t PARK_AT = 64;
+    static constexpr int COLUMNS = R == 1 ? 4 : R == 8 ? 1 : 2, K = COLUMNS * R * 2;      // columns, values finished together
+    // a cluster's: the transform of u, the message and e0, e1, u in two bits each, flags
+    static constexpr size_t UHAT = (size_t)n * 16, TERMS = (size_t)N * 8, E1 = N, UBITS = (size_t)NB * 4,
+                            SHARED = UHAT + TERMS + E1 + UBITS + 128;
+    // a thread block's: what waits, joined low pieces
+    static constexpr size_t WAIT = (size_t)WAIT_L2 * NB * 16, PARK = (size_t)N * 8, OWN = WAIT + PARK;
+    static constexpr size_t SMEM = (size_t)NB * 16 + (size_t)Tab::WORDS * 16 + (E_IN_SMEM ? N : 0);
+};
+
+// first unit (component, limb) of a ciphertext that begins at or after `pos` pieces
+__device__ __forceinline__ uint32_t fft_unit_at(const CtxDev &c, uint32_t pos) {
+    uint32_t half = pos >= c.fft_pieces ? 1 : 0, rest = pos - half * c.fft_pieces, j = 0;
     while (rest) {
         const uint32_t p = c.limb[j].split.pieces;
         rest = rest > p ? rest - p : 0;
         j++;
     }
-    return hc * c.L + j;
+    return half * c.L + j;
 }
 
-// A cluster of R thread blocks owns a range of (ciphertext, component, limb) units.  Per ciphertext: u is
-// drawn and transformed once (its transform waits in the blocks' scratch, i.e. in L2, read back by the threads
-// that wrote it), the slots are encoded in the transform buffers; per component the error terms are drawn,
-// e0 added to the message; per unit and piece of the key: product with the key's table, inverse transform,
-// rounding, joining, error and message terms, canonical residue.  HBM sees the slots and the ciphertext
-// once.  A cluster whose range begins inside a ciphertext repeats what it needs of the ciphertext's preparation.
+// value i (column, row, real or imaginary part) of a thread's columns from r0: its coefficient less the thread's number
+template <class G>
+__device__ __forceinline__ uint32_t enc_coefficient(uint32_t r0, int i) {
+    const int o = i >> 1;
+    return (o % G::R) * G::NB + G::NT * (r0 + o / G::R) + (i & 1) * G::n;
+}
+
+// Columns r0 .. r0 + COLUMNS - 1 of a product after the stages between blocks.
+template <class G>
+__device__ __forceinline__ void enc_columns(cpx (&v)[G::COLUMNS][G::R], const cpx (&x)[16], const double2 *buf, const double2 *wait,
+                                            uint32_t tm, const root_t *tab, uint32_t r0, uint32_t tid) {
+    if constexpr (G::R == 1) {
+#pragma unroll
+        for (int i = 0; i < G::COLUMNS; i++) v[i][0] = x[r0 + i];
+    } else if constexpr (G::R == 2) {
+        tmem_get(tm + r0 * 4, v[0][0], v[1][0]);
+        v[0][1] = x[r0];
+        v[1][1] = x[r0 + 1];
+    } else {
+#pragma unroll
+        for (int i = 0; i < G::COLUMNS; i++) {
+#pragma unroll
+            for (int a = G::WAIT_TMEM; a + 1 < G::R; a++) {
+                const double2 w = __ldcg(wait + (a - G::WAIT_TMEM) * G::NB + (r0 + i) * G::NT + tid);
+                v[i][a] = cpx{w.x, w.y};
+            }
+            const double2 w = buf[(r0 + i) * G::NT + tid];
+            v[i][G::R - 1] = cpx{w.x, w.y};
+        }
+        if constexpr (G::COLUMNS == 2) {
+#pragma unroll
+            for (int a = 0; a < 2; a++) tmem_get(tm + a * 64 + r0 * 4, v[0][a], v[1][a]);
+        } else {
+            // pairs of blocks side by side: words [column][block]
+            tmem_get(tm + r0 * 8, v[0][0], v[0][1]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < G::COLUMNS; i++) fft_outer_inverse<G::CL>(v[i], tab, tid, r0 + i);
+}
+
+// One block of a product waits for the last one.
+template <class G>
+__device__ __forceinline__ void enc_wait(const cpx (&x)[16], double2 *wait, uint32_t tm, uint32_t b, uint32_t tid) {
+    if (b < (uint32_t)G::WAIT_TMEM) {
+        if constexpr (G::R == 8) {
+#pragma unroll
+            for (int r = 0; r < 16; r++) {
+                asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(tm + r * 8 + b * 4),
+                             "r"(__double2loint(x[r].re)), "r"(__double2hiint(x[r].re)), "r"(__double2loint(x[r].im)),
+                             "r"(__double2hiint(x[r].im))
+                             : "memory");
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < 16; r += 2) tmem_put(tm + b * 64 + r * 4, x[r], x[r + 1]);
+        }
+        tmem_wait_put();
+    } else {
+        double2 *dst = wait + (b - G::WAIT_TMEM) * G::NB + tid;
+#pragma unroll
+        for (int r = 0; r < 16; r++) __stcg(dst + r * G::NT, make_double2(x[r].re, x[r].im));
+    }
+}
+
+__device__ __forceinline__ int64_t fft_round(double z) { return fft_round_bits(z) - FFT_ROUND_BITS; }
+
+// A low piece's values are parked for the same thread, which will join the top one.
+template <class G>
+__device__ __forceinline__ void enc_park(const cpx (&v)[G::COLUMNS][G::R], unsigned char *park, uint32_t tm, const FftSplit &f,
+                                         uint32_t piece, uint32_t r0, uint32_t tid) {
+    const uint32_t i0 = r0 * G::R * 2;
+    if (f.narrow) {
+        uint32_t w[G::K];
+#pragma unroll
+        for (int i = 0; i < G::K; i++) {
+            const cpx &c = v[i / (2 * G::R)][(i / 2) % G::R];
+            w[i] = (uint32_t)fft_round_bits((i & 1) ? c.im : c.re);
+        }
+        if constexpr (G::PARK_TMEM) {
+            static_assert(G::K == 8, "eight words at a time");
+            tmem_put8(tm + G::PARK_AT + i0, w);
+        } else {
+#pragma unroll
+            for (int i = 0; i < G::K; i++) __stcg(reinterpret_cast<uint32_t *>(park) + (i0 + i) * G::NT + tid, w[i]);
+        }
+    } else {
+        long long *p = reinterpret_cast<long long *>(park) + i0 * G::NT + tid;
+#pragma unroll
+        for (int i = 0; i < G::K; i++) {
+            const cpx &c = v[i / (2 * G::R)][(i / 2) % G::R];
+            long long w = fft_round((i & 1) ? c.im : c.re) << f.shift[piece];
+            if (piece) w += __ldcg(p + i * G::NT);
+            __stcg(p + i * G::NT, w);
+        }
+    }
+}
+template <class G>
+__device__ __forceinline__ void enc_parked(int64_t (&val)[G::K], const unsigned char *park, uint32_t tm, const FftSplit &f,
+                                           uint32_t r0, uint32_t tid) {
+    const uint32_t i0 = r0 * G::R * 2;
+    if (f.narrow) {
+        if constexpr (G::PARK_TMEM) {
+            uint32_t w[8];
+            tmem_get8(tm + G::PARK_AT + i0, w);
+#pragma unroll
+            for (int i = 0; i < G::K; i++) val[i] += (int)w[i];
+        } else {
+#pragma unroll
+            for (int i = 0; i < G::K; i++) val[i] += __ldcg(reinterpret_cast<const int *>(park) + (i0 + i) * G::NT + tid);
+        }
+    } else if (f.pieces > 1) {
+#pragma unroll
+        for (int i = 0; i < G::K; i++) val[i] += __ldcg(reinterpret_cast<const long long *>(park) + (i0 + i) * G::NT + tid);
+    }
+}
+
+// A cluster of thread blocks encrypts ciphertexts one after the other: first it prepares one together -- u
+// is drawn and transformed, the slots are encoded, e0 and the message added up, e1 drawn, all in R blocks
+// of 2^12 points that its thread blocks share out -- and then each of them works off its own units
+// (component, limb) of it: per piece of the key and block of the transform the product with the key's table
+// and the inverse transform, per piece the stages between blocks and the rounding, then joining, error and
+// message terms, canonical residues.  HBM sees the slots and the ciphertext once, the cluster meets three
+// times per ciphertext.  (With the blocks of every product spread over the cluster it met twice per
+// piece, and waiting for one another took 6, 9 and 11 of 19, 22 and 26 thousand clocks per block and piece for R = 2, 4, 8.)
 //
-// Two thread blocks fit on an SM on every ring, so that one's memory phases meet the other's arithmetic, and
-// what all of them keep in scratch (54 MB) stays in L2.
+// Two thread blocks fit on an SM on every ring, so that one's memory phases meet the other's arithmetic.
+// The clusters fetch ciphertexts as they finish (with equal shares dealt out beforehand the slowest took 16 %
+// longer than the mean).  Of the `rem` ciphertexts after the last whole round each is cut in `parts`: clusters that
+// all prepare it and share its units.
 template <int CL>
 __global__ void __launch_bounds__(FftLay::NT, 2)
 encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const float *sel, unsigned char *work,
-                   uint32_t t0, uint64_t seed, uint32_t client, uint64_t *ct, uint32_t T) {
-    using G = FftRing<CL>;
+                   uint32_t t0, uint64_t seed, uint32_t client, uint64_t *ct, uint32_t T, uint32_t S, uint32_t most_parts) {
+    using G = EncRing<CL>;
     constexpr uint32_t N = G::N, n = G::n, NB = G::NB, NT = G::NT, R = G::R;
     extern __shared__ __align__(128) unsigned char smem[];
     double2 *buf = reinterpret_cast<double2 *>(smem);
     root_t *tab = reinterpret_cast<root_t *>(smem + (size_t)NB * 16);
+    int8_t *e1_smem = reinterpret_cast<int8_t *>(tab + G::Tab::WORDS);
     __shared__ GaussTables gt;
-    __shared__ __align__(16) int8_t samples[2 * G::NB];   // e1 of the coefficients this block finishes
-    const uint32_t rank = blockIdx.x % R, cid = blockIdx.x / R, nc = gridDim.x / R;
+    __shared__ uint32_t tmem_base;
+    __shared__ __align__(8) uint64_t key_bar;
+    const uint32_t rank = blockIdx.x % S, cid = blockIdx.x / S, nc = gridDim.x / S;
     gauss_tables_init(gt, threadIdx.x, NT);
     for (uint32_t i = threadIdx.x; i < (uint32_t)G::Tab::WORDS; i += NT) tab[i] = c.fft_inv[i];
-    buffer_free<CL>();
-    unsigned char *shared_work = work + (size_t)cid * G::SCRATCH, *own = shared_work + rank * G::OWN;
-    double2 *uhat = reinterpret_cast<double2 *>(own);                           // [16][NT]
-    unsigned char *park = own + G::UHAT;
-    // message and e0 by residue of the coefficient's number: [2 halves][R][NB], coefficient R kk + b at kk of row b
-    long long *terms = reinterpret_cast<long long *>(shared_work + R * G::OWN);
-    // u, two bits (value + 1) per row of the column: [2 halves][NB]
-    uint16_t *ubits = reinterpret_cast<uint16_t *>(shared_work + R * G::OWN + G::TERMS);
+    if (threadIdx.x == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(&key_bar)) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    uint32_t key_parity = 0;
+    const uint32_t tm = tmem_take(&tmem_base);            // and the tables are there
+    unsigned char *common = work + (size_t)cid * (G::SHARED + S * G::OWN), *own = common + G::SHARED + rank * G::OWN;
+    double2 *uhat = reinterpret_cast<double2 *>(common);                        // [R][16][NT]
+    // message and e0 by residue of the coefficient's number, as the encoder's blocks leave them: [2 halves][R][NB],
+    // coefficient R kk + b at kk of row b
+    long long *terms = reinterpret_cast<long long *>(common + G::UHAT);
     auto term_of = [&](uint32_t coef) {
         return terms + ((coef & (n - 1)) >> CL) + ((coef & (R - 1)) + (coef >= n ? R : 0)) * NB;
     };
+    int8_t *e1 = reinterpret_cast<int8_t *>(terms + N);
+    uint16_t *ubits = reinterpret_cast<uint16_t *>(e1 + N);                     // value + 1 per row of the column: [2 halves][NB]
+    uint32_t *flags = reinterpret_cast<uint32_t *>(ubits + 2 * NB);
+    double2 *wait = reinterpret_cast<double2 *>(own);
+    unsigned char *park = own + G::WAIT;
+    auto meet = [&]() {                                   // everything the cluster wrote is visible to all of it
+        if (S > 1) {
+            asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+            asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        } else {
+            __syncthreads();
+        }
+    };
 
-    const uint32_t per_ct = 2 * c.L;
-    const uint64_t total = (uint64_t)T * 2 * c.fft_pieces;
-    const uint32_t u_end = fft_unit_at(c, total * (cid + 1) / nc);
-    uint32_t have_ct = 0xffffffffu, have_e = 0xffffffffu;
-    bool big = false;                                     // a term of this component needs reducing first
+    const uint32_t whole = T / nc * nc, rem = T - whole;
+    const uint32_t parts = rem ? (nc / rem < most_parts ? nc / rem : most_parts) : 1;
+    const uint32_t items = whole + rem * parts;           // at least as many as clusters
+    const uint32_t pieces = 2 * c.fft_pieces;
+    const bool leader = rank == 0 && threadIdx.x == 0;
+    uint32_t next_item = cid;
 #pragma unroll 1
-    for (uint32_t unit = fft_unit_at(c, total * cid / nc); unit < u_end; unit++) {
-        const uint32_t tl = unit / per_ct, comp = (unit / c.L) & 1u, j = unit % c.L, t = t0 + tl;
-        if (tl != have_ct) {
-            have_ct = tl;
-            // four columns of one half at a time
+    for (uint32_t it = 0; next_item < items; it++) {
+        const uint32_t item = next_item;
+        // words of two turns: a word is written again after the others have read it and met
+        if (leader) {
+            __stcg(flags + (it & 1u), 0u);
+            __stcg(flags + 2 + (it & 1u), nc + atomicAdd(c.deal, 1u));
+        }
+        uint32_t tl = item, part = 0, of = 1;
+        if (item >= whole) {
+            tl = whole + (item - whole) / parts;
+            part = (item - whole) % parts;
+            of = parts;
+        }
+        const uint32_t first = fft_unit_at(c, pieces * part / of), last = fft_unit_at(c, pieces * (part + 1) / of);
+        const uint32_t unit_end = fft_unit_at(c, pieces * (part * S + rank + 1) / (of * S));
+        uint32_t unit = fft_unit_at(c, pieces * (part * S + rank) / (of * S));
+        const bool c0_too = first < c.L, c1_too = last > c.L;
+        const uint32_t t = t0 + tl;
+
+        // ---- preparation: u, four columns of one half at a time ----
 #pragma unroll 1
-            for (uint32_t w = rank * (2 * NB / 4 / R) + threadIdx.x; w < (rank + 1) * (2 * NB / 4 / R); w += NT) {
-                uint32_t f[4] = {0, 0, 0, 0};
+        for (uint32_t w = rank * NT + threadIdx.x; w < 2 * NB / 4; w += S * NT) {
+            uint32_t f[4] = {0, 0, 0, 0};
 #pragma unroll
-                for (uint32_t a = 0; a < R; a++) {
-                    const uint32_t b = (w / (NB / 4)) * (n / 4) + a * (NB / 4) + w % (NB / 4);
-                    const u32x4 v = stream_block(seed, b, t, client, TAG_ENC_U);
-                    f[0] |= (uint32_t)(ternary_from_word(v.x) + 1) << (2 * a);
-                    f[1] |= (uint32_t)(ternary_from_word(v.y) + 1) << (2 * a);
-                    f[2] |= (uint32_t)(ternary_from_word(v.z) + 1) << (2 * a);
-                    f[3] |= (uint32_t)(ternary_from_word(v.w) + 1) << (2 * a);
-                }
-                __stcg(reinterpret_cast<uint2 *>(ubits) + w, make_uint2(f[0] | f[1] << 16, f[2] | f[3] << 16));
+            for (uint32_t a = 0; a < R; a++) {
+                const uint32_t b = (w / (NB / 4)) * (n / 4) + a * (NB / 4) + w % (NB / 4);
+                const u32x4 v = stream_block(seed, b, t, client, TAG_ENC_U);
+                f[0] |= (uint32_t)(ternary_from_word(v.x) + 1) << (2 * a);
+                f[1] |= (uint32_t)(ternary_from_word(v.y) + 1) << (2 * a);
+                f[2] |= (uint32_t)(ternary_from_word(v.z) + 1) << (2 * a);
+                f[3] |= (uint32_t)(ternary_from_word(v.w) + 1) << (2 * a);
             }
-            cluster_meet<CL>();                           // u is there, and nobody reads the last ciphertext's terms any more
-            cpx x[16];
-            {
-                const OuterPath<CL> outer(c.fft_fwd, rank);
-                const uint16_t *p = ubits + fresh_tid();
-                auto ternary = [](uint32_t f) {           // 0, 1, 2 -> -1.0, 0.0, 1.0
-                    return __hiloint2double(f == 1 ? 0 : 0x3ff00000 | (int)((f == 0 ? 1u : 0u) << 31), 0);
-                };
+            __stcg(reinterpret_cast<uint2 *>(ubits) + w, make_uint2(f[0] | f[1] << 16, f[2] | f[3] << 16));
+        }
+        meet();                                           // u is there, and nobody works on the last ciphertext any more
+        next_item = __ldcg(flags + 2 + (it & 1u));
+        if (first == last) continue;                      // more parts than units
+        // the transform of u and the encoder's network: 2 R blocks of 2^12 points
+#pragma unroll 1
+        for (uint32_t item = rank; item < 2 * R; item += S) {
+            const uint32_t b = item & (R - 1);
+            if (item < R) {
+                cpx x[16];
+                {
+                    const OuterPath<CL> outer(c.fft_fwd, b);
+                    const uint16_t *p = ubits + fresh_tid();
+                    auto ternary = [](uint32_t f) {       // 0, 1, 2 -> -1.0, 0.0, 1.0
+                        return __hiloint2double(f == 1 ? 0 : 0x3ff00000 | (int)((f == 0 ? 1u : 0u) << 31), 0);
+                    };
 #pragma unroll
-                for (int r = 0; r < 16; r++) {
-                    const uint32_t re = __ldcg(p + NT * r), im = __ldcg(p + NB + NT * r);
-                    cpx z[R];
+                    for (int r = 0; r < 16; r++) {
+                        const uint32_t re = __ldcg(p + NT * r), im = __ldcg(p + NB + NT * r);
+                        cpx z[R];
 #pragma unroll
-                    for (uint32_t a = 0; a < R; a++) z[a] = cpx{ternary((re >> (2 * a)) & 3u), ternary((im >> (2 * a)) & 3u)};
-                    x[r] = outer.apply(z);
+                        for (uint32_t a = 0; a < R; a++) z[a] = cpx{ternary((re >> (2 * a)) & 3u), ternary((im >> (2 * a)) & 3u)};
+                        x[r] = outer.apply(z);
+                    }
                 }
-            }
-            fft_forward<CL>(x, buf, c.fft_fwd, rank, fresh_tid());
-            {
-                double2 *dst = uhat + fresh_tid();
+                fft_forward<CL, true>(x, buf, c.fft_fwd, b, fresh_tid());
+                double2 *dst = uhat + b * NB + fresh_tid();
 #pragma unroll
                 for (int r = 0; r < 16; r++) __stcg(dst + r * NT, make_double2(x[r].re, x[r].im));
-            }
-            if (comp == 0) {
+            } else if (c0_too) {
                 const float *slots = sel + (size_t)tl * n;
-                long long *row = terms + (CL ? bitrev(rank, CL ? CL : 1) : 0u) * NB;
-                buffer_wait<CL>();
+                long long *row = terms + (CL ? bitrev(b, CL ? CL : 1) : 0u) * NB;
+                __syncthreads();                          // the buffer's last readers are done
                 if (encode_block_in_place<Lay<FftLay::LB, 4>>(
-                        c, [&](uint32_t i) { return encoder_stages<CL>(slots, c.ftw, n, rank, i); },
+                        c, [&](uint32_t i) { return encoder_stages<CL>(slots, c.ftw, n, b, i); },
                         reinterpret_cast<uint64_t *>(buf), CL,
                         [&](uint32_t kk, int64_t re, int64_t im) {
                             __stcg(row + kk, (long long)re);
                             __stcg(row + R * NB + kk, (long long)im);
                         }))
                     atomicOr(c.status, 1);
-                buffer_free<CL>();
-                if constexpr (CL > 0) cluster_meet<CL>(); // the message of all blocks is complete
             }
         }
-        if (2 * tl + comp != have_e) {
-            have_e = 2 * tl + comp;
-            __syncthreads();                              // nobody still reads the samples
+        meet();
+        // error terms, a pair of neighbours at a time
+#pragma unroll 1
+        for (int comp = c0_too ? 0 : 1; comp < (c1_too ? 2 : 1); comp++) {
             int far = 0;
-            // pairs of neighbours among the coefficients this block finishes: [2 R rows][COLS]
-            for (uint32_t pp = threadIdx.x; pp < NB; pp += NT) {
-                const uint32_t row = pp / (G::COLS / 2), lc = 2 * (pp % (G::COLS / 2));
-                const uint32_t coef = row * NB + rank * G::COLS + lc;
-                const u32x4 w = stream_block(seed, coef >> 1, t, client, comp == 0 ? TAG_ENC_E0 : TAG_ENC_E1);
-                const int ex = gauss_from_u64(gt, (uint64_t)w.x | ((uint64_t)w.y << 32));
-                const int ey = gauss_from_u64(gt, (uint64_t)w.z | ((uint64_t)w.w << 32));
+#pragma unroll 1
+            for (uint32_t b = rank * NT + threadIdx.x; b < N / 2; b += S * NT) {
                 if (comp == 0) {
-                    long long *px = term_of(coef), *py = term_of(coef + 1);
-                    const long long mx = __ldcg(px) + ex, my = __ldcg(py) + ey;
-                    far |= (mx < 0 ? -mx : mx) >= c.term_limit || (my < 0 ? -my : my) >= c.term_limit;
-                    __stcg(px, mx);
-                    __stcg(py, my);
+                    long long *p = term_of(2 * b);
+                    longlong2 m;
+                    if constexpr (CL == 0) m = __ldcg(reinterpret_cast<const longlong2 *>(p));
+                    else m = make_longlong2(__ldcg(p), __ldcg(p + NB));
+                    const int2 e = gauss_pair(gt, seed, b, t, client, TAG_ENC_E0);
+                    m.x += e.x;
+                    m.y += e.y;
+                    far |= (m.x < 0 ? -m.x : m.x) >= c.term_limit || (m.y < 0 ? -m.y : m.y) >= c.term_limit;
+                    if constexpr (CL == 0) {
+                        __stcg(reinterpret_cast<longlong2 *>(p), m);
+                    } else {
+                        __stcg(p, m.x);
+                        __stcg(p + NB, m.y);
+                    }
                 } else {
-                    *reinterpret_cast<char2 *>(samples + row * G::COLS + lc) = make_char2((signed char)ex, (signed char)ey);
+                    const int2 e = gauss_pair(gt, seed, b, t, client, TAG_ENC_E1);
+                    __stcg(reinterpret_cast<char2 *>(e1) + b, make_char2((signed char)e.x, (signed char)e.y));
                 }
             }
-            big = __syncthreads_or(far);                  // and the samples and terms are complete
+            if (far) atomicOr(flags + (it & 1u), 1u);
         }
-        const FftSplit &f = c.limb[j].split;
-        const uint64_t q = c.limb[j].q;
+        meet();
+        if (unit == unit_end) continue;
+        const bool big = __ldcg(flags + (it & 1u)) != 0;  // a term of c0 needs reducing first
+        if constexpr (G::E_IN_SMEM) {
+            if (c1_too) {
+                for (uint32_t i = threadIdx.x; i < N / 16; i += NT)
+                    reinterpret_cast<uint4 *>(e1_smem)[i] = __ldcg(reinterpret_cast<const uint4 *>(e1) + i);
+                __syncthreads();
+            }
+        }
+        const int8_t *e1_at = G::E_IN_SMEM ? e1_smem : e1;
+        if constexpr (R == 1) {
+            const double2 *uh = uhat + fresh_tid();
+#pragma unroll
+            for (int r = 0; r < 16; r += 2) {
+                const double2 a = __ldcg(uh + r * NT), b = __ldcg(uh + (r + 1) * NT);
+                tmem_put(tm + r * 4, cpx{a.x, a.y}, cpx{b.x, b.y});
+            }
+            tmem_wait_put();
+        }
+
+        // ---- this block's units ----
+        auto key_of = [&](uint32_t u, uint32_t pb) {
+            const uint32_t comp = u >= c.L ? 1 : 0;
+            const LimbDev &lb = c.limb[u - comp * c.L];
+            return k.fft_pk + lb.fft_key + ((size_t)comp * lb.split.pieces * R + pb) * NB;
+        };
+        if constexpr (!(G::E_IN_SMEM)) __syncthreads();   // the buffer's last readers are done
+        if (threadIdx.x == 0) key_fetch(buf, key_of(unit, 0), &key_bar);
 #pragma unroll 1
-        for (uint32_t p = 0; p < f.pieces; p++) {
-            cpx x[16];
-            {
+        for (; unit < unit_end; unit++) {
+            const uint32_t comp = unit >= c.L ? 1 : 0, j = unit - comp * c.L;
+            const FftSplit &f = c.limb[j].split;
+            const uint64_t q = c.limb[j].q;
+#pragma unroll 1
+            for (uint32_t pb = 0; pb < f.pieces * R; pb++) {
+                const uint32_t p = pb >> CL, b = pb & (R - 1);
+                cpx x[16];
+                {
+                    const uint32_t tid = fresh_tid();
+                    const double2 *key = buf + tid;
+                    if constexpr (R == 1) {
+                        if (!key_wait(&key_bar, key_parity)) atomicOr(c.status, 4);
+#pragma unroll
+                        for (int h = 0; h < 2; h++) {
+                            uint32_t w[32];
+                            tmem_get32(tm + h * 32, w);
+#pragma unroll
+                            for (int r = 0; r < 8; r++)
+                                x[8 * h + r] = cpx_mul(tmem_cpx(w + 4 * r), key[(8 * h + r) * NT].x, key[(8 * h + r) * NT].y);
+                        }
+                    } else {
+                        const double2 *uh = uhat + b * NB + tid;
+#pragma unroll
+                        for (int r = 0; r < 16; r++) {
+                            const double2 w = __ldcg(uh + r * NT);
+                            x[r] = cpx{w.x, w.y};
+                        }
+                        if (!key_wait(&key_bar, key_parity)) atomicOr(c.status, 4);
+#pragma unroll
+                        for (int r = 0; r < 16; r++) x[r] = cpx_mul(x[r], key[r * NT].x, key[r * NT].y);
+                    }
+                    key_parity ^= 1u;
+                }
+                // the next key may come as soon as the buffer is read; where a column loop needs the buffer, after it
+                const bool more = pb + 1 < f.pieces * R || unit + 1 < unit_end;
+                auto fetch_next = [&]() {
+                    __syncthreads();
+                    if (more && threadIdx.x == 0)
+                        key_fetch(buf, pb + 1 < f.pieces * R ? key_of(unit, pb + 1) : key_of(unit + 1, 0), &key_bar);
+                };
+                fft_inverse<0>(x, buf, tab, fresh_tid(), [&] {
+                    if (R <= 2 || b + 1 < R) fetch_next();
+                });
                 const uint32_t tid = fresh_tid();
-                const double2 *key = k.fft_pk + c.limb[j].fft_key + ((size_t)(comp * f.pieces + p) * R + rank) * NB + tid;
-                const double2 *uh = uhat + tid;
-#pragma unroll
-                for (int r = 0; r < 16; r++) x[r] = fft_mul(__ldcg(uh + r * NT), load_passing(key + r * NT));
-            }
-            fft_inverse<CL>(x, buf, tab, fresh_tid());
-            const uint32_t tid = fresh_tid();
-            fft_gather<G>(x, buf, tab, rank, tid);
-            if (p + 1 < f.pieces) {
-                fft_park<G>(x, park, f, p, tid);
-                continue;
-            }
-            uint64_t *out = ct + (((size_t)tl * 2 + comp) * c.L + j) * N + tid;
-            const FftJoin join(f, q);
-#pragma unroll
-            for (int i0 = 0; i0 < 32; i0 += G::BATCH) {
-                int64_t val[G::BATCH];
-                if (comp == 1) {
-#pragma unroll
-                    for (int i = 0; i < G::BATCH; i++) val[i] = samples[fft_own<G>(i0 + i) + tid];
-                } else if (big) {
-#pragma unroll
-                    for (int i = 0; i < G::BATCH; i++) val[i] = 0;
-                } else {
-#pragma unroll
-                    for (int i = 0; i < G::BATCH; i++) val[i] = __ldcg(term_of(fft_coefficient<G>(i0 + i, rank) + tid));
+                if (b + 1 < R) {
+                    enc_wait<G>(x, wait, tm, b, tid);
+                    continue;
                 }
-                fft_parked<G>(val, park, f, i0, tid);
-                // streaming stores: the finished ciphertext should not push tables and scratch out of L2
+                if constexpr (R > 2) {
+                    // the thread's own words: the columns are finished in a loop, which registers do not allow
 #pragma unroll
-                for (int i = 0; i < G::BATCH; i++) {
-                    const cpx &w = x[(i0 + i) >> 1];
-                    val[i] = join(val[i], (i & 1) ? w.im : w.re);
-                    __stcs(reinterpret_cast<unsigned long long *>(out + fft_coefficient<G>(i0 + i, rank)),
-                           (unsigned long long)fft_canonical(val[i], q));
+                    for (int r = 0; r < 16; r++) buf[r * NT + tid] = make_double2(x[r].re, x[r].im);
                 }
-            }
-            if (big && comp == 0) {
-                // terms beyond a quarter of the smallest prime: encoded updates are far below, so this is rare
-                const uint64_t mu = c.limb[j].mu;
+                constexpr int K = G::K;
+                if (p + 1 < f.pieces) {
+#pragma unroll(R <= 2 ? 16 : 1)
+                    for (uint32_t r0 = 0; r0 < 16; r0 += G::COLUMNS) {
+                        cpx v[G::COLUMNS][R];
+                        enc_columns<G>(v, x, buf, wait, tm, tab, r0, tid);
+                        enc_park<G>(v, park, tm, f, p, r0, tid);
+                    }
+                    if constexpr (G::PARK_TMEM) tmem_wait_put();
+                    if constexpr (R > 2) fetch_next();
+                    continue;
+                }
+                uint64_t *out = ct + (((size_t)tl * 2 + comp) * c.L + j) * N + tid;
+                const FftJoin join(f, q);
+                // the offsets of a thread's coefficients are multiples of R, so they split off the number of the first
+                const long long *my_terms = term_of(tid);
+                auto terms_of = [&](int64_t (&val)[K], uint32_t r0) {
+                    if (comp == 1) {
+#pragma unroll
+                        for (int i = 0; i < K; i++) val[i] = e1_at[enc_coefficient<G>(r0, i) + tid];
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < K; i++) {
+                            const uint32_t at = enc_coefficient<G>(r0, i);
+                            val[i] = __ldcg(my_terms + ((at & (n - 1)) >> CL) + (at >= n ? R * NB : 0));
+                        }
+                    }
+                };
+                int64_t next[K];
+                terms_of(next, 0);
+#pragma unroll(R <= 2 ? 16 : 1)
+                for (uint32_t r0 = 0; r0 < 16; r0 += G::COLUMNS) {
+                    int64_t val[K];
+#pragma unroll
+                    for (int i = 0; i < K; i++) val[i] = big && comp == 0 ? 0 : next[i];
+                    if (r0 + G::COLUMNS < 16) terms_of(next, r0 + G::COLUMNS);
+                    enc_parked<G>(val, park, tm, f, r0, tid);
+                    cpx v[G::COLUMNS][R];
+                    enc_columns<G>(v, x, buf, wait, tm, tab, r0, tid);
+                    // streaming stores: the finished ciphertext should not push tables and scratch out of L2
+#pragma unroll
+                    for (int i = 0; i < K; i++) {
+                        const cpx &w = v[i / (2 * (int)R)][(i / 2) % (int)R];
+                        __stcs(reinterpret_cast<unsigned long long *>(out + enc_coefficient<G>(r0, i)),
+                               (unsigned long long)fft_canonical(join(val[i], (i & 1) ? w.im : w.re), q));
+                    }
+                }
+                if constexpr (R > 2) fetch_next();
+                if (big && comp == 0) {
+                    // terms beyond a quarter of the smallest prime: encoded updates are far below, so this is rare
+                    const uint64_t mu = c.limb[j].mu;
 #pragma unroll 1
-                for (int i = 0; i < 32; i++) {
-                    const uint32_t at = fft_coefficient<G>(i, rank);
-                    out[at] = addmod(out[at], signed_residue(__ldcg(term_of(at + tid)), q, mu), q);
+                    for (uint32_t at = 0; at < N; at += NT)
+                        out[at] = addmod(out[at], signed_residue(__ldcg(term_of(at + tid)), q, mu), q);
                 }
             }
         }
     }
-    buffer_wait<CL>();                                    // the other blocks have read this one's buffer
+    if (leader && atomicAdd(c.deal + 1, 1u) + 1 == nc) {  // the last cluster leaves the words as it found them
+        c.deal[0] = 0;
+        c.deal[1] = 0;
+    }
+    tmem_give(tmem_base);
 }
 
 // ===========================================================================
@@ -400,7 +779,7 @@ decrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const uint
     const uint32_t rank = blockIdx.x % R, cid = blockIdx.x / R, nc = gridDim.x / R;
     for (uint32_t i = threadIdx.x; i < (uint32_t)G::Tab::WORDS; i += NT) tab[i] = c.fft_inv[i];
     buffer_free<CL>();
-    unsigned char *park = work + (size_t)cid * G::SCRATCH + rank * G::OWN + G::UHAT;
+    unsigned char *park = work + (size_t)cid * G::SCRATCH + rank * G::PARK;
     const FftSplit &f = c.dec_split;
     const uint64_t q = c.limb[0].q;
     const int64_t half_q = (int64_t)(q / 2);
@@ -516,22 +895,68 @@ static cudaError_t fft_grid(K kern, int n_sm, size_t want, cudaStream_t s, cudaL
     return cudaSuccess;
 }
 
-template <int CL>
-static size_t ring_scratch(int n_sm, size_t units) {
-    const size_t fit = 2 * (size_t)n_sm / FftRing<CL>::R;
-    return (units < fit ? units : fit) * FftRing<CL>::SCRATCH;
+// Asked how many thread blocks fit on an SM, the runtime answers 1 for any kernel that allocates tensor memory;
+// two that take half of it each do run side by side.  This kernel has the same shape without it.
+__global__ void __launch_bounds__(FftLay::NT, 2) enc_shape_kernel() {}
+
+// Thread blocks that work on one ciphertext together: as many as it has blocks of 2^12 points (less if its units
+// could not be shared out evenly), and more while the ciphertexts are too few to fill the device.
+static uint32_t enc_cluster(const CtxDev &c, int n_sm, size_t T) {
+    uint32_t S = 1;
+    while (S < 8 && S < (1u << (c.logN - 13)) && (2 * c.L) % (2 * S) == 0) S *= 2;
+    while (S < 8 && S < 2 * c.L && T * 2 * S <= 2 * (size_t)n_sm) S *= 2;
+    return S;
 }
-size_t fft_work_bytes(const CtxDev &c, int n_sm, size_t T) { FEDHE_FOR_RING(c, ring_scratch, n_sm, T * 2 * c.L) }
+// ... and the most clusters that a ciphertext is worth
+static uint32_t enc_parts(const CtxDev &c, uint32_t S) { return (2 * c.L + S - 1) / S; }
+
+template <int CL>
+static size_t ring_scratch(const CtxDev &c, int n_sm, size_t T) {
+    using G = EncRing<CL>;
+    size_t most = 0;                                   // of any number of ciphertexts up to T
+    for (uint32_t S = enc_cluster(c, n_sm, T); S <= 8; S *= 2) {
+        const size_t fit = 2 * (size_t)n_sm / S, want = T * enc_parts(c, S), bytes = (want < fit ? want : fit) * (G::SHARED + S * G::OWN);
+        if (bytes > most) most = bytes;
+    }
+    const size_t fit = 2 * (size_t)n_sm / FftRing<CL>::R, dec = (T < fit ? T : fit) * FftRing<CL>::SCRATCH;
+    return most > dec ? most : dec;
+}
+size_t fft_work_bytes(const CtxDev &c, int n_sm, size_t T) { FEDHE_FOR_RING(c, ring_scratch, c, n_sm, T) }
 
 template <int CL>
 static cudaError_t launch_encrypt_ring(const CtxDev &c, const KeysDev &k, const float *sel, void *work, int n_sm, uint32_t t0,
                                        size_t T, uint64_t seed, uint32_t client, uint64_t *ct, cudaStream_t s) {
+    using G = EncRing<CL>;
     auto kern = encrypt_fft_kernel<CL>;
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr;
     cudaError_t e;
-    if ((e = fft_grid<FftRing<CL>>(kern, n_sm, T * 2 * c.L, s, cfg, &attr))) return e;
-    if ((e = cudaLaunchKernelEx(&cfg, kern, c, k, sel, static_cast<unsigned char *>(work), t0, seed, client, ct, (uint32_t)T)))
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM))) return e;
+    const uint32_t S = enc_cluster(c, n_sm, T), parts = enc_parts(c, S);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr;
+    cfg.stream = s;
+    cfg.blockDim = dim3(G::NT, 1, 1);
+    cfg.dynamicSmemBytes = G::SMEM;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = S;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    size_t fit = 2 * (size_t)n_sm / S;
+    if (S > 1 && T * parts > fit / 2) {
+        cfg.gridDim = dim3(S, 1, 1);
+        int clusters = 0;
+        cfg.dynamicSmemBytes = G::SMEM + 4096;       // and the static part
+        if ((e = cudaFuncSetAttribute(enc_shape_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes))) return e;
+        if ((e = cudaOccupancyMaxActiveClusters(&clusters, enc_shape_kernel, &cfg))) return e;
+        cfg.dynamicSmemBytes = G::SMEM;
+        if (clusters < 1) return cudaErrorLaunchOutOfResources;
+        if ((size_t)clusters < fit) fit = (size_t)clusters;
+    }
+    // whole rounds of all clusters, or so many clusters to every ciphertext
+    size_t nc = T >= fit ? fit : T * (fit / T < parts ? fit / T : parts);
+    cfg.gridDim = dim3((unsigned)(nc * S), 1, 1);
+    if ((e = cudaLaunchKernelEx(&cfg, kern, c, k, sel, static_cast<unsigned char *>(work), t0, seed, client, ct, (uint32_t)T, S, parts)))
         return e;
     return FEDHE_LAUNCHED();
 }

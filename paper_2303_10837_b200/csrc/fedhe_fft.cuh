@@ -381,9 +381,10 @@ __device__ __forceinline__ void cluster_meet() {
     }
 }
 // x in layout A -> layout C (unscaled, with omega^-tid, without the registers' constants).  The
-// buffer is not given free: its words in layout C are the thread's own.
-template <int CL>
-__device__ __forceinline__ void fft_inverse(cpx (&x)[16], double2 *buf, const root_t *tab, uint32_t tid) {
+// buffer is not given free: its words in layout C are the thread's own.  has_read() runs when the thread has
+// taken its values from there.
+template <int CL, class Read>
+__device__ __forceinline__ void fft_inverse(cpx (&x)[16], double2 *buf, const root_t *tab, uint32_t tid, const Read &has_read) {
     using L = FftLay;
     const uint32_t lane = tid & 31u;
     double2 *wb = buf + (tid >> 5) * 512;
@@ -407,7 +408,13 @@ __device__ __forceinline__ void fft_inverse(cpx (&x)[16], double2 *buf, const ro
         const double2 v = buf[tid + L::NT * r];
         x[r] = cpx{v.x, v.y};
     }
+    has_read();
     inv_phase_c(x, tab + FftTab<0>::C, tid);
+}
+
+template <int CL>
+__device__ __forceinline__ void fft_inverse(cpx (&x)[16], double2 *buf, const root_t *tab, uint32_t tid) {
+    fft_inverse<CL>(x, buf, tab, tid, [] {});
 }
 
 // x in layout C -> layout A; block b of 2^CL blocks.  ALONE: outside a cluster.

@@ -82,6 +82,7 @@ struct CtxDev {
     FftSplit dec_split;                // of c1 on limb 0, for any c1
     uint32_t fft_pieces;               // of all limbs of a public-key half
     int64_t term_limit;                // a quarter of the smallest prime
+    uint32_t *deal;      // encryption hands out ciphertexts here: next one, thread blocks (clusters) that are done; 0 between calls
     int *status;         // sticky anomaly word
 };
 

@@ -18,6 +18,23 @@ static inline unsigned blocks_for(size_t count, unsigned per_block) {
     return (unsigned)((count + per_block - 1) / per_block);
 }
 
+// Words 1 and 3 of a stream block, the high halves of its two 64-bit values.  The last round makes them from two
+// low products, and the round before it only has to make the factors of these.
+__device__ __forceinline__ uint2 stream_block_high(uint64_t seed, uint32_t block, uint32_t t, uint32_t client, uint32_t tag_limb) {
+    uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+    u32x4 c = {block, t, client, tag_limb};
+#pragma unroll
+    for (int r = 0; r < 9; r++) {
+        uint32_t h0, l0, h1, l1;
+        mulhilo32(0xD2511F53u, c.x, h0, l0);
+        mulhilo32(0xCD9E8D57u, c.z, h1, l1);
+        c = u32x4{h1 ^ c.y ^ k0, l1, h0 ^ c.w ^ k1, l0};
+        k0 += 0x9E3779B9u;
+        k1 += 0xBB67AE85u;
+    }
+    return make_uint2(0xCD9E8D57u * c.z, 0xD2511F53u * c.x);
+}
+
 // ---------------------------------------------------------------------------
 // discrete Gaussian, sigma = 3.2 on [-19, 19]: thresholds floor(2^64 Pr[X <= x])
 // for x = -19 .. 18; a 64-bit uniform r maps to -19 + #{x : r >= T[x]}
@@ -41,16 +58,16 @@ __device__ __forceinline__ int gauss_from_u64(uint64_t r) {
     return v;
 }
 
-// The same map through shared-memory tables, by the high word of r.  An entry belongs to one value of
-// its top byte: in the entry's top byte the number of thresholds certainly not above r, below it the
-// next 24 bits of the one threshold that shares the byte, to be compared with those of r (an entry
-// without such a threshold counts one less and compares with 0).  The bytes 00 and ff share more than one
-// threshold (1 sample in 128) and have a second row each for the next byte; what is still undecided there
-// (1 in 32768, and equal bits, 1 in 2^24) is counted threshold by threshold.
-// One 4-byte load and a comparison per sample: a loop over the thresholds that share the byte cost a warp its longest one.
+// The same map through shared-memory tables, by the high word of r.  An entry belongs to one value of its
+// top byte: in the top byte the number of thresholds certainly not above r, below it 2^24 less the next 24 bits of the
+// one threshold that shares the byte.  Adding the next 24 bits of r carries into the top byte when r is not below that
+// threshold, so a sample costs one 4-byte load, an addition and a shift.  What this does not decide has the sum's
+// sign set (the bytes 00 and ff, which share more than one threshold: 1 sample in 128) or its low 24 bits zero
+// (r and the threshold agree so far): gauss_rare() looks at the next byte, and then at all thresholds (1 in 32768).
 struct GaussTables {
     uint32_t entry[3][256];
 };
+constexpr uint32_t GAUSS_UNDECIDED = 0x80000000u;
 
 __device__ __forceinline__ uint32_t gauss_entry(uint64_t lo, int width) {        // r in [lo, lo + 2^width)
     const uint64_t last = lo + ((1ull << width) - 1);
@@ -62,8 +79,8 @@ __device__ __forceinline__ uint32_t gauss_entry(uint64_t lo, int width) {       
         if (t <= lo) base++;
         else if (t <= last) { in++; t_in = t; }
     }
-    if (in > 1 || (in == 0 && base == 0)) return 0xffu << 24;
-    return in ? (base << 24) | ((uint32_t)(t_in >> (width - 24)) & 0xffffffu) : (base - 1) << 24;
+    if (in > 1) return GAUSS_UNDECIDED;
+    return (base << 24) + (in ? (1u << 24) - ((uint32_t)(t_in >> (width - 24)) & 0xffffffu) : 0u);
 }
 
 __device__ __forceinline__ void gauss_tables_init(GaussTables &g, uint32_t tid, uint32_t nthreads) {
@@ -74,21 +91,37 @@ __device__ __forceinline__ void gauss_tables_init(GaussTables &g, uint32_t tid, 
     }
 }
 
-static __device__ __noinline__ int gauss_counted(uint64_t r) {
+// value + 19 in the top byte, unless gauss_undecided()
+__device__ __forceinline__ uint32_t gauss_sum(const GaussTables &g, uint32_t hi) { return g.entry[0][hi >> 24] + (hi & 0xffffffu); }
+__device__ __forceinline__ bool gauss_undecided(uint32_t sum) { return (int)sum < 0 || (sum << 8) == 0; }
+static __device__ __noinline__ int gauss_rare(const GaussTables &g, uint64_t r) {
+    const uint32_t hi = (uint32_t)(r >> 32), byte = hi >> 24;
+    if (byte == 0 || byte == 255) {
+        const uint32_t sum = g.entry[byte ? 2 : 1][(hi >> 16) & 255u] + ((uint32_t)(r >> 24) & 0xffffffu);
+        if (!gauss_undecided(sum)) return (int)(sum >> 24) - 19;
+    }
     int v = -19;
 #pragma unroll 1
     for (int x = 0; x < 38; x++) v += (r >= c_gauss_cdf[x]) ? 1 : 0;
     return v;
 }
 __device__ __forceinline__ int gauss_from_u64(const GaussTables &g, uint64_t r) {
-    const uint32_t hi = (uint32_t)(r >> 32);
-    uint32_t e = g.entry[0][hi >> 24], rest = hi & 0xffffffu;
-    if ((e >> 24) == 0xffu) {
-        e = g.entry[(hi >> 31) + 1u][(hi >> 16) & 255u];
-        rest = (uint32_t)(r >> 24) & 0xffffffu;
+    const uint32_t sum = gauss_sum(g, (uint32_t)(r >> 32));
+    return gauss_undecided(sum) ? gauss_rare(g, r) : (int)(sum >> 24) - 19;
+}
+// The two samples of a stream block.  Only the high words decide nearly always, so the generator's last two
+// rounds make no others (stream_block_high); the rest of the warp waits for the whole block in 2 of 5 calls at most.
+__device__ __forceinline__ int2 gauss_pair(const GaussTables &g, uint64_t seed, uint32_t block, uint32_t t, uint32_t client,
+                                           uint32_t tag) {
+    const uint2 hi = stream_block_high(seed, block, t, client, tag);
+    const uint32_t s0 = gauss_sum(g, hi.x), s1 = gauss_sum(g, hi.y);
+    int2 v = make_int2((int)(s0 >> 24) - 19, (int)(s1 >> 24) - 19);
+    if ((int)(s0 | s1) < 0 || (s0 << 8) == 0 || (s1 << 8) == 0) {
+        const u32x4 w = stream_block(seed, block, t, client, tag);
+        v.x = gauss_from_u64(g, (uint64_t)w.x | ((uint64_t)w.y << 32));
+        v.y = gauss_from_u64(g, (uint64_t)w.z | ((uint64_t)w.w << 32));
     }
-    if ((e >> 24) == 0xffu || rest == (e & 0xffffffu)) return gauss_counted(r);
-    return (int)(e >> 24) + (rest >= (e & 0xffffffu) ? 1 : 0) - 19;
+    return v;
 }
 
 __device__ __forceinline__ uint64_t addmod(uint64_t a, uint64_t b, uint64_t q) { return csub(a + b, q); }
