@@ -363,28 +363,37 @@ static int build_mask(he_ctx *ctx, const float *score, size_t P, size_t k, const
         forced += ranges_host[2 * r + 1] - ranges_host[2 * r];
     }
     cudaStream_t st = as_stream(stream);
-    const size_t nblocks = (P + MASK_BLOCK - 1) / MASK_BLOCK, nwords = (P + 31) / 32;
+    const size_t tiles = (P + MASK_BLOCK - 1) / MASK_BLOCK, nwords = (P + 31) / 32;
     const size_t kmax = k + forced < P ? k + forced : P;
 
-    // Scratch in the context's work space (no allocation, and no free that would wait for the
-    // device): selection state (2) | totals (2) | three histograms (2048 each) | blk_a | blk_b | ranges
-    const size_t scratch_words = 4 + 3 * 2048 + 2 * nblocks + 4 * 64 + 2;
-    {
-        const int erc = ensure(&ctx->ws, &ctx->ws_bytes, scratch_words * sizeof(uint32_t));
-        if (erc != HE_OK) return erc;
+    // Scratch from the pool as well: what the selection clears | ranges | counts of runs | two counts per tile, a
+    // third with ranges | candidates
+    cudaMemPool_t pool = mask_pool(ctx->device);
+    if (!pool) return HE_ERR_CUDA;
+    const size_t scratch_words = SELECT_ZEROED + 4 * 64 + 2 * SELECT_RUNS + 3 * tiles + tiles * TILE_CANDIDATES;
+    uint32_t *scratch = nullptr;
+    if (cudaMallocFromPoolAsync(reinterpret_cast<void **>(&scratch), scratch_words * sizeof(uint32_t), pool, st) != cudaSuccess) {
+        cudaGetLastError();
+        return HE_ERR_ALLOC;
     }
-    uint32_t *scratch = static_cast<uint32_t *>(ctx->ws);
-    SelectState *state = reinterpret_cast<SelectState *>(scratch);
-    uint32_t *totals = scratch + 2, *hist = scratch + 4, *blk_eq = hist + 3 * 2048, *blk_sel = blk_eq + nblocks;
-    uint64_t *ranges_dev = reinterpret_cast<uint64_t *>(scratch + ((4 + 3 * 2048 + 2 * nblocks + 1) & ~(size_t)1));
+    SelectWork w;
+    w.hist = scratch;
+    w.done = scratch + 4096;
+    w.state = reinterpret_cast<SelectState *>(scratch + 4100);
+    w.total = scratch + 4102;
+    uint64_t *ranges_dev = reinterpret_cast<uint64_t *>(scratch + SELECT_ZEROED);
+    w.runs = ranges_dev + 2 * 64;
+    w.tile_above = reinterpret_cast<uint32_t *>(w.runs + SELECT_RUNS);
+    w.tile_cand = w.tile_above + tiles;
+    uint32_t *tile_sel = w.tile_cand + tiles, *total = w.total;
+    w.cand = tile_sel + tiles;
     // The mask owns one allocation: bit mask | per-word prefix counts | index list (its size is
     // known up to the overlap of the forced ranges with the top-k set and with each other).
     uint32_t *bits = nullptr;
-    cudaMemPool_t pool = mask_pool(ctx->device);
-    if (!pool) return HE_ERR_CUDA;
     if (cudaMallocFromPoolAsync(reinterpret_cast<void **>(&bits), (2 * nwords + (kmax ? kmax : 1)) * sizeof(uint32_t),
                                 pool, st) != cudaSuccess) {
         cudaGetLastError();
+        cudaFreeAsync(scratch, st);
         return HE_ERR_ALLOC;
     }
     uint32_t *wpre = bits + nwords, *idx = wpre + nwords;
@@ -392,33 +401,17 @@ static int build_mask(he_ctx *ctx, const float *score, size_t P, size_t k, const
     he_mask *m = nullptr;
     do {
 #define MCU(expr) if ((expr) != cudaSuccess) { rc = HE_ERR_CUDA; break; }
-        // Radix select of the k-th largest key, 11 + 11 + 10 bits, entirely on the device: the
-        // digit walk between two histogram passes is a one-block kernel, so nothing is read
-        // back before the end.
-        const SelectState init = {k ? 0u : 0xffffffffu, (uint32_t)k};      // k = 0: no key reaches the threshold
-        MCU(cudaMemcpyAsync(state, &init, sizeof(init), cudaMemcpyHostToDevice, st));
-        if (k) {
-            static const int digits[3] = {11, 11, 10};
-            MCU(cudaMemsetAsync(hist, 0, 3 * 2048 * sizeof(uint32_t), st));
-            int prefix_bits = 0;
-            bool fail = false;
-            for (int pass = 0; pass < 3 && !fail; pass++) {
-                uint32_t *h = hist + pass * 2048;
-                fail = launch_key_histogram(score, P, state, prefix_bits, digits[pass], ctx->sm_count, h, st) != cudaSuccess ||
-                       launch_radix_pick(h, digits[pass], state, st) != cudaSuccess;
-                prefix_bits += digits[pass];
-            }
-            if (fail) { rc = HE_ERR_CUDA; break; }
-        }
+        // Radix select of the k-th largest key, entirely on the device: nothing is read back before the end.
+        MCU(launch_select(score, P, k, w, ctx->sm_count, st));
         if (num_ranges)
             MCU(cudaMemcpyAsync(ranges_dev, ranges_host, 2 * num_ranges * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
-        MCU(launch_mask_count_eq(score, P, state, blk_eq, st));
-        MCU(launch_scan(blk_eq, nblocks, totals, st));
-        MCU(launch_mask_select(score, P, state, ranges_dev, (uint32_t)num_ranges, blk_eq, bits, blk_sel, st));
-        MCU(launch_scan(blk_sel, nblocks, totals + 1, st));
-        MCU(launch_mask_write(P, bits, blk_sel, wpre, idx, st));
+        MCU(launch_mask_mark(score, P, w, ranges_dev, (uint32_t)num_ranges, bits, wpre, idx, tile_sel, st));
+        if (num_ranges) {
+            MCU(launch_scan(tile_sel, tiles, total, st));
+            MCU(launch_mask_write(P, bits, tile_sel, wpre, idx, st));
+        }
         uint32_t ksel = 0;
-        MCU(cudaMemcpyAsync(&ksel, totals + 1, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+        MCU(cudaMemcpyAsync(&ksel, total, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
         MCU(cudaStreamSynchronize(st));                                      // the one wait of the call
         if ((num_ranges == 0 && ksel != k) || ksel > kmax) { rc = HE_ERR_CUDA; break; }     // cannot happen
         m = new (std::nothrow) he_mask();
@@ -431,6 +424,7 @@ static int build_mask(he_ctx *ctx, const float *score, size_t P, size_t k, const
         m->wpre = wpre;
 #undef MCU
     } while (0);
+    cudaFreeAsync(scratch, st);
     if (rc != HE_OK) {
         cudaStreamSynchronize(st);           // nothing may still write the allocation
         cudaFreeAsync(bits, st);

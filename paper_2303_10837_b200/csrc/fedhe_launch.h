@@ -92,22 +92,29 @@ cudaError_t launch_threshold_combine(const CtxDev &c, const uint64_t *ct, uint32
 // context-owned work space for T ciphertexts (2 * T * N words); implemented in fedhe_api.cu
 int ctx_workspace(he_ctx *ctx, size_t T, void **out);
 
-// mask construction (blocks of MASK_BLOCK consecutive parameters)
-constexpr uint32_t MASK_BLOCK = 4096;
+// mask construction (tiles of MASK_BLOCK consecutive parameters)
+constexpr uint32_t MASK_BLOCK = 1024, TILE_CANDIDATES = 128;
 // progress of the radix selection, in device memory: the key prefix found so far (tau after
 // the last step) and how many keys are still to be covered (after the last step: how many keys
 // equal to tau belong to the mask)
 struct SelectState { uint32_t prefix, need; };
-cudaError_t launch_key_histogram(const float *score, size_t P, const SelectState *state, int prefix_bits,
-                                 int digit_bits, int n_sm, uint32_t *hist, cudaStream_t s);
-cudaError_t launch_radix_pick(const uint32_t *hist, int digit_bits, SelectState *state, cudaStream_t s);
-cudaError_t launch_mask_count_eq(const float *score, size_t P, const SelectState *state, uint32_t *blk_eq,
-                                 cudaStream_t s);
+// work space of a selection; the SELECT_ZEROED words from `hist` are cleared at its start
+constexpr size_t SELECT_ZEROED = 4096 + 4 + 4;
+constexpr size_t SELECT_RUNS = 2 * 1024;          // thread blocks that a device holds at once, at most
+struct SelectWork {
+    uint32_t *hist;              // 2048, 1024, 1024
+    uint32_t *done;              // [4] thread blocks that finished a pass
+    SelectState *state;
+    uint32_t *total;             // selected parameters (without forced ranges)
+    uint32_t *tile_above, *tile_cand, *cand;     // per tile; [tiles][TILE_CANDIDATES]
+    uint64_t *runs;              // [SELECT_RUNS] counts before a run of tiles
+    uint32_t run;                // tiles of a run (set by launch_select)
+};
+cudaError_t launch_select(const float *score, size_t P, size_t k, SelectWork &w, int n_sm, cudaStream_t s);
 // in-place exclusive scan of a[0..count); the grand total goes to *total
 cudaError_t launch_scan(uint32_t *a, size_t count, uint32_t *total, cudaStream_t s);
-cudaError_t launch_mask_select(const float *score, size_t P, const SelectState *state,
-                               const uint64_t *ranges, uint32_t nranges, const uint32_t *blk_eq_prefix,
-                               uint32_t *bits, uint32_t *blk_sel, cudaStream_t s);
+cudaError_t launch_mask_mark(const float *score, size_t P, const SelectWork &w, const uint64_t *ranges, uint32_t nranges,
+                             uint32_t *bits, uint32_t *wpre, uint32_t *idx, uint32_t *tile_sel, cudaStream_t s);
 cudaError_t launch_mask_write(size_t P, const uint32_t *bits, const uint32_t *blk_sel_prefix,
                               uint32_t *wpre, uint32_t *idx, cudaStream_t s);
 

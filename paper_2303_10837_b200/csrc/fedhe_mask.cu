@@ -11,138 +11,321 @@ namespace fedhe {
 // non-negative number, 0 for negatives, -0 and NaN
 __device__ __forceinline__ uint32_t score_key(float s) {
     const uint32_t b = __float_as_uint(s);
-    return ((b & 0x80000000u) || b > 0x7f800000u) ? 0u : b;
+    return b > 0x7f800000u ? 0u : b;                       // the sign bit is above all of these
 }
 
 // exclusive prefix sum over the threads of a block (any whole number of warps up to 32); the block total goes to `total`
-__device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *warp_sums, uint32_t &total) {
+template <class T>
+__device__ __forceinline__ T block_exclusive_scan(T v, T *warp_sums, T &total) {
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t inc = v;
+    T inc = v;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t o = __shfl_up_sync(0xffffffffu, inc, d);
+        const T o = __shfl_up_sync(0xffffffffu, inc, d);
         if (lane >= (uint32_t)d) inc += o;
     }
     if (lane == 31) warp_sums[warp] = inc;
     __syncthreads();
     if (warp == 0) {
-        uint32_t w = lane < ((blockDim.x + 31u) >> 5) ? warp_sums[lane] : 0u, winc = w;
+        T w = lane < ((blockDim.x + 31u) >> 5) ? warp_sums[lane] : (T)0, winc = w;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t o = __shfl_up_sync(0xffffffffu, winc, d);
+            const T o = __shfl_up_sync(0xffffffffu, winc, d);
             if (lane >= (uint32_t)d) winc += o;
         }
         warp_sums[lane] = winc - w;          // exclusive warp offsets
         if (lane == 31) warp_sums[32] = winc;
     }
     __syncthreads();
-    const uint32_t res = warp_sums[warp] + inc - v;
+    const T res = warp_sums[warp] + inc - v;
     total = warp_sums[32];
     __syncthreads();
     return res;
 }
 
-// histogram of the next `digit_bits` key bits among the keys whose leading
-// `prefix_bits` bits equal the prefix found so far (state->prefix)
-__global__ void __launch_bounds__(512)
-key_histogram_kernel(const float *score, size_t P, const SelectState *state, int prefix_bits, int digit_bits,
-                     uint32_t *hist) {
-    extern __shared__ uint32_t sh[];
-    const uint32_t bins = 1u << digit_bits;
-    const uint32_t prefix = prefix_bits ? state->prefix : 0u;
-    for (uint32_t b = threadIdx.x; b < bins; b += blockDim.x) sh[b] = 0;
+// ---- radix selection of the k-th largest key: digits of 11, 10 and 10 bits (a key has 31) ----
+//
+// Three passes over the scores: the histogram of the first digit; the histogram of the second among the
+// keys that have the first (the candidates, a few per cent of real scores), which are also gathered by tiles;
+// and, when the threshold tau is known, the marking.  What lies between works on the candidates.  The
+// last thread block of a pass to finish does the one-block step that follows it: picking the digit, or
+// the scan over the tiles.  (With three histogram passes, a counting pass and one-block kernels between them
+// the selection of 2.56 M out of 25.6 M took 341 us; the first pass was bound by conflicts of its shared-memory
+// atomics, because neighbouring scores share an exponent.)
+
+// true in all threads of the block that finishes last; what the others wrote is visible to it
+__device__ __forceinline__ bool last_block(uint32_t *done) {
+    __shared__ uint32_t is_last;
+    __threadfence();
     __syncthreads();
-    const int shift = 32 - prefix_bits - digit_bits;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < P; i += (size_t)gridDim.x * blockDim.x) {
-        const uint32_t key = score_key(__ldg(score + i));
-        if (prefix_bits == 0 || (key >> (32 - prefix_bits)) == prefix)
-            atomicAdd(&sh[(key >> shift) & (bins - 1u)], 1u);
-    }
+    if (threadIdx.x == 0) is_last = atomicAdd(done, 1u) + 1u == gridDim.x ? 1u : 0u;
     __syncthreads();
-    for (uint32_t b = threadIdx.x; b < bins; b += blockDim.x)
-        if (sh[b]) atomicAdd(&hist[b], sh[b]);
+    if (is_last) __threadfence();
+    return is_last != 0;
 }
 
-cudaError_t launch_key_histogram(const float *score, size_t P, const SelectState *state, int prefix_bits,
-                                 int digit_bits, int n_sm, uint32_t *hist, cudaStream_t s) {
-    unsigned grid = blocks_for(P, 512);
-    const unsigned resident = (unsigned)n_sm * 4u;       // four blocks of 512 threads fit one SM
-    if (grid > resident) grid = resident;
-    if (grid == 0) grid = 1;
-    key_histogram_kernel<<<grid, 512, sizeof(uint32_t) << digit_bits, s>>>(score, P, state, prefix_bits,
-                                                                          digit_bits, hist);
-    return FEDHE_LAUNCHED();
-}
-
-// One step of the radix selection on the device: walks the digits of a
-// histogram from the largest down until `need` keys are covered, appends the
-// digit found to the prefix and takes the keys above it off `need`.  One block;
-// after the last step prefix is the threshold key tau and need the number of
-// keys equal to tau that belong to the mask.
-__global__ void __launch_bounds__(1024)
-radix_pick_kernel(const uint32_t *hist, int digit_bits, SelectState *state) {
+// Walks the digits of a histogram from the largest down until `need` keys are covered, appends the
+// digit found to the prefix and takes the keys above it off `need`.  By a block of 1024 threads.
+template <int BITS>
+__device__ __forceinline__ void radix_pick(const uint32_t *hist, uint32_t prefix, uint32_t need, SelectState *state) {
     __shared__ uint32_t warp_sums[33];
-    const uint32_t bins = 1u << digit_bits;
-    const uint32_t need = state->need;
-    // thread t looks at digits b = bins - 1 - (2 t), bins - 2 - (2 t): descending order
-    const uint32_t per = bins / 1024u ? bins / 1024u : 1u;       // 2 for 11 bits, 1 for 10 bits
-    uint32_t h[2] = {0u, 0u}, mine = 0u;
+    constexpr uint32_t bins = 1u << BITS, per = bins / 1024u;        // thread t: digits from bins - 1 - per t down
+    uint32_t h[per], mine = 0u;
+#pragma unroll
     for (uint32_t j = 0; j < per; j++) {
-        const uint32_t pos = threadIdx.x * per + j;              // position in descending order
-        h[j] = pos < bins ? hist[bins - 1u - pos] : 0u;
+        h[j] = __ldcg(hist + bins - 1u - (threadIdx.x * per + j));
         mine += h[j];
     }
     uint32_t tot;
-    uint32_t above = block_exclusive_scan(mine, warp_sums, tot);   // keys in digits above this thread's
-    __syncthreads();
+    uint32_t above = block_exclusive_scan(mine, warp_sums, tot);     // keys in digits above this thread's
+#pragma unroll
     for (uint32_t j = 0; j < per; j++) {
         const uint32_t pos = threadIdx.x * per + j;
-        // the digit where the running count first reaches `need` (digit 0 if it never does)
-        if (pos < bins && above < need && (above + h[j] >= need || pos == bins - 1u)) {
-            state->prefix = (state->prefix << digit_bits) | (bins - 1u - pos);
+        // the digit where the running count first reaches `need`
+        if (above < need && above + h[j] >= need) {
+            state->prefix = (prefix << BITS) | (bins - 1u - pos);
             state->need = need - above;
         }
         above += h[j];
     }
 }
 
-cudaError_t launch_radix_pick(const uint32_t *hist, int digit_bits, SelectState *state, cudaStream_t s) {
-    radix_pick_kernel<<<1, 1024, 0, s>>>(hist, digit_bits, state);
-    return FEDHE_LAUNCHED();
-}
+// First digit.  Every lane counts in a column of its own, so the lanes of a warp never meet in a word or a bank: two
+// 16-bit counters to a word, [1024][32].  A column takes a 32nd of the block's keys, and a block at most HIST_KEYS.
+constexpr int LOADS = 8, HIST_LOADS = 16;
+constexpr size_t HIST_KEYS = 32 * 65536 - 2048, HIST_SMEM = 1024 * 32 * sizeof(uint32_t);
 
-// Keys of the four neighbouring parameters a thread takes (one 16-byte load
-// where the pointer allows and all four exist; key 0 beyond the end).
-__device__ __forceinline__ void load_keys4(const float *score, size_t P, size_t i0, bool vec, uint32_t (&key)[4]) {
-    if (vec && i0 + 4 <= P) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(score + i0));
-        key[0] = score_key(v.x); key[1] = score_key(v.y); key[2] = score_key(v.z); key[3] = score_key(v.w);
-    } else {
+__global__ void __launch_bounds__(1024, 1)
+key_histogram_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
+    extern __shared__ uint32_t sh[];
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint32_t b = threadIdx.x; b < 1024u * 32u; b += 1024u) sh[b] = 0;
+    __syncthreads();
+    uint32_t *mine = sh + lane;
+    const size_t step = (size_t)gridDim.x * 1024u;
+    auto count = [&](float v) {
+        const uint32_t d = score_key(v) >> 20;
+        atomicAdd(mine + (d >> 1) * 32u, 1u << ((d & 1u) * 16u));
+    };
+    size_t i = (size_t)blockIdx.x * 1024u + threadIdx.x;
+    if (i + (HIST_LOADS - 1) * step < P) {
+        // the next loads are on their way while these are counted
+        float v[HIST_LOADS];
 #pragma unroll
-        for (int j = 0; j < 4; j++) key[j] = i0 + j < P ? score_key(__ldg(score + i0 + j)) : 0u;
+        for (int j = 0; j < HIST_LOADS; j++) v[j] = __ldg(score + i + j * step);
+        for (i += step * HIST_LOADS; i + (HIST_LOADS - 1) * step < P; i += step * HIST_LOADS) {
+            float next[HIST_LOADS];
+#pragma unroll
+            for (int j = 0; j < HIST_LOADS; j++) next[j] = __ldg(score + i + j * step);
+#pragma unroll
+            for (int j = 0; j < HIST_LOADS; j++) count(v[j]);
+#pragma unroll
+            for (int j = 0; j < HIST_LOADS; j++) v[j] = next[j];
+        }
+#pragma unroll
+        for (int j = 0; j < HIST_LOADS; j++) count(v[j]);
+    }
+    for (; i < P; i += step) count(__ldg(score + i));
+    __syncthreads();
+    uint32_t even = 0, odd = 0;
+#pragma unroll
+    for (uint32_t j = 0; j < 32u; j++) {
+        const uint32_t c = sh[threadIdx.x * 32u + ((lane + j) & 31u)];
+        even += c & 0xffffu;
+        odd += c >> 16;
+    }
+    if (even) atomicAdd(w.hist + 2 * threadIdx.x, even);
+    if (odd) atomicAdd(w.hist + 2 * threadIdx.x + 1, odd);
+    if (last_block(w.done)) {
+        if (k == 0) {
+            if (threadIdx.x == 0) *w.state = SelectState{0xffffffffu, 0u};       // no key reaches the threshold
+        } else {
+            radix_pick<11>(w.hist, 0u, k, w.state);
+        }
     }
 }
 
-// number of keys equal to tau in every block of MASK_BLOCK parameters (four per thread)
-__global__ void __launch_bounds__(MASK_BLOCK / 4)
-mask_count_eq_kernel(const float *score, size_t P, const SelectState *state, uint32_t *blk_eq, bool vec) {
-    __shared__ uint32_t warp_sums[33];
-    const uint32_t tau = state->prefix;
-    const size_t i0 = (size_t)blockIdx.x * MASK_BLOCK + 4 * threadIdx.x;
-    uint32_t key[4];
-    load_keys4(score, P, i0, vec, key);
-    uint32_t cnt = 0;
+// f(first word, words' keys) for LOADS words of a tile at a time, by a warp: lane l the l-th parameter of each word.
+// Beyond the end keys are 0, and f is told how many parameters are left (LOADS * 32 or less).
+template <class F>
+__device__ __forceinline__ void for_tile(const float *score, size_t P, size_t first, F f) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const float *p = score + first + lane;
+    const uint32_t left = P - first < MASK_BLOCK ? (uint32_t)(P - first) : MASK_BLOCK;
+#pragma unroll 1
+    for (uint32_t w0 = 0; w0 * 32 < left; w0 += LOADS) {
+        uint32_t key[LOADS];
+        if ((w0 + LOADS) * 32 <= left) {
 #pragma unroll
-    for (int j = 0; j < 4; j++) cnt += (i0 + j < P && key[j] == tau) ? 1u : 0u;
-    uint32_t tot;
-    block_exclusive_scan(cnt, warp_sums, tot);
-    if (threadIdx.x == 0) blk_eq[blockIdx.x] = tot;
+            for (int j = 0; j < LOADS; j++) key[j] = score_key(__ldg(p + (w0 + j) * 32));
+            f(w0, key, LOADS * 32u);
+        } else {
+#pragma unroll
+            for (int j = 0; j < LOADS; j++)
+                key[j] = (w0 + j) * 32 + lane < left ? score_key(__ldg(p + (w0 + j) * 32)) : 0u;
+            f(w0, key, left - w0 * 32);
+        }
+    }
 }
 
-cudaError_t launch_mask_count_eq(const float *score, size_t P, const SelectState *state, uint32_t *blk_eq,
-                                 cudaStream_t s) {
-    const bool vec = (reinterpret_cast<uintptr_t>(score) & 15u) == 0;
-    mask_count_eq_kernel<<<blocks_for(P, MASK_BLOCK), MASK_BLOCK / 4, 0, s>>>(score, P, state, blk_eq, vec);
+// Second digit.  A warp takes a tile of MASK_BLOCK scores, counts the keys above the first digit and
+// gathers the lower 20 bits of those that have it; a tile with more than TILE_CANDIDATES of them is read again instead.
+__global__ void __launch_bounds__(1024, 2)
+key_candidates_kernel(const float *score, size_t P, SelectWork w) {
+    __shared__ uint32_t sh[1024];
+    sh[threadIdx.x] = 0;
+    __syncthreads();
+    const uint32_t prefix = w.state->prefix, need = w.state->need;
+    const uint32_t lane = threadIdx.x & 31u;
+    const size_t tiles = (P + MASK_BLOCK - 1) / MASK_BLOCK;
+    for (size_t tile = (size_t)blockIdx.x * 32u + (threadIdx.x >> 5); tile < tiles; tile += (size_t)gridDim.x * 32u) {
+        const size_t first = tile * MASK_BLOCK;
+        uint32_t above = 0, found = 0;
+        uint32_t *cand = w.cand + tile * TILE_CANDIDATES;
+        for_tile(score, P, first, [&](uint32_t w0, const uint32_t (&key)[LOADS], uint32_t left) {
+            // a bit for every candidate among the lane's keys; the few there are get their places together
+            uint32_t mine = 0;
+#pragma unroll
+            for (int j = 0; j < LOADS; j++) {
+                const uint32_t top = key[j] >> 20;
+                if (top > prefix) above++;
+                if (top == prefix) mine |= 1u << j;
+            }
+            if (left < LOADS * 32u) {                              // keys beyond the end are 0 and not above any digit
+                const uint32_t words = left > lane ? (left - lane + 31u) / 32u : 0u;
+                mine &= (1u << words) - 1u;
+            }
+            const uint32_t n = __popc(mine);
+            uint32_t at = n;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t o = __shfl_up_sync(0xffffffffu, at, d);
+                if (lane >= (uint32_t)d) at += o;
+            }
+            const uint32_t all = __shfl_sync(0xffffffffu, at, 31);
+            at += found - n;
+            found += all;
+            while (mine) {
+                const uint32_t j = __ffs((int)mine) - 1;
+                mine &= mine - 1u;
+                const uint32_t low = score_key(__ldg(score + first + (w0 + j) * 32u + lane)) & 0xfffffu;
+                if (at < TILE_CANDIDATES) cand[at] = low;
+                at++;
+                atomicAdd(sh + (low >> 10), 1u);
+            }
+        });
+        above = __reduce_add_sync(0xffffffffu, above);
+        if (lane == 0) {
+            w.tile_above[tile] = above;
+            w.tile_cand[tile] = found;
+        }
+    }
+    __syncthreads();
+    if (sh[threadIdx.x]) atomicAdd(w.hist + 2048 + threadIdx.x, sh[threadIdx.x]);
+    if (last_block(w.done + 1)) radix_pick<10>(w.hist + 2048, prefix, need, w.state);
+}
+
+// f(in, lower 20 bits) for the candidates of a tile, by a whole warp: f may use warp operations
+template <class F>
+__device__ __forceinline__ void for_candidates(const float *score, size_t P, const SelectWork &w, size_t tile, uint32_t first_digit, F f) {
+    const uint32_t lane = threadIdx.x & 31u, found = w.tile_cand[tile];
+    if (found <= TILE_CANDIDATES) {
+        for (uint32_t i = 0; i < found; i += 32) {
+            const bool in = i + lane < found;
+            f(in, in ? w.cand[tile * TILE_CANDIDATES + i + lane] : 0u);
+        }
+    } else {
+        for (uint32_t i = 0; i < MASK_BLOCK; i += 32) {
+            const size_t at = tile * MASK_BLOCK + i + lane;
+            const uint32_t key = at < P ? score_key(__ldg(score + at)) : 0u;
+            f(at < P && (key >> 20) == first_digit, key & 0xfffffu);
+        }
+    }
+}
+
+// third digit, over the candidates
+__global__ void __launch_bounds__(1024, 2) key_last_digit_kernel(const float *score, size_t P, SelectWork w) {
+    __shared__ uint32_t sh[1024];
+    sh[threadIdx.x] = 0;
+    __syncthreads();
+    const uint32_t prefix = w.state->prefix, need = w.state->need;
+    const size_t tiles = (P + MASK_BLOCK - 1) / MASK_BLOCK;
+    for (size_t tile = (size_t)blockIdx.x * 32u + (threadIdx.x >> 5); tile < tiles; tile += (size_t)gridDim.x * 32u)
+        for_candidates(score, P, w, tile, prefix >> 10, [&](bool in, uint32_t low) {
+            if (in && (low >> 10) == (prefix & 1023u)) atomicAdd(sh + (low & 1023u), 1u);
+        });
+    __syncthreads();
+    if (sh[threadIdx.x]) atomicAdd(w.hist + 3072 + threadIdx.x, sh[threadIdx.x]);
+    if (last_block(w.done + 2)) radix_pick<10>(w.hist + 3072, prefix, need, w.state);
+}
+
+// Keys above and equal to tau: a block takes a run of tiles, and leaves for each the counts before it within the run
+// (equal keys in the upper half); the last block does the same for the runs.
+__global__ void __launch_bounds__(1024, 2) tile_counts_kernel(const float *score, size_t P, SelectWork w) {
+    __shared__ uint64_t warp_sums[33];
+    const uint32_t tau = w.state->prefix, need = w.state->need, lane = threadIdx.x & 31u;
+    const size_t tiles = (P + MASK_BLOCK - 1) / MASK_BLOCK;
+    const size_t begin = (size_t)blockIdx.x * w.run, end = begin + w.run < tiles ? begin + w.run : tiles;
+    for (size_t tile = begin + (threadIdx.x >> 5); tile < end; tile += 32u) {
+        uint32_t gt = 0, eq = 0;
+        for_candidates(score, P, w, tile, tau >> 20, [&](bool in, uint32_t low) {
+            gt += in && low > (tau & 0xfffffu) ? 1u : 0u;
+            eq += in && low == (tau & 0xfffffu) ? 1u : 0u;
+        });
+        gt = __reduce_add_sync(0xffffffffu, gt);
+        eq = __reduce_add_sync(0xffffffffu, eq);
+        if (lane == 0) {
+            w.tile_above[tile] += gt;
+            w.tile_cand[tile] = eq;
+        }
+    }
+    __syncthreads();
+    uint64_t before = 0, tot;
+    for (size_t t0 = begin; t0 < end; t0 += 1024u) {
+        const size_t tile = t0 + threadIdx.x;
+        const uint64_t c = tile < end ? ((uint64_t)w.tile_cand[tile] << 32) | w.tile_above[tile] : 0u;
+        const uint64_t at = before + block_exclusive_scan(c, warp_sums, tot);
+        before += tot;
+        if (tile < end) {
+            w.tile_cand[tile] = (uint32_t)(at >> 32);
+            w.tile_above[tile] = (uint32_t)at;
+        }
+    }
+    if (threadIdx.x == 0) __stcg(reinterpret_cast<unsigned long long *>(w.runs + blockIdx.x), (unsigned long long)before);
+    if (!last_block(w.done + 3)) return;
+    before = 0;
+    for (uint32_t r0 = 0; r0 < gridDim.x; r0 += 1024u) {
+        const uint32_t r = r0 + threadIdx.x;
+        const uint64_t c = r < gridDim.x ? __ldcg(reinterpret_cast<const unsigned long long *>(w.runs + r)) : 0u;
+        const uint64_t at = before + block_exclusive_scan(c, warp_sums, tot);
+        before += tot;
+        if (r < gridDim.x) w.runs[r] = at;
+    }
+    const uint32_t eq_all = (uint32_t)(before >> 32);
+    if (threadIdx.x == 0) *w.total = (uint32_t)before + (eq_all < need ? eq_all : need);
+}
+
+cudaError_t launch_select(const float *score, size_t P, size_t k, SelectWork &w, int n_sm, cudaStream_t s) {
+    cudaError_t e;
+    if ((e = cudaMemsetAsync(w.hist, 0, SELECT_ZEROED * sizeof(uint32_t), s))) return e;
+    if ((e = cudaFuncSetAttribute(key_histogram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HIST_SMEM))) return e;
+    // one thread block of the first pass to an SM, unless its counters could overflow
+    const unsigned want = blocks_for(P, 1024 * HIST_LOADS), least = blocks_for(P, (unsigned)HIST_KEYS);
+    unsigned g1 = want < (unsigned)n_sm ? want : (unsigned)n_sm;
+    if (g1 < least) g1 = least;
+    key_histogram_kernel<<<g1, 1024, HIST_SMEM, s>>>(score, P, w, (uint32_t)k);
+    if ((e = FEDHE_LAUNCHED())) return e;
+    auto grid = [&](unsigned per_block) {
+        const unsigned blocks = blocks_for(P, per_block), resident = n_sm < 1024 ? 2u * (unsigned)n_sm : (unsigned)SELECT_RUNS;
+        return blocks < resident ? blocks : resident;
+    };
+    key_candidates_kernel<<<grid(32 * MASK_BLOCK), 1024, 0, s>>>(score, P, w);
+    if ((e = FEDHE_LAUNCHED())) return e;
+    key_last_digit_kernel<<<grid(32 * MASK_BLOCK), 1024, 0, s>>>(score, P, w);
+    if ((e = FEDHE_LAUNCHED())) return e;
+    const size_t tiles = (P + MASK_BLOCK - 1) / MASK_BLOCK;
+    w.run = (uint32_t)((tiles + grid(32 * MASK_BLOCK) - 1) / grid(32 * MASK_BLOCK));
+    tile_counts_kernel<<<(unsigned)((tiles + w.run - 1) / w.run), 1024, 0, s>>>(score, P, w);
     return FEDHE_LAUNCHED();
 }
 
@@ -171,57 +354,68 @@ cudaError_t launch_scan(uint32_t *a, size_t count, uint32_t *total, cudaStream_t
     return FEDHE_LAUNCHED();
 }
 
-// membership bits: key > tau, or key == tau and fewer than `need` equal keys
-// at lower indices, or inside a forced index range.  A thread takes four
-// neighbouring parameters; eight neighbouring lanes put their four bits
-// together into one word of the bit mask.
-__global__ void __launch_bounds__(MASK_BLOCK / 4)
-mask_select_kernel(const float *score, size_t P, const SelectState *state, const uint64_t *ranges,
-                   uint32_t nranges, const uint32_t *blk_eq_prefix, uint32_t *bits, uint32_t *blk_sel, bool vec) {
-    __shared__ uint32_t warp_sums[33];
-    const uint32_t tau = state->prefix, need = state->need;
-    const size_t i0 = (size_t)blockIdx.x * MASK_BLOCK + 4 * threadIdx.x;
-    uint32_t key[4];
-    load_keys4(score, P, i0, vec, key);
-    uint32_t eqs = 0;
+// Membership: key > tau, or key == tau and fewer than `need` equal keys at lower indices, or (RANGES)
+// inside a forced index range.  A warp takes a tile, a lane the parameter of its number in every word of
+// the bit mask.  Without ranges the positions are known, and the prefix counts and the index list are written too.
+template <bool RANGES>
+__global__ void __launch_bounds__(256)
+mask_mark_kernel(const float *score, size_t P, SelectWork w, const uint64_t *ranges, uint32_t nranges, uint32_t *bits,
+                 uint32_t *wpre, uint32_t *idx, uint32_t *tile_sel) {
+    const uint32_t tau = w.state->prefix, need = w.state->need;
+    const uint32_t lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
+    const size_t tile = (size_t)blockIdx.x * 8u + (threadIdx.x >> 5), first = tile * MASK_BLOCK;
+    if (first >= P) return;
+    const uint64_t run = w.runs[tile / w.run];
+    uint32_t eq_before = w.tile_cand[tile] + (uint32_t)(run >> 32);
+    // selected before the tile: the keys above tau and the first `need` of the equal ones
+    uint32_t at = RANGES ? 0u : w.tile_above[tile] + (uint32_t)run + (eq_before < need ? eq_before : need);
+    // lane l keeps the bits and the prefix count of word l of the tile, which are stored together
+    uint32_t my_bits = 0, my_pre = 0;
+    static_assert(MASK_BLOCK == 1024, "a word of the tile for every lane");
+    for_tile(score, P, first, [&](uint32_t w0, const uint32_t (&key)[LOADS], uint32_t left) {
+        bool equal = false;
 #pragma unroll
-    for (int j = 0; j < 4; j++) eqs += (i0 + j < P && key[j] == tau) ? 1u : 0u;
-    uint32_t tot;
-    uint32_t eq_before = blk_eq_prefix[blockIdx.x] + block_exclusive_scan(eqs, warp_sums, tot);
-    uint32_t nibble = 0, cnt = 0;
+        for (int j = 0; j < LOADS; j++) equal = equal || key[j] == tau;
+        // keys equal to tau are rare (among real scores), and keys beyond the end are 0
+        const bool some = __any_sync(0xffffffffu, equal);
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
-        const size_t i = i0 + j;
-        if (i >= P) continue;
-        const bool eq = key[j] == tau;
-        bool sel = key[j] > tau || (eq && eq_before < need);
-        eq_before += eq ? 1u : 0u;
-        if (!sel)
-            for (uint32_t r = 0; r < nranges; r++)
-                if (i >= ranges[2 * r] && i < ranges[2 * r + 1]) sel = true;
-        nibble |= sel ? (1u << j) : 0u;
-        cnt += sel ? 1u : 0u;
+        for (int j = 0; j < LOADS; j++) {
+            const uint32_t i = (uint32_t)first + (w0 + j) * 32u + lane;        // parameters are fewer than 2^32
+            bool sel = key[j] > tau;
+            if (some || RANGES) {
+                const bool in = j * 32u + lane < left, eq = in && key[j] == tau;
+                const uint32_t eqs = __ballot_sync(0xffffffffu, eq);
+                sel = sel || (eq && eq_before + __popc(eqs & below) < need);
+                eq_before += __popc(eqs);
+                if (RANGES && in && !sel)
+                    for (uint32_t r = 0; r < nranges; r++)
+                        if (i >= ranges[2 * r] && i < ranges[2 * r + 1]) sel = true;
+            }
+            const uint32_t who = __ballot_sync(0xffffffffu, sel);
+            if (lane == w0 + j) {
+                my_bits = who;
+                my_pre = at;
+            }
+            if (!RANGES && sel) idx[at + __popc(who & below)] = i;
+            at += __popc(who);
+        }
+    });
+    if (first + lane * 32u < P) {
+        bits[(first >> 5) + lane] = my_bits;
+        if (!RANGES) wpre[(first >> 5) + lane] = my_pre;
     }
-    const uint32_t lane = threadIdx.x & 31u;
-    uint32_t word = nibble << (4u * (lane & 7u));
-    word |= __shfl_xor_sync(0xffffffffu, word, 1);
-    word |= __shfl_xor_sync(0xffffffffu, word, 2);
-    word |= __shfl_xor_sync(0xffffffffu, word, 4);
-    if ((lane & 7u) == 0 && i0 < P) bits[i0 >> 5] = word;
-    block_exclusive_scan(cnt, warp_sums, tot);
-    if (threadIdx.x == 0) blk_sel[blockIdx.x] = tot;
+    if (RANGES && lane == 0) tile_sel[tile] = at;
 }
 
-cudaError_t launch_mask_select(const float *score, size_t P, const SelectState *state,
-                               const uint64_t *ranges, uint32_t nranges, const uint32_t *blk_eq_prefix,
-                               uint32_t *bits, uint32_t *blk_sel, cudaStream_t s) {
-    const bool vec = (reinterpret_cast<uintptr_t>(score) & 15u) == 0;
-    mask_select_kernel<<<blocks_for(P, MASK_BLOCK), MASK_BLOCK / 4, 0, s>>>(score, P, state, ranges, nranges,
-                                                                            blk_eq_prefix, bits, blk_sel, vec);
+cudaError_t launch_mask_mark(const float *score, size_t P, const SelectWork &w, const uint64_t *ranges, uint32_t nranges,
+                             uint32_t *bits, uint32_t *wpre, uint32_t *idx, uint32_t *tile_sel, cudaStream_t s) {
+    const unsigned grid = blocks_for(P, 8 * MASK_BLOCK);
+    if (nranges) mask_mark_kernel<true><<<grid, 256, 0, s>>>(score, P, w, ranges, nranges, bits, wpre, idx, tile_sel);
+    else mask_mark_kernel<false><<<grid, 256, 0, s>>>(score, P, w, ranges, nranges, bits, wpre, idx, tile_sel);
     return FEDHE_LAUNCHED();
 }
 
-// per-word prefix counts and the ascending index list: a thread takes one word
+// With forced ranges: per-word prefix counts and the ascending index list; a thread takes one word
 // of the bit mask (32 parameters), a block the MASK_BLOCK / 32 words of one
 // counted block
 __global__ void __launch_bounds__(MASK_BLOCK / 32)

@@ -285,6 +285,21 @@ def test_select_mask_ties_and_special_values(he):
     assert list(got) == list(range(33))
 
 
+@pytest.mark.parametrize("P,spread", [(1, 1.0), (33, 1.0), (2047, 1.0), (2049, 1e-4), (300_001, 1e-4), (20_000_003, 1.0)])
+def test_select_mask_tiles_and_candidates(he, P, spread):
+    """Edges of the tiles, tiles with more candidates than their list holds (all scores within one
+    digit), more tiles than resident warps, and a start that is not 16-byte aligned."""
+    g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
+    rng = np.random.default_rng(P)
+    score = (1.0 + spread * rng.random(P + 1, dtype=np.float32)).astype(np.float32)
+    d = dev_f32(score)[1:]
+    score = score[1:]
+    for k in sorted({0, 1, P // 3, P - 1, P} if P < 1_000_000 else {P // 10}):
+        mask = he.he_select_mask(g, d, k)
+        got = he.he_mask_indices(mask).cpu().numpy().view(np.uint32)
+        assert mask.k == k and np.array_equal(got, oracle.select_mask(score, k)), k
+
+
 def test_mask_with_forced_ranges(he):
     """Top-k plus whole index ranges (first and last layers)."""
     g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
