@@ -186,6 +186,11 @@ int he_ctx_create(const he_params *p, he_ctx **out) {
         if (cudaMemset(st, 0, 4 * sizeof(int)) != cudaSuccess) { rc = HE_ERR_CUDA; break; }
         d.status = static_cast<int *>(st);
         d.deal = static_cast<uint32_t *>(st) + 2;
+        if (cudaMalloc(&st, gauss_table_bytes()) != cudaSuccess) { rc = HE_ERR_ALLOC; break; }
+        ctx->owned.push_back(st);
+        d.gauss = st;
+        if (fft_setup(d, ctx->sm_count) != cudaSuccess) { rc = HE_ERR_CUDA; break; }
+        if (launch_gauss_table(st, nullptr) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess) { rc = HE_ERR_CUDA; break; }
         // pointer and weight tables of the aggregation calls
         rc = ensure(&ctx->tab, &ctx->tab_bytes,
                     HE_MAX_CLIENTS * (2 * sizeof(void *) + sizeof(double) + HE_MAX_LIMBS * sizeof(tw_t)));
@@ -510,7 +515,7 @@ static int encrypt_range(he_ctx *ctx, const he_keys *keys, const float *sel_dev,
         CU(launch_encrypt_ntt(d, keys->dev, sel_dev, ctx->ws, ctx->sm_count, (uint32_t)t_begin, t_count, seed,
                               client_id, ct_dev, st));
     else
-        CU(launch_encrypt(d, keys->dev, sel_dev, ctx->ws, ctx->sm_count, (uint32_t)t_begin, t_count, seed,
+        CU(launch_encrypt(d, keys->dev, sel_dev, ctx->ws, (uint32_t)t_begin, t_count, seed,
                           client_id, ct_dev, st));
     return HE_OK;
 }

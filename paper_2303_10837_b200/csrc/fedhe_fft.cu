@@ -462,11 +462,13 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
     double2 *buf = reinterpret_cast<double2 *>(smem);
     root_t *tab = reinterpret_cast<root_t *>(smem + (size_t)NB * 16);
     int8_t *e1_smem = reinterpret_cast<int8_t *>(tab + G::Tab::WORDS);
-    __shared__ GaussTables gt;
+    __shared__ __align__(16) GaussTables gt;
     __shared__ uint32_t tmem_base;
     __shared__ __align__(8) uint64_t key_bar;
     const uint32_t rank = blockIdx.x % S, cid = blockIdx.x / S, nc = gridDim.x / S;
-    gauss_tables_init(gt, threadIdx.x, NT);
+    // (made once with the context: 768 entries from 38 thresholds each took 3 us of every call)
+    for (uint32_t i = threadIdx.x; i < sizeof(GaussTables) / 16; i += NT)
+        reinterpret_cast<uint4 *>(&gt)[i] = __ldg(reinterpret_cast<const uint4 *>(c.gauss) + i);
     for (uint32_t i = threadIdx.x; i < (uint32_t)G::Tab::WORDS; i += NT) tab[i] = c.fft_inv[i];
     if (threadIdx.x == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(&key_bar)) : "memory");
@@ -899,73 +901,111 @@ static cudaError_t fft_grid(K kern, int n_sm, size_t want, cudaStream_t s, cudaL
 // two that take half of it each do run side by side.  This kernel has the same shape without it.
 __global__ void __launch_bounds__(FftLay::NT, 2) enc_shape_kernel() {}
 
-// Thread blocks that work on one ciphertext together: as many as it has blocks of 2^12 points (less if its units
-// could not be shared out evenly), and more while the ciphertexts are too few to fill the device.
-static uint32_t enc_cluster(const CtxDev &c, int n_sm, size_t T) {
-    uint32_t S = 1;
-    while (S < 8 && S < (1u << (c.logN - 13)) && (2 * c.L) % (2 * S) == 0) S *= 2;
-    while (S < 8 && S < 2 * c.L && T * 2 * S <= 2 * (size_t)n_sm) S *= 2;
-    return S;
+// shared memory that leaves no room for a second thread block on the SM
+constexpr int ENC_ALONE_SMEM = 116 * 1024;
+
+// How many clusters of 1 .. ENC_MOST blocks the device holds at once, two blocks to an SM and one.
+template <int CL>
+static cudaError_t setup_ring(CtxDev &c, int n_sm) {
+    using G = EncRing<CL>;
+    static_assert(G::SMEM + 4096 <= ENC_ALONE_SMEM - 1024, "two thread blocks to an SM");
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(encrypt_fft_kernel<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, ENC_ALONE_SMEM))) return e;
+    if ((e = cudaFuncSetAttribute(enc_shape_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ENC_ALONE_SMEM))) return e;
+    for (uint32_t alone = 0; alone < 2; alone++)
+        for (uint32_t S = 1; S <= ENC_MOST; S++) {
+            cudaLaunchConfig_t cfg = {};
+            cudaLaunchAttribute attr;
+            cfg.blockDim = dim3(G::NT, 1, 1);
+            cfg.gridDim = dim3(S, 1, 1);
+            cfg.dynamicSmemBytes = alone ? ENC_ALONE_SMEM : G::SMEM + 4096;        // and the static part
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = S;
+            attr.val.clusterDim.y = 1;
+            attr.val.clusterDim.z = 1;
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            int clusters = 0;
+            if ((e = cudaOccupancyMaxActiveClusters(&clusters, enc_shape_kernel, &cfg))) return e;
+            const int most = (alone ? 1 : 2) * n_sm / (int)S;
+            c.enc_fit[alone][S] = (uint16_t)(clusters < most ? clusters : most);
+        }
+    return cudaSuccess;
 }
-// ... and the most clusters that a ciphertext is worth
-static uint32_t enc_parts(const CtxDev &c, uint32_t S) { return (2 * c.L + S - 1) / S; }
+cudaError_t fft_setup(CtxDev &c, int n_sm) { FEDHE_FOR_RING(c, setup_ring, c, n_sm) }
+
+// The thread blocks that work on a ciphertext together, whether they have their SMs to themselves, the clusters.
+struct EncPlan { uint32_t S, alone, clusters, parts; };
+
+// With ciphertexts enough to fill the device: as many blocks as the ciphertext has of 2^12 points, or the next
+// number below that shares its 2 L units out evenly.  With fewer, larger clusters, by these measurements (us, L = 3 or 4):
+//   N = 8192, 25 ciphertexts: 1, 2, 3, 4, 8 blocks 79, 52, 43, 40, 43 (8 of them share SMs); 60: 2, 4 blocks 52, 55;
+//     100: 1, 2 blocks 81, 72
+//   N = 16384, 40: 2, 3, 6 blocks 110, 86, 75; 60: 2, 4 blocks 111, 92
+// so the largest clusters that hold all ciphertexts at one block to an SM, if they can do the 2 R blocks of the
+// preparation side by side, and else the largest that hold them at two.
+static EncPlan enc_plan(const CtxDev &c, size_t T) {
+    const uint32_t R = 1u << (c.logN - 13), units = 2 * c.L, most = units < ENC_MOST ? units : ENC_MOST;
+    uint32_t base = R < most ? R : most;
+    while (units % base) base--;
+    EncPlan p = {base, 0, 0, (units + base - 1) / base};
+    uint32_t alone = most, shared = most;
+    while (alone > 1 && c.enc_fit[1][alone] < T) alone--;
+    while (shared > base && c.enc_fit[0][shared] < T) shared--;
+    if (c.enc_fit[1][alone] >= T && alone >= base && (alone >= 2 * R || alone == most)) p = EncPlan{alone, 1, 0, 1};
+    else if (shared > base) p = EncPlan{shared, 0, 0, 1};
+    const uint32_t fit = c.enc_fit[p.alone][p.S];
+    // what is left after whole rounds of all clusters, or too few ciphertexts for the largest clusters: several to each
+    if (p.S == most || T > fit) p.parts = (units + p.S - 1) / p.S;
+    p.clusters = T >= fit ? fit : (uint32_t)T * (fit / (uint32_t)T < p.parts ? fit / (uint32_t)T : p.parts);
+    return p;
+}
 
 template <int CL>
 static size_t ring_scratch(const CtxDev &c, int n_sm, size_t T) {
     using G = EncRing<CL>;
     size_t most = 0;                                   // of any number of ciphertexts up to T
-    for (uint32_t S = enc_cluster(c, n_sm, T); S <= 8; S *= 2) {
-        const size_t fit = 2 * (size_t)n_sm / S, want = T * enc_parts(c, S), bytes = (want < fit ? want : fit) * (G::SHARED + S * G::OWN);
+    for (uint32_t S = enc_plan(c, T).S; S <= ENC_MOST; S++) {
+        const size_t want = T * ((2 * c.L + S - 1) / S), fit = c.enc_fit[0][S], bytes = (want < fit ? want : fit) * (G::SHARED + S * G::OWN);
         if (bytes > most) most = bytes;
     }
     const size_t fit = 2 * (size_t)n_sm / FftRing<CL>::R, dec = (T < fit ? T : fit) * FftRing<CL>::SCRATCH;
     return most > dec ? most : dec;
 }
-size_t fft_work_bytes(const CtxDev &c, int n_sm, size_t T) { FEDHE_FOR_RING(c, ring_scratch, c, n_sm, T) }
+size_t fft_work_bytes(const CtxDev &c, int n_sm, size_t T) {
+    if (T == 0) return 0;
+    FEDHE_FOR_RING(c, ring_scratch, c, n_sm, T)
+}
 
 template <int CL>
-static cudaError_t launch_encrypt_ring(const CtxDev &c, const KeysDev &k, const float *sel, void *work, int n_sm, uint32_t t0,
+static cudaError_t launch_encrypt_ring(const CtxDev &c, const KeysDev &k, const float *sel, void *work, uint32_t t0,
                                        size_t T, uint64_t seed, uint32_t client, uint64_t *ct, cudaStream_t s) {
     using G = EncRing<CL>;
-    auto kern = encrypt_fft_kernel<CL>;
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM))) return e;
-    const uint32_t S = enc_cluster(c, n_sm, T), parts = enc_parts(c, S);
+    const EncPlan p = enc_plan(c, T);
+    if (p.clusters < 1) return cudaErrorLaunchOutOfResources;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;
     cfg.stream = s;
     cfg.blockDim = dim3(G::NT, 1, 1);
-    cfg.dynamicSmemBytes = G::SMEM;
+    cfg.gridDim = dim3(p.clusters * p.S, 1, 1);
+    cfg.dynamicSmemBytes = p.alone ? ENC_ALONE_SMEM : G::SMEM;
     attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = S;
+    attr.val.clusterDim.x = p.S;
     attr.val.clusterDim.y = 1;
     attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    size_t fit = 2 * (size_t)n_sm / S;
-    if (S > 1 && T * parts > fit / 2) {
-        cfg.gridDim = dim3(S, 1, 1);
-        int clusters = 0;
-        cfg.dynamicSmemBytes = G::SMEM + 4096;       // and the static part
-        if ((e = cudaFuncSetAttribute(enc_shape_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes))) return e;
-        if ((e = cudaOccupancyMaxActiveClusters(&clusters, enc_shape_kernel, &cfg))) return e;
-        cfg.dynamicSmemBytes = G::SMEM;
-        if (clusters < 1) return cudaErrorLaunchOutOfResources;
-        if ((size_t)clusters < fit) fit = (size_t)clusters;
-    }
-    // whole rounds of all clusters, or so many clusters to every ciphertext
-    size_t nc = T >= fit ? fit : T * (fit / T < parts ? fit / T : parts);
-    cfg.gridDim = dim3((unsigned)(nc * S), 1, 1);
-    if ((e = cudaLaunchKernelEx(&cfg, kern, c, k, sel, static_cast<unsigned char *>(work), t0, seed, client, ct, (uint32_t)T, S, parts)))
+    cudaError_t e;
+    if ((e = cudaLaunchKernelEx(&cfg, encrypt_fft_kernel<CL>, c, k, sel, static_cast<unsigned char *>(work), t0, seed, client, ct,
+                                (uint32_t)T, p.S, p.parts)))
         return e;
     return FEDHE_LAUNCHED();
 }
 
-cudaError_t launch_encrypt(const CtxDev &c, const KeysDev &k, const float *sel, void *work, int n_sm,
-                           uint32_t t0, size_t T, uint64_t seed, uint32_t client, uint64_t *ct,
-                           cudaStream_t s) {
+cudaError_t launch_encrypt(const CtxDev &c, const KeysDev &k, const float *sel, void *work, uint32_t t0, size_t T,
+                           uint64_t seed, uint32_t client, uint64_t *ct, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
-    FEDHE_FOR_RING(c, launch_encrypt_ring, c, k, sel, work, n_sm, t0, T, seed, client, ct, s)
+    FEDHE_FOR_RING(c, launch_encrypt_ring, c, k, sel, work, t0, T, seed, client, ct, s)
 }
 
 template <int CL>
@@ -984,6 +1024,13 @@ cudaError_t launch_decrypt_fft(const CtxDev &c, const KeysDev &k, const uint64_t
                                void *work, int n_sm, double *z, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
     FEDHE_FOR_RING(c, launch_decrypt_ring, c, k, ct, level, T, work, n_sm, z, s)
+}
+
+__global__ void __launch_bounds__(256) gauss_table_kernel(GaussTables *g) { gauss_tables_init(*g, threadIdx.x, blockDim.x); }
+size_t gauss_table_bytes() { return sizeof(GaussTables); }
+cudaError_t launch_gauss_table(void *table, cudaStream_t s) {
+    gauss_table_kernel<<<1, 256, 0, s>>>(static_cast<GaussTables *>(table));
+    return FEDHE_LAUNCHED();
 }
 
 // ---- key tables ------------------------------------------------------------------------

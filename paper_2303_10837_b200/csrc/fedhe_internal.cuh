@@ -70,6 +70,8 @@ struct LimbOf<ModF64> {
     static HD double wn(const LimbDev &lb) { return lb.wn_d; }
 };
 
+constexpr uint32_t ENC_MOST = 8;       // thread blocks of a cluster that encrypts, at most
+
 struct CtxDev {
     uint32_t N, logN, L;
     uint32_t LOGB, A;    // a length-N transform = 2^A blocks of 2^LOGB
@@ -82,6 +84,8 @@ struct CtxDev {
     FftSplit dec_split;                // of c1 on limb 0, for any c1
     uint32_t fft_pieces;               // of all limbs of a public-key half
     int64_t term_limit;                // a quarter of the smallest prime
+    uint16_t enc_fit[2][ENC_MOST + 1]; // clusters of a size that the device holds: two blocks to an SM, one
+    const void *gauss;   // GaussTables
     uint32_t *deal;      // encryption hands out ciphertexts here: next one, thread blocks (clusters) that are done; 0 between calls
     int *status;         // sticky anomaly word
 };
