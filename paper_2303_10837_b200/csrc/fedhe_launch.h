@@ -122,6 +122,13 @@ cudaError_t launch_mask_mark(const float *score, size_t P, const SelectWork &w, 
 cudaError_t launch_mask_write(size_t P, const uint32_t *bits, const uint32_t *blk_sel_prefix,
                               uint32_t *wpre, uint32_t *idx, cudaStream_t s);
 
+// the same for the parameters [first, first + count) of a mask, first a multiple of 32: x and w_glob point at the first
+// of them, sel, rest, z and rest_avg at the start of the whole arrays
+cudaError_t launch_pack_range(const he_mask *mask, const float *x, size_t first, size_t count, float *sel, float *rest,
+                              cudaStream_t s);
+cudaError_t launch_unpack_range(const he_mask *mask, const double *z, const double *rest_avg, size_t first, size_t count,
+                                double *w_glob, cudaStream_t s);
+cudaError_t launch_zero(float *dst, size_t count, cudaStream_t s);
 cudaError_t launch_pack(const he_mask *mask, const float *x, size_t P, size_t k, size_t padded,
                         float *sel, float *rest, cudaStream_t s);
 cudaError_t launch_unpack(const he_mask *mask, const double *z, const double *rest_avg, size_t P,

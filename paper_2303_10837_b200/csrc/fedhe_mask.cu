@@ -516,20 +516,28 @@ __global__ void __launch_bounds__(256) zero_tail_kernel(float *dst, size_t count
     if (i < count) dst[i] = 0.0f;
 }
 
+cudaError_t launch_pack_range(const he_mask *mask, const float *x, size_t first, size_t count, float *sel, float *rest,
+                              cudaStream_t s) {
+    if (count == 0) return cudaSuccess;
+    const size_t warps = (((count + 31) >> 5) + PACK_WORDS - 1) / PACK_WORDS;
+    // positions among the unselected count from the whole mask's start
+    pack_masked_kernel<<<blocks_for(warps * 32, 256), 256, 0, s>>>(mask->bits + (first >> 5), mask->wpre + (first >> 5), x, count,
+                                                                   sel, rest ? rest + first : nullptr);
+    return FEDHE_LAUNCHED();
+}
+
+cudaError_t launch_zero(float *dst, size_t count, cudaStream_t s) {
+    if (count == 0) return cudaSuccess;
+    zero_tail_kernel<<<blocks_for(count, 256), 256, 0, s>>>(dst, count);
+    return FEDHE_LAUNCHED();
+}
+
 cudaError_t launch_pack(const he_mask *mask, const float *x, size_t P, size_t k, size_t padded,
                         float *sel, float *rest, cudaStream_t s) {
     if (!mask) return launch_copy_pad<float, float4>(x, P, padded, sel, s);     // k = P: a copy and the zero tail
-    if (P) {
-        const size_t warps = (((P + 31) >> 5) + PACK_WORDS - 1) / PACK_WORDS;
-        pack_masked_kernel<<<blocks_for(warps * 32, 256), 256, 0, s>>>(mask->bits, mask->wpre, x, P, sel, rest);
-        const cudaError_t e = FEDHE_LAUNCHED();
-        if (e) return e;
-    }
-    if (padded > k) {                                                            // tail of the last ciphertext
-        zero_tail_kernel<<<blocks_for(padded - k, 256), 256, 0, s>>>(sel + k, padded - k);
-        return FEDHE_LAUNCHED();
-    }
-    return cudaSuccess;
+    const cudaError_t e = launch_pack_range(mask, x, 0, P, sel, rest, s);
+    if (e) return e;
+    return launch_zero(sel + k, padded - k, s);                                  // tail of the last ciphertext
 }
 
 // the reverse with a mask: w_glob[i] = z[r] for the r-th masked parameter, the remainder's
@@ -559,13 +567,20 @@ unpack_masked_kernel(const uint32_t *bits, const uint32_t *wpre, const double *z
     }
 }
 
+cudaError_t launch_unpack_range(const he_mask *mask, const double *z, const double *rest_avg, size_t first, size_t count,
+                                double *w_glob, cudaStream_t s) {
+    if (count == 0) return cudaSuccess;
+    const size_t warps = (((count + 31) >> 5) + PACK_WORDS - 1) / PACK_WORDS;
+    unpack_masked_kernel<<<blocks_for(warps * 32, 256), 256, 0, s>>>(mask->bits + (first >> 5), mask->wpre + (first >> 5), z,
+                                                                     rest_avg ? rest_avg + first : nullptr, count, w_glob);
+    return FEDHE_LAUNCHED();
+}
+
 cudaError_t launch_unpack(const he_mask *mask, const double *z, const double *rest_avg, size_t P,
                           double *w_glob, cudaStream_t s) {
     if (P == 0) return cudaSuccess;
     if (!mask) return launch_copy_pad<double, double2>(z, P, P, w_glob, s);
-    const size_t warps = (((P + 31) >> 5) + PACK_WORDS - 1) / PACK_WORDS;
-    unpack_masked_kernel<<<blocks_for(warps * 32, 256), 256, 0, s>>>(mask->bits, mask->wpre, z, rest_avg, P, w_glob);
-    return FEDHE_LAUNCHED();
+    return launch_unpack_range(mask, z, rest_avg, 0, P, w_glob, s);
 }
 
 }  // namespace fedhe

@@ -285,6 +285,30 @@ def test_select_mask_ties_and_special_values(he):
     assert list(got) == list(range(33))
 
 
+@pytest.mark.parametrize("P,k", [(1000, 10), (300_000, 4096), (1_300_003, 130_001), (1_300_003, 0), (1_300_003, 1_300_003),
+                                 (700_001, 1)])
+def test_host_round_by_ranges(he, P, k):
+    """A masked round from host buffers, cut along the parameters, against the same round step by step on the
+    device: one range and several, ranges that complete no ciphertext, nothing and everything masked."""
+    g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
+    keys = he.he_keygen(g, 5)
+    rng = np.random.default_rng(P + k)
+    xs = [(0.01 * rng.standard_normal(P)).astype(np.float32) for _ in range(3)]
+    alpha = [0.25, 0.5, 0.25]
+    mask = he.he_select_mask(g, dev_f32(rng.random(P, dtype=np.float32)), k)
+    rests, cts = [], []
+    for i, x in enumerate(xs):
+        sel, rest = he.he_pack(g, mask, dev_f32(x))
+        rests.append(rest)
+        cts.append(he.he_encrypt(g, keys, sel, 99, i))
+    z = he.he_decrypt(g, keys, he.he_weighted_aggregate(g, cts, alpha)) if k else torch.empty(0, dtype=torch.float64, device="cuda")
+    avg = he.he_plain_aggregate(g, rests, alpha)
+    want = he.he_unpack(g, mask, z, avg, P).cpu()
+    host = torch.empty(P, dtype=torch.float64)
+    he.he_round_host(g, keys, mask, [torch.from_numpy(x) for x in xs], alpha, 99, host)
+    assert torch.equal(host, want)
+
+
 @pytest.mark.parametrize("P,spread", [(1, 1.0), (33, 1.0), (2047, 1.0), (2049, 1e-4), (300_001, 1e-4), (20_000_003, 1.0)])
 def test_select_mask_tiles_and_candidates(he, P, spread):
     """Edges of the tiles, tiles with more candidates than their list holds (all scores within one
