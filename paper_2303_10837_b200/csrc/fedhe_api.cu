@@ -148,6 +148,8 @@ int he_ctx_create(const he_params *p, he_ctx **out) {
             ld.mu = hl.mu;
             ld.ninv = tw_t{hl.ninv.w, hl.ninv.wp};
             ld.wn = tw_t{hl.wn.w, hl.wn.wp};
+            const HostTw r64 = host_shoup((0 - hl.q) % hl.q, hl.q);
+            ld.r64 = tw_t{r64.w, r64.wp};
             if (j + 1 < p->L) {
                 HostTw qi = host_shoup(host_invmod(ql % hl.q, hl.q), hl.q);
                 ld.qlinv = tw_t{qi.w, qi.wp};

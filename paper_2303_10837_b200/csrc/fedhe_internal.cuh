@@ -37,6 +37,7 @@ struct LimbDev {
     uint64_t mu;         // floor(2^64 / q), Barrett
     tw_t ninv;           // 1/N
     tw_t wn;             // (inverse twiddle of stage 0) / N
+    tw_t r64;            // 2^64 mod q
     tw_t qlinv;          // 1 / q_{L-1} mod q (unused for the last prime)
     const tw_t *fwd;     // psi^brev(i)
     const tw_t *inv;     // psi^-brev(i)

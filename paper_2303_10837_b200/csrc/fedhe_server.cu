@@ -13,40 +13,73 @@ namespace fedhe {
 // (32 L C bytes per parameter), so the client pointers and weights are
 // staged in shared memory once per block and the loads of four clients are
 // issued before their multiply-adds to keep enough bytes in flight.
-__device__ __forceinline__ void weighted_sum_pair(const uint64_t *const *sp, const tw_t *sw, int C, uint32_t L,
-                                                  uint32_t j, size_t off, uint64_t q, uint64_t &ax,
-                                                  uint64_t &ay) {
-    const uint64_t q2 = 2 * q;
-    ax = 0;
-    ay = 0;
+//
+// A sum is not reduced as it grows: values and weights are cut at bit 30, their partial products are accumulated by
+// wide multiply-adds without carries (four clients fit 64 bits for every prime below 2^61), the accumulators
+// are joined into 128 bits after four clients, and the 128 bits are reduced after 64 and at the end.  A product costs the
+// multiply pipe 11 slots instead of the 20 of a modular one, which kept it two thirds busy beside HBM: the sum of
+// 64 clients and 25 ciphertexts of N = 8192 takes 115 us (5.5 TB/s) instead of 124.  Measured and not taken: a thread per
+// coefficient (8-byte loads: 130 us, and 752 instead of 627 us for 10 clients and 313 ciphertexts of N = 16384), a thread
+// per pair and limb (136 and 937 us), 48 or 40 registers for more resident blocks (151 and 616, 126 and 705 us).
+constexpr uint64_t LOW30 = (1ull << 30) - 1;
+
+__device__ __forceinline__ uint64_t reduce128(unsigned __int128 v, const LimbDev &lb) {
+    const uint64_t t = shoup_lazy((uint64_t)(v >> 64), lb.r64.w, lb.r64.wp, lb.q) + barrett64((uint64_t)v, lb.q, lb.mu);   // below 3q
+    return csub(csub(t, 2 * lb.q), lb.q);
+}
+
+struct SplitSum {
+    uint64_t low = 0, mid = 0, high = 0;
+    __device__ __forceinline__ void add(uint64_t x, uint64_t w) {        // w: its parts in the two words
+        const uint32_t x0 = (uint32_t)x & (uint32_t)LOW30, x1 = (uint32_t)(x >> 30), w0 = (uint32_t)w, w1 = (uint32_t)(w >> 32);
+        low += (uint64_t)x0 * w0;
+        mid += (uint64_t)x0 * w1;
+        mid += (uint64_t)x1 * w0;
+        high += (uint64_t)x1 * w1;
+    }
+    __device__ __forceinline__ unsigned __int128 joined() const {
+        return (unsigned __int128)low + ((unsigned __int128)mid << 30) + ((unsigned __int128)high << 60);
+    }
+};
+
+__device__ __forceinline__ void weighted_sum_pair(const uint64_t *const *sp, const uint64_t *sw, int C, uint32_t L,
+                                                  uint32_t j, size_t off, const LimbDev &lb, uint64_t &ax, uint64_t &ay) {
+    unsigned __int128 sx = 0, sy = 0;
     int cl = 0;
     for (; cl + 4 <= C; cl += 4) {
         ulonglong2 v[4];
 #pragma unroll
         for (int u = 0; u < 4; u++) v[u] = __ldg(reinterpret_cast<const ulonglong2 *>(sp[cl + u] + off));
+        SplitSum x, y;
 #pragma unroll
         for (int u = 0; u < 4; u++) {
-            const tw_t w = sw[(cl + u) * L + j];
-            ax = csub(ax + shoup_lazy(v[u].x, w.w, w.wp, q), q2);
-            ay = csub(ay + shoup_lazy(v[u].y, w.w, w.wp, q), q2);
+            const uint64_t w = sw[(cl + u) * L + j];
+            x.add(v[u].x, w);
+            y.add(v[u].y, w);
+        }
+        sx += x.joined();
+        sy += y.joined();
+        if ((cl & 63) == 60) {
+            sx = reduce128(sx, lb);
+            sy = reduce128(sy, lb);
         }
     }
+    SplitSum x, y;
     for (; cl < C; cl++) {
         const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(sp[cl] + off));
-        const tw_t w = sw[cl * L + j];
-        ax = csub(ax + shoup_lazy(v.x, w.w, w.wp, q), q2);
-        ay = csub(ay + shoup_lazy(v.y, w.w, w.wp, q), q2);
+        const uint64_t w = sw[cl * L + j];
+        x.add(v.x, w);
+        y.add(v.y, w);
     }
-    ax = csub(ax, q);
-    ay = csub(ay, q);
+    ax = reduce128(sx + x.joined(), lb);
+    ay = reduce128(sy + y.joined(), lb);
 }
 
 // The same sum for a limb whose prime is below 2^46, in the exact double-precision arithmetic of
-// the transforms: a product costs the shared multiply / double-precision pipe 6 slots instead of
-// about 19, which matters because this pass keeps that pipe two thirds busy beside HBM.  Every
+// the transforms: a product costs the shared multiply / double-precision pipe 6 slots.  Every
 // product has magnitude at most 3q/4 and the running sum is brought back below q after every 32
 // clients, so it stays below 25 q < 2^51 and every addition is exact.
-__device__ __forceinline__ void weighted_sum_pair_f64(const uint64_t *const *sp, const tw_t *sw, int C, uint32_t L,
+__device__ __forceinline__ void weighted_sum_pair_f64(const uint64_t *const *sp, const uint64_t *sw, int C, uint32_t L,
                                                       uint32_t j, size_t off, double q, double qi, uint64_t &ax,
                                                       uint64_t &ay) {
     double sx = 0.0, sy = 0.0;
@@ -57,7 +90,7 @@ __device__ __forceinline__ void weighted_sum_pair_f64(const uint64_t *const *sp,
         for (int u = 0; u < 4; u++) v[u] = __ldg(reinterpret_cast<const ulonglong2 *>(sp[cl + u] + off));
 #pragma unroll
         for (int u = 0; u < 4; u++) {
-            const double w = f64_from_u64(sw[(cl + u) * L + j].w);
+            const double w = f64_from_bits(sw[(cl + u) * L + j]);
             sx = f64_add(sx, f64_mulmod(f64_from_u64(v[u].x), w, q, qi));
             sy = f64_add(sy, f64_mulmod(f64_from_u64(v[u].y), w, q, qi));
         }
@@ -68,7 +101,7 @@ __device__ __forceinline__ void weighted_sum_pair_f64(const uint64_t *const *sp,
     }
     for (; cl < C; cl++) {
         const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(sp[cl] + off));
-        const double w = f64_from_u64(sw[cl * L + j].w);
+        const double w = f64_from_bits(sw[cl * L + j]);
         sx = f64_add(sx, f64_mulmod(f64_from_u64(v.x), w, q, qi));
         sy = f64_add(sy, f64_mulmod(f64_from_u64(v.y), w, q, qi));
     }
@@ -77,10 +110,14 @@ __device__ __forceinline__ void weighted_sum_pair_f64(const uint64_t *const *sp,
 }
 
 // a limb's sum in whichever arithmetic its prime allows
-__device__ __forceinline__ void weighted_sum_limb(const LimbDev &lb, const uint64_t *const *sp, const tw_t *sw, int C,
+__device__ __forceinline__ void weighted_sum_limb(const LimbDev &lb, const uint64_t *const *sp, const uint64_t *sw, int C,
                                                   uint32_t L, uint32_t j, size_t off, uint64_t &ax, uint64_t &ay) {
     if (lb.fwd_d) weighted_sum_pair_f64(sp, sw, C, L, j, off, lb.qd, lb.qi, ax, ay);
-    else weighted_sum_pair(sp, sw, C, L, j, off, lb.q, ax, ay);
+    else weighted_sum_pair(sp, sw, C, L, j, off, lb, ax, ay);
+}
+// what the sums read of a weight
+__device__ __forceinline__ uint64_t staged_weight(const LimbDev &lb, uint64_t w) {
+    return lb.fwd_d ? f64_bits(f64_from_u64(w)) : (w & LOW30) | (w >> 30) << 32;
 }
 
 __global__ void __launch_bounds__(256)
@@ -88,9 +125,9 @@ aggregate_rescale_kernel(const __grid_constant__ CtxDev c, const uint64_t *const
                          int C, uint64_t *out, size_t total) {
     extern __shared__ __align__(16) unsigned char agg_sm[];
     const uint32_t L = c.L;
-    tw_t *sw = reinterpret_cast<tw_t *>(agg_sm);                                    // [C][L]
+    uint64_t *sw = reinterpret_cast<uint64_t *>(agg_sm);                                    // [C][L]
     const uint64_t **sp = reinterpret_cast<const uint64_t **>(sw + (size_t)C * L);  // [C]
-    for (int e = threadIdx.x; e < C * (int)L; e += blockDim.x) sw[e] = wtab[e];
+    for (int e = threadIdx.x; e < C * (int)L; e += blockDim.x) sw[e] = staged_weight(c.limb[e % (int)L], __ldg(&wtab[e].w));
     for (int e = threadIdx.x; e < C; e += blockDim.x) sp[e] = ptrs[e];
     __syncthreads();
     const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -123,7 +160,7 @@ cudaError_t launch_aggregate(const CtxDev &c, const uint64_t *const *ptrs, const
                              size_t T, uint64_t *out, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
     const size_t total = T * 2 * (c.N >> 1);
-    const size_t smem = (size_t)C * c.L * sizeof(tw_t) + (size_t)C * sizeof(void *);
+    const size_t smem = (size_t)C * c.L * sizeof(uint64_t) + (size_t)C * sizeof(void *);
     cudaError_t e;
     if (smem > 48 * 1024 &&
         (e = cudaFuncSetAttribute(aggregate_rescale_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
@@ -148,9 +185,9 @@ aggregate_sum_kernel(const __grid_constant__ CtxDev c, const uint64_t *const *pt
                      uint64_t *out, uint64_t *last, size_t total) {
     extern __shared__ __align__(16) unsigned char agg_sm[];
     const uint32_t L = c.L;
-    tw_t *sw = reinterpret_cast<tw_t *>(agg_sm);
+    uint64_t *sw = reinterpret_cast<uint64_t *>(agg_sm);
     const uint64_t **sp = reinterpret_cast<const uint64_t **>(sw + (size_t)C * L);
-    for (int e = threadIdx.x; e < C * (int)L; e += blockDim.x) sw[e] = wtab[e];
+    for (int e = threadIdx.x; e < C * (int)L; e += blockDim.x) sw[e] = staged_weight(c.limb[e % (int)L], __ldg(&wtab[e].w));
     for (int e = threadIdx.x; e < C; e += blockDim.x) sp[e] = ptrs[e];
     __syncthreads();
     const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -214,7 +251,7 @@ rescale_partial_sum_kernel(const __grid_constant__ CtxDev c, const uint64_t *con
 cudaError_t launch_aggregate_partial(const CtxDev &c, const uint64_t *const *ptrs, const tw_t *wtab, int C,
                                      size_t T, uint64_t *out, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
-    const size_t smem = (size_t)C * c.L * sizeof(tw_t) + (size_t)C * sizeof(void *);
+    const size_t smem = (size_t)C * c.L * sizeof(uint64_t) + (size_t)C * sizeof(void *);
     cudaError_t e;
     if (smem > 48 * 1024 &&
         (e = cudaFuncSetAttribute(aggregate_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
@@ -265,7 +302,7 @@ cudaError_t launch_aggregate_ntt(const CtxDev &c, const uint64_t *const *ptrs, c
                                  size_t T, uint64_t *scratch, uint64_t *out, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
     uint64_t *last = scratch, *rem = scratch + 2 * T * c.N;
-    const size_t smem = (size_t)C * c.L * sizeof(tw_t) + (size_t)C * sizeof(void *);
+    const size_t smem = (size_t)C * c.L * sizeof(uint64_t) + (size_t)C * sizeof(void *);
     cudaError_t e;
     if (smem > 48 * 1024 &&
         (e = cudaFuncSetAttribute(aggregate_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
