@@ -238,7 +238,7 @@ int he_ctx_reserve(he_ctx *ctx, size_t max_k) {
     if (!good(ctx)) return HE_ERR_INVALID_ARG;
     const size_t T = he_num_ct(ctx, max_k);
     size_t need = encrypt_ntt_work_bytes(ctx->dev, ctx->sm_count, T);
-    const size_t fft = fft_work_bytes(ctx->dev, ctx->sm_count, T);
+    const size_t fft = fft_work_bytes(ctx->dev, T);
     if (fft > need) need = fft;
     return ensure(&ctx->ws, &ctx->ws_bytes, need);
 }
@@ -510,7 +510,7 @@ static int encrypt_range(he_ctx *ctx, const he_keys *keys, const float *sel_dev,
     if (!sel_dev || !ct_dev || !aligned16(ct_dev)) return HE_ERR_INVALID_ARG;
     const CtxDev &d = ctx->dev;
     int rc = ensure(&ctx->ws, &ctx->ws_bytes, ntt_out ? encrypt_ntt_work_bytes(d, ctx->sm_count, t_count)
-                                                      : fft_work_bytes(d, ctx->sm_count, t_count));
+                                                      : fft_work_bytes(d, t_count));
     if (rc != HE_OK) return rc;
     cudaStream_t st = as_stream(stream);
     if (ntt_out)
@@ -663,9 +663,7 @@ static int decrypt_level(he_ctx *ctx, const he_keys *keys, const uint64_t *ct_de
     cudaStream_t st = as_stream(stream);
     if (!ntt_in) {
         if (T >= (1ull << 32)) return HE_ERR_SIZE;
-        const int rc = ensure(&ctx->ws, &ctx->ws_bytes, fft_work_bytes(d, ctx->sm_count, T));
-        if (rc != HE_OK) return rc;
-        CU(launch_decrypt_fft(d, keys->dev, ct_dev, level, T, ctx->ws, ctx->sm_count, z_dev, st));
+        CU(launch_decrypt_fft(d, keys->dev, ct_dev, level, T, z_dev, st));
         return HE_OK;
     }
     if (d.logN <= 14) {                 // one fused kernel, no work buffer
@@ -866,7 +864,7 @@ static int round_host_full(he_ctx *ctx, const he_keys *keys, const float *const 
                  b_agg = align(Tmax * aggw * sizeof(uint64_t)), b_z = align(T * n * sizeof(double));
     int rc = ensure(&ctx->round_buf, &ctx->round_bytes, 2 * C * b_sel + b_cts + b_agg + b_z);
     if (rc != HE_OK) return rc;
-    if ((rc = ensure(&ctx->ws, &ctx->ws_bytes, fft_work_bytes(d, ctx->sm_count, Tmax))) != HE_OK) return rc;
+    if ((rc = ensure(&ctx->ws, &ctx->ws_bytes, fft_work_bytes(d, Tmax))) != HE_OK) return rc;
     if ((rc = round_host_streams(ctx)) != HE_OK) return rc;
     unsigned char *p = static_cast<unsigned char *>(ctx->round_buf);
     unsigned char *selbuf[2];
@@ -991,7 +989,7 @@ static int round_host_queued(he_ctx *ctx, const he_keys *keys, const he_mask *ma
                  b_ravg = align(restlen * sizeof(double)), b_out = align(P * sizeof(double));
     const size_t total = 2 * C * b_x + C * (b_sel + b_rest) + b_cts + b_agg + b_z + b_ravg + b_out;
     if ((rc = ensure(&ctx->round_buf, &ctx->round_bytes, total)) != HE_OK) return rc;
-    if ((rc = ensure(&ctx->ws, &ctx->ws_bytes, fft_work_bytes(d, ctx->sm_count, Tc))) != HE_OK) return rc;
+    if ((rc = ensure(&ctx->ws, &ctx->ws_bytes, fft_work_bytes(d, Tc))) != HE_OK) return rc;
     unsigned char *p = static_cast<unsigned char *>(ctx->round_buf);
     unsigned char *xbuf[2] = {p, p + C * b_x};
     p += 2 * C * b_x;

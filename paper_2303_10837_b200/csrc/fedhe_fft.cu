@@ -58,10 +58,7 @@ struct FftRing {
     using Tab = FftTab<CL_>;
     static constexpr int CL = CL_, R = 1 << CL, NB = FftLay::NB, NT = FftLay::NT, n = R * NB, N = 2 * n;
     static constexpr int PER = 16 / R, COLS = NB / R;     // columns of the R x NB view that a thread, a thread block finishes
-    // scratch in global memory (it lives in L2): a thread block's, then a cluster's
-    static constexpr size_t PARK = (size_t)NB * 16, SCRATCH = R * PARK;
     static constexpr size_t SMEM = (size_t)NB * 16 + (size_t)Tab::WORDS * 16;
-    static constexpr int BATCH = 8;                       // coefficients whose loads are in flight together
 };
 
 // a word of the buffer of block `a` of the cluster
@@ -131,45 +128,6 @@ __device__ __forceinline__ uint32_t fft_coefficient(int i, uint32_t rank) {
     const int o = i >> 1;
     return (o % G::R) * G::NB + G::NT * (rank * G::PER + o / G::R) + (i & 1) * G::n;
 }
-// the same in the block's own order of the coefficients it finishes: [2 halves][R rows][COLS]
-template <class G>
-__device__ __forceinline__ uint32_t fft_own(int i) {
-    const int o = i >> 1;
-    return (o % G::R) * G::COLS + G::NT * (o / G::R) + (i & 1) * G::NB;
-}
-
-// ---- joined lower pieces, parked for the thread that will join the top one ----
-template <class G>
-__device__ __forceinline__ void fft_park(const cpx (&x)[16], unsigned char *park, const FftSplit &f, uint32_t piece,
-                                         uint32_t tid) {
-    if (f.narrow) {
-        int *p = reinterpret_cast<int *>(park) + tid;
-#pragma unroll
-        for (int i = 0; i < 32; i++) __stcg(p + i * G::NT, (int)fft_round_bits((i & 1) ? x[i >> 1].im : x[i >> 1].re));
-    } else {
-        long long *p = reinterpret_cast<long long *>(park) + tid;
-        const uint32_t sh = f.shift[piece];
-#pragma unroll
-        for (int i = 0; i < 32; i++) {
-            long long w = (fft_round_bits((i & 1) ? x[i >> 1].im : x[i >> 1].re) - FFT_ROUND_BITS) << sh;
-            if (piece) w += __ldcg(p + i * G::NT);
-            __stcg(p + i * G::NT, w);
-        }
-    }
-}
-// val += the parked sums of values i0 .. i0 + BATCH - 1
-template <class G>
-__device__ __forceinline__ void fft_parked(int64_t (&val)[G::BATCH], const unsigned char *park, const FftSplit &f, int i0,
-                                           uint32_t tid) {
-    if (f.narrow) {
-#pragma unroll
-        for (int i = 0; i < G::BATCH; i++) val[i] += __ldcg(reinterpret_cast<const int *>(park) + (i0 + i) * G::NT + tid);
-    } else if (f.pieces > 1) {
-#pragma unroll
-        for (int i = 0; i < G::BATCH; i++) val[i] += __ldcg(reinterpret_cast<const long long *>(park) + (i0 + i) * G::NT + tid);
-    }
-}
-
 // the value that position i of block `blk` (of 2^LEV) has after LEV stages of the encoder's network
 template <int LEV>
 __device__ __forceinline__ cpx encoder_stages(const float *slots, const double2 *ftw, uint32_t n, uint32_t blk, uint32_t i) {
@@ -763,31 +721,53 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
 // decryption + decoding:  d = c0 + c1 s on limb 0, centred, then the slot transform
 // ===========================================================================
 
+// a double from a 32-bit integer: the integer plus 2^31 as the low word of 2^52 + ...
+__device__ __forceinline__ double fft_from_int32(int v) {
+    return f64_sub(__hiloint2double(0x43300000, (int)((uint32_t)v ^ 0x80000000u)), 4503601774854144.0);      // 2^52 + 2^31
+}
+
 // A cluster decrypts and decodes a range of ciphertexts: per piece of c1 a forward
 // transform, the product with the transformed secret, an inverse transform; joining, c0, centring;
 // then the slot transform, which is the forward transform again (a slot is the value at one of the
 // roots; `slot_of` puts the values in order through shared memory).  Only the two limb-0
 // polynomials are read and the n decoded values written.
+//
+// c0 and the joined lower pieces wait in tensor memory, in the words of the threads that will join them; c1 is read
+// by all its loads at once, and cut in 32-bit arithmetic if its pieces are two.  (Reading eight values at a time from L2
+// and cutting in 64 bits, loading and joining took 28 of 65 thousand clocks per ciphertext of N = 8192.)
 template <int CL>
 __global__ void __launch_bounds__(FftLay::NT, 2)
 decrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const uint64_t *ct, uint32_t level,
-                   unsigned char *work, double *z, uint32_t T) {
+                   double *z, uint32_t T) {
     using G = FftRing<CL>;
     constexpr uint32_t n = G::n, NB = G::NB, NT = G::NT, R = G::R;
     constexpr size_t N = G::N;
     extern __shared__ __align__(128) unsigned char smem[];
     double2 *buf = reinterpret_cast<double2 *>(smem);
     root_t *tab = reinterpret_cast<root_t *>(smem + (size_t)NB * 16);
+    __shared__ uint32_t tmem_base;
     const uint32_t rank = blockIdx.x % R, cid = blockIdx.x / R, nc = gridDim.x / R;
     for (uint32_t i = threadIdx.x; i < (uint32_t)G::Tab::WORDS; i += NT) tab[i] = c.fft_inv[i];
     buffer_free<CL>();
-    unsigned char *park = work + (size_t)cid * G::SCRATCH + rank * G::PARK;
+    const uint32_t tm = tmem_take(&tmem_base);            // and the tables are there
+    constexpr uint32_t C0_AT = 0, PARK_AT = 64;           // 32 values of two words each
     const FftSplit &f = c.dec_split;
     const uint64_t q = c.limb[0].q;
     const int64_t half_q = (int64_t)(q / 2);
     const double inv_delta = __longlong_as_double((long long)(1023 - c.log2_delta) << 52);
     const uint32_t t_end = (uint32_t)((uint64_t)T * (cid + 1) / nc);
-    __syncthreads();
+    auto centred = [&](uint64_t v) { return v > (uint64_t)half_q ? (int64_t)(v - q) : (int64_t)v; };
+    auto get4 = [&](uint32_t at, int64_t (&v)[4]) {
+        uint32_t w[8];
+        tmem_get8(tm + at, w);
+#pragma unroll
+        for (int i = 0; i < 4; i++) v[i] = (int64_t)(((uint64_t)w[2 * i + 1] << 32) | w[2 * i]);
+    };
+    auto put4 = [&](uint32_t at, const int64_t (&v)[4]) {
+        const uint32_t w[8] = {(uint32_t)v[0], (uint32_t)((uint64_t)v[0] >> 32), (uint32_t)v[1], (uint32_t)((uint64_t)v[1] >> 32),
+                               (uint32_t)v[2], (uint32_t)((uint64_t)v[2] >> 32), (uint32_t)v[3], (uint32_t)((uint64_t)v[3] >> 32)};
+        tmem_put8(tm + at, w);
+    };
 #pragma unroll 1
     for (uint32_t t = (uint32_t)((uint64_t)T * cid / nc); t < t_end; t++) {
         const uint64_t *c0 = ct + ((size_t)t * 2 * level) * N, *c1 = c0 + level * N;
@@ -797,13 +777,28 @@ decrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const uint
         for (uint32_t p = 0; p <= f.pieces; p++) {
             if (p < f.pieces) {
                 const uint64_t *src = c1 + fresh_tid();
-                auto value = [&](uint64_t v) {
-                    return fft_from_int(fft_piece(f, v > (uint64_t)half_q ? (int64_t)(v - q) : (int64_t)v, p));
-                };
+                uint64_t raw[32];
 #pragma unroll
-                for (int o = 0; o < 16; o++) {
-                    const uint64_t re = __ldg(src + fft_coefficient<G>(2 * o, rank)), im = __ldg(src + fft_coefficient<G>(2 * o + 1, rank));
-                    x[o] = cpx{value(re), value(im)};
+                for (int i = 0; i < 32; i++) raw[i] = __ldg(src + fft_coefficient<G>(i, rank));
+                if (f.pieces == 2) {
+                    const uint32_t w = f.shift[1];                       // at most 30
+                    if (p == 0) {
+#pragma unroll
+                        for (int o = 0; o < 16; o++) {
+                            const uint32_t re = (uint32_t)centred(raw[2 * o]), im = (uint32_t)centred(raw[2 * o + 1]);
+                            x[o] = cpx{fft_from_int32((int)(re << (32 - w)) >> (32 - w)), fft_from_int32((int)(im << (32 - w)) >> (32 - w))};
+                        }
+                    } else {
+                        const int64_t round = (int64_t)1 << (w - 1);
+#pragma unroll
+                        for (int o = 0; o < 16; o++)
+                            x[o] = cpx{fft_from_int32((int)((centred(raw[2 * o]) + round) >> w)),
+                                       fft_from_int32((int)((centred(raw[2 * o + 1]) + round) >> w))};
+                    }
+                } else {
+#pragma unroll
+                    for (int o = 0; o < 16; o++)
+                        x[o] = cpx{fft_from_int(fft_piece(f, centred(raw[2 * o]), p)), fft_from_int(fft_piece(f, centred(raw[2 * o + 1]), p))};
                 }
             }
             fft_spread<G>(x, buf, c.fft_fwd, rank, fresh_tid());
@@ -818,26 +813,54 @@ decrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const uint
                 }
             }
             fft_inverse<CL>(x, buf, tab, fresh_tid());
-            const uint32_t tid = fresh_tid();
-            fft_gather<G>(x, buf, tab, rank, tid);
+            fft_gather<G>(x, buf, tab, rank, fresh_tid());
             if (p + 1 < f.pieces) {
-                fft_park<G>(x, park, f, p, tid);
+                const uint32_t sh = f.shift[p];
+#pragma unroll
+                for (int i0 = 0; i0 < 32; i0 += 4) {
+                    int64_t v[4];
+                    if (p) get4(PARK_AT + 2 * i0, v);
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        const int64_t low = fft_round((i & 1) ? x[(i0 + i) >> 1].im : x[(i0 + i) >> 1].re) << sh;
+                        v[i] = p ? v[i] + low : low;
+                    }
+                    put4(PARK_AT + 2 * i0, v);
+                }
+                if (p + 2 == f.pieces) {
+                    // c0, while nothing else is wanted of the registers
+                    const uint64_t *src = c0 + fresh_tid();
+                    uint64_t raw[32];
+#pragma unroll
+                    for (int i = 0; i < 32; i++) raw[i] = __ldg(src + fft_coefficient<G>(i, rank));
+#pragma unroll
+                    for (int i0 = 0; i0 < 32; i0 += 4) {
+                        const int64_t v[4] = {centred(raw[i0]), centred(raw[i0 + 1]), centred(raw[i0 + 2]), centred(raw[i0 + 3])};
+                        put4(C0_AT + 2 * i0, v);
+                    }
+                }
+                tmem_wait_put();
                 continue;
             }
             const FftJoin join(f, q);
+            const uint64_t *src = c0 + fresh_tid();
 #pragma unroll
-            for (int i0 = 0; i0 < 32; i0 += G::BATCH) {
-                int64_t val[G::BATCH];
+            for (int i0 = 0; i0 < 32; i0 += 4) {
+                int64_t add[4], low[4] = {0, 0, 0, 0};
+                if (f.pieces > 1) {
+                    get4(C0_AT + 2 * i0, add);
+                    get4(PARK_AT + 2 * i0, low);
+                } else {
 #pragma unroll
-                for (int i = 0; i < G::BATCH; i++) val[i] = (int64_t)__ldg(c0 + fft_coefficient<G>(i0 + i, rank) + tid);
-                fft_parked<G>(val, park, f, i0, tid);
+                    for (int i = 0; i < 4; i++) add[i] = centred(__ldg(src + fft_coefficient<G>(i0 + i, rank)));
+                }
 #pragma unroll
-                for (int i = 0; i < G::BATCH; i++) {
+                for (int i = 0; i < 4; i++) {
                     cpx &w = x[(i0 + i) >> 1];
-                    int64_t d = join(val[i], (i & 1) ? w.im : w.re);      // (-q, 2q)
-                    d -= d > half_q ? (int64_t)q : 0;
-                    d -= d > half_q ? (int64_t)q : 0;
-                    d += d < -half_q ? (int64_t)q : 0;
+                    // |the product| <= q / 2 and a little, |c0| <= q / 2
+                    int64_t d = join(low[i] + add[i], (i & 1) ? w.im : w.re);
+                    if (d > half_q) d -= (int64_t)q;
+                    else if (d < -half_q) d += (int64_t)q;
                     ((i & 1) ? w.im : w.re) = __ll2double_rn(d) * inv_delta;
                 }
             }
@@ -856,6 +879,7 @@ decrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const uint
         buffer_free<CL>();
     }
     buffer_wait<CL>();
+    tmem_give(tmem_base);
 }
 
 // ---- launch --------------------------------------------------------------------------
@@ -867,35 +891,6 @@ decrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const uint
     case 15: return FN<2>(__VA_ARGS__);                     \
     default: return FN<3>(__VA_ARGS__);                     \
     }
-
-// as many clusters as the device holds at once, no more than there is work
-template <class G, class K>
-static cudaError_t fft_grid(K kern, int n_sm, size_t want, cudaStream_t s, cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr) {
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM))) return e;
-    cfg = {};
-    cfg.stream = s;
-    cfg.blockDim = dim3(G::NT, 1, 1);
-    cfg.dynamicSmemBytes = G::SMEM;
-    size_t fit = 2 * (size_t)n_sm / G::R;
-    if constexpr (G::CL > 0) {
-        attr->id = cudaLaunchAttributeClusterDimension;
-        attr->val.clusterDim.x = G::R;
-        attr->val.clusterDim.y = 1;
-        attr->val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (want > fit / 2) {
-            cfg.gridDim = dim3(G::R, 1, 1);
-            int clusters = 0;
-            if ((e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg))) return e;
-            if (clusters < 1) return cudaErrorLaunchOutOfResources;
-            if ((size_t)clusters < fit) fit = (size_t)clusters;
-        }
-    }
-    cfg.gridDim = dim3((unsigned)((want < fit ? want : fit) * G::R), 1, 1);
-    return cudaSuccess;
-}
 
 // Asked how many thread blocks fit on an SM, the runtime answers 1 for any kernel that allocates tensor memory;
 // two that take half of it each do run side by side.  This kernel has the same shape without it.
@@ -911,6 +906,7 @@ static cudaError_t setup_ring(CtxDev &c, int n_sm) {
     static_assert(G::SMEM + 4096 <= ENC_ALONE_SMEM - 1024, "two thread blocks to an SM");
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(encrypt_fft_kernel<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, ENC_ALONE_SMEM))) return e;
+    if ((e = cudaFuncSetAttribute(decrypt_fft_kernel<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FftRing<CL>::SMEM))) return e;
     if ((e = cudaFuncSetAttribute(enc_shape_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ENC_ALONE_SMEM))) return e;
     for (uint32_t alone = 0; alone < 2; alone++)
         for (uint32_t S = 1; S <= ENC_MOST; S++) {
@@ -962,19 +958,18 @@ static EncPlan enc_plan(const CtxDev &c, size_t T) {
 }
 
 template <int CL>
-static size_t ring_scratch(const CtxDev &c, int n_sm, size_t T) {
+static size_t ring_scratch(const CtxDev &c, size_t T) {
     using G = EncRing<CL>;
     size_t most = 0;                                   // of any number of ciphertexts up to T
     for (uint32_t S = enc_plan(c, T).S; S <= ENC_MOST; S++) {
         const size_t want = T * ((2 * c.L + S - 1) / S), fit = c.enc_fit[0][S], bytes = (want < fit ? want : fit) * (G::SHARED + S * G::OWN);
         if (bytes > most) most = bytes;
     }
-    const size_t fit = 2 * (size_t)n_sm / FftRing<CL>::R, dec = (T < fit ? T : fit) * FftRing<CL>::SCRATCH;
-    return most > dec ? most : dec;
+    return most;
 }
-size_t fft_work_bytes(const CtxDev &c, int n_sm, size_t T) {
+size_t fft_work_bytes(const CtxDev &c, size_t T) {
     if (T == 0) return 0;
-    FEDHE_FOR_RING(c, ring_scratch, c, n_sm, T)
+    FEDHE_FOR_RING(c, ring_scratch, c, T)
 }
 
 template <int CL>
@@ -1010,20 +1005,32 @@ cudaError_t launch_encrypt(const CtxDev &c, const KeysDev &k, const float *sel, 
 
 template <int CL>
 static cudaError_t launch_decrypt_ring(const CtxDev &c, const KeysDev &k, const uint64_t *ct, uint32_t level, size_t T,
-                                       void *work, int n_sm, double *z, cudaStream_t s) {
+                                       double *z, cudaStream_t s) {
+    using G = FftRing<CL>;
     auto kern = decrypt_fft_kernel<CL>;
-    cudaLaunchConfig_t cfg;
+    const size_t fit = c.enc_fit[0][G::R], clusters = T < fit ? T : fit;       // of the same shape as encryption's
+    if (clusters < 1) return cudaErrorLaunchOutOfResources;
+    cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr;
+    cfg.stream = s;
+    cfg.blockDim = dim3(G::NT, 1, 1);
+    cfg.gridDim = dim3((unsigned)(clusters * G::R), 1, 1);
+    cfg.dynamicSmemBytes = G::SMEM;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = G::R;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = G::R > 1 ? 1 : 0;
     cudaError_t e;
-    if ((e = fft_grid<FftRing<CL>>(kern, n_sm, T, s, cfg, &attr))) return e;
-    if ((e = cudaLaunchKernelEx(&cfg, kern, c, k, ct, level, static_cast<unsigned char *>(work), z, (uint32_t)T))) return e;
+    if ((e = cudaLaunchKernelEx(&cfg, kern, c, k, ct, level, z, (uint32_t)T))) return e;
     return FEDHE_LAUNCHED();
 }
 
 cudaError_t launch_decrypt_fft(const CtxDev &c, const KeysDev &k, const uint64_t *ct, uint32_t level, size_t T,
-                               void *work, int n_sm, double *z, cudaStream_t s) {
+                               double *z, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
-    FEDHE_FOR_RING(c, launch_decrypt_ring, c, k, ct, level, T, work, n_sm, z, s)
+    FEDHE_FOR_RING(c, launch_decrypt_ring, c, k, ct, level, T, z, s)
 }
 
 __global__ void __launch_bounds__(256) gauss_table_kernel(GaussTables *g) { gauss_tables_init(*g, threadIdx.x, blockDim.x); }

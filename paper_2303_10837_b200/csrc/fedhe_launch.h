@@ -30,15 +30,15 @@ cudaError_t launch_decode(const CtxDev &c, const int64_t *d, size_t T, double2 *
 
 // Encode + encrypt ciphertexts t0 .. t0+T-1 (sel and ct point at the first of
 // them).  `work` is scratch of fft_work_bytes() bytes, what the resident thread
-// blocks keep in L2.  n_sm: the device's SM count.
-size_t fft_work_bytes(const CtxDev &c, int n_sm, size_t T);
+// blocks keep in L2.
+size_t fft_work_bytes(const CtxDev &c, size_t T);
 cudaError_t launch_encrypt(const CtxDev &c, const KeysDev &k, const float *sel, void *work, uint32_t t0, size_t T,
                            uint64_t seed, uint32_t client, uint64_t *ct, cudaStream_t s);
 // Once per context, on its device: what the device holds of these kernels (CtxDev::enc_fit).
 cudaError_t fft_setup(CtxDev &c, int n_sm);
-// Decrypt + decode T coefficient-domain ciphertexts; the same scratch.
+// Decrypt + decode T coefficient-domain ciphertexts.
 cudaError_t launch_decrypt_fft(const CtxDev &c, const KeysDev &k, const uint64_t *ct, uint32_t level, size_t T,
-                               void *work, int n_sm, double *z, cudaStream_t s);
+                               double *z, cudaStream_t s);
 // The table of the discrete Gaussian that encryption reads (CtxDev::gauss).
 size_t gauss_table_bytes();
 cudaError_t launch_gauss_table(void *table, cudaStream_t s);
