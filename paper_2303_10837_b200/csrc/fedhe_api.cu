@@ -50,34 +50,6 @@ int upload(he_ctx *ctx, const T *host, size_t count, const T **dev) {
     return HE_OK;
 }
 
-// How the exact products cut the residues of prime q: the top pieces `most` bits wide, the lowest
-// with what remains.  narrow_bits: widest low piece whose product fits 32 bits.
-void split_residues(uint64_t q, int most, int narrow_bits, FftSplit &f) {
-    int bits = 0;
-    while (q >> bits) bits++;
-    f.pieces = (uint32_t)((bits + most - 1) / most);
-    for (uint32_t p = 0; p < FFT_MAX_PIECES; p++) f.shift[p] = p && p < f.pieces ? (uint32_t)(bits - most * (int)(f.pieces - p)) : 0;
-    f.narrow = f.pieces == 2 && (int)f.shift[1] <= narrow_bits;
-    f.top_scale = ldexp(1.0, (int)f.shift[f.pieces - 1]) / (double)q;
-}
-
-// The public key's residues.  A limb of two pieces is cut as low as the low piece's product is sure to fit
-// 32 bits (a coefficient is below N 2^(width - 1)) or else as high as the top one may be wide: then the
-// product, a sum of N independent terms u_k p_k with variance 2^(2 width) / 18, stays below 2^31 (a ternary
-// u_k is strictly sub-Gaussian, so the chance of a larger one is at most 2 exp(-2^62 9 / (N 2^(2 width))):
-// under e^-95 for every width let in here).
-void split_limb(const CtxDev &d, uint64_t q, LimbDev &lb, size_t &words) {
-    const int sure = fft_sure_bits((int)d.logN), wide = fft_wide_bits((int)d.logN);
-    int bits = 0;
-    while (q >> bits) bits++;
-    const bool low_fits = bits > wide && bits - sure + (int)d.logN - 1 < 31;
-    int narrow = 0;
-    while (ldexp(9.0, 62 - (int)d.logN - 2 * (narrow + 1)) >= 95.0) narrow++;
-    split_residues(q, low_fits ? sure : wide, narrow, lb.split);
-    lb.fft_key = words;
-    words += 2 * (size_t)lb.split.pieces * (d.N / 2);
-}
-
 size_t work_bytes(const he_ctx *ctx, size_t T) { return 2 * T * (size_t)ctx->dev.N * sizeof(uint64_t); }
 
 }  // namespace
@@ -134,13 +106,7 @@ int he_ctx_create(const he_params *p, he_ctx **out) {
         d.LOGB = d.logN <= 14 ? d.logN : 13;   // longer transforms: 2^13 blocks, two per SM
         d.A = d.logN - d.LOGB;
         const uint64_t ql = p->q[p->L - 1];
-        size_t fft_words = 0;
-        split_residues(p->q[0], fft_sure_bits((int)d.logN), 30 - (int)d.logN + 1, d.dec_split);
-        d.term_limit = INT64_MAX;
         for (uint32_t j = 0; j < p->L && rc == HE_OK; j++) {
-            split_limb(d, p->q[j], d.limb[j], fft_words);
-            d.fft_pieces += d.limb[j].split.pieces;
-            if ((int64_t)(p->q[j] / 4) < d.term_limit) d.term_limit = (int64_t)(p->q[j] / 4);
             HostLimb hl;
             host_build_limb(d.N, p->q[j], hl);
             LimbDev &ld = d.limb[j];
@@ -175,6 +141,7 @@ int he_ctx_create(const he_params *p, he_ctx **out) {
         host_unit_roots(d.N, roots);
         host_slot_twiddles(d.N, roots, ftw);
         rc = upload(ctx, reinterpret_cast<const double2 *>(ftw.data()), ftw.size() / 2, &d.ftw);
+        fft_cut(d);
         host_fft_tables(d.N, roots, fwd, inv, slot_of);
         if (rc == HE_OK) rc = upload(ctx, reinterpret_cast<const root_t *>(fwd.data()), fwd.size() / 2, &d.fft_fwd);
         if (rc == HE_OK) rc = upload(ctx, reinterpret_cast<const root_t *>(inv.data()), inv.size() / 2, &d.fft_inv);

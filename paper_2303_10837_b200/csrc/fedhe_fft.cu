@@ -269,15 +269,15 @@ struct EncRing {
     static constexpr size_t SMEM = (size_t)NB * 16 + (size_t)Tab::WORDS * 16 + (E_IN_SMEM ? N : 0);
 };
 
-// first unit (component, limb) of a ciphertext that begins at or after `pos` pieces
+// first unit of a ciphertext, of both components, that begins at or after `pos` products
 __device__ __forceinline__ uint32_t fft_unit_at(const CtxDev &c, uint32_t pos) {
     uint32_t half = pos >= c.fft_pieces ? 1 : 0, rest = pos - half * c.fft_pieces, j = 0;
     while (rest) {
-        const uint32_t p = c.limb[j].split.pieces;
+        const uint32_t p = c.enc_unit[j].products;
         rest = rest > p ? rest - p : 0;
         j++;
     }
-    return half * c.L + j;
+    return half * c.enc_units + j;
 }
 
 // value i (column, row, real or imaginary part) of a thread's columns from r0: its coefficient less the thread's number
@@ -379,17 +379,22 @@ __device__ __forceinline__ void enc_park(const cpx (&v)[G::COLUMNS][G::R], unsig
 }
 template <class G>
 __device__ __forceinline__ void enc_parked(int64_t (&val)[G::K], const unsigned char *park, uint32_t tm, const FftSplit &f,
-                                           uint32_t r0, uint32_t tid) {
+                                           uint32_t of_pair, uint32_t r0, uint32_t tid) {
     const uint32_t i0 = r0 * G::R * 2;
+    // the low piece's product: the word itself, or, of a pair, its lower 16 bits (signed) or what they leave
+    auto low_of = [&](int w) {
+        if (of_pair == 0) return w;
+        return of_pair == 1 ? (int)(int16_t)w : (w - (int)(int16_t)w) >> 16;
+    };
     if (f.narrow) {
         if constexpr (G::PARK_TMEM) {
             uint32_t w[8];
             tmem_get8(tm + G::PARK_AT + i0, w);
 #pragma unroll
-            for (int i = 0; i < G::K; i++) val[i] += (int)w[i];
+            for (int i = 0; i < G::K; i++) val[i] += low_of((int)w[i]);
         } else {
 #pragma unroll
-            for (int i = 0; i < G::K; i++) val[i] += __ldcg(reinterpret_cast<const int *>(park) + (i0 + i) * G::NT + tid);
+            for (int i = 0; i < G::K; i++) val[i] += low_of(__ldcg(reinterpret_cast<const int *>(park) + (i0 + i) * G::NT + tid));
         }
     } else if (f.pieces > 1) {
 #pragma unroll
@@ -410,7 +415,8 @@ __device__ __forceinline__ void enc_parked(int64_t (&val)[G::K], const unsigned 
 // The clusters fetch ciphertexts as they finish (with equal shares dealt out beforehand the slowest took 16 %
 // longer than the mean).  Of the `rem` ciphertexts after the last whole round each is cut in `parts`: clusters that
 // all prepare it and share its units.
-template <int CL>
+// PAIRS: some units are of two limbs (the code for both kinds costs the others 1.5 %).
+template <int CL, bool PAIRS>
 __global__ void __launch_bounds__(FftLay::NT, 2)
 encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const float *sel, unsigned char *work,
                    uint32_t t0, uint64_t seed, uint32_t client, uint64_t *ct, uint32_t T, uint32_t S, uint32_t most_parts) {
@@ -479,7 +485,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
         const uint32_t first = fft_unit_at(c, pieces * part / of), last = fft_unit_at(c, pieces * (part + 1) / of);
         const uint32_t unit_end = fft_unit_at(c, pieces * (part * S + rank + 1) / (of * S));
         uint32_t unit = fft_unit_at(c, pieces * (part * S + rank) / (of * S));
-        const bool c0_too = first < c.L, c1_too = last > c.L;
+        const bool c0_too = first < c.enc_units, c1_too = last > c.enc_units;
         const uint32_t t = t0 + tl;
 
         // ---- preparation: u, four columns of one half at a time ----
@@ -591,20 +597,23 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
 
         // ---- this block's units ----
         auto key_of = [&](uint32_t u, uint32_t pb) {
-            const uint32_t comp = u >= c.L ? 1 : 0;
-            const LimbDev &lb = c.limb[u - comp * c.L];
-            return k.fft_pk + lb.fft_key + ((size_t)comp * lb.split.pieces * R + pb) * NB;
+            const uint32_t comp = u >= c.enc_units ? 1 : 0;
+            const EncUnit &e = c.enc_unit[u - comp * c.enc_units];
+            return k.fft_pk + e.fft_key + ((size_t)comp * e.products * R + pb) * NB;
         };
         if constexpr (!(G::E_IN_SMEM)) __syncthreads();   // the buffer's last readers are done
         if (threadIdx.x == 0) key_fetch(buf, key_of(unit, 0), &key_bar);
 #pragma unroll 1
         for (; unit < unit_end; unit++) {
-            const uint32_t comp = unit >= c.L ? 1 : 0, j = unit - comp * c.L;
-            const FftSplit &f = c.limb[j].split;
-            const uint64_t q = c.limb[j].q;
+            const uint32_t comp = unit >= c.enc_units ? 1 : 0;
+            const EncUnit &e = c.enc_unit[unit - comp * c.enc_units];
+            const bool pair = PAIRS && e.limb2 != NO_LIMB;
 #pragma unroll 1
-            for (uint32_t pb = 0; pb < f.pieces * R; pb++) {
+            for (uint32_t pb = 0; pb < e.products * R; pb++) {
                 const uint32_t p = pb >> CL, b = pb & (R - 1);
+                const uint32_t j = pair && p == 2 ? e.limb2 : e.limb;
+                const FftSplit &f = c.limb[j].split;
+                const uint64_t q = c.limb[j].q;
                 cpx x[16];
                 {
                     const uint32_t tid = fresh_tid();
@@ -633,11 +642,11 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
                     key_parity ^= 1u;
                 }
                 // the next key may come as soon as the buffer is read; where a column loop needs the buffer, after it
-                const bool more = pb + 1 < f.pieces * R || unit + 1 < unit_end;
+                const bool more = pb + 1 < e.products * R || unit + 1 < unit_end;
                 auto fetch_next = [&]() {
                     __syncthreads();
                     if (more && threadIdx.x == 0)
-                        key_fetch(buf, pb + 1 < f.pieces * R ? key_of(unit, pb + 1) : key_of(unit + 1, 0), &key_bar);
+                        key_fetch(buf, pb + 1 < e.products * R ? key_of(unit, pb + 1) : key_of(unit + 1, 0), &key_bar);
                 };
                 fft_inverse<0>(x, buf, tab, fresh_tid(), [&] {
                     if (R <= 2 || b + 1 < R) fetch_next();
@@ -653,7 +662,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
                     for (int r = 0; r < 16; r++) buf[r * NT + tid] = make_double2(x[r].re, x[r].im);
                 }
                 constexpr int K = G::K;
-                if (p + 1 < f.pieces) {
+                if (pair ? p == 0 : p + 1 < f.pieces) {
 #pragma unroll(R <= 2 ? 16 : 1)
                     for (uint32_t r0 = 0; r0 < 16; r0 += G::COLUMNS) {
                         cpx v[G::COLUMNS][R];
@@ -688,7 +697,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
 #pragma unroll
                     for (int i = 0; i < K; i++) val[i] = big && comp == 0 ? 0 : next[i];
                     if (r0 + G::COLUMNS < 16) terms_of(next, r0 + G::COLUMNS);
-                    enc_parked<G>(val, park, tm, f, r0, tid);
+                    enc_parked<G>(val, park, tm, f, pair ? p : 0, r0, tid);
                     cpx v[G::COLUMNS][R];
                     enc_columns<G>(v, x, buf, wait, tm, tab, r0, tid);
                     // streaming stores: the finished ciphertext should not push tables and scratch out of L2
@@ -892,6 +901,70 @@ decrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const uint
     default: return FN<3>(__VA_ARGS__);                     \
     }
 
+// ---- how residues are cut -----------------------------------------------------------
+
+static int bits_of(uint64_t q) {
+    int bits = 0;
+    while (q >> bits) bits++;
+    return bits;
+}
+// the top pieces `most` bits wide, the lowest with what remains; narrow_bits: widest low piece whose product fits 32 bits
+static void cut_residues(uint64_t q, int most, int narrow_bits, FftSplit &f) {
+    const int bits = bits_of(q);
+    f.pieces = (uint32_t)((bits + most - 1) / most);
+    for (uint32_t p = 0; p < FFT_MAX_PIECES; p++) f.shift[p] = p && p < f.pieces ? (uint32_t)(bits - most * (int)(f.pieces - p)) : 0;
+    f.narrow = f.pieces == 2 && (int)f.shift[1] <= narrow_bits;
+    f.top_scale = ldexp(1.0, (int)f.shift[f.pieces - 1]) / (double)q;
+}
+// Widest random piece whose product stays below 2^(t - 1).  A coefficient is a sum of N independent terms u_k p_k,
+// strictly sub-Gaussian with variance 2^(2 width) / 18 each, so the chance of a larger one is at most
+// 2 exp(-9 2^(2 t - 2) / (N 2^(2 width))); `least` is what the exponent has to reach.
+static int random_bits(int logN, int t, double least) {
+    int w = 0;
+    while (ldexp(9.0, 2 * t - 2 - logN - 2 * (w + 1)) >= least) w++;
+    return w;
+}
+
+// Decryption cuts for any c1.  Of the public key's limbs, two whose low pieces have products of 16 bits (up to 6 bits wide
+// for N = 2^15, at 12 standard deviations: under 2^-102 a coefficient) share one product for both: three instead of
+// four, for instance for primes of 45 bits.  Another limb of two pieces is cut as low as the low piece's product is sure
+// to fit 32 bits (a coefficient is below N 2^(width - 1)), or else as high as the top one may be wide, where it
+// fits all the same (exponent 95: under 2^-136).
+void fft_cut(CtxDev &c) {
+    const int logN = (int)c.logN, sure = fft_sure_bits(logN), wide = fft_wide_bits(logN);
+    cut_residues(c.limb[0].q, sure, 31 - logN, c.dec_split);
+    c.term_limit = INT64_MAX;
+    uint32_t waiting = NO_LIMB;                        // unit of a limb that could share its low product
+    size_t words = 0;
+    c.enc_units = 0;
+    for (uint32_t j = 0; j < c.L; j++) {
+        const uint64_t q = c.limb[j].q;
+        if ((int64_t)(q / 4) < c.term_limit) c.term_limit = (int64_t)(q / 4);
+        const int bits = bits_of(q);
+        const bool shares = bits > wide && bits - wide <= random_bits(logN, 16, 72.0);
+        const bool low_fits = bits > wide && bits - sure + logN - 1 < 31;
+        if (shares && waiting != NO_LIMB) {
+            EncUnit &e = c.enc_unit[waiting];
+            cut_residues(c.limb[e.limb].q, wide, random_bits(logN, 32, 95.0), c.limb[e.limb].split);
+            cut_residues(q, wide, random_bits(logN, 32, 95.0), c.limb[j].split);
+            e.limb2 = j;
+            e.products = 3;
+            waiting = NO_LIMB;
+            continue;
+        }
+        cut_residues(q, low_fits ? sure : wide, random_bits(logN, 32, 95.0), c.limb[j].split);
+        c.enc_unit[c.enc_units] = EncUnit{j, NO_LIMB, c.limb[j].split.pieces, 0};
+        if (shares) waiting = c.enc_units;
+        c.enc_units++;
+    }
+    c.fft_pieces = 0;
+    for (uint32_t u = 0; u < c.enc_units; u++) {
+        c.enc_unit[u].fft_key = words;
+        words += 2 * (size_t)c.enc_unit[u].products * (c.N / 2);
+        c.fft_pieces += c.enc_unit[u].products;
+    }
+}
+
 // Asked how many thread blocks fit on an SM, the runtime answers 1 for any kernel that allocates tensor memory;
 // two that take half of it each do run side by side.  This kernel has the same shape without it.
 __global__ void __launch_bounds__(FftLay::NT, 2) enc_shape_kernel() {}
@@ -905,7 +978,10 @@ static cudaError_t setup_ring(CtxDev &c, int n_sm) {
     using G = EncRing<CL>;
     static_assert(G::SMEM + 4096 <= ENC_ALONE_SMEM - 1024, "two thread blocks to an SM");
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(encrypt_fft_kernel<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, ENC_ALONE_SMEM))) return e;
+    const bool pairs = c.enc_units < c.L;
+    if ((e = cudaFuncSetAttribute(pairs ? encrypt_fft_kernel<CL, true> : encrypt_fft_kernel<CL, false>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, ENC_ALONE_SMEM)))
+        return e;
     if ((e = cudaFuncSetAttribute(decrypt_fft_kernel<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FftRing<CL>::SMEM))) return e;
     if ((e = cudaFuncSetAttribute(enc_shape_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ENC_ALONE_SMEM))) return e;
     for (uint32_t alone = 0; alone < 2; alone++)
@@ -934,14 +1010,14 @@ cudaError_t fft_setup(CtxDev &c, int n_sm) { FEDHE_FOR_RING(c, setup_ring, c, n_
 struct EncPlan { uint32_t S, alone, clusters, parts; };
 
 // With ciphertexts enough to fill the device: as many blocks as the ciphertext has of 2^12 points, or the next
-// number below that shares its 2 L units out evenly.  With fewer, larger clusters, by these measurements (us, L = 3 or 4):
+// number below that shares its units out evenly.  With fewer, larger clusters, by these measurements (us, L = 3 or 4):
 //   N = 8192, 25 ciphertexts: 1, 2, 3, 4, 8 blocks 79, 52, 43, 40, 43 (8 of them share SMs); 60: 2, 4 blocks 52, 55;
 //     100: 1, 2 blocks 81, 72
 //   N = 16384, 40: 2, 3, 6 blocks 110, 86, 75; 60: 2, 4 blocks 111, 92
 // so the largest clusters that hold all ciphertexts at one block to an SM, if they can do the 2 R blocks of the
 // preparation side by side, and else the largest that hold them at two.
 static EncPlan enc_plan(const CtxDev &c, size_t T) {
-    const uint32_t R = 1u << (c.logN - 13), units = 2 * c.L, most = units < ENC_MOST ? units : ENC_MOST;
+    const uint32_t R = 1u << (c.logN - 13), units = 2 * c.enc_units, most = units < ENC_MOST ? units : ENC_MOST;
     uint32_t base = R < most ? R : most;
     while (units % base) base--;
     EncPlan p = {base, 0, 0, (units + base - 1) / base};
@@ -962,7 +1038,7 @@ static size_t ring_scratch(const CtxDev &c, size_t T) {
     using G = EncRing<CL>;
     size_t most = 0;                                   // of any number of ciphertexts up to T
     for (uint32_t S = enc_plan(c, T).S; S <= ENC_MOST; S++) {
-        const size_t want = T * ((2 * c.L + S - 1) / S), fit = c.enc_fit[0][S], bytes = (want < fit ? want : fit) * (G::SHARED + S * G::OWN);
+        const size_t want = T * ((2 * c.enc_units + S - 1) / S), fit = c.enc_fit[0][S], bytes = (want < fit ? want : fit) * (G::SHARED + S * G::OWN);
         if (bytes > most) most = bytes;
     }
     return most;
@@ -991,7 +1067,7 @@ static cudaError_t launch_encrypt_ring(const CtxDev &c, const KeysDev &k, const 
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     cudaError_t e;
-    if ((e = cudaLaunchKernelEx(&cfg, encrypt_fft_kernel<CL>, c, k, sel, static_cast<unsigned char *>(work), t0, seed, client, ct,
+    if ((e = cudaLaunchKernelEx(&cfg, c.enc_units < c.L ? encrypt_fft_kernel<CL, true> : encrypt_fft_kernel<CL, false>, c, k, sel, static_cast<unsigned char *>(work), t0, seed, client, ct,
                                 (uint32_t)T, p.S, p.parts)))
         return e;
     return FEDHE_LAUNCHED();
@@ -1043,7 +1119,7 @@ cudaError_t launch_gauss_table(void *table, cudaStream_t s) {
 // ---- key tables ------------------------------------------------------------------------
 
 // One thread block per (polynomial, block of its transform).  `pk`: the public key's coefficients
-// [2][L][N], canonical; polynomial number -> (limb, component, piece) in the order of the tables;
+// [2][L][N], canonical; polynomial number -> (unit, component, product) in the order of the tables;
 // the last one is the secret key.
 template <int CL>
 __global__ void __launch_bounds__(FftLay::NT)
@@ -1053,16 +1129,20 @@ fft_key_kernel(const __grid_constant__ CtxDev c, const uint64_t *pk, const int8_
     extern __shared__ __align__(128) unsigned char smem[];
     double2 *buf = reinterpret_cast<double2 *>(smem);
     const uint32_t tid = threadIdx.x, b = blockIdx.x % R;
-    uint32_t poly = blockIdx.x / R, j = 0;
-    while (j < c.L && poly >= 2 * c.limb[j].split.pieces) poly -= 2 * c.limb[j++].split.pieces;
-    const bool secret = j == c.L;
-    const LimbDev &lb = c.limb[secret ? 0 : j];
-    const uint32_t comp = secret ? 0 : poly / lb.split.pieces, piece = secret ? 0 : poly % lb.split.pieces;
-    const uint64_t *src = pk + ((size_t)comp * c.L + (secret ? 0 : j)) * c.N;
+    uint32_t poly = blockIdx.x / R, u = 0;
+    while (u < c.enc_units && poly >= 2 * c.enc_unit[u].products) poly -= 2 * c.enc_unit[u++].products;
+    const bool secret = u == c.enc_units;
+    const EncUnit &e = c.enc_unit[secret ? 0 : u];
+    const uint32_t comp = secret ? 0 : poly / e.products, product = secret ? 0 : poly % e.products;
+    auto piece = [&](uint32_t j, uint32_t of, uint32_t i) {
+        const uint64_t v = pk[((size_t)comp * c.L + j) * c.N + i], q = c.limb[j].q;
+        return fft_piece(c.limb[j].split, v > q / 2 ? (int64_t)(v - q) : (int64_t)v, of);
+    };
     auto value = [&](uint32_t i) {
         if (secret) return (double)s8[i];
-        const uint64_t v = src[i];
-        return (double)fft_piece(lb.split, v > lb.q / 2 ? (int64_t)(v - lb.q) : (int64_t)v, piece);
+        if (e.limb2 == NO_LIMB) return (double)piece(e.limb, product, i);
+        if (product == 0) return (double)(piece(e.limb, 0, i) + 65536 * piece(e.limb2, 0, i));
+        return (double)piece(product == 1 ? e.limb : e.limb2, 1, i);
     };
     const OuterPath<CL> outer(c.fft_fwd, b);
     // the columns, in a loop, wait in the thread's own words of the buffer
@@ -1081,7 +1161,7 @@ fft_key_kernel(const __grid_constant__ CtxDev c, const uint64_t *pk, const int8_
 #pragma unroll
     for (int r = 0; r < 16; r++) x[r] = cpx{buf[tid + NT * r].x, buf[tid + NT * r].y};
     fft_forward<CL, true>(x, buf, c.fft_fwd, b, tid);
-    double2 *dst = (secret ? fft_s : fft_pk + lb.fft_key + (size_t)poly * n) + (size_t)b * NB + tid;
+    double2 *dst = (secret ? fft_s : fft_pk + e.fft_key + (size_t)poly * n) + (size_t)b * NB + tid;
     const double scale = 1.0 / n;                  // a power of two
 #pragma unroll
     for (int r = 0; r < 16; r++) dst[r * NT] = make_double2(x[r].re * scale, x[r].im * scale);

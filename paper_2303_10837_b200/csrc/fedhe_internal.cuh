@@ -31,6 +31,16 @@ HD int64_t fft_piece(const FftSplit &f, int64_t v, uint32_t p) {
     return v;
 }
 
+// What an encryption computes together: a limb, by the products of its pieces from the lowest to the top one, or
+// two limbs whose low pieces are a few bits wide, by one product of both of them, the first's plus 2^16 times
+// the second's, and their top ones.
+constexpr uint32_t NO_LIMB = 0xffffffffu;
+struct EncUnit {
+    uint32_t limb, limb2;        // limb2 = NO_LIMB: a single one
+    uint32_t products;
+    size_t fft_key;              // first word of its key tables: [2 components][products][n]
+};
+
 // Per-prime constants and table pointers, passed to kernels by value.
 struct LimbDev {
     uint64_t q;          // the prime
@@ -48,7 +58,6 @@ struct LimbDev {
     double qd, qi;       // q and 1/q rounded
     double ninv_d, wn_d; // 1/N and (inverse twiddle of stage 0)/N
     FftSplit split;      // of the public key's residues for the exact products by complex transforms
-    size_t fft_key;      // first word of the limb's key tables: [2 components][pieces][n]
 };
 
 // the pieces of a limb that a transform in arithmetic M needs
@@ -83,7 +92,8 @@ struct CtxDev {
     const root_t *fft_fwd, *fft_inv;   // complex transforms of the exact products (fedhe_fft.cuh)
     const uint32_t *slot_of;           // slot of every value that the forward transform leaves
     FftSplit dec_split;                // of c1 on limb 0, for any c1
-    uint32_t fft_pieces;               // of all limbs of a public-key half
+    uint32_t enc_units, fft_pieces;    // units and products of a public-key half
+    EncUnit enc_unit[HE_MAX_LIMBS];
     int64_t term_limit;                // a quarter of the smallest prime
     uint16_t enc_fit[2][ENC_MOST + 1]; // clusters of a size that the device holds: two blocks to an SM, one
     const void *gauss;   // GaussTables

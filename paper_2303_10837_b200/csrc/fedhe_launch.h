@@ -34,7 +34,8 @@ cudaError_t launch_decode(const CtxDev &c, const int64_t *d, size_t T, double2 *
 size_t fft_work_bytes(const CtxDev &c, size_t T);
 cudaError_t launch_encrypt(const CtxDev &c, const KeysDev &k, const float *sel, void *work, uint32_t t0, size_t T,
                            uint64_t seed, uint32_t client, uint64_t *ct, cudaStream_t s);
-// Once per context, on its device: what the device holds of these kernels (CtxDev::enc_fit).
+// Once per context: how the products cut the residues (from the primes); then, on its device, what the device holds of these kernels (CtxDev::enc_fit).
+void fft_cut(CtxDev &c);
 cudaError_t fft_setup(CtxDev &c, int n_sm);
 // Decrypt + decode T coefficient-domain ciphertexts.
 cudaError_t launch_decrypt_fft(const CtxDev &c, const KeysDev &k, const uint64_t *ct, uint32_t level, size_t T,
