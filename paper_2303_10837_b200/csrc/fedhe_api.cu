@@ -919,9 +919,10 @@ static int round_host_queued(he_ctx *ctx, const he_keys *keys, const he_mask *ma
     int rc;
     if ((rc = round_host_streams(ctx)) != HE_OK) return rc;
 
-    // Ranges: a twelfth each, but not so small that launches count, the last one halved twice because
+    // Ranges: a twelfth each, but so large that a client's part takes longer to come up (76 us for 2^20 parameters)
+    // than its few ciphertexts take to be encrypted (45 us), the last one halved twice because
     // nothing hides its way through the chip and back.
-    const size_t UNIT = 8192, least = (size_t)1 << 18;
+    const size_t UNIT = 8192, least = (size_t)1 << 20;
     size_t len = (P + 11) / 12 > least ? (P + 11) / 12 : least;
     len = (len + UNIT - 1) / UNIT * UNIT;
     std::vector<size_t> cut = {0};                    // boundaries
@@ -971,41 +972,39 @@ static int round_host_queued(he_ctx *ctx, const he_keys *keys, const he_mask *ma
 
     CU(cudaEventRecord(ctx->ev_free[0], st));       // earlier work on `st` may still use the buffers
     CU(cudaEventRecord(ctx->ev_free[1], st));
-    auto upload = [&](size_t c) -> int {
-        const int b = (int)(c & 1);
-        CU(cudaStreamWaitEvent(ctx->copy_stream, ctx->ev_free[b], 0));
-        for (int i = 0; i < C; i++)
-            CU(cudaMemcpyAsync(xbuf[b] + (size_t)i * b_x, xs_host[i] + cut[c], (cut[c + 1] - cut[c]) * sizeof(float),
-                               cudaMemcpyHostToDevice, ctx->copy_stream));
-        CU(cudaEventRecord(ctx->ev_ready[b], ctx->copy_stream));
-        return HE_OK;
-    };
-    if ((rc = upload(0)) != HE_OK) return rc;
     std::vector<const uint64_t *> cptr(C);
     std::vector<const float *> rptr(C);
     size_t t = 0, r = 0, home = 0;                    // ciphertexts, remainder entries and ranges that are done
     for (size_t c = 0; c < R; c++) {
         const int b = (int)(c & 1);
-        CU(cudaStreamWaitEvent(st, ctx->ev_ready[b], 0));
-        if (c + 1 < R && (rc = upload(c + 1)) != HE_OK) return rc;
+        const size_t end = ready(c), now = end - t < Tc ? end - t : Tc;
+        auto encrypt = [&](int i, size_t tc) -> int {
+            uint64_t *ci = cts + (size_t)i * Tc * ctw;
+            cptr[i] = ci;
+            return he_encrypt_range(ctx, keys, sel[i] + t * n, t, tc, enc_seed, (uint32_t)i, ci, stream);
+        };
+        CU(cudaStreamWaitEvent(ctx->copy_stream, ctx->ev_free[b], 0));
         for (int i = 0; i < C; i++) {
-            CU(launch_pack_range(mask, reinterpret_cast<const float *>(xbuf[b] + (size_t)i * b_x), cut[c], cut[c + 1] - cut[c], sel[i],
-                                 restlen ? rest[i] : nullptr, st));
+            // client by client: one's ciphertexts are encrypted while the next one's part comes up (a wait
+            // takes the event's latest record at the time of the call)
+            float *x = reinterpret_cast<float *>(xbuf[b] + (size_t)i * b_x);
+            CU(cudaMemcpyAsync(x, xs_host[i] + cut[c], (cut[c + 1] - cut[c]) * sizeof(float), cudaMemcpyHostToDevice, ctx->copy_stream));
+            CU(cudaEventRecord(ctx->ev_ready[b], ctx->copy_stream));
+            CU(cudaStreamWaitEvent(st, ctx->ev_ready[b], 0));
+            CU(launch_pack_range(mask, x, cut[c], cut[c + 1] - cut[c], sel[i], restlen ? rest[i] : nullptr, st));
             if (c + 1 == R) CU(launch_zero(sel[i] + k, padded - k, st));
+            if (i + 1 == C) CU(cudaEventRecord(ctx->ev_free[b], st));
+            if (now && (rc = encrypt(i, now)) != HE_OK) return rc;
         }
-        CU(cudaEventRecord(ctx->ev_free[b], st));
-        for (const size_t end = ready(c); t < end;) {
-            const size_t tc = end - t < Tc ? end - t : Tc;
-            for (int i = 0; i < C; i++) {
-                uint64_t *ci = cts + (size_t)i * Tc * ctw;
-                rc = he_encrypt_range(ctx, keys, sel[i] + t * n, t, tc, enc_seed, (uint32_t)i, ci, stream);
-                if (rc != HE_OK) return rc;
-                cptr[i] = ci;
-            }
+        for (size_t tc = now; t < end; tc = end - t < Tc ? end - t : Tc) {
             rc = he_weighted_aggregate(ctx, cptr.data(), alpha_host, C, tc, agg, stream);
             if (rc != HE_OK) return rc;
             if ((rc = he_decrypt(ctx, keys, agg, tc, z + t * n, stream)) != HE_OK) return rc;
             t += tc;
+            if (t == end) break;
+            const size_t more = end - t < Tc ? end - t : Tc;
+            for (int i = 0; i < C; i++)
+                if ((rc = encrypt(i, more)) != HE_OK) return rc;
         }
         // the remainder so far, in whole vectors until the end
         const size_t r_end = c + 1 == R ? restlen : (cut[c + 1] - before[c + 1]) & ~(size_t)3;
