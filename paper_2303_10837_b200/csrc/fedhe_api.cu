@@ -919,18 +919,30 @@ static int round_host_queued(he_ctx *ctx, const he_keys *keys, const he_mask *ma
     int rc;
     if ((rc = round_host_streams(ctx)) != HE_OK) return rc;
 
-    // Ranges: a twelfth each, but so large that a client's part takes longer to come up (76 us for 2^20 parameters)
-    // than its few ciphertexts take to be encrypted (45 us), the last one halved twice because
-    // nothing hides its way through the chip and back.
-    const size_t UNIT = 8192, least = (size_t)1 << 20;
-    size_t len = (P + 11) / 12 > least ? (P + 11) / 12 : least;
-    len = (len + UNIT - 1) / UNIT * UNIT;
+    // Equal ranges, as many as make the call shortest by this account (us): a client's part of a range comes up
+    // at 55 GB/s; its ciphertexts take 35, 55, 115 or 200 (N = 2^13 .. 2^16) and 0.4, 1, 4 or 9 each; a range costs
+    // 50 besides; after the last upload come one client's ciphertexts, and the range's download.  (With ranges of
+    // 2^20 parameters, 12 clients and 3 M parameters at N = 2^15 spent 5.0 instead of 3.5 ms on short encryptions.)
+    const size_t UNIT = 8192;
+    const double PCIE = 55e3, first_ct[4] = {35, 55, 115, 200}, each_ct[4] = {0.4, 1.0, 4.0, 9.0};
+    const int ring = (int)d.logN - 13;
+    auto part_us = [&](double params) { return 4.0 * params / PCIE; };
+    auto encrypt_us = [&](double params) { return T ? first_ct[ring] + each_ct[ring] * (double)T * params / (double)P : 0.0; };
+    size_t ranges = 1;
+    double best = 0;
+    for (size_t m = 1; m <= 32 && m * UNIT <= P + UNIT; m++) {
+        const double params = (double)P / (double)m, part = part_us(params), enc = encrypt_us(params);
+        const double us = (double)m * (C * (part > enc ? part : enc) + 50.0) + enc + 2.0 * part;
+        if (m == 1) best = 0.95 * us;                 // a cut has to be worth its while
+        else if (us < best) { best = us; ranges = m; }
+    }
+    size_t len = ((P + ranges - 1) / ranges + UNIT - 1) / UNIT * UNIT;
     std::vector<size_t> cut = {0};                    // boundaries
     while (P - cut.back() > len) cut.push_back(cut.back() + len);
-    for (int half = 0; half < 2; half++) {
-        const size_t left = (P - cut.back()) / 2 / UNIT * UNIT;
-        if (cut.size() > 1 && left >= least / 2) cut.push_back(cut.back() + left);
-    }
+    // nothing hides the last range's way through the chip and back
+    for (size_t left = (P - cut.back()) / 2 / UNIT * UNIT; cut.size() > 1 && left && encrypt_us((double)left) <= part_us((double)left);
+         left = left / 2 / UNIT * UNIT)
+        cut.push_back(cut.back() + left);
     cut.push_back(P);
     const size_t R = cut.size() - 1;
     size_t most = 0;
