@@ -1,5 +1,5 @@
-// Encryption into the transform-domain wire format (part 3 of the kernels); the coefficient
-// format is in fedhe_fft.cu.
+// Encryption into the transform-domain wire format, and into the coefficient format by passes where that is
+// faster (part 3 of the kernels); the coefficient format otherwise is in fedhe_fft.cu.
 #include "fedhe_kernels.cuh"
 #include "fedhe_slots.cuh"
 
@@ -79,7 +79,7 @@ encrypt_fused_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const fl
     int8_t *se0 = su + B, *se1 = se0 + B;
     const uint32_t tid = threadIdx.x;
     __shared__ GaussTables gt;
-    gauss_tables_init(gt, tid, blockDim.x);
+    gauss_tables_load(gt, c.gauss, tid, blockDim.x);
 
     // Work units are (ciphertext, limb) pairs in ciphertext-major order, dealt
     // evenly to the blocks of the grid (one block per SM), so that the last
@@ -104,14 +104,9 @@ encrypt_fused_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const fl
                 *reinterpret_cast<char4 *>(su + bswz(4 * b)) = v;
             }
             for (uint32_t b = tid; b < B / 2; b += RT) {
-                u32x4 w0 = stream_block(seed, b, t, client, TAG_ENC_E0);
-                u32x4 w1 = stream_block(seed, b, t, client, TAG_ENC_E1);
-                char2 a = make_char2((signed char)gauss_from_u64(gt, (uint64_t)w0.x | ((uint64_t)w0.y << 32)),
-                                     (signed char)gauss_from_u64(gt, (uint64_t)w0.z | ((uint64_t)w0.w << 32)));
-                char2 e = make_char2((signed char)gauss_from_u64(gt, (uint64_t)w1.x | ((uint64_t)w1.y << 32)),
-                                     (signed char)gauss_from_u64(gt, (uint64_t)w1.z | ((uint64_t)w1.w << 32)));
-                *reinterpret_cast<char2 *>(se0 + bswz(2 * b)) = a;
-                *reinterpret_cast<char2 *>(se1 + bswz(2 * b)) = e;
+                const int2 a = gauss_pair(gt, seed, b, t, client, TAG_ENC_E0), e = gauss_pair(gt, seed, b, t, client, TAG_ENC_E1);
+                *reinterpret_cast<char2 *>(se0 + bswz(2 * b)) = make_char2((signed char)a.x, (signed char)a.y);
+                *reinterpret_cast<char2 *>(se1 + bswz(2 * b)) = make_char2((signed char)e.x, (signed char)e.y);
             }
             // the ciphertext's message: slot transform, scaling and rounding in the limb buffer
             if (encode_in_block<LF>(c, sel + (size_t)tl * (B / 2), sm, mblk)) atomicOr(c.status, 1);
@@ -211,7 +206,7 @@ encrypt_fused2_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const f
     int8_t *se0 = su + B, *se1 = se0 + B;
     const uint32_t tid = threadIdx.x;
     __shared__ GaussTables gt_tab;
-    gauss_tables_init(gt_tab, tid, blockDim.x);
+    gauss_tables_load(gt_tab, c.gauss, tid, blockDim.x);
 
     const uint64_t units = (uint64_t)T * c.L;
     const uint32_t u_begin = (uint32_t)(units * blockIdx.x / gridDim.x);
@@ -232,14 +227,9 @@ encrypt_fused2_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const f
                 *reinterpret_cast<char4 *>(su + bswz(4 * b)) = v;
             }
             for (uint32_t b = tid; b < B / 2; b += RT) {
-                u32x4 w0 = stream_block(seed, b, t, client, TAG_ENC_E0);
-                u32x4 w1 = stream_block(seed, b, t, client, TAG_ENC_E1);
-                char2 a = make_char2((signed char)gauss_from_u64(gt_tab, (uint64_t)w0.x | ((uint64_t)w0.y << 32)),
-                                     (signed char)gauss_from_u64(gt_tab, (uint64_t)w0.z | ((uint64_t)w0.w << 32)));
-                char2 e = make_char2((signed char)gauss_from_u64(gt_tab, (uint64_t)w1.x | ((uint64_t)w1.y << 32)),
-                                     (signed char)gauss_from_u64(gt_tab, (uint64_t)w1.z | ((uint64_t)w1.w << 32)));
-                *reinterpret_cast<char2 *>(se0 + bswz(2 * b)) = a;
-                *reinterpret_cast<char2 *>(se1 + bswz(2 * b)) = e;
+                const int2 a = gauss_pair(gt_tab, seed, b, t, client, TAG_ENC_E0), e = gauss_pair(gt_tab, seed, b, t, client, TAG_ENC_E1);
+                *reinterpret_cast<char2 *>(se0 + bswz(2 * b)) = make_char2((signed char)a.x, (signed char)a.y);
+                *reinterpret_cast<char2 *>(se1 + bswz(2 * b)) = make_char2((signed char)e.x, (signed char)e.y);
             }
             // the ciphertext's message: slot transform, scaling and rounding in the limb buffer
             if (encode_in_block<LF>(c, sel + (size_t)tl * H, sm, mblk)) atomicOr(c.status, 1);
@@ -298,10 +288,9 @@ enc_outer_sample_kernel(const __grid_constant__ CtxDev c, uint32_t t0, uint64_t 
     }
 }
 
-// one thread block per (ciphertext, limb, block): forward block transform of u, from `ubuf`
-// ([T][L][N]), whose products with both halves of the public key are added, on the way out, to
-// the canonical residues in the ciphertext's slots
-template <class M, class L, int V>
+// one thread block per (ciphertext, limb, block): forward block transform of u, products with both halves
+// of the public key on the way out
+template <class M, class L, int V, bool ACC>
 __device__ __forceinline__ void enc_block_forward(const CtxDev &c, const LimbDev &lb, uint64_t *sm, uint32_t blk,
                                                   const tw_t *p0, const tw_t *p1, const uint64_t *u,
                                                   uint64_t *c0, uint64_t *c1) {
@@ -313,17 +302,28 @@ __device__ __forceinline__ void enc_block_forward(const CtxDev &c, const LimbDev
         [&](uint32_t p, val x, val y) {
             const auto a0 = M::load_key(p0 + p), a1 = M::load_key(p0 + p + 1);
             const auto b0 = M::load_key(p1 + p), b1 = M::load_key(p1 + p + 1);
-            u64x2 v0 = *reinterpret_cast<const u64x2 *>(c0 + p), v1 = *reinterpret_cast<const u64x2 *>(c1 + p);
-            v0.x = ar.canon_add(ar.mul_key(x, a0), v0.x);
-            v0.y = ar.canon_add(ar.mul_key(y, a1), v0.y);
-            v1.x = ar.canon_add(ar.mul_key(x, b0), v1.x);
-            v1.y = ar.canon_add(ar.mul_key(y, b1), v1.y);
+            u64x2 v0, v1;
+            if constexpr (ACC) {       // the slots hold canonical residues to add to
+                v0 = *reinterpret_cast<const u64x2 *>(c0 + p);
+                v1 = *reinterpret_cast<const u64x2 *>(c1 + p);
+                v0.x = ar.canon_add(ar.mul_key(x, a0), v0.x);
+                v0.y = ar.canon_add(ar.mul_key(y, a1), v0.y);
+                v1.x = ar.canon_add(ar.mul_key(x, b0), v1.x);
+                v1.y = ar.canon_add(ar.mul_key(y, b1), v1.y);
+            } else {
+                v0.x = ar.to_residue(ar.mul_key(x, a0));
+                v0.y = ar.to_residue(ar.mul_key(y, a1));
+                v1.x = ar.to_residue(ar.mul_key(x, b0));
+                v1.y = ar.to_residue(ar.mul_key(y, b1));
+            }
             *reinterpret_cast<u64x2 *>(c0 + p) = v0;
             *reinterpret_cast<u64x2 *>(c1 + p) = v1;
         });
 }
 
-template <class L, int V>
+// ACC = false: u comes from the c1 slot and the products replace both slots;
+// ACC = true: u comes from `ubuf` ([T][L][N]) and the products are added to the slots
+template <class L, int V, bool ACC>
 __global__ void __launch_bounds__(L::NT / V, (L::NT / V) <= 512 ? 2 : 1)
 enc_block_forward_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const uint64_t *ubuf, uint64_t *ct) {
     extern __shared__ __align__(128) uint64_t sm[];
@@ -336,9 +336,9 @@ enc_block_forward_kernel(const __grid_constant__ CtxDev c, const KeysDev k, cons
     const size_t off = ((size_t)blk << L::LOGB);
     uint64_t *c0 = ct + ((tl * 2 + 0) * c.L + j) * c.N + off;
     uint64_t *c1 = ct + ((tl * 2 + 1) * c.L + j) * c.N + off;
-    const uint64_t *u = ubuf + (tl * c.L + j) * c.N + off;
+    const uint64_t *u = ACC ? ubuf + (tl * c.L + j) * c.N + off : c1;
     const tw_t *p0 = k.pk0_hat + (size_t)j * c.N + off, *p1 = k.pk1_hat + (size_t)j * c.N + off;
-    FEDHE_FOR_ARITH(lb, (enc_block_forward<M_, L, V>(c, lb, sm, blk, p0, p1, u, c0, c1)));
+    FEDHE_FOR_ARITH(lb, (enc_block_forward<M_, L, V, ACC>(c, lb, sm, blk, p0, p1, u, c0, c1)));
 }
 
 // residues of e0 + m into the c0 slots and
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(256)
 enc_fill_errors_kernel(const __grid_constant__ CtxDev c, const int64_t *m, uint32_t t0, uint64_t seed,
                        uint32_t client, uint64_t *ct, size_t total) {
     __shared__ GaussTables gt;
-    gauss_tables_init(gt, threadIdx.x, blockDim.x);
+    gauss_tables_load(gt, c.gauss, threadIdx.x, blockDim.x);
     __syncthreads();
     const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= total) return;
@@ -355,13 +355,10 @@ enc_fill_errors_kernel(const __grid_constant__ CtxDev c, const int64_t *m, uint3
     const uint32_t b = (uint32_t)(g % pairs), i = 2 * b;   // one Philox block per pair
     const size_t tl = g / pairs;
     const uint32_t t = t0 + (uint32_t)tl;
-    const u32x4 w0 = stream_block(seed, b, t, client, TAG_ENC_E0);
-    const u32x4 w1 = stream_block(seed, b, t, client, TAG_ENC_E1);
+    const int2 e0 = gauss_pair(gt, seed, b, t, client, TAG_ENC_E0), e1 = gauss_pair(gt, seed, b, t, client, TAG_ENC_E1);
     const longlong2 mm = *reinterpret_cast<const longlong2 *>(m + tl * c.N + i);
-    const int64_t ax = mm.x + gauss_from_u64(gt, (uint64_t)w0.x | ((uint64_t)w0.y << 32));
-    const int64_t ay = mm.y + gauss_from_u64(gt, (uint64_t)w0.z | ((uint64_t)w0.w << 32));
-    const int ex = gauss_from_u64(gt, (uint64_t)w1.x | ((uint64_t)w1.y << 32));
-    const int ey = gauss_from_u64(gt, (uint64_t)w1.z | ((uint64_t)w1.w << 32));
+    const int64_t ax = mm.x + e0.x, ay = mm.y + e0.y;
+    const int ex = e1.x, ey = e1.y;
     for (uint32_t j = 0; j < c.L; j++) {
         const LimbDev &lb = c.limb[j];
         const uint64_t q = lb.q;
@@ -369,6 +366,69 @@ enc_fill_errors_kernel(const __grid_constant__ CtxDev c, const int64_t *m, uint3
             u64x2{signed_residue(ax, q, lb.mu), signed_residue(ay, q, lb.mu)};
         *reinterpret_cast<u64x2 *>(ct + ((tl * 2 + 1) * c.L + j) * c.N + i) =
             u64x2{small_residue(ex, q), small_residue(ey, q)};
+    }
+}
+
+template <class M, uint32_t A>
+__device__ __forceinline__ void enc_outer_inverse_add_limb(const LimbDev &lb, uint64_t *p, uint32_t B,
+                                                           const int64_t (&add)[1u << A][2]) {
+    constexpr uint32_t rows = 1u << A;
+    const uint64_t q = lb.q;
+    const auto t = LimbOf<M>::args(lb, false, 0, 0);
+    typename M::val x[rows], y[rows];
+#pragma unroll
+    for (uint32_t a = 0; a < rows; a++) {
+        const u64x2 v = *reinterpret_cast<const u64x2 *>(p + (size_t)a * B);
+        x[a] = M::from_bits(v.x);
+        y[a] = M::from_bits(v.y);
+    }
+    outer_inverse<A>(x, y, t, LimbOf<M>::ninv(lb), LimbOf<M>::wn(lb));
+#pragma unroll
+    for (uint32_t a = 0; a < rows; a++) {
+        u64x2 o;
+        o.x = t.m.canon_add(x[a], signed_residue(add[a][0], q, lb.mu));
+        o.y = t.m.canon_add(y[a], signed_residue(add[a][1], q, lb.mu));
+        *reinterpret_cast<u64x2 *>(p + (size_t)a * B) = o;
+    }
+}
+
+// one thread per pair of neighbouring columns of one ciphertext: for each
+// component draws its error terms once (e0 + m, then e1), then finishes every limb
+template <uint32_t A>
+__global__ void __launch_bounds__(256, A == 3 ? 2 : 4)
+enc_outer_inverse_add_kernel(const __grid_constant__ CtxDev c, const int64_t *m, uint32_t t0, uint64_t seed,
+                             uint32_t client, uint64_t *ct, size_t total) {
+    __shared__ GaussTables gt;
+    gauss_tables_load(gt, c.gauss, threadIdx.x, blockDim.x);
+    __syncthreads();
+    size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= total) return;
+    const uint32_t B = 1u << c.LOGB, half = B >> 1;
+    constexpr uint32_t rows = 1u << A;
+    const uint32_t col = (uint32_t)(g % half) * 2;
+    const size_t tl = g / half;
+    const uint32_t t = t0 + (uint32_t)tl;
+#pragma unroll 1
+    for (uint32_t comp = 0; comp < 2; comp++) {
+        int64_t add[rows][2];                          // e0 + m, or e1
+#pragma unroll
+        for (uint32_t a = 0; a < rows; a++) {
+            const uint32_t i = a * B + col;           // one Philox block per pair of coefficients
+            const int2 e = gauss_pair(gt, seed, i >> 1, t, client, comp == 0 ? TAG_ENC_E0 : TAG_ENC_E1);
+            add[a][0] = e.x;
+            add[a][1] = e.y;
+            if (comp == 0) {
+                const longlong2 mm = *reinterpret_cast<const longlong2 *>(m + tl * c.N + i);
+                add[a][0] += mm.x;
+                add[a][1] += mm.y;
+            }
+        }
+#pragma unroll 1
+        for (uint32_t j = 0; j < c.L; j++) {
+            const LimbDev &lb = c.limb[j];
+            uint64_t *p = ct + ((tl * 2 + comp) * c.L + j) * c.N + col;
+            FEDHE_FOR_ARITH(lb, (enc_outer_inverse_add_limb<M_, A>(lb, p, B, add)));
+        }
     }
 }
 
@@ -398,12 +458,13 @@ static cudaError_t launch_encrypt_fused(const CtxDev &c, const KeysDev &k, const
 }
 
 // launches the block forward kernel of the long-ring paths
+template <bool ACC>
 static cudaError_t launch_enc_block_forward(const CtxDev &c, const KeysDev &k, const uint64_t *ubuf, size_t T,
                                             uint64_t *ct, cudaStream_t s) {
     using L = WLay<13>;                                 // long rings are cut into 2^13 blocks
     constexpr int V = 2;
     const size_t smem = sizeof(uint64_t) << L::LOGB;
-    auto kern = enc_block_forward_kernel<L, V>;
+    auto kern = enc_block_forward_kernel<L, V, ACC>;
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
     kern<<<(unsigned)((T * c.L) << c.A), L::NT / V, smem, s>>>(c, k, ubuf, ct);
@@ -443,7 +504,48 @@ cudaError_t launch_encrypt_ntt(const CtxDev &c, const KeysDev &k, const float *s
     FEDHE_FOR_A(c, (enc_outer_sample_kernel<A_><<<blocks_for(cols, 256), 256, 0, s>>>(c, t0, seed, client, ubuf, LN,
                                                                                      cols)));
     if ((e = FEDHE_LAUNCHED())) return e;
-    return launch_enc_block_forward(c, k, ubuf, T, ct, s);
+    return launch_enc_block_forward<true>(c, k, ubuf, T, ct, s);
+}
+
+// Coefficient format on the longest ring by passes over the ciphertext itself, which is the work space: (1) draw u
+// and run the outer forward stages into the c1 slots; (2) block transforms of the c1 slots whose last phase
+// writes both products u^ pk0^ -> c0 and u^ pk1^ -> c1; (3) inverse block transforms of all slots; (4) outer
+// inverse stages fused with the error and message terms.  `work`: the encoded messages and the encoder's complex buffer.
+//
+// A limb of N = 2^16 is eight blocks of the complex transforms, which one thread block computes one after the other, so
+// few ciphertexts of few limbs take long there, and 45-bit limbs, two pieces each, are cheap here.  Measured (us, the
+// passes and the complex transforms; 1, 7, 31 and 92 ciphertexts): two 60-bit limbs 93, 115, 274, 690 and 183, 198, 232,
+// 546; four of 45 bits 88, 124, 301, 786 and 154, 170, 298, 830; eight of 60 bits 148, 271, 783, 2109 and 157, 183, 518, 1477.
+// The two sides below are lines through these; a first turn of the complex transforms takes 170 us whatever it holds.
+bool encrypt_by_passes(const CtxDev &c, size_t T) {
+    if (c.logN < 16) return false;
+    double per_ct = 1.8;
+    for (uint32_t j = 0; j < c.L; j++) per_ct += c.limb[j].fwd_d ? 1.54 : 2.48;
+    const double passes = 60.0 + 6.0 * c.L + per_ct * (double)T;
+    const double transforms = 40.0 + (1.5 + 0.89 * c.fft_pieces) * (double)T;
+    return passes < (transforms > 170.0 ? transforms : 170.0);
+}
+size_t encrypt_passes_work_bytes(const CtxDev &c, size_t T) {
+    if (c.logN < 16) return 0;
+    size_t most = T;               // the passes are taken for T itself or, if at all, up to a number below it
+    while (most && !encrypt_by_passes(c, most)) most /= 2;
+    most = 2 * most + 1 < T ? 2 * most + 1 : T;
+    return 2 * most * c.N * sizeof(uint64_t);
+}
+cudaError_t launch_encrypt_passes(const CtxDev &c, const KeysDev &k, const float *sel, void *work, uint32_t t0, size_t T,
+                                  uint64_t seed, uint32_t client, uint64_t *ct, cudaStream_t s) {
+    if (T == 0) return cudaSuccess;
+    int64_t *m = static_cast<int64_t *>(work);
+    cudaError_t e;
+    if ((e = launch_encode(c, sel, T, reinterpret_cast<double2 *>(m + T * c.N), m, s))) return e;
+    const size_t cols = T * ((size_t)1 << (c.LOGB - 1));      // pairs of columns
+    const size_t LN = (size_t)c.L * c.N;
+    enc_outer_sample_kernel<3><<<blocks_for(cols, 256), 256, 0, s>>>(c, t0, seed, client, ct + LN, 2 * LN, cols);
+    if ((e = FEDHE_LAUNCHED())) return e;
+    if ((e = launch_enc_block_forward<false>(c, k, nullptr, T, ct, s))) return e;
+    if ((e = launch_ntt_inner(c, false, ct, 2 * T, LN, 0, c.L, s))) return e;
+    enc_outer_inverse_add_kernel<3><<<blocks_for(cols, 256), 256, 0, s>>>(c, m, t0, seed, client, ct, cols);
+    return FEDHE_LAUNCHED();
 }
 
 }  // namespace fedhe

@@ -426,13 +426,11 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
     double2 *buf = reinterpret_cast<double2 *>(smem);
     root_t *tab = reinterpret_cast<root_t *>(smem + (size_t)NB * 16);
     int8_t *e1_smem = reinterpret_cast<int8_t *>(tab + G::Tab::WORDS);
-    __shared__ __align__(16) GaussTables gt;
+    __shared__ GaussTables gt;
     __shared__ uint32_t tmem_base;
     __shared__ __align__(8) uint64_t key_bar;
     const uint32_t rank = blockIdx.x % S, cid = blockIdx.x / S, nc = gridDim.x / S;
-    // (made once with the context: 768 entries from 38 thresholds each took 3 us of every call)
-    for (uint32_t i = threadIdx.x; i < sizeof(GaussTables) / 16; i += NT)
-        reinterpret_cast<uint4 *>(&gt)[i] = __ldg(reinterpret_cast<const uint4 *>(c.gauss) + i);
+    gauss_tables_load(gt, c.gauss, threadIdx.x, NT);
     for (uint32_t i = threadIdx.x; i < (uint32_t)G::Tab::WORDS; i += NT) tab[i] = c.fft_inv[i];
     if (threadIdx.x == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(&key_bar)) : "memory");
@@ -1043,9 +1041,14 @@ static size_t ring_scratch(const CtxDev &c, size_t T) {
     }
     return most;
 }
+template <int CL>
+static size_t ring_work(const CtxDev &c, size_t T) {
+    const size_t a = ring_scratch<CL>(c, T), b = encrypt_passes_work_bytes(c, T);
+    return a > b ? a : b;
+}
 size_t fft_work_bytes(const CtxDev &c, size_t T) {
     if (T == 0) return 0;
-    FEDHE_FOR_RING(c, ring_scratch, c, T)
+    FEDHE_FOR_RING(c, ring_work, c, T)
 }
 
 template <int CL>
@@ -1076,6 +1079,7 @@ static cudaError_t launch_encrypt_ring(const CtxDev &c, const KeysDev &k, const 
 cudaError_t launch_encrypt(const CtxDev &c, const KeysDev &k, const float *sel, void *work, uint32_t t0, size_t T,
                            uint64_t seed, uint32_t client, uint64_t *ct, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
+    if (encrypt_by_passes(c, T)) return launch_encrypt_passes(c, k, sel, work, t0, T, seed, client, ct, s);
     FEDHE_FOR_RING(c, launch_encrypt_ring, c, k, sel, work, t0, T, seed, client, ct, s)
 }
 

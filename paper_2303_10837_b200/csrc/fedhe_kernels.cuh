@@ -64,7 +64,7 @@ __device__ __forceinline__ int gauss_from_u64(uint64_t r) {
 // threshold, so a sample costs one 4-byte load, an addition and a shift.  What this does not decide has the sum's
 // sign set (the bytes 00 and ff, which share more than one threshold: 1 sample in 128) or its low 24 bits zero
 // (r and the threshold agree so far): gauss_rare() looks at the next byte, and then at all thresholds (1 in 32768).
-struct GaussTables {
+struct __align__(16) GaussTables {
     uint32_t entry[3][256];
 };
 constexpr uint32_t GAUSS_UNDECIDED = 0x80000000u;
@@ -89,6 +89,12 @@ __device__ __forceinline__ void gauss_tables_init(GaussTables &g, uint32_t tid, 
         const uint64_t b = i & 255u;
         g.entry[row][b] = row == 0 ? gauss_entry(b << 56, 56) : gauss_entry((row == 2 ? 0xffull << 56 : 0) | (b << 48), 48);
     }
+}
+
+// a copy of the context's table (768 entries from 38 thresholds each took 3 us of every call)
+__device__ __forceinline__ void gauss_tables_load(GaussTables &g, const void *made, uint32_t tid, uint32_t nthreads) {
+    for (uint32_t i = tid; i < sizeof(GaussTables) / 16; i += nthreads)
+        reinterpret_cast<uint4 *>(&g)[i] = __ldg(static_cast<const uint4 *>(made) + i);
 }
 
 // value + 19 in the top byte, unless gauss_undecided()

@@ -194,6 +194,57 @@ def test_encrypt_large_messages_bit_exact(he, base):
     assert np.array_equal(to_host_u64(ct), ct_o)
 
 
+def primes_below(limit, N, count):
+    """The largest `count` primes = 1 mod 2N below `limit` (Miller-Rabin with bases that decide below 2^64)."""
+    def prime(q):
+        d = (q - 1) // ((q - 1) & (1 - q))
+        for a in (2, 3, 5, 7, 11, 13, 17, 19, 23, 29, 31, 37):
+            x, e = pow(a, d, q), d
+            while e != q - 1 and x not in (1, q - 1):
+                x, e = x * x % q, 2 * e
+            if x != q - 1 and e % 2 == 0:
+                return False
+        return True
+    q, out = (limit - 1) // (2 * N) * 2 * N + 1, []
+    while len(out) < count:
+        q -= 2 * N
+        if prime(q):
+            out.append(q)
+    return tuple(out)
+
+
+@pytest.mark.parametrize("N,primes,T", [
+    (8192, (si.PRIMES_SWEEP[0], si.PRIMES_SWEEP_45[0]), 1),           # a 45-bit limb that pairs with none
+    (8192, si.PRIMES_SWEEP_45[:3], 149),                              # a pair and a single; one ciphertext more than SMs
+    (8192, (si.PRIMES_SWEEP[0],) + si.PRIMES_SWEEP_45[:5], 40),       # clusters of several sizes
+    (16384, si.PRIMES_SWEEP_45[:2] + (si.PRIMES_SWEEP[0],), 75),
+    (32768, si.PRIMES_SWEEP_45[:5], 38),
+    (65536, si.PRIMES_SWEEP[:2], 14),                                 # the last count that goes by passes ...
+    (65536, si.PRIMES_SWEEP[:2], 15),                                 # ... and the first that does not
+    (65536, si.PRIMES_SWEEP_45[:3], 38),                              # more than the clusters of the device
+    (8192, primes_below(1 << 61, 8192, 2), 3),                        # the largest primes: pieces that take 64 bits
+    (65536, primes_below(1 << 61, 65536, 2), 15),
+])
+def test_encrypt_counts_and_limbs_bit_exact(he, N, primes, T):
+    """Each way of sharing out the work gives the same words: all ciphertexts of a call, the same one
+    by one and in a ragged second half, and the oracle's first ciphertext."""
+    g, o = contexts(he, N, primes, 40)
+    keys = he.he_keygen(g, 15)
+    _, pk_o = o.keygen(15)
+    n, L = N // 2, len(primes)
+    x = np.random.default_rng(T).normal(0, 0.02, T * n).astype(np.float32)
+    sel = dev_f32(x)
+    ct = he.he_encrypt(g, keys, sel, 31, 2)
+    ct_o, bad = o.encrypt(pk_o, x[:n], 31, 2)
+    assert bad == 0 and np.array_equal(to_host_u64(ct[:1]), ct_o)
+    part = torch.empty((T, 2, L, N), dtype=torch.int64, device="cuda")
+    for t in {0, T // 2, T - 1}:
+        he.he_encrypt_range(g, keys, sel[t * n:], t, 1, 31, 2, part[t:])
+        assert torch.equal(part[t], ct[t])
+    he.he_encrypt_range(g, keys, sel[T // 2 * n:], T // 2, T - T // 2, 31, 2, part[T // 2:])
+    assert torch.equal(part[T // 2:], ct[T // 2:])
+
+
 def oracle_ntt_of(o, ct):
     """Every limb polynomial of an oracle ciphertext [T][2][level][N] through the oracle's forward transform."""
     out = np.empty_like(ct)
