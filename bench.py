@@ -31,6 +31,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import math
 import os
 import statistics
 import subprocess
@@ -60,18 +61,14 @@ UNIT = "params/s"
 # operations for the modular product, 2 for the sum and difference, and in the
 # inverse transform 1 more per butterfly for keeping the sums small.
 # Additions, shifts and logic go to another pipe.
-# DRAM bytes (read + write) per ciphertext of the encrypt kernel, by (N, L), from ncu captures of
-# the profile_case.py encrypt case (summaries under profiles/; traffic grows in proportion to the
-# number of ciphertexts).  An entry is dropped (None is reported) when the kernel has changed
-# since its counters were taken.
-ENCRYPT_DRAM_BYTES_PER_CT = {(16384, 4): 372.248832e6 / 296,       # encrypt_fused2_kernel, 296 ciphertexts
-                             (32768, 6): 478.248704e6 / 148}       # encrypt_cluster_kernel, 148 ciphertexts
+# The encryption of the coefficient format multiplies by complex transforms of N / 2 points instead: one of u, one of
+# the slots, and one inverse per product of u with a piece of the public key.
 SLOTS_PER_SM_CLK = 64.0
 WIDE_COST = 2.5
 INT_SLOTS_PER_BUTTERFLY = 6 * WIDE_COST + 4
 F64_SLOTS_FORWARD, F64_SLOTS_INVERSE = 8.0, 9.0
 F64_PRIME_LIMIT = 1 << 46
-ENCODE_SLOTS_PER_BUTTERFLY = 10.0     # complex product (4 multiplies, 2 add/sub) and complex sum and difference
+COMPLEX_SLOTS_PER_BUTTERFLY = 10.0    # complex product (4 multiplies, 2 add/sub) and complex sum and difference
 
 
 def transform_slots(primes, N, forward, inverse):
@@ -84,6 +81,26 @@ def transform_slots(primes, N, forward, inverse):
         else:
             total += bf * (forward + inverse) * INT_SLOTS_PER_BUTTERFLY
     return total
+
+
+def key_products(primes, N):
+    """Products of u with pieces of one half of the public key: a piece is as wide as 24 standard deviations of the
+    transform's error allow, and of two limbs whose low pieces are small these share one product."""
+    logN = N.bit_length() - 1
+    wide = 44
+    while 24.0 * 1.3 * math.sqrt((logN - 1) * N / 18.0) * 2.0 ** (wide - 53) >= 0.5:
+        wide -= 1
+    small = (27 - logN) // 2                       # bits of two low pieces whose products fit 16 bits each
+    pieces = [-(-q.bit_length() // wide) for q in primes]
+    share = sum(1 for q in primes if 0 < q.bit_length() - wide <= small)
+    return sum(pieces) - share // 2
+
+
+def encrypt_slots(primes, N):
+    """Pipe slots of one ciphertext's encryption by complex transforms: the butterflies, and the products between."""
+    n, products = N // 2, 2 * key_products(primes, N)
+    transform = (n // 2) * (n.bit_length() - 1) * COMPLEX_SLOTS_PER_BUTTERFLY
+    return (2 + products) * transform, products * n * 4.0
 
 
 def fallback_peaks():
@@ -485,27 +502,23 @@ def measure(job, w, steps, warmup, with_cpu_baseline):
     logN = w.N.bit_length() - 1
     per_launch = Tr                                          # ciphertexts of one client's he_encrypt calls
     butterflies = 3 * w.L * (w.N // 2) * logN * per_launch
-    # coefficient format: one forward and two inverse transforms per limb; transform format: three forward
-    slots_per_ct = transform_slots(w.primes, w.N, 3 if transform else 1, 0 if transform else 2)
-    if launches_per_encrypt == 1:
-        # the encoder runs inside the kernel: (n/2) log2 n complex butterflies of 10 double-precision operations
-        slots_per_ct += (n // 2) * (n.bit_length() - 1) * ENCODE_SLOTS_PER_BUTTERFLY
+    if transform:                                            # three forward transforms per limb
+        slots_per_ct, extra_per_ct = transform_slots(w.primes, w.N, 3, 0), 0.0
+        if launches_per_encrypt == 1:                        # the encoder runs inside the kernel
+            slots_per_ct += (n // 2) * (n.bit_length() - 1) * COMPLEX_SLOTS_PER_BUTTERFLY
+    else:
+        slots_per_ct, extra_per_ct = encrypt_slots(w.primes, w.N)
+        butterflies = (2 + 2 * key_products(w.primes, w.N)) * (n // 2) * (logN - 1) * per_launch
+        # Philox4x32-10: ten rounds of two 32x32->64 products for each of the N/4 + N/2 + N/2 blocks behind u, e0, e1
+        extra_per_ct += 1.25 * w.N * 20 * WIDE_COST
     achieved = slots_per_ct * per_launch / (kern_ms * 1e-3) / 1e12
-    # Everything else the method makes the kernel compute on the same pipe, per ciphertext:
-    # Philox4x32-10 (ten rounds of two 32x32->64 products for each of the N/4 + N/2 + N/2 blocks behind
-    # u, e0, e1), the two products with the public key per coefficient and limb, and the factor 1/N
-    # (one more product per butterfly of the last stage of both inverse transforms).
-    ints = sum(1 for q in w.primes if q >= F64_PRIME_LIMIT)
-    f64s = w.L - ints
-    per_product = ints * INT_SLOTS_PER_BUTTERFLY + f64s * 6.0
-    extra_per_ct = 1.25 * w.N * 20 * WIDE_COST + (2 * w.N + w.N) * per_product
-    achieved_all = (slots_per_ct + (0 if transform else extra_per_ct)) * per_launch / (kern_ms * 1e-3) / 1e12
+    achieved_all = (slots_per_ct + extra_per_ct) * per_launch / (kern_ms * 1e-3) / 1e12
     peak = job.n_sm * SLOTS_PER_SM_CLK * job.peaks["sm_max_mhz"] * 1e6 / 1e12
     alg_bytes = (4.0 + 32.0 * w.L) * n * per_launch          # read the slots, write the ciphertext
-    if w.N <= 16384:
+    if not transform and launches_per_encrypt == 1:
+        kname = "encrypt_fft_kernel"
+    elif w.N <= 16384:
         kname = "encrypt_fused2_kernel" if w.N == 16384 else "encrypt_fused_kernel"
-    elif launches_per_encrypt == 1:
-        kname = "encrypt_cluster_kernel"                     # one limb per pair of thread blocks (N = 32768)
     else:
         kname = "the %d kernels of he_encrypt on this ring, timed as one call" % launches_per_encrypt
     roofline = {
@@ -514,8 +527,7 @@ def measure(job, w, steps, warmup, with_cpu_baseline):
         "unit": "T slots/s (integer-multiply / double-precision pipe)",
         "frac": achieved / peak,
         "frac_all_required_work": achieved_all / peak,
-        "traffic": (ENCRYPT_DRAM_BYTES_PER_CT[(w.N, w.L)] * per_launch
-                    if (w.N, w.L) in ENCRYPT_DRAM_BYTES_PER_CT and not transform else None),
+        "traffic": None,                                     # no counters of this kernel are kept here
         "algorithmic_bytes": alg_bytes,
         "ms_per_launch": kern_ms, "launches_per_step": w.clients, "kernels_per_he_encrypt": int(launches_per_encrypt),
         "butterflies_per_launch": butterflies,
