@@ -415,6 +415,14 @@ __device__ __forceinline__ void enc_parked(int64_t (&val)[G::K], const unsigned 
 // The clusters fetch ciphertexts as they finish (with equal shares dealt out beforehand the slowest took 16 %
 // longer than the mean).  Of the `rem` ciphertexts after the last whole round each is cut in `parts`: clusters that
 // all prepare it and share its units.
+//
+// What bounds it is latency: registers leave 16 warps to an SM, the fp64 pipe is 31 to 35 % busy, the load and store
+// path half, and on N = 2^15 part of the 98 MB of scratch misses L2.  Measured, against modular transforms of every limb:
+//   N = 2^13, L = 3, 1 ciphertext       67.7 us -> 30.7 us
+//   N = 2^14, L = 4, 313 ciphertexts    0.69 ms -> 0.32 ms
+//   N = 2^14, L = 4, 1429 ciphertexts   2.82 ms -> 1.38 ms (1.1 TB/s of ciphertext)
+//   N = 2^15, L = 6, 6714 ciphertexts   40.2 ms -> 26.8 ms (0.8 TB/s)
+//
 // PAIRS: some units are of two limbs (the code for both kinds costs the others 1.5 %).
 template <int CL, bool PAIRS>
 __global__ void __launch_bounds__(FftLay::NT, 2)
@@ -742,6 +750,9 @@ __device__ __forceinline__ double fft_from_int32(int v) {
 // c0 and the joined lower pieces wait in tensor memory, in the words of the threads that will join them; c1 is read
 // by all its loads at once, and cut in 32-bit arithmetic if its pieces are two.  (Reading eight values at a time from L2
 // and cutting in 64 bits, loading and joining took 28 of 65 thousand clocks per ciphertext of N = 8192.)
+//
+// Bound by its chain of transforms, exchanges and loads on few ciphertexts: 68 of N = 2^15 take 141 us by modular transforms in
+// separate kernels and 84 us here.
 template <int CL>
 __global__ void __launch_bounds__(FftLay::NT, 2)
 decrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const uint64_t *ct, uint32_t level,
