@@ -63,6 +63,9 @@ UNIT = "params/s"
 # Additions, shifts and logic go to another pipe.
 # The encryption of the coefficient format multiplies by complex transforms of N / 2 points instead: one of u, one of
 # the slots, and one inverse per product of u with a piece of the public key.
+# DRAM bytes (read + write) per ciphertext of the encrypt kernel, by (N, L), from an ncu capture of
+# the profile_case.py encrypt case (traffic grows in proportion to the number of ciphertexts).
+ENCRYPT_DRAM_BYTES_PER_CT = {(16384, 4): 339.017984e6 / 296}       # encrypt_fft_kernel, 296 ciphertexts
 SLOTS_PER_SM_CLK = 64.0
 WIDE_COST = 2.5
 INT_SLOTS_PER_BUTTERFLY = 6 * WIDE_COST + 4
@@ -527,7 +530,8 @@ def measure(job, w, steps, warmup, with_cpu_baseline):
         "unit": "T slots/s (integer-multiply / double-precision pipe)",
         "frac": achieved / peak,
         "frac_all_required_work": achieved_all / peak,
-        "traffic": None,                                     # no counters of this kernel are kept here
+        "traffic": (ENCRYPT_DRAM_BYTES_PER_CT[(w.N, w.L)] * per_launch
+                    if (w.N, w.L) in ENCRYPT_DRAM_BYTES_PER_CT and not transform else None),
         "algorithmic_bytes": alg_bytes,
         "ms_per_launch": kern_ms, "launches_per_step": w.clients, "kernels_per_he_encrypt": int(launches_per_encrypt),
         "butterflies_per_launch": butterflies,
