@@ -313,11 +313,14 @@ int he_ntt_inverse(he_ctx *ctx, uint64_t *polys_dev, size_t B, void *stream);
  * encryption the slots of the next chunk of ciphertext indices (a contiguous
  * piece of every update) go up while the current chunk is computed, and the
  * decoded slots of a finished chunk go home while the next is computed; with
- * a mask the whole update of the next client goes up while the current one is
- * packed and encrypted.  They overlap the arithmetic only when xs and w_glob
+ * a mask the round is cut along the parameters, and the part of the model that
+ * a range of every update completes goes home while the next range comes up.
+ * They overlap the arithmetic only when xs and w_glob
  * are page-locked (pinned) host memory; pageable memory is correct but
- * serialises.  With full encryption parts of w_glob are written
- * before the call returns; after an error return its contents are unspecified.
+ * serialises.  Parts of w_glob are written before the call returns; after an
+ * error return its contents are unspecified.  With a mask w_glob may share
+ * memory with updates (it is then written after the last upload); with full
+ * encryption it must not.
  * Bad arguments (a NULL xs[i], a weight outside [0, 1]) are refused before
  * anything is queued.  On every return, error or not, all streams have been
  * waited for: no copy is still reading xs or writing w_glob. */

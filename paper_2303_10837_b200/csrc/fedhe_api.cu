@@ -982,6 +982,14 @@ static int round_host_queued(he_ctx *ctx, const he_keys *keys, const he_mask *ma
     double *ravg = reinterpret_cast<double *>(p); p += b_ravg;
     double *out = reinterpret_cast<double *>(p);
 
+    // A model that shares memory with an update may only be written when every update has come up.
+    bool shared = false;
+    const uintptr_t w_at = reinterpret_cast<uintptr_t>(w_glob_host);
+    for (int i = 0; i < C; i++) {
+        const uintptr_t x_at = reinterpret_cast<uintptr_t>(xs_host[i]);
+        shared = shared || (x_at < w_at + P * sizeof(double) && w_at < x_at + P * sizeof(float));
+    }
+
     CU(cudaEventRecord(ctx->ev_free[0], st));       // earlier work on `st` may still use the buffers
     CU(cudaEventRecord(ctx->ev_free[1], st));
     std::vector<const uint64_t *> cptr(C);
@@ -1028,7 +1036,7 @@ static int round_host_queued(he_ctx *ctx, const he_keys *keys, const he_mask *ma
         }
         // ranges of which everything is decoded go home
         size_t done = home;
-        while (done <= c && (before[done + 1] <= t * n) && (cut[done + 1] - before[done + 1] <= r)) done++;
+        while ((!shared || c + 1 == R) && done <= c && (before[done + 1] <= t * n) && (cut[done + 1] - before[done + 1] <= r)) done++;
         if (done > home) {
             const size_t first = cut[home], count = cut[done] - first;
             CU(launch_unpack_range(mask, z, restlen ? ravg : nullptr, first, count, out + first, st));

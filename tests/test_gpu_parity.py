@@ -360,6 +360,24 @@ def test_host_round_by_ranges(he, P, k):
     assert torch.equal(host, want)
 
 
+def test_masked_host_round_into_memory_of_an_update(he):
+    """The model may share memory with an update: here the last client's update, which comes up last, lies in the
+    first half of the model's buffer, where finished ranges would overwrite what has yet to come up."""
+    P, clients = 5_300_003, 8
+    g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
+    keys = he.he_keygen(g, 5)
+    rng = np.random.default_rng(3)
+    xs = [torch.from_numpy((0.01 * rng.standard_normal(P)).astype(np.float32)).pin_memory() for _ in range(clients)]
+    alpha = [1.0 / clients] * clients
+    mask = he.he_select_mask(g, dev_f32(rng.random(P, dtype=np.float32)), P // 10)
+    want = he.he_round_host(g, keys, mask, xs, alpha, 99, torch.empty(P, dtype=torch.float64).pin_memory())
+    out = torch.empty(P, dtype=torch.float64).pin_memory()
+    last = out.view(torch.float32)[:P]
+    last.copy_(xs[-1])
+    he.he_round_host(g, keys, mask, xs[:-1] + [last], alpha, 99, out)
+    assert torch.equal(out, want)
+
+
 @pytest.mark.parametrize("P,spread", [(1, 1.0), (33, 1.0), (2047, 1.0), (2049, 1e-4), (300_001, 1e-4), (20_000_003, 1.0)])
 def test_select_mask_tiles_and_candidates(he, P, spread):
     """Edges of the tiles, tiles with more candidates than their list holds (all scores within one
