@@ -37,7 +37,9 @@
  *     he_ctx_reserve does that ahead of time.
  *   - Kernels never trap or assert.  A numeric anomaly (an encoded
  *     coefficient of magnitude >= 2^62, or a non-finite input) sets a sticky
- *     status word read by he_ctx_status().
+ *     status word read by he_ctx_status(), and so does a copy inside a kernel
+ *     that has not arrived after seconds (an error of the device): the kernel
+ *     leaves out what depends on it and ends.
  *   - Ring R = Z[X]/(X^N+1), N a power of two, RNS primes q_0..q_{L-1} (all
  *     of them ciphertext limbs; the rescale drops q_{L-1}); n = N/2 real
  *     slots per ciphertext; scale Delta = 2^log2_delta.
@@ -89,8 +91,10 @@ const char *he_strerror(int code);
  * them.  Synchronous. */
 int he_ctx_create(const he_params *params, he_ctx **out);
 int he_ctx_destroy(he_ctx *ctx);
-/* Synchronises the device, returns the sticky status (HE_OK or
- * HE_ERR_OVERFLOW) in *status and clears it. */
+/* Synchronises the device, returns the sticky status (HE_OK; HE_ERR_OVERFLOW,
+ * an encoded coefficient out of range or an input that is not finite;
+ * HE_ERR_CUDA, a copy inside a kernel did not arrive and results since the
+ * last call are incomplete) in *status and clears it. */
 int he_ctx_status(he_ctx *ctx, int *status);
 /* Pre-sizes the library-owned work buffers for encryptions/decryptions of up
  * to max_k encrypted parameters so that later calls allocate nothing.

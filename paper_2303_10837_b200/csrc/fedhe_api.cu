@@ -197,7 +197,7 @@ int he_ctx_status(he_ctx *ctx, int *status) {
     CU(cudaDeviceSynchronize());
     CU(cudaMemcpy(&word, ctx->dev.status, sizeof(int), cudaMemcpyDeviceToHost));
     if (word) CU(cudaMemset(ctx->dev.status, 0, sizeof(int)));
-    *status = word ? HE_ERR_OVERFLOW : HE_OK;
+    *status = host_status_code(word);
     return HE_OK;
 }
 

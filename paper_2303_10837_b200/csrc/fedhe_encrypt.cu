@@ -109,7 +109,7 @@ encrypt_fused_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const fl
                 *reinterpret_cast<char2 *>(se1 + bswz(2 * b)) = make_char2((signed char)e.x, (signed char)e.y);
             }
             // the ciphertext's message: slot transform, scaling and rounding in the limb buffer
-            if (encode_in_block<LF>(c, sel + (size_t)tl * (B / 2), sm, mblk)) atomicOr(c.status, 1);
+            if (encode_in_block<LF>(c, sel + (size_t)tl * (B / 2), sm, mblk)) atomicOr(c.status, STATUS_RANGE);
         }
         const LimbDev &lb = c.limb[j];
         uint64_t *cbase = ct + (((size_t)tl * 2 + 0) * c.L + j) * B;
@@ -232,7 +232,7 @@ encrypt_fused2_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const f
                 *reinterpret_cast<char2 *>(se1 + bswz(2 * b)) = make_char2((signed char)e.x, (signed char)e.y);
             }
             // the ciphertext's message: slot transform, scaling and rounding in the limb buffer
-            if (encode_in_block<LF>(c, sel + (size_t)tl * H, sm, mblk)) atomicOr(c.status, 1);
+            if (encode_in_block<LF>(c, sel + (size_t)tl * H, sm, mblk)) atomicOr(c.status, STATUS_RANGE);
         }
         const LimbDev &lb = c.limb[j];
         uint64_t *cbase = ct + (((size_t)tl * 2 + 0) * c.L + j) * B;

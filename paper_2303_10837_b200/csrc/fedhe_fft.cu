@@ -223,17 +223,17 @@ __device__ __forceinline__ void key_fetch(double2 *buf, const double2 *key, uint
                  "n"(KEY_BYTES), "r"(b)
                  : "memory");
 }
-// false if the copy has not come after many tries, which would be an error of the device
-__device__ __forceinline__ bool key_wait(uint64_t *bar, uint32_t parity) {
+// whether the copy is there, after 10 ms at most
+__device__ __forceinline__ bool key_try(uint64_t *bar, uint32_t parity) {
     const uint32_t b = (uint32_t)__cvta_generic_to_shared(bar);
-    uint32_t done = 0;
-    for (int i = 0; i < 256 && !done; i++)
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 0x989680;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(done)
-                     : "r"(b), "r"(parity)
-                     : "memory");
-    return done;
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 0x989680;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done)
+                 : "r"(b), "r"(parity)
+                 : "memory");
+    return done != 0;
 }
+constexpr uint32_t KEY_TRIES = 256;
 
 // two complex values
 __device__ __forceinline__ void tmem_put(uint32_t at, cpx a, cpx b) {
@@ -444,7 +444,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(&key_bar)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    uint32_t key_parity = 0;
+    CopyTurns turns(KEY_TRIES);
     const uint32_t tm = tmem_take(&tmem_base);            // and the tables are there
     unsigned char *common = work + (size_t)cid * (G::SHARED + S * G::OWN), *own = common + G::SHARED + rank * G::OWN;
     double2 *uhat = reinterpret_cast<double2 *>(common);                        // [R][16][NT]
@@ -548,7 +548,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
                             __stcg(row + kk, (long long)re);
                             __stcg(row + R * NB + kk, (long long)im);
                         }))
-                    atomicOr(c.status, 1);
+                    atomicOr(c.status, STATUS_RANGE);
             }
         }
         meet();
@@ -602,13 +602,16 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
         }
 
         // ---- this block's units ----
+        auto wait_for_key = [&]() {
+            if (!turns.take([&](uint32_t parity) { return key_try(&key_bar, parity); })) atomicOr(c.status, STATUS_COPY);
+        };
         auto key_of = [&](uint32_t u, uint32_t pb) {
             const uint32_t comp = u >= c.enc_units ? 1 : 0;
             const EncUnit &e = c.enc_unit[u - comp * c.enc_units];
             return k.fft_pk + e.fft_key + ((size_t)comp * e.products * R + pb) * NB;
         };
         if constexpr (!(G::E_IN_SMEM)) __syncthreads();   // the buffer's last readers are done
-        if (threadIdx.x == 0) key_fetch(buf, key_of(unit, 0), &key_bar);
+        if (threadIdx.x == 0 && !turns.lost()) key_fetch(buf, key_of(unit, 0), &key_bar);
 #pragma unroll 1
         for (; unit < unit_end; unit++) {
             const uint32_t comp = unit >= c.enc_units ? 1 : 0;
@@ -625,7 +628,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
                     const uint32_t tid = fresh_tid();
                     const double2 *key = buf + tid;
                     if constexpr (R == 1) {
-                        if (!key_wait(&key_bar, key_parity)) atomicOr(c.status, 4);
+                        wait_for_key();
 #pragma unroll
                         for (int h = 0; h < 2; h++) {
                             uint32_t w[32];
@@ -641,17 +644,16 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
                             const double2 w = __ldcg(uh + r * NT);
                             x[r] = cpx{w.x, w.y};
                         }
-                        if (!key_wait(&key_bar, key_parity)) atomicOr(c.status, 4);
+                        wait_for_key();
 #pragma unroll
                         for (int r = 0; r < 16; r++) x[r] = cpx_mul(x[r], key[r * NT].x, key[r * NT].y);
                     }
-                    key_parity ^= 1u;
                 }
                 // the next key may come as soon as the buffer is read; where a column loop needs the buffer, after it
                 const bool more = pb + 1 < e.products * R || unit + 1 < unit_end;
                 auto fetch_next = [&]() {
                     __syncthreads();
-                    if (more && threadIdx.x == 0)
+                    if (more && threadIdx.x == 0 && !turns.lost())
                         key_fetch(buf, pb + 1 < e.products * R ? key_of(unit, pb + 1) : key_of(unit + 1, 0), &key_bar);
                 };
                 fft_inverse<0>(x, buf, tab, fresh_tid(), [&] {
@@ -725,6 +727,8 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
             }
         }
     }
+    if (threadIdx.x == 0 && turns.lost())                 // that copy may still be on its way into this block's memory
+        for (uint32_t i = 0; i < KEY_TRIES && !key_try(&key_bar, turns.parity()); i++) {}
     if (leader && atomicAdd(c.deal + 1, 1u) + 1 == nc) {  // the last cluster leaves the words as it found them
         c.deal[0] = 0;
         c.deal[1] = 0;

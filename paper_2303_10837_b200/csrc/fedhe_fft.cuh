@@ -351,6 +351,31 @@ HD void fft_outer_inverse(cpx (&v)[1 << CL], const root_t *tab, uint32_t tid, ui
     for (int a = 0; a < R; a++) v[a] = cpx_mul(v[a], turn[next + a].re, turn[next + a].im);
 }
 
+// ---- copies a thread block waits for, one after the other ----
+//
+// Every thread waits for the copy of a turn; one thread starts the next copy, behind a barrier of the block.  A thread has a
+// number of tries for all its waits together, of which copies that come in time take none.  When they are used up it
+// waits no more, and what it reads means nothing; if it is the one that starts the copies it starts no more, so
+// that there are never two on their way, and it stays at the turn that it lost.
+struct CopyTurns {
+    uint32_t state;                                    // tries left, and the parity of the copy to come in bit 0
+    explicit HD CopyTurns(uint32_t tries) : state(2 * tries) {}
+    HD uint32_t parity() const { return state & 1u; }
+    HD bool lost() const { return state < 2; }
+    // try_once(parity): whether the copy is there, after a while
+    template <class Try>
+    HD bool take(const Try &try_once) {
+        while (!lost()) {
+            if (try_once(parity())) {
+                state ^= 1u;
+                return true;
+            }
+            state -= 2;
+        }
+        return false;
+    }
+};
+
 #if defined(__CUDACC__)
 // ---- whole blocks (device) -----------------------------------------------------------
 

@@ -3,9 +3,16 @@
 
 #include <quadmath.h>
 
+#include "../../include/fedhe.h"
+
 namespace fedhe {
 
 typedef unsigned __int128 u128;
+
+int host_status_code(int word) {
+    if (word & STATUS_COPY) return HE_ERR_CUDA;
+    return word ? HE_ERR_OVERFLOW : HE_OK;
+}
 
 uint64_t host_mulmod(uint64_t a, uint64_t b, uint64_t q) { return (uint64_t)((u128)a * b % q); }
 

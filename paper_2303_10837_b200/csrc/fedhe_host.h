@@ -21,6 +21,11 @@ struct HostLimb {
     std::vector<HostTw> inv;   // inv[i] = psi^-brev(i)
 };
 
+// Bits of a context's status word, raised by the kernels: an encoded coefficient out of range or an input that is not
+// finite; a copy inside a kernel that did not arrive.  And what the word amounts to, the graver first.
+enum { STATUS_RANGE = 1, STATUS_COPY = 4 };
+int host_status_code(int word);
+
 uint64_t host_mulmod(uint64_t a, uint64_t b, uint64_t q);
 uint64_t host_powmod(uint64_t a, uint64_t e, uint64_t q);
 uint64_t host_invmod(uint64_t a, uint64_t q);

@@ -8,6 +8,7 @@
 
 #include "../../include/fedhe.h"
 #include "fedhe_fft.cuh"
+#include "fedhe_host.h"
 #include "fedhe_ntt.cuh"
 
 namespace fedhe {

@@ -57,7 +57,7 @@ encode_block_kernel(const __grid_constant__ CtxDev c, const float *sel, const do
         mt[k] = stage[stage_swz(kk)];
         mt[k + n] = stage[NB + stage_swz(kk)];
     }
-    if (bad) atomicOr(c.status, 1);
+    if (bad) atomicOr(c.status, STATUS_RANGE);
 }
 
 // Outer stages of the encoder for n > block: each thread owns one column of

@@ -1,11 +1,13 @@
 // Plays the complex transforms behind the exact products on the host, thread by thread, with the
 // device's own index arithmetic, and compares products of a ternary polynomial and one of the largest
-// pieces with the exact integers.  usage: host_fft_check logN
+// pieces with the exact integers.  usage: host_fft_check logN, or 0 for the
+// turns of a kernel's copies
 #include <cstdio>
 #include <cstdlib>
 #include <random>
 #include <vector>
 
+#include "../include/fedhe.h"
 #include "../paper_2303_10837_b200/csrc/fedhe_fft.cuh"
 #include "../paper_2303_10837_b200/csrc/fedhe_host.h"
 
@@ -160,9 +162,63 @@ static int check(uint32_t N) {
     return bad;
 }
 
+// A thread block whose threads, in any order, wait for copies of which one comes late or never: there are never two on
+// their way, none is started after the starting thread lost one, and every wait ends.
+static void copies_that_do_not_come() {
+    std::mt19937 rng(7);
+    const int NT = 8, TURNS = 8;
+    const uint32_t TRIES = 6;
+    for (int trial = 0; trial < 20000; trial++) {
+        const int bad = (int)(rng() % (TURNS + 1));          // TURNS: every copy comes in time
+        const bool never = rng() % 2;
+        struct Thread { CopyTurns turns{TRIES}; int turn = 0; uint32_t tries = 0; bool behind = false; } th[NT];
+        int arrived[TURNS] = {}, started = 1, phases = 0, running = NT;      // phases of the copies' barrier that are over
+        while (running) {
+            const int id = (int)(rng() % NT);
+            Thread &t = th[id];
+            if (t.turn == TURNS) continue;
+            if (!t.behind) {
+                // a try goes on for longer than a copy that comes in time takes, and than the others' way to the barrier
+                if (started <= t.turn && !th[0].turns.lost() && !t.turns.lost()) continue;
+                t.turns.take([&](uint32_t parity) {
+                    if (phases < started && (phases != bad || (!never && rng() % 16 == 0))) phases++;
+                    const bool here = (uint32_t)(phases & 1) != parity;
+                    t.tries += !here;
+                    return here;
+                });
+                arrived[t.turn]++;
+                t.behind = true;
+            } else if (arrived[t.turn] == NT) {
+                if (id == 0 && t.turn + 1 < TURNS && !t.turns.lost()) {
+                    if (phases != started) { std::printf("two copies at once\n"); std::exit(1); }
+                    started++;
+                }
+                t.behind = false;
+                running -= ++t.turn == TURNS;
+            }
+        }
+        bool lost = false;
+        for (const Thread &t : th) {
+            lost = lost || t.turns.lost();
+            if (t.tries > TRIES) { std::printf("the waits are too long\n"); std::exit(1); }
+        }
+        if ((lost && bad == TURNS) || (!th[0].turns.lost() && started != TURNS) ||
+            (th[0].turns.lost() && (started != bad + 1 || th[0].turns.parity() != (uint32_t)(bad & 1)))) {
+            std::printf("a lost copy is not the last\n");
+            std::exit(1);
+        }
+    }
+    if (host_status_code(0) != HE_OK || host_status_code(STATUS_RANGE) != HE_ERR_OVERFLOW || host_status_code(STATUS_COPY) != HE_ERR_CUDA ||
+        host_status_code(STATUS_RANGE | STATUS_COPY) != HE_ERR_CUDA) {
+        std::printf("status codes\n");
+        std::exit(1);
+    }
+}
+
 int main(int argc, char **argv) {
     const int logN = argc > 1 ? std::atoi(argv[1]) : 13;
     int bad = 0;
+    if (logN == 0) copies_that_do_not_come();
     if (logN == 13) bad |= check<0>(1u << 13);
     if (logN == 14) bad |= check<1>(1u << 14);
     if (logN == 15) bad |= check<2>(1u << 15);

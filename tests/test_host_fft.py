@@ -1,5 +1,5 @@
 """The complex transforms behind the exact products of encryption and decryption, compiled for
-the CPU and run thread by thread: index arithmetic, tables and the rounding-error bounds."""
+the CPU and run thread by thread: index arithmetic, tables and the rounding-error bounds; and what a kernel does when a copy does not come."""
 import os
 import subprocess
 
@@ -8,7 +8,7 @@ import pytest
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
-@pytest.mark.parametrize("logn", [13, 14, 15, 16])
+@pytest.mark.parametrize("logn", [0, 13, 14, 15, 16])
 def test_exact_products_on_the_host(tmp_path, logn):
     exe = str(tmp_path / "host_fft_check")
     cmd = ["g++", "-O2", "-std=gnu++17", "-ffp-contract=off", "-o", exe,
