@@ -121,8 +121,9 @@ int he_keys_export(he_ctx *ctx, const he_keys *keys, uint64_t *pk_dev, int8_t *s
  * the first k form the mask.  score: dev float[P], P < 2^32, 0 <= k <= P.
  * Synchronous (the result sizes are needed on the host).  The mask's device
  * buffers come from a per-device memory pool that the library creates on
- * first use and keeps until the process ends; he_mask_destroy returns them
- * to the pool, which holds at most 256 MiB of unused memory. */
+ * first use; he_mask_destroy, which may be called with another device current,
+ * returns them to the pool, which holds at most 256 MiB of unused memory and
+ * is given back with the last context and mask of the device. */
 int he_select_mask(he_ctx *ctx, const float *score_dev, size_t P, size_t k, he_mask **out, void *stream);
 /* Variant for the paper's empirical selection recipe (the top-p most
  * sensitive parameters as well as whole layers, e.g. the first and last):

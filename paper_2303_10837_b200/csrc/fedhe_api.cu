@@ -50,6 +50,55 @@ int upload(he_ctx *ctx, const T *host, size_t count, const T **dev) {
     return HE_OK;
 }
 
+// Masks are made and dropped once per round, and a plain device allocation costs more than the
+// kernels of the selection.  Their buffers therefore come from one memory pool per device, which hands freed
+// buffers out again and gives back to the driver at once only what it holds beyond MASK_POOL_KEEP bytes.  The pool
+// is made for the first mask and lives as long as a context or a mask of the device does.
+constexpr uint64_t MASK_POOL_KEEP = 256ull << 20;
+struct MaskPool {
+    cudaMemPool_t pool = nullptr;
+    size_t users = 0;                                 // contexts and masks
+};
+constexpr int MAX_DEVICES = 64;
+std::mutex mask_pool_mu;
+MaskPool mask_pools[MAX_DEVICES];
+
+void mask_pool_join(int device) {
+    std::lock_guard<std::mutex> lock(mask_pool_mu);
+    if (device >= 0 && device < MAX_DEVICES) mask_pools[device].users++;
+}
+// nothing of the pool is in use by the device any more when its last user leaves
+void mask_pool_leave(int device) {
+    std::lock_guard<std::mutex> lock(mask_pool_mu);
+    if (device < 0 || device >= MAX_DEVICES) return;
+    MaskPool &m = mask_pools[device];
+    if (--m.users == 0 && m.pool) {
+        cudaMemPoolDestroy(m.pool);
+        m.pool = nullptr;
+    }
+}
+// by a user of it
+cudaMemPool_t mask_pool(int device) {
+    std::lock_guard<std::mutex> lock(mask_pool_mu);
+    if (device < 0 || device >= MAX_DEVICES) return nullptr;
+    MaskPool &m = mask_pools[device];
+    if (!m.pool) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.handleTypes = cudaMemHandleTypeNone;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        if (cudaMemPoolCreate(&m.pool, &props) != cudaSuccess) {
+            cudaGetLastError();
+            m.pool = nullptr;
+            return nullptr;
+        }
+        uint64_t keep = MASK_POOL_KEEP;
+        cudaMemPoolSetAttribute(m.pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    }
+    return m.pool;
+}
+
 size_t work_bytes(const he_ctx *ctx, size_t T) { return 2 * T * (size_t)ctx->dev.N * sizeof(uint64_t); }
 
 }  // namespace
@@ -91,7 +140,8 @@ int he_ctx_create(const he_params *p, he_ctx **out) {
     ctx->params = *p;
     int rc = HE_OK;
     do {
-        if (cudaGetDevice(&ctx->device) != cudaSuccess) { rc = HE_ERR_CUDA; break; }
+        if (cudaGetDevice(&ctx->device) != cudaSuccess) { rc = HE_ERR_CUDA; ctx->device = -1; break; }
+        mask_pool_join(ctx->device);
         if (cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess ||
             ctx->sm_count < 1) {
             rc = HE_ERR_CUDA;
@@ -186,6 +236,7 @@ int he_ctx_destroy(he_ctx *ctx) {
         if (ctx->ev_free[i]) cudaEventDestroy(ctx->ev_free[i]);
     }
     if (ctx->ev_chunk) cudaEventDestroy(ctx->ev_chunk);
+    mask_pool_leave(ctx->device);
     ctx->magic = 0;
     delete ctx;
     return HE_OK;
@@ -299,31 +350,6 @@ int he_keys_export(he_ctx *ctx, const he_keys *keys, uint64_t *pk_dev, int8_t *s
 // mask
 // ---------------------------------------------------------------------------
 
-// Masks are made and dropped once per round, and a plain device allocation costs more than the
-// kernels of the selection.  Their buffers therefore come from one memory pool per device, made
-// on first use and kept for the life of the process; the pool hands freed buffers out again and
-// gives back to the driver only what it holds beyond MASK_POOL_KEEP bytes.
-static constexpr uint64_t MASK_POOL_KEEP = 256ull << 20;
-static cudaMemPool_t mask_pool(int device) {
-    static std::mutex mu;
-    static cudaMemPool_t pools[64] = {};
-    if (device < 0 || device >= 64) return nullptr;
-    std::lock_guard<std::mutex> lock(mu);
-    if (!pools[device]) {
-        cudaMemPoolProps props = {};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.handleTypes = cudaMemHandleTypeNone;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = device;
-        cudaMemPool_t pool = nullptr;
-        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-        uint64_t keep = MASK_POOL_KEEP;
-        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-        pools[device] = pool;
-    }
-    return pools[device];
-}
-
 static int build_mask(he_ctx *ctx, const float *score, size_t P, size_t k, const uint64_t *ranges_host,
                       size_t num_ranges, he_mask **out, void *stream) {
     if (!good(ctx) || !out || (!score && P) || k > P) return HE_ERR_INVALID_ARG;
@@ -391,6 +417,8 @@ static int build_mask(he_ctx *ctx, const float *score, size_t P, size_t k, const
         m = new (std::nothrow) he_mask();
         if (!m) { rc = HE_ERR_ALLOC; break; }
         m->magic = MASK_MAGIC;
+        m->device = ctx->device;
+        mask_pool_join(m->device);
         m->P = P;
         m->k = ksel;
         m->idx = idx;
@@ -433,8 +461,14 @@ int he_mask_copy_indices(const he_mask *mask, uint32_t *out_dev, void *stream) {
 
 int he_mask_destroy(he_mask *mask) {
     if (!good(mask)) return HE_ERR_INVALID_ARG;
+    // the mask's device need not be the current one, and it is that device's work that has to be over
+    int current = mask->device;
+    cudaGetDevice(&current);
+    if (current != mask->device) cudaSetDevice(mask->device);
     cudaDeviceSynchronize();
     cudaFreeAsync(mask->bits, nullptr);      // back to the pool; prefix counts and index list are parts of this allocation
+    mask_pool_leave(mask->device);
+    if (current != mask->device) cudaSetDevice(current);
     mask->magic = 0;
     delete mask;
     return HE_OK;

@@ -143,6 +143,7 @@ struct he_keys {
 
 struct he_mask {
     uint32_t magic;
+    int device;
     size_t P, k;
     uint32_t *idx;       // [k] ascending
     uint32_t *bits;      // [ceil(P/32)] bit i of word i/32 set if parameter i is encrypted
