@@ -997,16 +997,20 @@ static int round_host_queued(he_ctx *ctx, const he_keys *keys, const he_mask *ma
     if (Tc < 1) Tc = 1;
 
     auto align = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    const size_t b_x = align(most * sizeof(float)), b_sel = align(padded * sizeof(float)),
+    // Parts of updates come up into two sets of buffers, for as many clients each as a whole update has room for, or
+    // 256 MiB: for all of them, unless they are very many (256 clients and eight ranges would hold 64 updates).
+    const size_t b_x = align(most * sizeof(float)), room = P * sizeof(float) > (256u << 20) ? P * sizeof(float) : 256u << 20;
+    const size_t lanes = (size_t)C * b_x <= room ? (size_t)C : room / b_x > 1 ? room / b_x : 1;
+    const size_t b_sel = align(padded * sizeof(float)),
                  b_rest = align(restlen * sizeof(float)), b_cts = align(C * Tc * ctw * sizeof(uint64_t)),
                  b_agg = align(Tc * aggw * sizeof(uint64_t)), b_z = align(padded * sizeof(double)),
                  b_ravg = align(restlen * sizeof(double)), b_out = align(P * sizeof(double));
-    const size_t total = 2 * C * b_x + C * (b_sel + b_rest) + b_cts + b_agg + b_z + b_ravg + b_out;
+    const size_t total = 2 * lanes * b_x + C * (b_sel + b_rest) + b_cts + b_agg + b_z + b_ravg + b_out;
     if ((rc = ensure(&ctx->round_buf, &ctx->round_bytes, total)) != HE_OK) return rc;
     if ((rc = ensure(&ctx->ws, &ctx->ws_bytes, fft_work_bytes(d, Tc))) != HE_OK) return rc;
     unsigned char *p = static_cast<unsigned char *>(ctx->round_buf);
-    unsigned char *xbuf[2] = {p, p + C * b_x};
-    p += 2 * C * b_x;
+    unsigned char *xbuf[2] = {p, p + lanes * b_x};
+    p += 2 * lanes * b_x;
     std::vector<float *> sel(C), rest(C);
     for (int i = 0; i < C; i++) { sel[i] = reinterpret_cast<float *>(p); p += b_sel; }
     for (int i = 0; i < C; i++) { rest[i] = reinterpret_cast<float *>(p); p += b_rest; }
@@ -1029,25 +1033,28 @@ static int round_host_queued(he_ctx *ctx, const he_keys *keys, const he_mask *ma
     std::vector<const uint64_t *> cptr(C);
     std::vector<const float *> rptr(C);
     size_t t = 0, r = 0, home = 0;                    // ciphertexts, remainder entries and ranges that are done
+    int b = 1;                                        // the set of buffers in use
     for (size_t c = 0; c < R; c++) {
-        const int b = (int)(c & 1);
         const size_t end = ready(c), now = end - t < Tc ? end - t : Tc;
         auto encrypt = [&](int i, size_t tc) -> int {
             uint64_t *ci = cts + (size_t)i * Tc * ctw;
             cptr[i] = ci;
             return he_encrypt_range(ctx, keys, sel[i] + t * n, t, tc, enc_seed, (uint32_t)i, ci, stream);
         };
-        CU(cudaStreamWaitEvent(ctx->copy_stream, ctx->ev_free[b], 0));
         for (int i = 0; i < C; i++) {
+            if (i % lanes == 0) {
+                b ^= 1;
+                CU(cudaStreamWaitEvent(ctx->copy_stream, ctx->ev_free[b], 0));
+            }
             // client by client: one's ciphertexts are encrypted while the next one's part comes up (a wait
             // takes the event's latest record at the time of the call)
-            float *x = reinterpret_cast<float *>(xbuf[b] + (size_t)i * b_x);
+            float *x = reinterpret_cast<float *>(xbuf[b] + i % lanes * b_x);
             CU(cudaMemcpyAsync(x, xs_host[i] + cut[c], (cut[c + 1] - cut[c]) * sizeof(float), cudaMemcpyHostToDevice, ctx->copy_stream));
             CU(cudaEventRecord(ctx->ev_ready[b], ctx->copy_stream));
             CU(cudaStreamWaitEvent(st, ctx->ev_ready[b], 0));
             CU(launch_pack_range(mask, x, cut[c], cut[c + 1] - cut[c], sel[i], restlen ? rest[i] : nullptr, st));
             if (c + 1 == R) CU(launch_zero(sel[i] + k, padded - k, st));
-            if (i + 1 == C) CU(cudaEventRecord(ctx->ev_free[b], st));
+            if (i + 1 == C || (i + 1) % lanes == 0) CU(cudaEventRecord(ctx->ev_free[b], st));
             if (now && (rc = encrypt(i, now)) != HE_OK) return rc;
         }
         for (size_t tc = now; t < end; tc = end - t < Tc ? end - t : Tc) {

@@ -378,6 +378,40 @@ def test_masked_host_round_into_memory_of_an_update(he):
     assert torch.equal(out, want)
 
 
+def test_masked_host_round_of_many_clients(he):
+    """Many clients do not multiply the memory of the uploads: beside every client's packed update the call may hold two whole
+    updates, or 512 MiB; and the model is that of the steps one by one."""
+    P, k, clients = 6_000_011, 4096, 256
+    torch.cuda.empty_cache()
+    g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
+    keys = he.he_keygen(g, 5)
+    he.he_ctx_reserve(g, k)
+    rng = np.random.default_rng(8)
+    xs = [torch.from_numpy((0.01 * rng.standard_normal(P)).astype(np.float32)).pin_memory() for _ in range(3)]
+    pick = [i % 3 for i in range(clients)]
+    alpha = [1.0 / clients] * clients
+    mask = he.he_select_mask(g, dev_f32(rng.random(P, dtype=np.float32)), k)
+    host = torch.empty(P, dtype=torch.float64).pin_memory()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    before = torch.cuda.mem_get_info()[0]
+    he.he_round_host(g, keys, mask, [xs[p] for p in pick], alpha, 99, host)
+    used = before - torch.cuda.mem_get_info()[0]
+    n, L = g.n, g.L
+    T = he.he_num_ct(g, k)
+    own = (clients * (T * n + P - k) * 4 + clients * T * 2 * L * g.N * 8 + T * 2 * (L - 1) * g.N * 8
+           + (T * n + (P - k) + P) * 8)
+    assert used <= own + 2 * max(4 * P, 256 << 20) + (64 << 20), (used, own)
+    rests, cts = [], []
+    for i, p in enumerate(pick):
+        sel, rest = he.he_pack(g, mask, xs[p].cuda())
+        rests.append(rest)
+        cts.append(he.he_encrypt(g, keys, sel, 99, i))
+    z = he.he_decrypt(g, keys, he.he_weighted_aggregate(g, cts, alpha))
+    want = he.he_unpack(g, mask, z, he.he_plain_aggregate(g, rests, alpha), P).cpu()
+    assert torch.equal(host, want)
+
+
 @pytest.mark.parametrize("P,spread", [(1, 1.0), (33, 1.0), (2047, 1.0), (2049, 1e-4), (300_001, 1e-4), (20_000_003, 1.0)])
 def test_select_mask_tiles_and_candidates(he, P, spread):
     """Edges of the tiles, tiles with more candidates than their list holds (all scores within one
