@@ -574,11 +574,11 @@ static int weighted_aggregate(he_ctx *ctx, const uint64_t *const *cts_host, cons
     if (mode == AGG_NTT) {
         int rc = ensure(&ctx->ws, &ctx->ws_bytes, 2 * T * (size_t)L * d.N * sizeof(uint64_t));
         if (rc != HE_OK) return rc;
-        CU(launch_aggregate_ntt(d, dptrs, dw, C, T, static_cast<uint64_t *>(ctx->ws), agg_dev, st));
+        CU(launch_aggregate_ntt(d, dptrs, dw, C, T, static_cast<uint64_t *>(ctx->ws), agg_dev, ctx->sm_count, st));
     } else if (mode == AGG_PARTIAL) {
-        CU(launch_aggregate_partial(d, dptrs, dw, C, T, agg_dev, st));
+        CU(launch_aggregate_partial(d, dptrs, dw, C, T, agg_dev, ctx->sm_count, st));
     } else {
-        CU(launch_aggregate(d, dptrs, dw, C, T, agg_dev, st));
+        CU(launch_aggregate(d, dptrs, dw, C, T, agg_dev, ctx->sm_count, st));
     }
     return HE_OK;
 }

@@ -63,14 +63,14 @@ cudaError_t launch_encrypt_ntt(const CtxDev &c, const KeysDev &k, const float *s
 
 // ptrs: device array of C ciphertext pointers; wtab: device [C][L] weights
 cudaError_t launch_aggregate(const CtxDev &c, const uint64_t *const *ptrs, const tw_t *wtab, int C,
-                             size_t T, uint64_t *out, cudaStream_t s);
+                             size_t T, uint64_t *out, int n_sm, cudaStream_t s);
 // transform-domain ciphertexts in and out; scratch: uint64 [T][2][L][N]
 cudaError_t launch_aggregate_ntt(const CtxDev &c, const uint64_t *const *ptrs, const tw_t *wtab, int C,
-                                 size_t T, uint64_t *scratch, uint64_t *out, cudaStream_t s);
+                                 size_t T, uint64_t *scratch, uint64_t *out, int n_sm, cudaStream_t s);
 // aligned16: every client's pointer is 16-byte aligned (the caller knows the host copies)
 // the clients' weighted sum on all L limbs without the rescale, and the rescale of a sum of such sums
 cudaError_t launch_aggregate_partial(const CtxDev &c, const uint64_t *const *ptrs, const tw_t *wtab, int C,
-                                     size_t T, uint64_t *out, cudaStream_t s);
+                                     size_t T, uint64_t *out, int n_sm, cudaStream_t s);
 cudaError_t launch_rescale_partial_sum(const CtxDev &c, const uint64_t *const *parts, int P, size_t T,
                                        uint64_t *out, cudaStream_t s);
 cudaError_t launch_plain_aggregate(const float *const *ptrs, const double *alpha, int C, size_t len,

@@ -42,6 +42,39 @@ struct SplitSum {
     }
 };
 
+// what a block stages of a weight: the word that the split or the double-precision sum reads, or that and its Shoup factor
+template <bool SPLIT> using staged_t = std::conditional_t<SPLIT, uint64_t, tw_t>;
+__device__ __forceinline__ double staged_f64(uint64_t w) { return f64_from_bits(w); }
+__device__ __forceinline__ double staged_f64(const tw_t &w) { return f64_from_u64(w.w); }
+
+// the sum of few clients: every product reduced
+__device__ __forceinline__ void weighted_sum_pair(const uint64_t *const *sp, const tw_t *sw, int C, uint32_t L,
+                                                  uint32_t j, size_t off, const LimbDev &lb, uint64_t &ax, uint64_t &ay) {
+    const uint64_t q = lb.q, q2 = 2 * q;
+    ax = 0;
+    ay = 0;
+    int cl = 0;
+    for (; cl + 4 <= C; cl += 4) {
+        ulonglong2 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) v[u] = __ldg(reinterpret_cast<const ulonglong2 *>(sp[cl + u] + off));
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const tw_t w = sw[(cl + u) * L + j];
+            ax = csub(ax + shoup_lazy(v[u].x, w.w, w.wp, q), q2);
+            ay = csub(ay + shoup_lazy(v[u].y, w.w, w.wp, q), q2);
+        }
+    }
+    for (; cl < C; cl++) {
+        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(sp[cl] + off));
+        const tw_t w = sw[cl * L + j];
+        ax = csub(ax + shoup_lazy(v.x, w.w, w.wp, q), q2);
+        ay = csub(ay + shoup_lazy(v.y, w.w, w.wp, q), q2);
+    }
+    ax = csub(ax, q);
+    ay = csub(ay, q);
+}
+
 __device__ __forceinline__ void weighted_sum_pair(const uint64_t *const *sp, const uint64_t *sw, int C, uint32_t L,
                                                   uint32_t j, size_t off, const LimbDev &lb, uint64_t &ax, uint64_t &ay) {
     unsigned __int128 sx = 0, sy = 0;
@@ -79,7 +112,8 @@ __device__ __forceinline__ void weighted_sum_pair(const uint64_t *const *sp, con
 // the transforms: a product costs the shared multiply / double-precision pipe 6 slots.  Every
 // product has magnitude at most 3q/4 and the running sum is brought back below q after every 32
 // clients, so it stays below 25 q < 2^51 and every addition is exact.
-__device__ __forceinline__ void weighted_sum_pair_f64(const uint64_t *const *sp, const uint64_t *sw, int C, uint32_t L,
+template <class W>
+__device__ __forceinline__ void weighted_sum_pair_f64(const uint64_t *const *sp, const W *sw, int C, uint32_t L,
                                                       uint32_t j, size_t off, double q, double qi, uint64_t &ax,
                                                       uint64_t &ay) {
     double sx = 0.0, sy = 0.0;
@@ -90,7 +124,7 @@ __device__ __forceinline__ void weighted_sum_pair_f64(const uint64_t *const *sp,
         for (int u = 0; u < 4; u++) v[u] = __ldg(reinterpret_cast<const ulonglong2 *>(sp[cl + u] + off));
 #pragma unroll
         for (int u = 0; u < 4; u++) {
-            const double w = f64_from_bits(sw[(cl + u) * L + j]);
+            const double w = staged_f64(sw[(cl + u) * L + j]);
             sx = f64_add(sx, f64_mulmod(f64_from_u64(v[u].x), w, q, qi));
             sy = f64_add(sy, f64_mulmod(f64_from_u64(v[u].y), w, q, qi));
         }
@@ -101,7 +135,7 @@ __device__ __forceinline__ void weighted_sum_pair_f64(const uint64_t *const *sp,
     }
     for (; cl < C; cl++) {
         const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(sp[cl] + off));
-        const double w = f64_from_bits(sw[cl * L + j]);
+        const double w = staged_f64(sw[cl * L + j]);
         sx = f64_add(sx, f64_mulmod(f64_from_u64(v.x), w, q, qi));
         sy = f64_add(sy, f64_mulmod(f64_from_u64(v.y), w, q, qi));
     }
@@ -110,24 +144,28 @@ __device__ __forceinline__ void weighted_sum_pair_f64(const uint64_t *const *sp,
 }
 
 // a limb's sum in whichever arithmetic its prime allows
-__device__ __forceinline__ void weighted_sum_limb(const LimbDev &lb, const uint64_t *const *sp, const uint64_t *sw, int C,
+template <class W>
+__device__ __forceinline__ void weighted_sum_limb(const LimbDev &lb, const uint64_t *const *sp, const W *sw, int C,
                                                   uint32_t L, uint32_t j, size_t off, uint64_t &ax, uint64_t &ay) {
     if (lb.fwd_d) weighted_sum_pair_f64(sp, sw, C, L, j, off, lb.qd, lb.qi, ax, ay);
     else weighted_sum_pair(sp, sw, C, L, j, off, lb, ax, ay);
 }
-// what the sums read of a weight
-__device__ __forceinline__ uint64_t staged_weight(const LimbDev &lb, uint64_t w) {
-    return lb.fwd_d ? f64_bits(f64_from_u64(w)) : (w & LOW30) | (w >> 30) << 32;
+template <bool SPLIT>
+__device__ __forceinline__ staged_t<SPLIT> staged_weight(const LimbDev &lb, const tw_t *w) {
+    const uint64_t v = __ldg(&w->w);
+    if constexpr (SPLIT) return lb.fwd_d ? f64_bits(f64_from_u64(v)) : (v & LOW30) | (v >> 30) << 32;
+    else return tw_t{v, __ldg(&w->wp)};
 }
 
+template <bool SPLIT>
 __global__ void __launch_bounds__(256)
 aggregate_rescale_kernel(const __grid_constant__ CtxDev c, const uint64_t *const *ptrs, const tw_t *wtab,
                          int C, uint64_t *out, size_t total) {
     extern __shared__ __align__(16) unsigned char agg_sm[];
     const uint32_t L = c.L;
-    uint64_t *sw = reinterpret_cast<uint64_t *>(agg_sm);                                    // [C][L]
+    auto *sw = reinterpret_cast<staged_t<SPLIT> *>(agg_sm);                         // [C][L]
     const uint64_t **sp = reinterpret_cast<const uint64_t **>(sw + (size_t)C * L);  // [C]
-    for (int e = threadIdx.x; e < C * (int)L; e += blockDim.x) sw[e] = staged_weight(c.limb[e % (int)L], __ldg(&wtab[e].w));
+    for (int e = threadIdx.x; e < C * (int)L; e += blockDim.x) sw[e] = staged_weight<SPLIT>(c.limb[e % (int)L], wtab + e);
     for (int e = threadIdx.x; e < C; e += blockDim.x) sp[e] = ptrs[e];
     __syncthreads();
     const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -156,17 +194,41 @@ aggregate_rescale_kernel(const __grid_constant__ CtxDev c, const uint64_t *const
     }
 }
 
+// Which sum is the faster one.  The split sum saves 9 slots a product and pays some 45 a coefficient at the end, and with the rescale it
+// takes 60 registers instead of 40: four thread blocks to an SM, not six.  Measured (us, every product reduced and split):
+//   many blocks: N = 16384, 60/40/40/60 bits, 100 ciphertexts, 2, 6, 8, 16 and 64 clients   86 98, 145 150, 172 168, 303 278, (25:) 297 264
+//   one wave either way: 5 of them, 2, 4, 6, 16 and 100 clients   16 14, 18 16, 22 20, 37 29, 176 113; 8 of them, 4 and 6   20 20, 25 22
+//   a wave of six blocks to an SM, but not of four: 11 of them, 6, 16 and 100 clients   27 29, 47 47, 222 228; with one limb of three
+//     below 2^46 (N = 8192, 22 ciphertexts, 100 clients) 176 176, with four of six (N = 32768, 5) 305 327, with all 148 170
+// Without the rescale both are bound by their loads: 5 and 100 ciphertexts, 33 clients   59 49, 565 545; 50 of N = 8192   119 129.
+static bool split_pays(const CtxDev &c, int C, size_t pairs, int n_sm, bool rescale) {
+    const size_t blocks = blocks_for(pairs, 256), sm = (size_t)n_sm;
+    if (!rescale) return blocks <= 5 * sm ? C >= 8 : blocks > 24 * sm && C >= 16;
+    if (blocks <= 4 * sm) return C >= (2 * blocks <= 5 * sm ? 2 : 6);
+    if (blocks > 6 * sm) return C >= 8;
+    uint32_t in_doubles = 0;
+    for (uint32_t j = 0; j < c.L; j++) in_doubles += c.limb[j].fwd_d ? 1 : 0;
+    return C >= 12 && 2 * in_doubles <= c.L;
+}
+static size_t sum_smem(const CtxDev &c, int C, bool split) {
+    return (size_t)C * c.L * (split ? sizeof(staged_t<true>) : sizeof(staged_t<false>)) + (size_t)C * sizeof(void *);
+}
+// kernels of the two sums, launched with what they stage
+template <class K, class... Args>
+static cudaError_t launch_sum(K kernel, size_t smem, size_t total, cudaStream_t s, const Args &...args) {
+    cudaError_t e;
+    if (smem > 48 * 1024 && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
+    kernel<<<blocks_for(total, 256), 256, smem, s>>>(args...);
+    return FEDHE_LAUNCHED();
+}
+
 cudaError_t launch_aggregate(const CtxDev &c, const uint64_t *const *ptrs, const tw_t *wtab, int C,
-                             size_t T, uint64_t *out, cudaStream_t s) {
+                             size_t T, uint64_t *out, int n_sm, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
     const size_t total = T * 2 * (c.N >> 1);
-    const size_t smem = (size_t)C * c.L * sizeof(uint64_t) + (size_t)C * sizeof(void *);
-    cudaError_t e;
-    if (smem > 48 * 1024 &&
-        (e = cudaFuncSetAttribute(aggregate_rescale_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
-        return e;
-    aggregate_rescale_kernel<<<blocks_for(total, 256), 256, smem, s>>>(c, ptrs, wtab, C, out, total);
-    return FEDHE_LAUNCHED();
+    const bool split = split_pays(c, C, total, n_sm, true);
+    return launch_sum(split ? aggregate_rescale_kernel<true> : aggregate_rescale_kernel<false>, sum_smem(c, C, split), total, s,
+                      c, ptrs, wtab, C, out, total);
 }
 
 // ---------------------------------------------------------------------------
@@ -180,14 +242,15 @@ cudaError_t launch_aggregate(const CtxDev &c, const uint64_t *const *ptrs, const
 // acc_j = sum_i W_i ct_i for all limbs: limbs below the last go to `out`
 // ([T][2][L-1][N]), the last limb to `last` ([T][2][N]); with `last` null all L
 // limbs go to `out` ([T][2][L][N]): the partial sum of a subset of the clients
+template <bool SPLIT>
 __global__ void __launch_bounds__(256)
 aggregate_sum_kernel(const __grid_constant__ CtxDev c, const uint64_t *const *ptrs, const tw_t *wtab, int C,
                      uint64_t *out, uint64_t *last, size_t total) {
     extern __shared__ __align__(16) unsigned char agg_sm[];
     const uint32_t L = c.L;
-    uint64_t *sw = reinterpret_cast<uint64_t *>(agg_sm);
+    auto *sw = reinterpret_cast<staged_t<SPLIT> *>(agg_sm);
     const uint64_t **sp = reinterpret_cast<const uint64_t **>(sw + (size_t)C * L);
-    for (int e = threadIdx.x; e < C * (int)L; e += blockDim.x) sw[e] = staged_weight(c.limb[e % (int)L], __ldg(&wtab[e].w));
+    for (int e = threadIdx.x; e < C * (int)L; e += blockDim.x) sw[e] = staged_weight<SPLIT>(c.limb[e % (int)L], wtab + e);
     for (int e = threadIdx.x; e < C; e += blockDim.x) sp[e] = ptrs[e];
     __syncthreads();
     const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -248,17 +311,18 @@ rescale_partial_sum_kernel(const __grid_constant__ CtxDev c, const uint64_t *con
     }
 }
 
+static cudaError_t launch_limb_sums(const CtxDev &c, const uint64_t *const *ptrs, const tw_t *wtab, int C, uint64_t *out,
+                                    uint64_t *last, size_t pairs, int n_sm, cudaStream_t s) {
+    const bool split = split_pays(c, C, pairs, n_sm, false);
+    return launch_sum(split ? aggregate_sum_kernel<true> : aggregate_sum_kernel<false>, sum_smem(c, C, split), pairs, s, c, ptrs, wtab,
+                      C, out, last, pairs);
+}
+
 cudaError_t launch_aggregate_partial(const CtxDev &c, const uint64_t *const *ptrs, const tw_t *wtab, int C,
-                                     size_t T, uint64_t *out, cudaStream_t s) {
+                                     size_t T, uint64_t *out, int n_sm, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
-    const size_t smem = (size_t)C * c.L * sizeof(uint64_t) + (size_t)C * sizeof(void *);
-    cudaError_t e;
-    if (smem > 48 * 1024 &&
-        (e = cudaFuncSetAttribute(aggregate_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
-        return e;
     const size_t pairs = T * 2 * (c.N >> 1);
-    aggregate_sum_kernel<<<blocks_for(pairs, 256), 256, smem, s>>>(c, ptrs, wtab, C, out, nullptr, pairs);
-    return FEDHE_LAUNCHED();
+    return launch_limb_sums(c, ptrs, wtab, C, out, nullptr, pairs, n_sm, s);
 }
 
 cudaError_t launch_rescale_partial_sum(const CtxDev &c, const uint64_t *const *parts, int P, size_t T,
@@ -299,17 +363,12 @@ aggregate_finish_kernel(const __grid_constant__ CtxDev c, const uint64_t *rem, u
 
 // scratch: [T][2][N] + [T][2][L-1][N] words
 cudaError_t launch_aggregate_ntt(const CtxDev &c, const uint64_t *const *ptrs, const tw_t *wtab, int C,
-                                 size_t T, uint64_t *scratch, uint64_t *out, cudaStream_t s) {
+                                 size_t T, uint64_t *scratch, uint64_t *out, int n_sm, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
     uint64_t *last = scratch, *rem = scratch + 2 * T * c.N;
-    const size_t smem = (size_t)C * c.L * sizeof(uint64_t) + (size_t)C * sizeof(void *);
     cudaError_t e;
-    if (smem > 48 * 1024 &&
-        (e = cudaFuncSetAttribute(aggregate_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
-        return e;
     const size_t pairs = T * 2 * (c.N >> 1);
-    aggregate_sum_kernel<<<blocks_for(pairs, 256), 256, smem, s>>>(c, ptrs, wtab, C, out, last, pairs);
-    if ((e = FEDHE_LAUNCHED())) return e;
+    if ((e = launch_limb_sums(c, ptrs, wtab, C, out, last, pairs, n_sm, s))) return e;
     if ((e = launch_ntt(c, false, last, 2 * T, c.N, c.L - 1, 1, s))) return e;
     if (c.L > 1) {
         const size_t n_last = 2 * T * c.N, n_out = n_last * (c.L - 1);

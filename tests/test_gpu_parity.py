@@ -680,6 +680,23 @@ def test_weighted_aggregate_many_clients_bit_exact(he, primes, C):
     assert np.array_equal(to_host_u64(he.he_rescale_partial_parts(g, parts)), want)
 
 
+@pytest.mark.parametrize("primes", [si.PRIMES_N8192, si.PRIMES_SWEEP[:3]], ids=["60-40-60", "60"])
+@pytest.mark.parametrize("C,T", [(1, 1), (2, 18), (3, 18), (7, 18), (8, 18), (3, 19), (11, 19), (12, 27), (7, 28), (8, 28)])
+def test_weighted_aggregate_either_sum_bit_exact(he, primes, C, T):
+    """Client and ciphertext counts on either side of what chooses between the sums (with 148 SMs: one wave of four thread
+    blocks each, 18 ciphertexts of N = 8192; one of six, 27; more)."""
+    N = 8192
+    g, o = contexts(he, N, primes, 30)
+    cts_o = [si.random_residues(7 * C + i, (T, 2, len(primes), N), primes) for i in range(C)]
+    alpha = np.random.default_rng(C).random(C)
+    alpha /= alpha.sum()
+    cts = [to_dev_u64(c) for c in cts_o]
+    W = o.weights(alpha)
+    summed = o.weighted_sum(cts_o, W)
+    assert np.array_equal(to_host_u64(he.he_weighted_partial(g, cts, alpha)), summed)
+    assert np.array_equal(to_host_u64(he.he_weighted_aggregate(g, cts, alpha)), o.rescale(summed))
+
+
 @pytest.mark.parametrize("N,primes,ld", [(8192, si.PRIMES_N8192, 40), (16384, si.PRIMES_N16384, 40),
                                          (32768, si.PRIMES_N32768, 45)],
                          ids=["n8192", "n16384", "n32768"])
