@@ -191,7 +191,8 @@ int he_ctx_create(const he_params *p, he_ctx **out) {
         host_unit_roots(d.N, roots);
         host_slot_twiddles(d.N, roots, ftw);
         rc = upload(ctx, reinterpret_cast<const double2 *>(ftw.data()), ftw.size() / 2, &d.ftw);
-        fft_cut(d);
+        fft_cut(d, ctx->enc);
+        d.enc = &ctx->enc;
         host_fft_tables(d.N, roots, fwd, inv, slot_of);
         if (rc == HE_OK) rc = upload(ctx, reinterpret_cast<const root_t *>(fwd.data()), fwd.size() / 2, &d.fft_fwd);
         if (rc == HE_OK) rc = upload(ctx, reinterpret_cast<const root_t *>(inv.data()), inv.size() / 2, &d.fft_inv);
@@ -285,7 +286,7 @@ int he_keygen(he_ctx *ctx, uint64_t seed, he_keys **out, void *stream) {
     k->magic = KEYS_MAGIC;
     k->ctx = ctx;
     k->storage = nullptr;
-    const size_t fft_words = (1 + 2 * (size_t)d.fft_pieces) * (d.N / 2);     // the secret, then the pieces of the public key
+    const size_t fft_words = d.N / 2 + fft_key_words(d);     // the secret, then the pieces of the public key
     const size_t bytes = 3 * LN * sizeof(tw_t) + fft_words * sizeof(double2) + d.N;
     void *tmp = nullptr;
     int rc = HE_OK;

@@ -522,7 +522,7 @@ bool encrypt_by_passes(const CtxDev &c, size_t T) {
     double per_ct = 1.8;
     for (uint32_t j = 0; j < c.L; j++) per_ct += c.limb[j].fwd_d ? 1.54 : 2.48;
     const double passes = 60.0 + 6.0 * c.L + per_ct * (double)T;
-    const double transforms = 40.0 + (1.5 + 0.89 * c.fft_pieces) * (double)T;
+    const double transforms = 40.0 + (1.5 + 0.89 * c.enc->way[0].products) * (double)T;
     return passes < (transforms > 170.0 ? transforms : 170.0);
 }
 size_t encrypt_passes_work_bytes(const CtxDev &c, size_t T) {

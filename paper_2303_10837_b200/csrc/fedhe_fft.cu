@@ -270,14 +270,14 @@ struct EncRing {
 };
 
 // first unit of a ciphertext, of both components, that begins at or after `pos` products
-__device__ __forceinline__ uint32_t fft_unit_at(const CtxDev &c, uint32_t pos) {
-    uint32_t half = pos >= c.fft_pieces ? 1 : 0, rest = pos - half * c.fft_pieces, j = 0;
+__host__ __device__ __forceinline__ uint32_t fft_unit_at(const EncWay &w, uint32_t pos) {
+    uint32_t half = pos >= w.products ? 1 : 0, rest = pos - half * w.products, j = 0;
     while (rest) {
-        const uint32_t p = c.enc_unit[j].products;
+        const uint32_t p = w.unit[j].products;
         rest = rest > p ? rest - p : 0;
         j++;
     }
-    return half * c.enc_units + j;
+    return half * w.units + j;
 }
 
 // value i (column, row, real or imaginary part) of a thread's columns from r0: its coefficient less the thread's number
@@ -426,7 +426,7 @@ __device__ __forceinline__ void enc_parked(int64_t (&val)[G::K], const unsigned 
 // PAIRS: some units are of two limbs (the code for both kinds costs the others 1.5 %).
 template <int CL, bool PAIRS>
 __global__ void __launch_bounds__(FftLay::NT, 2)
-encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const float *sel, unsigned char *work,
+encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ EncWay way, const KeysDev k, const float *sel, unsigned char *work,
                    uint32_t t0, uint64_t seed, uint32_t client, uint64_t *ct, uint32_t T, uint32_t S, uint32_t most_parts) {
     using G = EncRing<CL>;
     constexpr uint32_t N = G::N, n = G::n, NB = G::NB, NT = G::NT, R = G::R;
@@ -471,7 +471,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
     const uint32_t whole = T / nc * nc, rem = T - whole;
     const uint32_t parts = rem ? (nc / rem < most_parts ? nc / rem : most_parts) : 1;
     const uint32_t items = whole + rem * parts;           // at least as many as clusters
-    const uint32_t pieces = 2 * c.fft_pieces;
+    const uint32_t pieces = 2 * way.products;
     const bool leader = rank == 0 && threadIdx.x == 0;
     uint32_t next_item = cid;
 #pragma unroll 1
@@ -488,10 +488,10 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
             part = (item - whole) % parts;
             of = parts;
         }
-        const uint32_t first = fft_unit_at(c, pieces * part / of), last = fft_unit_at(c, pieces * (part + 1) / of);
-        const uint32_t unit_end = fft_unit_at(c, pieces * (part * S + rank + 1) / (of * S));
-        uint32_t unit = fft_unit_at(c, pieces * (part * S + rank) / (of * S));
-        const bool c0_too = first < c.enc_units, c1_too = last > c.enc_units;
+        const uint32_t first = fft_unit_at(way, pieces * part / of), last = fft_unit_at(way, pieces * (part + 1) / of);
+        const uint32_t unit_end = fft_unit_at(way, pieces * (part * S + rank + 1) / (of * S));
+        uint32_t unit = fft_unit_at(way, pieces * (part * S + rank) / (of * S));
+        const bool c0_too = first < way.units, c1_too = last > way.units;
         const uint32_t t = t0 + tl;
 
         // ---- preparation: u, four columns of one half at a time ----
@@ -606,22 +606,22 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const KeysDev k, const floa
             if (!turns.take([&](uint32_t parity) { return key_try(&key_bar, parity); })) atomicOr(c.status, STATUS_COPY);
         };
         auto key_of = [&](uint32_t u, uint32_t pb) {
-            const uint32_t comp = u >= c.enc_units ? 1 : 0;
-            const EncUnit &e = c.enc_unit[u - comp * c.enc_units];
+            const uint32_t comp = u >= way.units ? 1 : 0;
+            const EncUnit &e = way.unit[u - comp * way.units];
             return k.fft_pk + e.fft_key + ((size_t)comp * e.products * R + pb) * NB;
         };
         if constexpr (!(G::E_IN_SMEM)) __syncthreads();   // the buffer's last readers are done
         if (threadIdx.x == 0 && !turns.lost()) key_fetch(buf, key_of(unit, 0), &key_bar);
 #pragma unroll 1
         for (; unit < unit_end; unit++) {
-            const uint32_t comp = unit >= c.enc_units ? 1 : 0;
-            const EncUnit &e = c.enc_unit[unit - comp * c.enc_units];
+            const uint32_t comp = unit >= way.units ? 1 : 0;
+            const EncUnit &e = way.unit[unit - comp * way.units];
             const bool pair = PAIRS && e.limb2 != NO_LIMB;
 #pragma unroll 1
             for (uint32_t pb = 0; pb < e.products * R; pb++) {
                 const uint32_t p = pb >> CL, b = pb & (R - 1);
                 const uint32_t j = pair && p == 2 ? e.limb2 : e.limb;
-                const FftSplit &f = c.limb[j].split;
+                const FftSplit &f = c.limb[j].split[PAIRS];
                 const uint64_t q = c.limb[j].q;
                 cpx x[16];
                 {
@@ -938,44 +938,71 @@ static int random_bits(int logN, int t, double least) {
     return w;
 }
 
-// Decryption cuts for any c1.  Of the public key's limbs, two whose low pieces have products of 16 bits (up to 6 bits wide
+// Decryption cuts for any c1.  Of the public key's limbs, if they go in pairs, two whose low pieces have products of 16 bits (up to 6 bits wide
 // for N = 2^15, at 12 standard deviations: under 2^-102 a coefficient) share one product for both: three instead of
 // four, for instance for primes of 45 bits.  Another limb of two pieces is cut as low as the low piece's product is sure
 // to fit 32 bits (a coefficient is below N 2^(width - 1)), or else as high as the top one may be wide, where it
 // fits all the same (exponent 95: under 2^-136).
-void fft_cut(CtxDev &c) {
-    const int logN = (int)c.logN, sure = fft_sure_bits(logN), wide = fft_wide_bits(logN);
-    cut_residues(c.limb[0].q, sure, 31 - logN, c.dec_split);
-    c.term_limit = INT64_MAX;
+static void cut_limbs(CtxDev &c, bool in_pairs, EncWay &w, size_t &words) {
+    const int logN = (int)c.logN, sure = fft_sure_bits(logN), wide = fft_wide_bits(logN), narrow = random_bits(logN, 32, 95.0);
     uint32_t waiting = NO_LIMB;                        // unit of a limb that could share its low product
-    size_t words = 0;
-    c.enc_units = 0;
+    w.units = 0;
     for (uint32_t j = 0; j < c.L; j++) {
         const uint64_t q = c.limb[j].q;
-        if ((int64_t)(q / 4) < c.term_limit) c.term_limit = (int64_t)(q / 4);
         const int bits = bits_of(q);
-        const bool shares = bits > wide && bits - wide <= random_bits(logN, 16, 72.0);
+        const bool shares = in_pairs && bits > wide && bits - wide <= random_bits(logN, 16, 72.0);
         const bool low_fits = bits > wide && bits - sure + logN - 1 < 31;
         if (shares && waiting != NO_LIMB) {
-            EncUnit &e = c.enc_unit[waiting];
-            cut_residues(c.limb[e.limb].q, wide, random_bits(logN, 32, 95.0), c.limb[e.limb].split);
-            cut_residues(q, wide, random_bits(logN, 32, 95.0), c.limb[j].split);
+            EncUnit &e = w.unit[waiting];
+            cut_residues(c.limb[e.limb].q, wide, narrow, c.limb[e.limb].split[1]);
+            cut_residues(q, wide, narrow, c.limb[j].split[1]);
             e.limb2 = j;
             e.products = 3;
             waiting = NO_LIMB;
             continue;
         }
-        cut_residues(q, low_fits ? sure : wide, random_bits(logN, 32, 95.0), c.limb[j].split);
-        c.enc_unit[c.enc_units] = EncUnit{j, NO_LIMB, c.limb[j].split.pieces, 0};
-        if (shares) waiting = c.enc_units;
-        c.enc_units++;
+        FftSplit &f = c.limb[j].split[in_pairs];
+        cut_residues(q, low_fits ? sure : wide, narrow, f);
+        w.unit[w.units] = EncUnit{j, NO_LIMB, f.pieces, 0};
+        if (shares) waiting = w.units;
+        w.units++;
     }
-    c.fft_pieces = 0;
-    for (uint32_t u = 0; u < c.enc_units; u++) {
-        c.enc_unit[u].fft_key = words;
-        words += 2 * (size_t)c.enc_unit[u].products * (c.N / 2);
-        c.fft_pieces += c.enc_unit[u].products;
+    w.products = 0;
+    for (uint32_t u = 0; u < w.units; u++) {
+        w.unit[u].fft_key = words;
+        words += 2 * (size_t)w.unit[u].products * (c.N / 2);
+        w.products += w.unit[u].products;
     }
+}
+void fft_cut(CtxDev &c, EncWays &e) {
+    cut_residues(c.limb[0].q, fft_sure_bits((int)c.logN), 31 - (int)c.logN, c.dec_split);
+    c.term_limit = INT64_MAX;
+    for (uint32_t j = 0; j < c.L; j++)
+        if ((int64_t)(c.limb[j].q / 4) < c.term_limit) c.term_limit = (int64_t)(c.limb[j].q / 4);
+    size_t words = 0;
+    cut_limbs(c, true, e.way[0], words);
+    e.count = e.way[0].units < c.L ? 2 : 1;
+    if (e.count == 1) words = 0;
+    cut_limbs(c, false, e.way[e.count - 1], words);
+    for (uint32_t i = 0; i < e.count; i++) {
+        const EncWay &w = e.way[i];
+        for (uint32_t of = 1; of < ENC_SHARES; of++) {
+            uint32_t most = 0;
+            for (uint32_t part = 0; part < of; part++) {
+                uint32_t sum = 0;
+                const uint32_t end = fft_unit_at(w, 2 * w.products * (part + 1) / of);
+                for (uint32_t u = fft_unit_at(w, 2 * w.products * part / of); u < end; u++) sum += w.unit[u % w.units].products;
+                most = sum > most ? sum : most;
+            }
+            e.most[i][of] = (uint16_t)most;
+        }
+    }
+}
+static bool pairs_limbs(const CtxDev &c, uint32_t way) { return c.enc->way[way].units < c.L; }
+size_t fft_key_words(const CtxDev &c) {
+    size_t words = 0;
+    for (uint32_t i = 0; i < c.enc->count; i++) words += 2 * (size_t)c.enc->way[i].products * (c.N / 2);
+    return words;
 }
 
 // Asked how many thread blocks fit on an SM, the runtime answers 1 for any kernel that allocates tensor memory;
@@ -991,10 +1018,10 @@ static cudaError_t setup_ring(CtxDev &c, int n_sm) {
     using G = EncRing<CL>;
     static_assert(G::SMEM + 4096 <= ENC_ALONE_SMEM - 1024, "two thread blocks to an SM");
     cudaError_t e;
-    const bool pairs = c.enc_units < c.L;
-    if ((e = cudaFuncSetAttribute(pairs ? encrypt_fft_kernel<CL, true> : encrypt_fft_kernel<CL, false>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, ENC_ALONE_SMEM)))
-        return e;
+    for (uint32_t i = 0; i < c.enc->count; i++)
+        if ((e = cudaFuncSetAttribute(pairs_limbs(c, i) ? encrypt_fft_kernel<CL, true> : encrypt_fft_kernel<CL, false>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, ENC_ALONE_SMEM)))
+            return e;
     if ((e = cudaFuncSetAttribute(decrypt_fft_kernel<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FftRing<CL>::SMEM))) return e;
     if ((e = cudaFuncSetAttribute(enc_shape_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ENC_ALONE_SMEM))) return e;
     for (uint32_t alone = 0; alone < 2; alone++)
@@ -1019,8 +1046,14 @@ static cudaError_t setup_ring(CtxDev &c, int n_sm) {
 }
 cudaError_t fft_setup(CtxDev &c, int n_sm) { FEDHE_FOR_RING(c, setup_ring, c, n_sm) }
 
-// The thread blocks that work on a ciphertext together, whether they have their SMs to themselves, the clusters.
-struct EncPlan { uint32_t S, alone, clusters, parts; };
+// The units' way, the thread blocks that work on a ciphertext together, whether they have their SMs to themselves, the
+// clusters, and the clusters that may share a ciphertext of the last round.
+struct EncPlan { uint32_t way, S, alone, clusters, parts; };
+
+static EncPlan enc_plan_of(const CtxDev &c, uint32_t way, uint32_t S, uint32_t alone, uint32_t fit, uint32_t parts, size_t T) {
+    const size_t each = fit / T < parts ? fit / T : parts;
+    return EncPlan{way, S, alone, T >= fit ? fit : (uint32_t)(T * each), parts};
+}
 
 // With ciphertexts enough to fill the device: as many blocks as the ciphertext has of 2^12 points, or the next
 // number below that shares its units out evenly.  With fewer, larger clusters, by these measurements (us, L = 3 or 4):
@@ -1029,29 +1062,81 @@ struct EncPlan { uint32_t S, alone, clusters, parts; };
 //   N = 16384, 40: 2, 3, 6 blocks 110, 86, 75; 60: 2, 4 blocks 111, 92
 // so the largest clusters that hold all ciphertexts at one block to an SM, if they can do the 2 R blocks of the
 // preparation side by side, and else the largest that hold them at two.
-static EncPlan enc_plan(const CtxDev &c, size_t T) {
-    const uint32_t R = 1u << (c.logN - 13), units = 2 * c.enc_units, most = units < ENC_MOST ? units : ENC_MOST;
+static EncPlan enc_plan_by_size(const CtxDev &c, size_t T) {
+    const uint32_t R = 1u << (c.logN - 13), units = 2 * c.enc->way[0].units, most = units < ENC_MOST ? units : ENC_MOST;
     uint32_t base = R < most ? R : most;
     while (units % base) base--;
-    EncPlan p = {base, 0, 0, (units + base - 1) / base};
+    uint32_t S = base, one = 0, parts = (units + base - 1) / base;
     uint32_t alone = most, shared = most;
     while (alone > 1 && c.enc_fit[1][alone] < T) alone--;
     while (shared > base && c.enc_fit[0][shared] < T) shared--;
-    if (c.enc_fit[1][alone] >= T && alone >= base && (alone >= 2 * R || alone == most)) p = EncPlan{alone, 1, 0, 1};
-    else if (shared > base) p = EncPlan{shared, 0, 0, 1};
-    const uint32_t fit = c.enc_fit[p.alone][p.S];
+    if (c.enc_fit[1][alone] >= T && alone >= base && (alone >= 2 * R || alone == most)) S = alone, one = 1, parts = 1;
+    else if (shared > base) S = shared, parts = 1;
+    const uint32_t fit = c.enc_fit[one][S];
     // what is left after whole rounds of all clusters, or too few ciphertexts for the largest clusters: several to each
-    if (p.S == most || T > fit) p.parts = (units + p.S - 1) / p.S;
-    p.clusters = T >= fit ? fit : (uint32_t)T * (fit / (uint32_t)T < p.parts ? fit / (uint32_t)T : p.parts);
-    return p;
+    if (S == most || T > fit) parts = (units + S - 1) / S;
+    return enc_plan_of(c, 0, S, one, fit, parts, T);
+}
+
+// clusters that surely run at once: with sizes that do not divide the SMs of a part of the chip the last one may have to wait
+static uint32_t enc_sure_fit(const CtxDev &c, uint32_t alone, uint32_t S) {
+    const uint32_t fit = c.enc_fit[alone][S];
+    return S > 2 && S < 8 && fit > 1 ? fit - 1 : fit;
+}
+
+// What a plan takes, in us: a round is fixed + by_size / S + product * (block transforms of the busiest block's products),
+// fitted to 10,000 measurements of all plans for up to 200 ciphertexts of 2 to 12 limbs of 45 and 60 bits (nine of ten within
+// 10 %), for two blocks to an SM and for one.
+struct EncCost { double fixed, by_size, product; };
+static const EncCost ENC_COST[4][2] = {{{27.3, 12.7, 7.7}, {33.1, 2.2, 4.9}},
+                                       {{27.4, 40.1, 9.1}, {43.5, 13.7, 5.7}},
+                                       {{-2.2, 160.6, 12.6}, {26.2, 76.9, 6.8}},
+                                       {{-27.8, 410.0, 15.6}, {15.8, 226.7, 8.3}}};
+static double enc_plan_us(const CtxDev &c, const EncPlan &p, size_t T) {
+    const uint32_t ring = c.logN - 13;
+    auto round = [&](uint32_t clusters, uint32_t parts) {
+        const EncCost &k = ENC_COST[ring][p.alone || clusters <= enc_sure_fit(c, 1, p.S)];
+        return k.fixed + k.by_size / p.S + k.product * (c.enc->most[p.way][p.S * parts] << ring);
+    };
+    const size_t whole = T / p.clusters;
+    const uint32_t rem = (uint32_t)(T % p.clusters);
+    double us = whole ? (double)whole * round(p.clusters, 1) : 0.0;
+    if (rem) {
+        const uint32_t parts = p.clusters / rem < p.parts ? p.clusters / rem : p.parts;
+        us += round(rem * parts, parts);
+    }
+    return us;
+}
+
+// The plan by size, or for up to a round or two of ciphertexts of N = 16384 and up another one if it should be 5 % faster:
+// clusters of 2, 4 or 8, several of them to a ciphertext, and limbs by themselves.  Measured (us, by size and so; primes of 45 bits):
+//   N = 16384, L = 2, 1 ciphertext 106, 81; L = 12, 9 of them 116, 68; L = 4, 74 of them 159, 102
+//   N = 32768, L = 2, 1 of them 173, 101; L = 6, 9 of them 128, 92; L = 8, 36 of them 322, 236
+static EncPlan enc_plan(const CtxDev &c, size_t T) {
+    EncPlan best = enc_plan_by_size(c, T);
+    const uint32_t R = 1u << (c.logN - 13);
+    if (best.clusters < 1 || R == 1 || T > (R == 8 ? 1u : 2u) * c.enc_fit[0][R]) return best;
+    double us = 0.95 * enc_plan_us(c, best, T);
+    for (uint32_t way = 0; way < c.enc->count; way++)
+        for (uint32_t S = 2; S <= ENC_MOST; S *= 2)
+            for (uint32_t alone = 0; alone < 2; alone++) {
+                const uint32_t fit = enc_sure_fit(c, alone, S), units = 2 * c.enc->way[way].units;
+                if (fit < 1) continue;
+                const EncPlan p = enc_plan_of(c, way, S, alone, fit, (units + S - 1) / S, T);
+                const double t = enc_plan_us(c, p, T);
+                if (t < us) us = t, best = p;
+            }
+    return best;
 }
 
 template <int CL>
 static size_t ring_scratch(const CtxDev &c, size_t T) {
     using G = EncRing<CL>;
-    size_t most = 0;                                   // of any number of ciphertexts up to T
-    for (uint32_t S = enc_plan(c, T).S; S <= ENC_MOST; S++) {
-        const size_t want = T * ((2 * c.enc_units + S - 1) / S), fit = c.enc_fit[0][S], bytes = (want < fit ? want : fit) * (G::SHARED + S * G::OWN);
+    size_t most = 0;                                   // of any number of ciphertexts up to T, on any plan
+    for (uint32_t S = 1; S <= ENC_MOST; S++) {
+        const uint32_t units = 2 * c.enc->way[c.enc->count - 1].units;
+        if (S == 1 && enc_plan_by_size(c, T).S > 1) continue;
+        const size_t want = T * ((units + S - 1) / S), fit = c.enc_fit[0][S], bytes = (want < fit ? want : fit) * (G::SHARED + S * G::OWN);
         if (bytes > most) most = bytes;
     }
     return most;
@@ -1085,8 +1170,8 @@ static cudaError_t launch_encrypt_ring(const CtxDev &c, const KeysDev &k, const 
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     cudaError_t e;
-    if ((e = cudaLaunchKernelEx(&cfg, c.enc_units < c.L ? encrypt_fft_kernel<CL, true> : encrypt_fft_kernel<CL, false>, c, k, sel, static_cast<unsigned char *>(work), t0, seed, client, ct,
-                                (uint32_t)T, p.S, p.parts)))
+    if ((e = cudaLaunchKernelEx(&cfg, pairs_limbs(c, p.way) ? encrypt_fft_kernel<CL, true> : encrypt_fft_kernel<CL, false>, c, c.enc->way[p.way],
+                                k, sel, static_cast<unsigned char *>(work), t0, seed, client, ct, (uint32_t)T, p.S, p.parts)))
         return e;
     return FEDHE_LAUNCHED();
 }
@@ -1142,26 +1227,27 @@ cudaError_t launch_gauss_table(void *table, cudaStream_t s) {
 // the last one is the secret key.
 template <int CL>
 __global__ void __launch_bounds__(FftLay::NT)
-fft_key_kernel(const __grid_constant__ CtxDev c, const uint64_t *pk, const int8_t *s8, double2 *fft_pk, double2 *fft_s) {
+fft_key_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ EncWay way, const uint64_t *pk, const int8_t *s8, double2 *fft_pk, double2 *fft_s) {
     using G = FftRing<CL>;
     constexpr uint32_t NB = G::NB, NT = G::NT, R = G::R, n = G::n;
     extern __shared__ __align__(128) unsigned char smem[];
     double2 *buf = reinterpret_cast<double2 *>(smem);
     const uint32_t tid = threadIdx.x, b = blockIdx.x % R;
     uint32_t poly = blockIdx.x / R, u = 0;
-    while (u < c.enc_units && poly >= 2 * c.enc_unit[u].products) poly -= 2 * c.enc_unit[u++].products;
-    const bool secret = u == c.enc_units;
-    const EncUnit &e = c.enc_unit[secret ? 0 : u];
+    while (u < way.units && poly >= 2 * way.unit[u].products) poly -= 2 * way.unit[u++].products;
+    const bool secret = u == way.units;
+    const EncUnit &e = way.unit[secret ? 0 : u];
     const uint32_t comp = secret ? 0 : poly / e.products, product = secret ? 0 : poly % e.products;
-    auto piece = [&](uint32_t j, uint32_t of, uint32_t i) {
+    auto piece = [&](uint32_t second, uint32_t of, uint32_t i) {
+        const uint32_t j = second ? e.limb2 : e.limb;
         const uint64_t v = pk[((size_t)comp * c.L + j) * c.N + i], q = c.limb[j].q;
-        return fft_piece(c.limb[j].split, v > q / 2 ? (int64_t)(v - q) : (int64_t)v, of);
+        return fft_piece(c.limb[j].split[way.units < c.L], v > q / 2 ? (int64_t)(v - q) : (int64_t)v, of);
     };
     auto value = [&](uint32_t i) {
         if (secret) return (double)s8[i];
-        if (e.limb2 == NO_LIMB) return (double)piece(e.limb, product, i);
-        if (product == 0) return (double)(piece(e.limb, 0, i) + 65536 * piece(e.limb2, 0, i));
-        return (double)piece(product == 1 ? e.limb : e.limb2, 1, i);
+        if (e.limb2 == NO_LIMB) return (double)piece(0, product, i);
+        if (product == 0) return (double)(piece(0, 0, i) + 65536 * piece(1, 0, i));
+        return (double)piece(product == 1 ? 0 : 1, 1, i);
     };
     const OuterPath<CL> outer(c.fft_fwd, b);
     // the columns, in a loop, wait in the thread's own words of the buffer
@@ -1193,8 +1279,12 @@ static cudaError_t launch_fft_keys_ring(const CtxDev &c, const uint64_t *pk, con
     const size_t smem = (size_t)G::NB * 16;
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(fft_key_kernel<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))) return e;
-    fft_key_kernel<CL><<<(2 * c.fft_pieces + 1) * G::R, G::NT, smem, s>>>(c, pk, s8, fft_pk, fft_s);
-    return FEDHE_LAUNCHED();
+    for (uint32_t i = 0; i < c.enc->count; i++) {         // the secret with the first
+        const EncWay &way = c.enc->way[i];
+        fft_key_kernel<CL><<<(2 * way.products + (i == 0 ? 1 : 0)) * G::R, G::NT, smem, s>>>(c, way, pk, s8, fft_pk, fft_s);
+        if ((e = FEDHE_LAUNCHED())) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_fft_keys(const CtxDev &c, const uint64_t *pk, const int8_t *s8, double2 *fft_pk, double2 *fft_s,

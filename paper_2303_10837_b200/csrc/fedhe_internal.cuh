@@ -41,6 +41,19 @@ struct EncUnit {
     uint32_t products;
     size_t fft_key;              // first word of its key tables: [2 components][products][n]
 };
+// The units of a public-key half.
+struct EncWay {
+    uint32_t units, products;    // of all units
+    EncUnit unit[HE_MAX_LIMBS];
+};
+// Limbs in pairs where that is possible, and, if any are, every limb by itself too: fewer products, or more units to share out.
+constexpr uint32_t ENC_MOST = 8;       // thread blocks of a cluster that encrypts, at most
+constexpr uint32_t ENC_SHARES = 2 * HE_MAX_LIMBS + ENC_MOST;
+struct EncWays {
+    uint32_t count;
+    EncWay way[2];
+    uint16_t most[2][ENC_SHARES];      // of the products of a ciphertext shared out to so many blocks, the most that one has
+};
 
 // Per-prime constants and table pointers, passed to kernels by value.
 struct LimbDev {
@@ -58,7 +71,7 @@ struct LimbDev {
     const double *inv_d;
     double qd, qi;       // q and 1/q rounded
     double ninv_d, wn_d; // 1/N and (inverse twiddle of stage 0)/N
-    FftSplit split;      // of the public key's residues for the exact products by complex transforms
+    FftSplit split[2];   // of the public key's residues: for a limb by itself, and where limbs go in pairs
 };
 
 // the pieces of a limb that a transform in arithmetic M needs
@@ -81,8 +94,6 @@ struct LimbOf<ModF64> {
     static HD double wn(const LimbDev &lb) { return lb.wn_d; }
 };
 
-constexpr uint32_t ENC_MOST = 8;       // thread blocks of a cluster that encrypts, at most
-
 struct CtxDev {
     uint32_t N, logN, L;
     uint32_t LOGB, A;    // a length-N transform = 2^A blocks of 2^LOGB
@@ -93,8 +104,7 @@ struct CtxDev {
     const root_t *fft_fwd, *fft_inv;   // complex transforms of the exact products (fedhe_fft.cuh)
     const uint32_t *slot_of;           // slot of every value that the forward transform leaves
     FftSplit dec_split;                // of c1 on limb 0, for any c1
-    uint32_t enc_units, fft_pieces;    // units and products of a public-key half
-    EncUnit enc_unit[HE_MAX_LIMBS];
+    const EncWays *enc;                // host memory (the context's): kernels get the way they take by value
     int64_t term_limit;                // a quarter of the smallest prime
     uint16_t enc_fit[2][ENC_MOST + 1]; // clusters of a size that the device holds: two blocks to an SM, one
     const void *gauss;   // GaussTables
@@ -117,6 +127,7 @@ struct he_ctx {
     uint32_t magic;
     int device;
     fedhe::CtxDev dev;
+    fedhe::EncWays enc;
     he_params params;
     std::vector<void *> owned;     // device allocations freed with the context
     // growable work buffers (device)

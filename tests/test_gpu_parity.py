@@ -219,6 +219,14 @@ def primes_below(limit, N, count):
     (8192, (si.PRIMES_SWEEP[0],) + si.PRIMES_SWEEP_45[:5], 40),       # clusters of several sizes
     (16384, si.PRIMES_SWEEP_45[:2] + (si.PRIMES_SWEEP[0],), 75),
     (32768, si.PRIMES_SWEEP_45[:5], 38),
+    # few ciphertexts of limbs that could go in pairs: limbs by themselves, clusters with more blocks than units,
+    # several clusters to a ciphertext, pairs in clusters of two
+    (16384, si.PRIMES_SWEEP_45[:2], 1),
+    (16384, si.PRIMES_SWEEP_45[:12], 10),
+    (16384, si.PRIMES_SWEEP_45[:4], 74),
+    (32768, si.PRIMES_SWEEP_45[:2], 1),
+    (32768, si.PRIMES_SWEEP_45[:6], 9),
+    (32768, si.PRIMES_SWEEP_45[:8], 36),
     (65536, si.PRIMES_SWEEP[:2], 14),                                 # the last count that goes by passes ...
     (65536, si.PRIMES_SWEEP[:2], 15),                                 # ... and the first that does not
     (65536, si.PRIMES_SWEEP_45[:3], 38),                              # more than the clusters of the device
