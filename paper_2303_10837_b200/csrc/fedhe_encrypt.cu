@@ -512,25 +512,37 @@ cudaError_t launch_encrypt_ntt(const CtxDev &c, const KeysDev &k, const float *s
 // writes both products u^ pk0^ -> c0 and u^ pk1^ -> c1; (3) inverse block transforms of all slots; (4) outer
 // inverse stages fused with the error and message terms.  `work`: the encoded messages and the encoder's complex buffer.
 //
-// A limb of N = 2^16 is eight blocks of the complex transforms, which one thread block computes one after the other, so
-// few ciphertexts of few limbs take long there, and 45-bit limbs, two pieces each, are cheap here.  Measured (us, the
-// passes and the complex transforms; 1, 7, 31 and 92 ciphertexts): two 60-bit limbs 93, 115, 274, 690 and 183, 198, 232,
-// 546; four of 45 bits 88, 124, 301, 786 and 154, 170, 298, 830; eight of 60 bits 148, 271, 783, 2109 and 157, 183, 518, 1477.
-// The two sides below are lines through these; a first turn of the complex transforms takes 170 us whatever it holds.
+// A limb of N = 2^16 is eight blocks of the complex transforms, which one thread block computes one after the other, and what a
+// number of ciphertexts takes rises in steps with the rounds of clusters; the passes take the same for every ciphertext, less for limbs
+// below 2^46.  So with 60-bit limbs the passes are faster for few ciphertexts, and with 45-bit ones but for some counts just short of
+// a round, and again for many.  Measured (us, passes and transforms):
+//   two 60-bit limbs: 10, 24, 40, 92, 600 ciphertexts   143 214, 216 224, 341 333, 653 546, 3961 2870
+//   eight: 3, 5, 18, 40   180 177, 214 173, 452 478, 986 642;      four of 45 bits: 10, 31, 40, 92, 600   147 185, 298 298, 394 439, 761 824, 4608 4919
+//   twelve of 45 bits: 3, 10, 31, 92, 300   165 179, 300 407, 718 732, 1949 2141, 6166 6578
+// The passes by the line through these (up to 20 % low short of a whole wave of their thread blocks, hence 4 to 7 % in their favour),
+// the transforms by the cost of their plan.
 bool encrypt_by_passes(const CtxDev &c, size_t T) {
     if (c.logN < 16) return false;
-    double per_ct = 1.8;
-    for (uint32_t j = 0; j < c.L; j++) per_ct += c.limb[j].fwd_d ? 1.54 : 2.48;
-    const double passes = 60.0 + 6.0 * c.L + per_ct * (double)T;
-    const double transforms = 40.0 + (1.5 + 0.89 * c.enc->way[0].products) * (double)T;
-    return passes < (transforms > 170.0 ? transforms : 170.0);
+    if (T > PASSES_KNOWN) return c.passes_most > PASSES_KNOWN;
+    double fixed = 40.0, per_ct = 1.5, favour = 1.04;
+    for (uint32_t j = 0; j < c.L; j++) {
+        const bool in_doubles = c.limb[j].fwd_d != nullptr;
+        fixed += in_doubles ? 4.0 : 6.0 + 20.0 / c.L;
+        per_ct += in_doubles ? 1.54 : 2.48;
+        if (in_doubles) favour = 1.07;
+    }
+    return fixed + per_ct * (double)T < favour * enc_transforms_us(c, T);
 }
-size_t encrypt_passes_work_bytes(const CtxDev &c, size_t T) {
+// The largest number of ciphertexts that goes by passes: up to PASSES_KNOWN by the rule, beyond like the last counts before.
+uint32_t passes_most(const CtxDev &c) {
     if (c.logN < 16) return 0;
-    size_t most = T;               // the passes are taken for T itself or, if at all, up to a number below it
-    while (most && !encrypt_by_passes(c, most)) most /= 2;
-    most = 2 * most + 1 < T ? 2 * most + 1 : T;
-    return 2 * most * c.N * sizeof(uint64_t);
+    uint32_t T = PASSES_KNOWN;
+    while (T && !encrypt_by_passes(c, T)) T--;
+    return T > PASSES_KNOWN - 64 ? UINT32_MAX : T;
+}
+// what the passes need for any number of ciphertexts up to T
+size_t encrypt_passes_work_bytes(const CtxDev &c, size_t T) {
+    return 2 * (T < c.passes_most ? T : (size_t)c.passes_most) * c.N * sizeof(uint64_t);
 }
 cudaError_t launch_encrypt_passes(const CtxDev &c, const KeysDev &k, const float *sel, void *work, uint32_t t0, size_t T,
                                   uint64_t seed, uint32_t client, uint64_t *ct, cudaStream_t s) {

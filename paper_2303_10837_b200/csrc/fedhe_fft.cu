@@ -1044,7 +1044,13 @@ static cudaError_t setup_ring(CtxDev &c, int n_sm) {
         }
     return cudaSuccess;
 }
-cudaError_t fft_setup(CtxDev &c, int n_sm) { FEDHE_FOR_RING(c, setup_ring, c, n_sm) }
+static cudaError_t setup_this_ring(CtxDev &c, int n_sm) { FEDHE_FOR_RING(c, setup_ring, c, n_sm) }
+cudaError_t fft_setup(CtxDev &c, int n_sm) {
+    const cudaError_t e = setup_this_ring(c, n_sm);
+    if (e) return e;
+    c.passes_most = passes_most(c);
+    return cudaSuccess;
+}
 
 // The units' way, the thread blocks that work on a ciphertext together, whether they have their SMs to themselves, the
 // clusters, and the clusters that may share a ciphertext of the last round.
@@ -1108,7 +1114,7 @@ static double enc_plan_us(const CtxDev &c, const EncPlan &p, size_t T) {
     return us;
 }
 
-// The plan by size, or for up to a round or two of ciphertexts of N = 16384 and up another one if it should be 5 % faster:
+// The plan by size, or for up to a round or two of ciphertexts of N = 16384 and up another one if it should be 5 % faster (10 % at N = 65536):
 // clusters of 2, 4 or 8, several of them to a ciphertext, and limbs by themselves.  Measured (us, by size and so; primes of 45 bits):
 //   N = 16384, L = 2, 1 ciphertext 106, 81; L = 12, 9 of them 116, 68; L = 4, 74 of them 159, 102
 //   N = 32768, L = 2, 1 of them 173, 101; L = 6, 9 of them 128, 92; L = 8, 36 of them 322, 236
@@ -1116,7 +1122,7 @@ static EncPlan enc_plan(const CtxDev &c, size_t T) {
     EncPlan best = enc_plan_by_size(c, T);
     const uint32_t R = 1u << (c.logN - 13);
     if (best.clusters < 1 || R == 1 || T > (R == 8 ? 1u : 2u) * c.enc_fit[0][R]) return best;
-    double us = 0.95 * enc_plan_us(c, best, T);
+    double us = (R == 8 ? 0.9 : 0.95) * enc_plan_us(c, best, T);
     for (uint32_t way = 0; way < c.enc->count; way++)
         for (uint32_t S = 2; S <= ENC_MOST; S *= 2)
             for (uint32_t alone = 0; alone < 2; alone++) {
@@ -1127,6 +1133,11 @@ static EncPlan enc_plan(const CtxDev &c, size_t T) {
                 if (t < us) us = t, best = p;
             }
     return best;
+}
+
+double enc_transforms_us(const CtxDev &c, size_t T) {
+    const EncPlan p = enc_plan(c, T);
+    return p.clusters ? enc_plan_us(c, p, T) : 0.0;
 }
 
 template <int CL>

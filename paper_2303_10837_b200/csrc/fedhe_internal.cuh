@@ -107,6 +107,7 @@ struct CtxDev {
     const EncWays *enc;                // host memory (the context's): kernels get the way they take by value
     int64_t term_limit;                // a quarter of the smallest prime
     uint16_t enc_fit[2][ENC_MOST + 1]; // clusters of a size that the device holds: two blocks to an SM, one
+    uint32_t passes_most;              // encryption by passes (N = 2^16): the most ciphertexts that go by them
     const void *gauss;   // GaussTables
     uint32_t *deal;      // encryption hands out ciphertexts here: next one, thread blocks (clusters) that are done; 0 between calls
     int *status;         // sticky anomaly word

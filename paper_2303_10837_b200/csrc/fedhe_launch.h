@@ -29,8 +29,8 @@ cudaError_t launch_decode(const CtxDev &c, const int64_t *d, size_t T, double2 *
                           cudaStream_t s);
 
 // Encode + encrypt ciphertexts t0 .. t0+T-1 (sel and ct point at the first of
-// them).  `work` is scratch of fft_work_bytes() bytes, what the resident thread
-// blocks keep in L2.
+// them).  `work` is scratch of fft_work_bytes() bytes: what the resident thread
+// blocks keep in L2, or, by passes, what those need.
 size_t fft_work_bytes(const CtxDev &c, size_t T);
 cudaError_t launch_encrypt(const CtxDev &c, const KeysDev &k, const float *sel, void *work, uint32_t t0, size_t T,
                            uint64_t seed, uint32_t client, uint64_t *ct, cudaStream_t s);
@@ -38,9 +38,12 @@ cudaError_t launch_encrypt(const CtxDev &c, const KeysDev &k, const float *sel, 
 void fft_cut(CtxDev &c, EncWays &e);
 size_t fft_key_words(const CtxDev &c);
 cudaError_t fft_setup(CtxDev &c, int n_sm);
-// The same by passes over the ciphertext, on the longest ring, where encrypt_by_passes() says that it is faster; scratch
-// of encrypt_passes_work_bytes() for any number of ciphertexts up to T.
+// The same by passes over the ciphertext, on the longest ring, for the numbers of ciphertexts where encrypt_by_passes() says that it
+// is faster; scratch of encrypt_passes_work_bytes() for any number up to T (16 N bytes for each that may go by passes).
+constexpr uint32_t PASSES_KNOWN = 1024;
 bool encrypt_by_passes(const CtxDev &c, size_t T);
+uint32_t passes_most(const CtxDev &c);                // sets CtxDev::passes_most
+double enc_transforms_us(const CtxDev &c, size_t T);   // estimate of the time by transforms
 size_t encrypt_passes_work_bytes(const CtxDev &c, size_t T);
 cudaError_t launch_encrypt_passes(const CtxDev &c, const KeysDev &k, const float *sel, void *work, uint32_t t0, size_t T,
                                   uint64_t seed, uint32_t client, uint64_t *ct, cudaStream_t s);

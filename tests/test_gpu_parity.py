@@ -227,9 +227,14 @@ def primes_below(limit, N, count):
     (32768, si.PRIMES_SWEEP_45[:2], 1),
     (32768, si.PRIMES_SWEEP_45[:6], 9),
     (32768, si.PRIMES_SWEEP_45[:8], 36),
-    (65536, si.PRIMES_SWEEP[:2], 14),                                 # the last count that goes by passes ...
-    (65536, si.PRIMES_SWEEP[:2], 15),                                 # ... and the first that does not
-    (65536, si.PRIMES_SWEEP_45[:3], 38),                              # more than the clusters of the device
+    (65536, si.PRIMES_SWEEP[:2], 14),
+    (65536, si.PRIMES_SWEEP[:2], 15),
+    (65536, si.PRIMES_SWEEP[:2], 21),                                 # the last count that goes by passes ...
+    (65536, si.PRIMES_SWEEP[:2], 22),                                 # ... and the first that does not
+    (65536, si.PRIMES_SWEEP[:2], 38),                                 # more than the clusters of the device; by passes again,
+    (65536, si.PRIMES_SWEEP[:2], 45),                                 # and by transforms
+    (65536, si.PRIMES_SWEEP_45[:3], 38),
+    (65536, si.PRIMES_SWEEP_45[:12], 40),                             # primes below 2^46: by passes at any larger count
     (8192, primes_below(1 << 61, 8192, 2), 3),                        # the largest primes: pieces that take 64 bits
     (65536, primes_below(1 << 61, 65536, 2), 15),
 ])
