@@ -30,10 +30,11 @@
  *     Calls are asynchronous on it unless stated otherwise.  A context keeps
  *     library-owned work buffers; calls that share a context must be issued
  *     on one stream at a time.  A call that needs more work space than the
- *     context holds (he_encode, he_encrypt*, he_decrypt*,
- *     he_threshold_combine, he_weighted_aggregate_ntt, he_round_host with a
- *     larger problem than before) frees and reallocates it, which
- *     synchronises the whole device once;
+ *     context holds (he_encode, he_encrypt*, he_decrypt* at N = 65536,
+ *     he_decrypt_level_ntt above N = 16384, he_threshold_combine,
+ *     he_weighted_aggregate_ntt, he_round_host with a larger problem than
+ *     before) frees and reallocates it, which synchronises the whole device
+ *     once;
  *     he_ctx_reserve does that ahead of time.
  *   - Kernels never trap or assert.  A numeric anomaly (an encoded
  *     coefficient of magnitude >= 2^62, or a non-finite input) sets a sticky

@@ -101,6 +101,12 @@ cudaMemPool_t mask_pool(int device) {
 
 size_t work_bytes(const he_ctx *ctx, size_t T) { return 2 * T * (size_t)ctx->dev.N * sizeof(uint64_t); }
 
+// of encryption and decryption in the coefficient format, any number of ciphertexts up to T
+size_t round_work_bytes(const he_ctx *ctx, size_t T) {
+    const size_t fft = fft_work_bytes(ctx->dev, T), dec = ctx->dev.logN < 16 ? 0 : work_bytes(ctx, T);
+    return fft > dec ? fft : dec;
+}
+
 }  // namespace
 
 namespace fedhe {
@@ -257,8 +263,8 @@ int he_ctx_reserve(he_ctx *ctx, size_t max_k) {
     if (!good(ctx)) return HE_ERR_INVALID_ARG;
     const size_t T = he_num_ct(ctx, max_k);
     size_t need = encrypt_ntt_work_bytes(ctx->dev, ctx->sm_count, T);
-    const size_t fft = fft_work_bytes(ctx->dev, T);
-    if (fft > need) need = fft;
+    const size_t round = round_work_bytes(ctx, T);
+    if (round > need) need = round;
     return ensure(&ctx->ws, &ctx->ws_bytes, need);
 }
 
@@ -663,12 +669,12 @@ static int decrypt_level(he_ctx *ctx, const he_keys *keys, const uint64_t *ct_de
     if (!ct_dev || !z_dev || !aligned16(ct_dev)) return HE_ERR_INVALID_ARG;
     const CtxDev &d = ctx->dev;
     cudaStream_t st = as_stream(stream);
-    if (!ntt_in) {
+    if (!ntt_in && !decrypt_by_passes(d, T)) {
         if (T >= (1ull << 32)) return HE_ERR_SIZE;
         CU(launch_decrypt_fft(d, keys->dev, ct_dev, level, T, z_dev, st));
         return HE_OK;
     }
-    if (d.logN <= 14) {                 // one fused kernel, no work buffer
+    if (ntt_in && d.logN <= 14) {       // one fused kernel, no work buffer
         CU(launch_decrypt_ntt_fused(d, keys->dev, ct_dev, level, T, z_dev, st));
         return HE_OK;
     }
@@ -676,7 +682,8 @@ static int decrypt_level(he_ctx *ctx, const he_keys *keys, const uint64_t *ct_de
     if (rc != HE_OK) return rc;
     uint64_t *scratch = static_cast<uint64_t *>(ctx->ws);
     double2 *cplx = reinterpret_cast<double2 *>(scratch + T * d.N);
-    CU(launch_decrypt_ntt(d, keys->dev, ct_dev, level, T, scratch, st));
+    if (ntt_in) CU(launch_decrypt_ntt(d, keys->dev, ct_dev, level, T, scratch, st));
+    else CU(launch_decrypt(d, keys->dev, ct_dev, level, T, scratch, st));
     CU(launch_decode(d, reinterpret_cast<const int64_t *>(scratch), T, cplx, z_dev, st));
     return HE_OK;
 }
@@ -866,7 +873,7 @@ static int round_host_full(he_ctx *ctx, const he_keys *keys, const float *const 
                  b_agg = align(Tmax * aggw * sizeof(uint64_t)), b_z = align(T * n * sizeof(double));
     int rc = ensure(&ctx->round_buf, &ctx->round_bytes, 2 * C * b_sel + b_cts + b_agg + b_z);
     if (rc != HE_OK) return rc;
-    if ((rc = ensure(&ctx->ws, &ctx->ws_bytes, fft_work_bytes(d, Tmax))) != HE_OK) return rc;
+    if ((rc = ensure(&ctx->ws, &ctx->ws_bytes, round_work_bytes(ctx, Tmax))) != HE_OK) return rc;
     if ((rc = round_host_streams(ctx)) != HE_OK) return rc;
     unsigned char *p = static_cast<unsigned char *>(ctx->round_buf);
     unsigned char *selbuf[2];
@@ -1008,7 +1015,7 @@ static int round_host_queued(he_ctx *ctx, const he_keys *keys, const he_mask *ma
                  b_ravg = align(restlen * sizeof(double)), b_out = align(P * sizeof(double));
     const size_t total = 2 * lanes * b_x + C * (b_sel + b_rest) + b_cts + b_agg + b_z + b_ravg + b_out;
     if ((rc = ensure(&ctx->round_buf, &ctx->round_bytes, total)) != HE_OK) return rc;
-    if ((rc = ensure(&ctx->ws, &ctx->ws_bytes, fft_work_bytes(d, Tc))) != HE_OK) return rc;
+    if ((rc = ensure(&ctx->ws, &ctx->ws_bytes, round_work_bytes(ctx, Tc))) != HE_OK) return rc;
     unsigned char *p = static_cast<unsigned char *>(ctx->round_buf);
     unsigned char *xbuf[2] = {p, p + lanes * b_x};
     p += 2 * lanes * b_x;

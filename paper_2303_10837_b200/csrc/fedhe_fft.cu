@@ -1218,6 +1218,22 @@ static cudaError_t launch_decrypt_ring(const CtxDev &c, const KeysDev &k, const 
     return FEDHE_LAUNCHED();
 }
 
+// At N = 2^16 a ciphertext takes a cluster of eight blocks, the device holds 33 of them (15 with their SMs to themselves), and c1
+// of 60 bits needs three pieces, so that the kernels of launch_decrypt(), which share out every ciphertext, are often faster.
+// Measured (us, those and the transforms):
+//   three pieces: 1, 14, 18, 28, 37, 75, 150, 600 ciphertexts   89 104, 99 98, 104 117, 139 117, 149 213, 296 320, 540 557, 1984 2055
+//   two pieces: 1, 14, 28, 37, 56, 110, 300, 600                71 80, 83 74, 114 88, 122 143, 186 171, 298 313, 827 762, 1572 1452
+// Both sides below are lines and steps through these.
+bool decrypt_by_passes(const CtxDev &c, size_t T) {
+    const uint32_t pieces = c.dec_split.pieces, fit = c.enc_fit[0][8], alone = c.enc_fit[1][8];
+    if (c.logN < 16 || pieces < 2 || fit < 1) return false;
+    const bool three = pieces > 2;
+    const double t = (double)T, rounds = (double)((T + fit - 1) / fit);
+    const double transforms = T <= alone ? (three ? 98.0 : 75.0) : T <= fit ? (three ? 118.0 : 90.0) : three ? 36.0 + 105.0 * rounds : 26.0 + 78.0 * rounds;
+    const double passes = T <= 18 ? (three ? 88.0 : 70.0) + t : T <= 37 ? (three ? 105.0 + 1.25 * t : 85.0 + 1.07 * t) : three ? 45.0 + 3.3 * t : 47.0 + 2.6 * t;
+    return passes < transforms;
+}
+
 cudaError_t launch_decrypt_fft(const CtxDev &c, const KeysDev &k, const uint64_t *ct, uint32_t level, size_t T,
                                double *z, cudaStream_t s) {
     if (T == 0) return cudaSuccess;

@@ -47,7 +47,9 @@ double enc_transforms_us(const CtxDev &c, size_t T);   // estimate of the time b
 size_t encrypt_passes_work_bytes(const CtxDev &c, size_t T);
 cudaError_t launch_encrypt_passes(const CtxDev &c, const KeysDev &k, const float *sel, void *work, uint32_t t0, size_t T,
                                   uint64_t seed, uint32_t client, uint64_t *ct, cudaStream_t s);
-// Decrypt + decode T coefficient-domain ciphertexts.
+// Decrypt + decode T coefficient-domain ciphertexts; by launch_decrypt() and launch_decode() where decrypt_by_passes() says that
+// those are faster.
+bool decrypt_by_passes(const CtxDev &c, size_t T);
 cudaError_t launch_decrypt_fft(const CtxDev &c, const KeysDev &k, const uint64_t *ct, uint32_t level, size_t T,
                                double *z, cudaStream_t s);
 // The table of the discrete Gaussian that encryption reads (CtxDev::gauss).

@@ -10,8 +10,8 @@
 // synchronisation that cudaMalloc/cudaFree imply.  For the rings this entry
 // point accepts (N <= 16384) he_decrypt itself runs one fused kernel that needs
 // no work buffer and allocates nothing either, and is the faster call; the
-// multi-kernel path is what he_decrypt uses on the longer rings, where it may
-// grow the context's work buffer.  This entry point gives a caller that path
+// multi-kernel path is what he_decrypt uses at N = 65536 for some counts, where it
+// may grow the context's work buffer.  This entry point gives a caller that path
 // with a guarantee that does not depend on which kernel the library picks: it
 // never allocates, at the price of a size limit and of about three extra
 // passes over T * N words.

@@ -258,6 +258,28 @@ def test_encrypt_counts_and_limbs_bit_exact(he, N, primes, T):
     assert torch.equal(part[T // 2:], ct[T // 2:])
 
 
+@pytest.mark.parametrize("primes", [si.PRIMES_SWEEP[:2], si.PRIMES_SWEEP_45[:2]], ids=["60", "45"])
+def test_decrypt_counts_on_the_longest_ring(he, primes):
+    """Counts on either side of what chooses between the two ways of decryption (one wave of clusters alone on their SMs and
+    with two blocks to an SM, and beyond): the first and the last ciphertext against the oracle."""
+    N, most = 65536, 57
+    g, o = contexts(he, N, primes, 40)
+    keys = he.he_keygen(g, 15)
+    s_o, _ = o.keygen(15)
+    n = N // 2
+    x = np.random.default_rng(4).normal(0, 0.02, most * n).astype(np.float32)
+    ct = he.he_encrypt(g, keys, dev_f32(x), 31, 2)
+    agg = he.he_weighted_aggregate(g, [ct], [1.0])
+    ref = {}
+    for T in (1, 14, 16, 18, 19, 33, 34, 40, 57):
+        z = he.he_decrypt(g, keys, agg[:T].contiguous()).cpu().numpy().reshape(T, n)
+        for t in {0, T - 1}:
+            if t not in ref:
+                ref[t] = o.decode(o.decrypt(s_o, to_host_u64(agg[t : t + 1]), 1)).reshape(-1)
+            assert np.abs(z[t] - ref[t]).max() <= DECODE_TOL, (T, t)
+        assert np.abs(z.reshape(-1) - x[: T * n]).max() <= fresh_noise_bound(N, 40)
+
+
 def oracle_ntt_of(o, ct):
     """Every limb polynomial of an oracle ciphertext [T][2][level][N] through the oracle's forward transform."""
     out = np.empty_like(ct)
