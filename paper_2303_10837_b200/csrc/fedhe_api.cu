@@ -962,27 +962,34 @@ static int round_host_queued(he_ctx *ctx, const he_keys *keys, const he_mask *ma
     if ((rc = round_host_streams(ctx)) != HE_OK) return rc;
 
     // Equal ranges, as many as make the call shortest by this account (us): a client's part of a range comes up
-    // at 55 GB/s; its ciphertexts take 35, 55, 115 or 200 (N = 2^13 .. 2^16) and 0.4, 1, 4 or 9 each; a range costs
-    // 50 besides; after the last upload come one client's ciphertexts, and the range's download.  (With ranges of
-    // 2^20 parameters, 12 clients and 3 M parameters at N = 2^15 spent 5.0 instead of 3.5 ms on short encryptions.)
+    // at 55 GB/s (the link of the machine that this was measured on); its ciphertexts take `first` (N = 2^13 .. 2^16) and, each,
+    // `product` for every product of a public-key half and two more; a range costs range_us besides; after the last upload
+    // come one client's ciphertexts, and the range's download.  (With ranges of 2^20 parameters, 12 clients and 3 M
+    // parameters at N = 2^15 spent 5.0 instead of 3.5 ms on short encryptions; with the cost of a ciphertext by the ring alone, 10
+    // clients and 3 M parameters, half of them masked, at N = 2^13 with twelve 60-bit primes 9.6 instead of 7.0 ms.)
     const size_t UNIT = 8192;
-    const double PCIE = 55e3, first_ct[4] = {35, 55, 115, 200}, each_ct[4] = {0.4, 1.0, 4.0, 9.0};
     const int ring = (int)d.logN - 13;
+    const double PCIE = 55e3, first_ct[4] = {35, 55, 115, 100}, range_us[4] = {50, 50, 50, 150}, product[4] = {0.057, 0.125, 0.33, 0.9};
+    const double first = first_ct[ring], each = product[ring] * (2 + d.enc->way[0].products);
     auto part_us = [&](double params) { return 4.0 * params / PCIE; };
-    auto encrypt_us = [&](double params) { return T ? first_ct[ring] + each_ct[ring] * (double)T * params / (double)P : 0.0; };
+    auto encrypt_us = [&](double params) { return T ? first + each * (double)T * params / (double)P : 0.0; };
     size_t ranges = 1;
     double best = 0;
     for (size_t m = 1; m <= 32 && m * UNIT <= P + UNIT; m++) {
         const double params = (double)P / (double)m, part = part_us(params), enc = encrypt_us(params);
-        const double us = (double)m * (C * (part > enc ? part : enc) + 50.0) + enc + 2.0 * part;
+        const double us = (double)m * (C * (part > enc ? part : enc) + range_us[ring]) + enc + 2.0 * part;
         if (m == 1) best = 0.95 * us;                 // a cut has to be worth its while
         else if (us < best) { best = us; ranges = m; }
     }
     size_t len = ((P + ranges - 1) / ranges + UNIT - 1) / UNIT * UNIT;
     std::vector<size_t> cut = {0};                    // boundaries
     while (P - cut.back() > len) cut.push_back(cut.back() + len);
-    // nothing hides the last range's way through the chip and back
-    for (size_t left = (P - cut.back()) / 2 / UNIT * UNIT; cut.size() > 1 && left && encrypt_us((double)left) <= part_us((double)left);
+    // nothing hides the last range's way through the chip and back: it is halved while the chip keeps up, or while its download
+    // takes longer than another range
+    auto worth_it = [&](double params) {
+        return encrypt_us(params) <= part_us(params) || part_us(params) > C * first + range_us[ring];
+    };
+    for (size_t left = (P - cut.back()) / 2 / UNIT * UNIT; cut.size() > 1 && left && worth_it((double)left);
          left = left / 2 / UNIT * UNIT)
         cut.push_back(cut.back() + left);
     cut.push_back(P);

@@ -376,7 +376,18 @@ def test_select_mask_ties_and_special_values(he):
 def test_host_round_by_ranges(he, P, k):
     """A masked round from host buffers, cut along the parameters, against the same round step by step on the
     device: one range and several, ranges that complete no ciphertext, nothing and everything masked."""
-    g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
+    host_round_against_the_steps(he, 8192, si.PRIMES_N8192, P, k)
+
+
+@pytest.mark.parametrize("N,primes", [(8192, si.PRIMES_SWEEP[:8]), (16384, si.PRIMES_SWEEP_45[:5]), (32768, si.PRIMES_SWEEP[:2]),
+                                      (65536, si.PRIMES_SWEEP[:2])])
+def test_host_round_by_ranges_of_other_contexts(he, N, primes):
+    """The same where ciphertexts cost more or less than those of the workloads' primes."""
+    host_round_against_the_steps(he, N, primes, 3_000_001, 700_000)
+
+
+def host_round_against_the_steps(he, N, primes, P, k):
+    g, _ = contexts(he, N, primes, 40)
     keys = he.he_keygen(g, 5)
     rng = np.random.default_rng(P + k)
     xs = [(0.01 * rng.standard_normal(P)).astype(np.float32) for _ in range(3)]
