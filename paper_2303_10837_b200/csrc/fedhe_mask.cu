@@ -125,7 +125,14 @@ key_histogram_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
 #pragma unroll
         for (int j = 0; j < HIST_LOADS; j++) count(v[j]);
     }
-    for (; i < P; i += step) count(__ldg(score + i));
+    for (; i < P; i += 4 * step) {
+        float v[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) v[j] = i + j * step < P ? __ldg(score + i + j * step) : 0.0f;
+#pragma unroll
+        for (int j = 0; j < 4; j++)
+            if (i + j * step < P) count(v[j]);
+    }
     __syncthreads();
     uint32_t even = 0, odd = 0;
 #pragma unroll
@@ -235,11 +242,10 @@ __device__ __forceinline__ void for_candidates(const float *score, size_t P, con
             f(in, in ? w.cand[tile * TILE_CANDIDATES + i + lane] : 0u);
         }
     } else {
-        for (uint32_t i = 0; i < MASK_BLOCK; i += 32) {
-            const size_t at = tile * MASK_BLOCK + i + lane;
-            const uint32_t key = at < P ? score_key(__ldg(score + at)) : 0u;
-            f(at < P && (key >> 20) == first_digit, key & 0xfffffu);
-        }
+        for_tile(score, P, tile * MASK_BLOCK, [&](uint32_t, const uint32_t (&key)[LOADS], uint32_t left) {
+#pragma unroll
+            for (int j = 0; j < LOADS; j++) f(j * 32u + lane < left && (key[j] >> 20) == first_digit, key[j] & 0xfffffu);
+        });
     }
 }
 
@@ -309,8 +315,9 @@ cudaError_t launch_select(const float *score, size_t P, size_t k, SelectWork &w,
     cudaError_t e;
     if ((e = cudaMemsetAsync(w.hist, 0, SELECT_ZEROED * sizeof(uint32_t), s))) return e;
     if ((e = cudaFuncSetAttribute(key_histogram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HIST_SMEM))) return e;
-    // one thread block of the first pass to an SM, unless its counters could overflow
-    const unsigned want = blocks_for(P, 1024 * HIST_LOADS), least = blocks_for(P, (unsigned)HIST_KEYS);
+    // One thread block of the first pass to an SM, unless its counters could overflow; two keys to a thread are enough (with
+    // sixteen, 100 k scores left a thread fourteen loads one after the other: 10 us more).
+    const unsigned want = blocks_for(P, 1024 * 2), least = blocks_for(P, (unsigned)HIST_KEYS);
     unsigned g1 = want < (unsigned)n_sm ? want : (unsigned)n_sm;
     if (g1 < least) g1 = least;
     key_histogram_kernel<<<g1, 1024, HIST_SMEM, s>>>(score, P, w, (uint32_t)k);
