@@ -197,7 +197,7 @@ int he_ctx_create(const he_params *p, he_ctx **out) {
         host_unit_roots(d.N, roots);
         host_slot_twiddles(d.N, roots, ftw);
         rc = upload(ctx, reinterpret_cast<const double2 *>(ftw.data()), ftw.size() / 2, &d.ftw);
-        fft_cut(d, ctx->enc);
+        if (!fft_cut(d, ctx->enc)) { rc = HE_ERR_PARAMS; break; }     // no prime that host_check_params() lets pass
         d.enc = &ctx->enc;
         host_fft_tables(d.N, roots, fwd, inv, slot_of);
         if (rc == HE_OK) rc = upload(ctx, reinterpret_cast<const root_t *>(fwd.data()), fwd.size() / 2, &d.fft_fwd);

@@ -14,8 +14,6 @@ __device__ __forceinline__ double fft_from_int(int64_t v) {
 }
 __device__ __forceinline__ int64_t fft_round_bits(double z) { return __double_as_longlong(f64_add(z, FFT_ROUND)); }
 
-__device__ __forceinline__ cpx fft_mul(double2 a, double2 b) { return cpx_mul(cpx{a.x, a.y}, b.x, b.y); }
-
 // The thread's number, read anew: what is computed from it cannot be kept in registers across a
 // transform, whose sixteen points need them (the kernels would spill addresses instead).
 __device__ __forceinline__ uint32_t fresh_tid() {
@@ -57,7 +55,7 @@ template <int CL_>
 struct FftRing {
     using Tab = FftTab<CL_>;
     static constexpr int CL = CL_, R = 1 << CL, NB = FftLay::NB, NT = FftLay::NT, n = R * NB, N = 2 * n;
-    static constexpr int PER = 16 / R, COLS = NB / R;     // columns of the R x NB view that a thread, a thread block finishes
+    static constexpr int PER = 16 / R;     // columns of the R x NB view that a thread finishes
     static constexpr size_t SMEM = (size_t)NB * 16 + (size_t)Tab::WORDS * 16;
 };
 
@@ -177,19 +175,6 @@ __device__ __forceinline__ void tmem_put8(uint32_t at, const uint32_t (&w)[8]) {
                  : "memory");
 }
 __device__ __forceinline__ void tmem_wait_put() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-// A load in two halves: the words count only after tmem_wait_get8().
-__device__ __forceinline__ void tmem_start_get8(uint32_t at, uint32_t (&w)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
-                 : "r"(at)
-                 : "memory");
-}
-__device__ __forceinline__ void tmem_wait_get8(uint32_t (&w)[8]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3]), "+r"(w[4]), "+r"(w[5]), "+r"(w[6]), "+r"(w[7])
-                 :
-                 : "memory");
-}
 __device__ __forceinline__ void tmem_get32(uint32_t at, uint32_t (&w)[32]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\ttcgen05.wait::ld.sync.aligned;"
                  : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]),
@@ -260,12 +245,14 @@ struct EncRing {
     // ... and for R <= 2 the 32-bit products of low pieces do, in the words from PARK_AT; for R = 1 the transform of u, from 0
     static constexpr bool PARK_TMEM = R <= 2;
     static constexpr uint32_t PARK_AT = 64;
+    // for R <= 2 those are all there are: of a prime below 2^61 the low piece has 21 bits at most, and 22 fit (cut_limbs() checks)
+    static constexpr bool ALL_NARROW = R <= 2;
     static constexpr int COLUMNS = R == 1 ? 4 : R == 8 ? 1 : 2, K = COLUMNS * R * 2;      // columns, values finished together
     // a cluster's: the transform of u, the message and e0, e1, u in two bits each, flags
     static constexpr size_t UHAT = (size_t)n * 16, TERMS = (size_t)N * 8, E1 = N, UBITS = (size_t)NB * 4,
                             SHARED = UHAT + TERMS + E1 + UBITS + 128;
     // a thread block's: what waits, joined low pieces
-    static constexpr size_t WAIT = (size_t)WAIT_L2 * NB * 16, PARK = (size_t)N * 8, OWN = WAIT + PARK;
+    static constexpr size_t WAIT = (size_t)WAIT_L2 * NB * 16, PARK = ALL_NARROW ? 0 : (size_t)N * 8, OWN = WAIT + PARK;
     static constexpr size_t SMEM = (size_t)NB * 16 + (size_t)Tab::WORDS * 16 + (E_IN_SMEM ? N : 0);
 };
 
@@ -324,7 +311,7 @@ __device__ __forceinline__ void enc_columns(cpx (&v)[G::COLUMNS][G::R], const cp
 // One block of a product waits for the last one.
 template <class G>
 __device__ __forceinline__ void enc_wait(const cpx (&x)[16], double2 *wait, uint32_t tm, uint32_t b, uint32_t tid) {
-    if (b < (uint32_t)G::WAIT_TMEM) {
+    if (G::WAIT_TMEM > 0 && (int)b < G::WAIT_TMEM) {
         if constexpr (G::R == 8) {
 #pragma unroll
             for (int r = 0; r < 16; r++) {
@@ -350,9 +337,9 @@ __device__ __forceinline__ int64_t fft_round(double z) { return fft_round_bits(z
 // A low piece's values are parked for the same thread, which will join the top one.
 template <class G>
 __device__ __forceinline__ void enc_park(const cpx (&v)[G::COLUMNS][G::R], unsigned char *park, uint32_t tm, const FftSplit &f,
-                                         uint32_t piece, uint32_t r0, uint32_t tid) {
+                                         uint32_t r0, uint32_t tid) {
     const uint32_t i0 = r0 * G::R * 2;
-    if (f.narrow) {
+    if (G::ALL_NARROW || f.narrow) {
         uint32_t w[G::K];
 #pragma unroll
         for (int i = 0; i < G::K; i++) {
@@ -366,14 +353,12 @@ __device__ __forceinline__ void enc_park(const cpx (&v)[G::COLUMNS][G::R], unsig
 #pragma unroll
             for (int i = 0; i < G::K; i++) __stcg(reinterpret_cast<uint32_t *>(park) + (i0 + i) * G::NT + tid, w[i]);
         }
-    } else {
+    } else {                                              // two pieces, 61 bits on the longer rings
         long long *p = reinterpret_cast<long long *>(park) + i0 * G::NT + tid;
 #pragma unroll
         for (int i = 0; i < G::K; i++) {
             const cpx &c = v[i / (2 * G::R)][(i / 2) % G::R];
-            long long w = fft_round((i & 1) ? c.im : c.re) << f.shift[piece];
-            if (piece) w += __ldcg(p + i * G::NT);
-            __stcg(p + i * G::NT, w);
+            __stcg(p + i * G::NT, (long long)fft_round((i & 1) ? c.im : c.re));
         }
     }
 }
@@ -396,7 +381,7 @@ __device__ __forceinline__ void enc_parked(int64_t (&val)[G::K], const unsigned 
 #pragma unroll
             for (int i = 0; i < G::K; i++) val[i] += low_of(__ldcg(reinterpret_cast<const int *>(park) + (i0 + i) * G::NT + tid));
         }
-    } else if (f.pieces > 1) {
+    } else if (!G::ALL_NARROW && f.pieces > 1) {
 #pragma unroll
         for (int i = 0; i < G::K; i++) val[i] += __ldcg(reinterpret_cast<const long long *>(park) + (i0 + i) * G::NT + tid);
     }
@@ -675,7 +660,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
                     for (uint32_t r0 = 0; r0 < 16; r0 += G::COLUMNS) {
                         cpx v[G::COLUMNS][R];
                         enc_columns<G>(v, x, buf, wait, tm, tab, r0, tid);
-                        enc_park<G>(v, park, tm, f, p, r0, tid);
+                        enc_park<G>(v, park, tm, f, r0, tid);
                     }
                     if constexpr (G::PARK_TMEM) tmem_wait_put();
                     if constexpr (R > 2) fetch_next();
@@ -943,7 +928,8 @@ static int random_bits(int logN, int t, double least) {
 // four, for instance for primes of 45 bits.  Another limb of two pieces is cut as low as the low piece's product is sure
 // to fit 32 bits (a coefficient is below N 2^(width - 1)), or else as high as the top one may be wide, where it
 // fits all the same (exponent 95: under 2^-136).
-static void cut_limbs(CtxDev &c, bool in_pairs, EncWay &w, size_t &words) {
+// False for a prime that the kernels are not made for: more than two pieces, or, for N <= 2^14, a wide low one.
+static bool cut_limbs(CtxDev &c, bool in_pairs, EncWay &w, size_t &words) {
     const int logN = (int)c.logN, sure = fft_sure_bits(logN), wide = fft_wide_bits(logN), narrow = random_bits(logN, 32, 95.0);
     uint32_t waiting = NO_LIMB;                        // unit of a limb that could share its low product
     w.units = 0;
@@ -967,23 +953,28 @@ static void cut_limbs(CtxDev &c, bool in_pairs, EncWay &w, size_t &words) {
         if (shares) waiting = w.units;
         w.units++;
     }
+    for (uint32_t j = 0; j < c.L; j++) {
+        const FftSplit &f = c.limb[j].split[in_pairs];
+        if (f.pieces > 2 || (f.pieces == 2 && !f.narrow && logN <= 14)) return false;
+    }
     w.products = 0;
     for (uint32_t u = 0; u < w.units; u++) {
         w.unit[u].fft_key = words;
         words += 2 * (size_t)w.unit[u].products * (c.N / 2);
         w.products += w.unit[u].products;
     }
+    return true;
 }
-void fft_cut(CtxDev &c, EncWays &e) {
+bool fft_cut(CtxDev &c, EncWays &e) {
     cut_residues(c.limb[0].q, fft_sure_bits((int)c.logN), 31 - (int)c.logN, c.dec_split);
     c.term_limit = INT64_MAX;
     for (uint32_t j = 0; j < c.L; j++)
         if ((int64_t)(c.limb[j].q / 4) < c.term_limit) c.term_limit = (int64_t)(c.limb[j].q / 4);
     size_t words = 0;
-    cut_limbs(c, true, e.way[0], words);
+    if (!cut_limbs(c, true, e.way[0], words)) return false;
     e.count = e.way[0].units < c.L ? 2 : 1;
     if (e.count == 1) words = 0;
-    cut_limbs(c, false, e.way[e.count - 1], words);
+    if (!cut_limbs(c, false, e.way[e.count - 1], words)) return false;
     for (uint32_t i = 0; i < e.count; i++) {
         const EncWay &w = e.way[i];
         for (uint32_t of = 1; of < ENC_SHARES; of++) {
@@ -997,6 +988,7 @@ void fft_cut(CtxDev &c, EncWays &e) {
             e.most[i][of] = (uint16_t)most;
         }
     }
+    return true;
 }
 static bool pairs_limbs(const CtxDev &c, uint32_t way) { return c.enc->way[way].units < c.L; }
 size_t fft_key_words(const CtxDev &c) {

@@ -395,16 +395,6 @@ template <int CL>
 __device__ __forceinline__ void buffer_free() {
     if constexpr (CL > 0) cluster_arrive();
 }
-// everything that any thread of the cluster wrote is visible to all
-template <int CL>
-__device__ __forceinline__ void cluster_meet() {
-    buffer_wait<CL>();
-    if constexpr (CL > 0) {
-        cluster_arrive();
-        cluster_wait();
-        cluster_arrive();
-    }
-}
 // x in layout A -> layout C (unscaled, with omega^-tid, without the registers' constants).  The
 // buffer is not given free: its words in layout C are the thread's own.  has_read() runs when the thread has
 // taken its values from there.

@@ -35,7 +35,7 @@ size_t fft_work_bytes(const CtxDev &c, size_t T);
 cudaError_t launch_encrypt(const CtxDev &c, const KeysDev &k, const float *sel, void *work, uint32_t t0, size_t T,
                            uint64_t seed, uint32_t client, uint64_t *ct, cudaStream_t s);
 // Once per context: how the products cut the residues (from the primes); then, on its device, what the device holds of these kernels (CtxDev::enc_fit).
-void fft_cut(CtxDev &c, EncWays &e);
+bool fft_cut(CtxDev &c, EncWays &e);
 size_t fft_key_words(const CtxDev &c);
 cudaError_t fft_setup(CtxDev &c, int n_sm);
 // The same by passes over the ciphertext, on the longest ring, for the numbers of ciphertexts where encrypt_by_passes() says that it
