@@ -914,15 +914,6 @@ static void cut_residues(uint64_t q, int most, int narrow_bits, FftSplit &f) {
     f.narrow = f.pieces == 2 && (int)f.shift[1] <= narrow_bits;
     f.top_scale = ldexp(1.0, (int)f.shift[f.pieces - 1]) / (double)q;
 }
-// Widest random piece whose product stays below 2^(t - 1).  A coefficient is a sum of N independent terms u_k p_k,
-// strictly sub-Gaussian with variance 2^(2 width) / 18 each, so the chance of a larger one is at most
-// 2 exp(-9 2^(2 t - 2) / (N 2^(2 width))); `least` is what the exponent has to reach.
-static int random_bits(int logN, int t, double least) {
-    int w = 0;
-    while (ldexp(9.0, 2 * t - 2 - logN - 2 * (w + 1)) >= least) w++;
-    return w;
-}
-
 // Decryption cuts for any c1.  Of the public key's limbs, if they go in pairs, two whose low pieces have products of 16 bits (up to 6 bits wide
 // for N = 2^15, at 12 standard deviations: under 2^-102 a coefficient) share one product for both: three instead of
 // four, for instance for primes of 45 bits.  Another limb of two pieces is cut as low as the low piece's product is sure
@@ -930,13 +921,13 @@ static int random_bits(int logN, int t, double least) {
 // fits all the same (exponent 95: under 2^-136).
 // False for a prime that the kernels are not made for: more than two pieces, or, for N <= 2^14, a wide low one.
 static bool cut_limbs(CtxDev &c, bool in_pairs, EncWay &w, size_t &words) {
-    const int logN = (int)c.logN, sure = fft_sure_bits(logN), wide = fft_wide_bits(logN), narrow = random_bits(logN, 32, 95.0);
+    const int logN = (int)c.logN, sure = fft_sure_bits(logN), wide = fft_wide_bits(logN), narrow = fft_random_bits(logN, 32, FFT_NARROW_EXPONENT);
     uint32_t waiting = NO_LIMB;                        // unit of a limb that could share its low product
     w.units = 0;
     for (uint32_t j = 0; j < c.L; j++) {
         const uint64_t q = c.limb[j].q;
         const int bits = bits_of(q);
-        const bool shares = in_pairs && bits > wide && bits - wide <= random_bits(logN, 16, 72.0);
+        const bool shares = in_pairs && bits > wide && bits - wide <= fft_random_bits(logN, 16, FFT_PAIR_EXPONENT);
         const bool low_fits = bits > wide && bits - sure + logN - 1 < 31;
         if (shares && waiting != NO_LIMB) {
             EncUnit &e = w.unit[waiting];

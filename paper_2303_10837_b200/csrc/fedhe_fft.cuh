@@ -77,6 +77,17 @@ inline int fft_wide_bits(int logN) {
     return b;
 }
 
+// Widest random piece whose product stays below 2^(t - 1).  A coefficient is a sum of N independent terms u_k p_k,
+// strictly sub-Gaussian with variance 2^(2 width) / 18 each, so the chance of a larger one is at most
+// 2 exp(-9 2^(2 t - 2) / (N 2^(2 width))); `least` is what the exponent has to reach.
+inline int fft_random_bits(int logN, int t, double least) {
+    int w = 0;
+    while (ldexp(9.0, 2 * t - 2 - logN - 2 * (w + 1)) >= least) w++;
+    return w;
+}
+// `least` for the 16-bit products of two limbs' low pieces, and for 32-bit ones
+constexpr double FFT_PAIR_EXPONENT = 72.0, FFT_NARROW_EXPONENT = 95.0;
+
 // ---- geometry ------------------------------------------------------------------
 //
 // A block of NB = 2^12 points is transformed by NT = 256 threads with 16 points

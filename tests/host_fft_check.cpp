@@ -75,16 +75,21 @@ static int check(uint32_t N) {
     const root_t *ft = reinterpret_cast<const root_t *>(fwd.data()), *it = reinterpret_cast<const root_t *>(inv.data());
     std::mt19937_64 rng(N);
     int bad = 0;
-    for (int kind = 0; kind < 4; kind++) {
-        // sure pieces: uniform, largest values with random signs, largest values of one sign; wide ones: uniform
-        const int b = kind == 3 ? fft_wide_bits(logN) : fft_sure_bits(logN);
+    for (int kind = 0; kind < 8; kind++) {
+        // sure pieces: uniform, largest values with random signs, largest values of one sign; wide ones: uniform, of several
+        // keys; and the low pieces of two limbs in one operand
+        const bool wide = kind >= 3 && kind < 7, pair = kind == 7;
+        const int low_bits = fft_random_bits(logN, 16, FFT_PAIR_EXPONENT);
+        const int b = wide ? fft_wide_bits(logN) : pair ? 16 + low_bits : fft_sure_bits(logN);
         const double sd = fft_error_sd(logN, b);
         // of 2^16 errors the largest is near 4.3 standard deviations, and 8 are never seen
-        const double bound = kind == 3 ? 8 * sd : (11.4 * (logN - 1) + 23.0) * std::ldexp(1.0, logN + b - 1 - 53);
-        std::vector<int64_t> p(N), u(N);
+        const double bound = wide || pair ? 8 * sd : (11.4 * (logN - 1) + 23.0) * std::ldexp(1.0, logN + b - 1 - 53);
+        std::vector<int64_t> p(N), u(N), low[2] = {std::vector<int64_t>(N), std::vector<int64_t>(N)};
         const int64_t top = (int64_t)1 << (b - 1);
         for (uint32_t i = 0; i < N; i++) {
-            p[i] = kind == 0 || kind == 3 ? (int64_t)(rng() >> (64 - b)) - top : kind == 1 ? ((rng() & 1) ? top : -top) : top;
+            low[0][i] = (int64_t)(rng() >> (64 - low_bits)) - ((int64_t)1 << (low_bits - 1));
+            low[1][i] = (int64_t)(rng() >> (64 - low_bits)) - ((int64_t)1 << (low_bits - 1));
+            p[i] = pair ? low[0][i] + 65536 * low[1][i] : kind == 0 || wide ? (int64_t)(rng() >> (64 - b)) - top : kind == 1 ? ((rng() & 1) ? top : -top) : top;
             u[i] = kind == 2 ? 1 : (int64_t)(rng() % 3) - 1;
         }
         auto transform = [&](const std::vector<int64_t> &a, uint32_t blk, Block &B) {
@@ -144,8 +149,16 @@ static int check(uint32_t N) {
         double worst = 0;
         for (int s = 0; s < 300; s++) {           // single coefficients against the schoolbook sum
             const uint32_t k = s < 4 ? (s & 1 ? N - 1 - s / 2 : s / 2) : (uint32_t)(rng() % N);
-            int64_t want = 0;
-            for (uint32_t i = 0; i < N; i++) want += i <= k ? u[i] * p[k - i] : -u[i] * p[N + k - i];
+            auto product = [&](const std::vector<int64_t> &a) {
+                int64_t sum = 0;
+                for (uint32_t i = 0; i < N; i++) sum += i <= k ? u[i] * a[k - i] : -u[i] * a[N + k - i];
+                return sum;
+            };
+            const int64_t want = product(p);
+            if (pair) {                           // each limb's product out of the rounded word
+                const int64_t z = (int64_t)std::nearbyint(c[k]), first = (int16_t)z;
+                if (first != product(low[0]) || (z - first) >> 16 != product(low[1])) { std::printf("pair of limbs\n"); bad = 1; }
+            }
             worst = std::max(worst, std::fabs(c[k] - (double)want));
         }
         double off = 0, sq = 0;                   // and the distance of all of them to an integer
@@ -157,7 +170,7 @@ static int check(uint32_t N) {
         std::printf("N %u, %d bits, kind %d: error %.3g, off an integer %.3g (rms %.3g, model %.3g), bound %.3g\n", N, b, kind, worst,
                     off, std::sqrt(sq / N), sd, bound);
         if (!(worst < bound) || !(off < bound)) bad = 1;
-        if (kind == 3 && std::sqrt(sq / N) > sd) bad = 1;
+        if (wide && std::sqrt(sq / N) > sd) bad = 1;
     }
     return bad;
 }

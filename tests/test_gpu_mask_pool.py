@@ -39,7 +39,8 @@ for mask_last in (False, True, False):
     torch.cuda.empty_cache()
     after = torch.cuda.mem_get_info()[0]
     assert before - inside > 70 << 20, (before, inside)
-    assert after == before, (mask_last, before, after)
+    # the figures are the device's, so other programs move them a little; the pool would hold all of what was used inside
+    assert before - after < 8 << 20, (mask_last, before, after)
 print("ok")
 """
 

@@ -235,8 +235,13 @@ def primes_below(limit, N, count):
     (65536, si.PRIMES_SWEEP[:2], 45),                                 # and by transforms
     (65536, si.PRIMES_SWEEP_45[:3], 38),
     (65536, si.PRIMES_SWEEP_45[:12], 40),                             # primes below 2^46: by passes at any larger count
-    (8192, primes_below(1 << 61, 8192, 2), 3),                        # the largest primes: pieces that take 64 bits
-    (65536, primes_below(1 << 61, 65536, 2), 15),
+    (8192, primes_below(1 << 61, 8192, 2), 3),                        # the largest primes,
+    (16384, primes_below(1 << 61, 16384, 2), 3),
+    (32768, primes_below(1 << 61, 32768, 2), 3),                      # whose low pieces take 64 bits from here on
+    (65536, primes_below(1 << 61, 65536, 2), 15),                     # by passes
+    (65536, primes_below(1 << 61, 65536, 2), 24),                     # and by transforms
+    (65536, primes_below(1 << 44, 65536, 4), 31),                     # limbs that go in pairs on the longest ring
+    (65536, primes_below(1 << 44, 65536, 4), 56),
 ])
 def test_encrypt_counts_and_limbs_bit_exact(he, N, primes, T):
     """Each way of sharing out the work gives the same words: all ciphertexts of a call, the same one
@@ -278,6 +283,22 @@ def test_decrypt_counts_on_the_longest_ring(he, primes):
                 ref[t] = o.decode(o.decrypt(s_o, to_host_u64(agg[t : t + 1]), 1)).reshape(-1)
             assert np.abs(z[t] - ref[t]).max() <= DECODE_TOL, (T, t)
         assert np.abs(z.reshape(-1) - x[: T * n]).max() <= fresh_noise_bound(N, 40)
+
+
+@pytest.mark.parametrize("N,bits", [(8192, 30), (16384, 30), (32768, 30), (65536, 29), (65536, 30)])
+def test_decrypt_small_first_prime(he, N, bits):
+    """A first prime whose residues are one piece for the products with the secret (two for 30 bits at N = 65536)."""
+    primes = primes_below(1 << bits, N, 1) + si.PRIMES_SWEEP[:1]
+    g, o = contexts(he, N, primes, 20)
+    keys = he.he_keygen(g, 15)
+    s_o, pk_o = o.keygen(15)
+    T = 3
+    x = np.random.default_rng(bits).normal(0, 0.02, T * N // 2).astype(np.float32)
+    ct = he.he_encrypt(g, keys, dev_f32(x), 31, 2)
+    ct_o, bad = o.encrypt(pk_o, x, 31, 2)
+    assert bad == 0 and np.array_equal(to_host_u64(ct), ct_o)
+    z = he.he_decrypt_level(g, keys, ct, 2).cpu().numpy()
+    assert np.abs(z - o.decode(o.decrypt(s_o, ct_o, 2)).reshape(-1)).max() <= DECODE_TOL
 
 
 def oracle_ntt_of(o, ct):
@@ -386,12 +407,18 @@ def test_host_round_by_ranges_of_other_contexts(he, N, primes):
     host_round_against_the_steps(he, N, primes, 3_000_001, 700_000)
 
 
-def host_round_against_the_steps(he, N, primes, P, k):
+def test_host_round_with_many_ciphertexts_to_a_range(he):
+    """More ciphertexts in one range than 8 GiB hold for all clients: they are encrypted and summed in turns."""
+    host_round_against_the_steps(he, 8192, si.PRIMES_SWEEP, 600_000, 600_000, clients=64)
+
+
+def host_round_against_the_steps(he, N, primes, P, k, clients=3):
     g, _ = contexts(he, N, primes, 40)
     keys = he.he_keygen(g, 5)
     rng = np.random.default_rng(P + k)
-    xs = [(0.01 * rng.standard_normal(P)).astype(np.float32) for _ in range(3)]
-    alpha = [0.25, 0.5, 0.25]
+    xs = [(0.01 * rng.standard_normal(P)).astype(np.float32) for _ in range(3)] * (clients // 3 + 1)
+    xs = xs[:clients]
+    alpha = [0.25, 0.5, 0.25] if clients == 3 else [1.0 / clients] * clients
     mask = he.he_select_mask(g, dev_f32(rng.random(P, dtype=np.float32)), k)
     rests, cts = [], []
     for i, x in enumerate(xs):
@@ -724,6 +751,30 @@ def test_weighted_aggregate_many_clients_bit_exact(he, primes, C):
     parts = [he.he_weighted_partial(g, cts[:half], alpha[:half]), he.he_weighted_partial(g, cts[half:], alpha[half:])]
     assert np.array_equal(to_host_u64(parts[0]), o.weighted_sum(cts_o[:half], W[:half]))
     assert np.array_equal(to_host_u64(he.he_rescale_partial_parts(g, parts)), want)
+
+
+@pytest.mark.parametrize("C", [3, 4, 63, 64, 65, 128, 256])
+def test_weighted_aggregate_largest_values_bit_exact(he, C):
+    """The split sum where its accumulators are fullest: the largest primes, residues and weights, and client counts at
+    the ends of its groups (4 clients to 64 bits, 64 to 128)."""
+    N = 8192
+    primes = primes_below(1 << 61, N, 3)
+    g, o = contexts(he, N, primes, 30)
+    rng = np.random.default_rng(C)
+    cts_o, kinds = [], []
+    for i in range(4):
+        ct = np.empty((1, 2, 3, N), np.uint64)
+        for j, q in enumerate(primes):
+            ct[:, :, j] = q - 1 - (rng.integers(0, 3, (1, 2, N), dtype=np.uint64) if i else 0)
+        kinds.append(ct)
+    for i in range(C):
+        cts_o.append(kinds[i % 4 if i % 7 == 0 else 0])
+    alpha = [1.0] * C
+    dev = [to_dev_u64(k) for k in kinds]
+    cts = [dev[next(n for n, k in enumerate(kinds) if k is c)] for c in cts_o]
+    summed = o.weighted_sum(cts_o, o.weights(alpha))
+    assert np.array_equal(to_host_u64(he.he_weighted_partial(g, cts, alpha)), summed)
+    assert np.array_equal(to_host_u64(he.he_weighted_aggregate(g, cts, alpha)), o.rescale(summed))
 
 
 @pytest.mark.parametrize("primes", [si.PRIMES_N8192, si.PRIMES_SWEEP[:3]], ids=["60-40-60", "60"])
