@@ -71,7 +71,8 @@ WIDE_COST = 2.5
 INT_SLOTS_PER_BUTTERFLY = 6 * WIDE_COST + 4
 F64_SLOTS_FORWARD, F64_SLOTS_INVERSE = 8.0, 9.0
 F64_PRIME_LIMIT = 1 << 46
-COMPLEX_SLOTS_PER_BUTTERFLY = 10.0    # complex product (4 multiplies, 2 add/sub) and complex sum and difference
+ENCODER_SLOTS_PER_BUTTERFLY = 10.0    # complex product (4 multiplies, 2 add/sub) and complex sum and difference, each rounded
+PRODUCT_SLOTS_PER_BUTTERFLY = 6.0     # of the transforms behind the products: fused multiply-adds
 
 
 def transform_slots(primes, N, forward, inverse):
@@ -102,8 +103,8 @@ def key_products(primes, N):
 def encrypt_slots(primes, N):
     """Pipe slots of one ciphertext's encryption by complex transforms: the butterflies, and the products between."""
     n, products = N // 2, 2 * key_products(primes, N)
-    transform = (n // 2) * (n.bit_length() - 1) * COMPLEX_SLOTS_PER_BUTTERFLY
-    return (2 + products) * transform, products * n * 4.0
+    butterflies = (n // 2) * (n.bit_length() - 1)
+    return butterflies * (ENCODER_SLOTS_PER_BUTTERFLY + (1 + products) * PRODUCT_SLOTS_PER_BUTTERFLY), products * n * 4.0
 
 
 def fallback_peaks():
@@ -508,7 +509,7 @@ def measure(job, w, steps, warmup, with_cpu_baseline):
     if transform:                                            # three forward transforms per limb
         slots_per_ct, extra_per_ct = transform_slots(w.primes, w.N, 3, 0), 0.0
         if launches_per_encrypt == 1:                        # the encoder runs inside the kernel
-            slots_per_ct += (n // 2) * (n.bit_length() - 1) * COMPLEX_SLOTS_PER_BUTTERFLY
+            slots_per_ct += (n // 2) * (n.bit_length() - 1) * ENCODER_SLOTS_PER_BUTTERFLY
     else:
         slots_per_ct, extra_per_ct = encrypt_slots(w.primes, w.N)
         butterflies = (2 + 2 * key_products(w.primes, w.N)) * (n // 2) * (logN - 1) * per_launch
