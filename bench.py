@@ -65,7 +65,7 @@ UNIT = "params/s"
 # the slots, and one inverse per product of u with a piece of the public key.
 # DRAM bytes (read + write) per ciphertext of the encrypt kernel, by (N, L), from an ncu capture of
 # the profile_case.py encrypt case (traffic grows in proportion to the number of ciphertexts).
-ENCRYPT_DRAM_BYTES_PER_CT = {(16384, 4): 339.017984e6 / 296}       # encrypt_fft_kernel, 296 ciphertexts
+ENCRYPT_DRAM_BYTES_PER_CT = {(8192, 3): 110.983168e6 / 296, (16384, 4): 332.172544e6 / 296, (32768, 6): 999.883776e6 / 142}
 SLOTS_PER_SM_CLK = 64.0
 WIDE_COST = 2.5
 INT_SLOTS_PER_BUTTERFLY = 6 * WIDE_COST + 4
@@ -502,7 +502,7 @@ def measure(job, w, steps, warmup, with_cpu_baseline):
     if rank != 0:
         return None
 
-    # roofline of the dominant kernel (bound by the multiply / double-precision pipe)
+    # the dominant kernel against the pipe that its arithmetic takes (what bounds it is latency)
     logN = w.N.bit_length() - 1
     per_launch = Tr                                          # ciphertexts of one client's he_encrypt calls
     butterflies = 3 * w.L * (w.N // 2) * logN * per_launch

@@ -127,7 +127,7 @@ def kernels(workload):
     outs = [torch.empty(P, dtype=torch.float64, device="cuda") for _ in range(3)]
     zs = [z, z.clone(), z.clone()]
     rows = [
-        ("he_select_mask (k = P/10)", lambda i: he.he_select_mask(g, score, P // 10), 6 * 4.0 * P, 4),
+        ("he_select_mask (k = P/10)", lambda i: he.he_select_mask(g, score, P // 10), 4.0 * P + 4.0 * P / 10, 4),
         ("he_pack (full)", lambda i: he.he_pack(g, None, xs[i % C]), 8.0 * P, 8),
         ("he_pack (masked, 10 %)", lambda i: he.he_pack(g, mask, xs[i % C]), 8.0 * P + 4.0 * P / 10, 8),
         ("he_encode", lambda i: he.he_encode(g, sel), 4.0 * T * n + 8.0 * T * N, 4),
