@@ -156,7 +156,11 @@ int he_encode(he_ctx *ctx, const float *sel_dev, size_t k, int64_t *m_dev, void 
  * e0, e1 (Gaussian) from Philox streams of (seed, t, client_id):
  *   c0 = pk0 u + e0 + m,  c1 = pk1 u + e1  (mod q_j).
  * ct: dev uint64 [T][2][L][N].  A (seed, client_id, t) triple must not be
- * reused across rounds. */
+ * reused across rounds.
+ * The products pk u are computed by double-precision transforms of pieces of
+ * pk and rounded to the exact integers: not for every conceivable pk, but for
+ * all keys that he_keygen may draw except with a chance below 2^-100 for each
+ * coefficient (he_decrypt* rounds exactly whatever the ciphertext). */
 int he_encrypt(he_ctx *ctx, const he_keys *keys, const float *sel_dev, size_t k, uint64_t seed,
                uint32_t client_id, uint64_t *ct_dev, void *stream);
 
