@@ -301,6 +301,29 @@ def test_decrypt_small_first_prime(he, N, bits):
     assert np.abs(z - o.decode(o.decrypt(s_o, ct_o, 2)).reshape(-1)).max() <= DECODE_TOL
 
 
+@pytest.mark.parametrize("N,primes", [(8192, si.PRIMES_N8192), (16384, si.PRIMES_SWEEP_45[:4]), (32768, si.PRIMES_N32768),
+                                      (65536, si.PRIMES_SWEEP[:2])])
+def test_reserve_covers_every_smaller_call(he, N, primes):
+    """After he_ctx_reserve no encryption or decryption of that many ciphertexts or fewer allocates, whichever plan it takes."""
+    T, n, L = 45, N // 2, len(primes)
+    g, _ = contexts(he, N, primes, 40)
+    keys = he.he_keygen(g, 15)
+    sel = torch.zeros(T * n, device="cuda")
+    ct = torch.empty((T, 2, L, N), dtype=torch.int64, device="cuda")
+    agg = torch.zeros((T, 2, L - 1, N), dtype=torch.int64, device="cuda")
+    z = torch.empty(T * n, dtype=torch.float64, device="cuda")
+    he.he_ctx_reserve(g, T * n)
+    he.he_encrypt(g, keys, sel[:n], 1, 0, out=ct[:1])                # loads the kernels
+    he.he_decrypt(g, keys, agg[:1], out=z[:n])
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    for t in (1, 2, 3, 9, 14, 16, 20, 22, 34, 37, 44, T):
+        he.he_encrypt(g, keys, sel[: t * n], 1, 0, out=ct[:t])
+        he.he_decrypt(g, keys, agg[:t], out=z[: t * n])
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] < 4 << 20           # the figure is the device's: other programs move it a little
+
+
 def oracle_ntt_of(o, ct):
     """Every limb polynomial of an oracle ciphertext [T][2][level][N] through the oracle's forward transform."""
     out = np.empty_like(ct)
