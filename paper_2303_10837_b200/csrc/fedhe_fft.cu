@@ -1098,7 +1098,7 @@ static double enc_plan_us(const CtxDev &c, const EncPlan &p, size_t T) {
 }
 
 // The plan by size, or for up to a round or two of ciphertexts of N = 16384 and up another one if it should be 5 % faster (10 % at N = 65536):
-// clusters of 2, 4 or 8, several of them to a ciphertext, and limbs by themselves.  Measured (us, by size and so; primes of 45 bits):
+// clusters of 2, 4, 6 or 8, several of them to a ciphertext, and limbs by themselves.  Measured (us, by size and so; primes of 45 bits):
 //   N = 16384, L = 2, 1 ciphertext 106, 81; L = 12, 9 of them 116, 68; L = 4, 74 of them 159, 102
 //   N = 32768, L = 2, 1 of them 173, 101; L = 6, 9 of them 128, 92; L = 8, 36 of them 322, 236
 static EncPlan enc_plan(const CtxDev &c, size_t T) {
@@ -1107,7 +1107,7 @@ static EncPlan enc_plan(const CtxDev &c, size_t T) {
     if (best.clusters < 1 || R == 1 || T > (R == 8 ? 1u : 2u) * c.enc_fit[0][R]) return best;
     double us = (R == 8 ? 0.9 : 0.95) * enc_plan_us(c, best, T);
     for (uint32_t way = 0; way < c.enc->count; way++)
-        for (uint32_t S = 2; S <= ENC_MOST; S *= 2)
+        for (uint32_t S = 2; S <= ENC_MOST; S += 2)
             for (uint32_t alone = 0; alone < 2; alone++) {
                 const uint32_t fit = enc_sure_fit(c, alone, S), units = 2 * c.enc->way[way].units;
                 if (fit < 1) continue;

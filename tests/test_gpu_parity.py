@@ -225,12 +225,13 @@ def primes_below(limit, N, count):
     (16384, si.PRIMES_SWEEP_45[:12], 10),
     (16384, si.PRIMES_SWEEP_45[:4], 74),
     (32768, si.PRIMES_SWEEP_45[:2], 1),
+    (32768, si.PRIMES_SWEEP_45[:3], 20),                              # clusters of six
     (32768, si.PRIMES_SWEEP_45[:6], 9),
     (32768, si.PRIMES_SWEEP_45[:8], 36),
     (65536, si.PRIMES_SWEEP[:2], 14),
     (65536, si.PRIMES_SWEEP[:2], 15),
-    (65536, si.PRIMES_SWEEP[:2], 21),                                 # the last count that goes by passes ...
-    (65536, si.PRIMES_SWEEP[:2], 22),                                 # ... and the first that does not
+    (65536, si.PRIMES_SWEEP[:2], 18),                                 # the last count that goes by passes ...
+    (65536, si.PRIMES_SWEEP[:2], 19),                                 # ... and the first that does not
     (65536, si.PRIMES_SWEEP[:2], 38),                                 # more than the clusters of the device; by passes again,
     (65536, si.PRIMES_SWEEP[:2], 45),                                 # and by transforms
     (65536, si.PRIMES_SWEEP_45[:3], 38),
