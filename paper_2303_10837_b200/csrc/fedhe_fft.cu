@@ -247,7 +247,9 @@ struct EncRing {
     static constexpr uint32_t PARK_AT = 64;
     // for R <= 2 those are all there are: of a prime below 2^61 the low piece has 21 bits at most, and 22 fit (cut_limbs() checks)
     static constexpr bool ALL_NARROW = R <= 2;
-    static constexpr int COLUMNS = R == 1 ? 4 : R == 8 ? 1 : 2, K = COLUMNS * R * 2;      // columns, values finished together
+    static constexpr int COLUMNS = R == 1 ? 4 : R == 2 ? 2 : 1, K = COLUMNS * R * 2;      // columns, values finished together
+    // whether what a column needs from L2 is fetched a column ahead: of R = 8 it does not fit the registers
+    static constexpr bool FAR_AHEAD = R == 4;
     // a cluster's: the transform of u, the message and e0, e1, u in two bits each, flags
     static constexpr size_t UHAT = (size_t)n * 16, TERMS = (size_t)N * 8, E1 = N, UBITS = (size_t)NB * 4,
                             SHARED = UHAT + TERMS + E1 + UBITS + 128;
@@ -274,10 +276,38 @@ __device__ __forceinline__ uint32_t enc_coefficient(uint32_t r0, int i) {
     return (o % G::R) * G::NB + G::NT * (r0 + o / G::R) + (i & 1) * G::n;
 }
 
-// Columns r0 .. r0 + COLUMNS - 1 of a product after the stages between blocks.
+// What columns need from L2 is fetched ahead: a loop that loads it where it is used waits for every column.
 template <class G>
-__device__ __forceinline__ void enc_columns(cpx (&v)[G::COLUMNS][G::R], const cpx (&x)[16], const double2 *buf, const double2 *wait,
-                                            uint32_t tm, const root_t *tab, uint32_t r0, uint32_t tid) {
+struct EncAhead {
+    static constexpr int W = G::WAIT_L2 ? G::WAIT_L2 : 1;
+    cpx w[W];                              // the column in the blocks that wait in L2
+    int low[G::PARK_TMEM ? 1 : G::K];      // its parked words
+    __device__ __forceinline__ void fetch_wait(const double2 *wait, uint32_t r, uint32_t tid) {
+#pragma unroll
+        for (int a = 0; a < G::WAIT_L2; a++) {
+            const double2 v = __ldcg(wait + a * G::NB + r * G::NT + tid);
+            w[a] = cpx{v.x, v.y};
+        }
+    }
+    __device__ __forceinline__ void fetch_low(const unsigned char *park, uint32_t r, uint32_t tid) {
+        if constexpr (!G::PARK_TMEM) {
+            static_assert(G::COLUMNS == 1 && G::K % 4 == 0, "whole 16-byte words of one column");
+#pragma unroll
+            for (int i = 0; i < G::K; i += 4) {
+                const int4 v = __ldcg(reinterpret_cast<const int4 *>(park) + (r * (G::K / 4) + i / 4) * G::NT + tid);
+                low[i] = v.x;
+                low[i + 1] = v.y;
+                low[i + 2] = v.z;
+                low[i + 3] = v.w;
+            }
+        }
+    }
+};
+
+// Columns r0 .. r0 + COLUMNS - 1 of a product as they enter the stages between blocks ...
+template <class G>
+__device__ __forceinline__ void enc_columns(cpx (&v)[G::COLUMNS][G::R], const cpx (&x)[16], const double2 *buf, const EncAhead<G> &ahead,
+                                            uint32_t tm, uint32_t r0, uint32_t tid) {
     if constexpr (G::R == 1) {
 #pragma unroll
         for (int i = 0; i < G::COLUMNS; i++) v[i][0] = x[r0 + i];
@@ -286,24 +316,17 @@ __device__ __forceinline__ void enc_columns(cpx (&v)[G::COLUMNS][G::R], const cp
         v[0][1] = x[r0];
         v[1][1] = x[r0 + 1];
     } else {
+        // pairs of blocks side by side: words [column][block]
+        tmem_get(tm + r0 * 8, v[0][0], v[0][1]);
 #pragma unroll
-        for (int i = 0; i < G::COLUMNS; i++) {
-#pragma unroll
-            for (int a = G::WAIT_TMEM; a + 1 < G::R; a++) {
-                const double2 w = __ldcg(wait + (a - G::WAIT_TMEM) * G::NB + (r0 + i) * G::NT + tid);
-                v[i][a] = cpx{w.x, w.y};
-            }
-            const double2 w = buf[(r0 + i) * G::NT + tid];
-            v[i][G::R - 1] = cpx{w.x, w.y};
-        }
-        if constexpr (G::COLUMNS == 2) {
-#pragma unroll
-            for (int a = 0; a < 2; a++) tmem_get(tm + a * 64 + r0 * 4, v[0][a], v[1][a]);
-        } else {
-            // pairs of blocks side by side: words [column][block]
-            tmem_get(tm + r0 * 8, v[0][0], v[0][1]);
-        }
+        for (int a = G::WAIT_TMEM; a + 1 < G::R; a++) v[0][a] = ahead.w[a - G::WAIT_TMEM];
+        const double2 w = buf[r0 * G::NT + tid];
+        v[0][G::R - 1] = cpx{w.x, w.y};
     }
+}
+// ... and after them
+template <class G>
+__device__ __forceinline__ void enc_between(cpx (&v)[G::COLUMNS][G::R], const root_t *tab, uint32_t r0, uint32_t tid) {
 #pragma unroll
     for (int i = 0; i < G::COLUMNS; i++) fft_outer_inverse<G::CL>(v[i], tab, tid, r0 + i);
 }
@@ -312,7 +335,7 @@ __device__ __forceinline__ void enc_columns(cpx (&v)[G::COLUMNS][G::R], const cp
 template <class G>
 __device__ __forceinline__ void enc_wait(const cpx (&x)[16], double2 *wait, uint32_t tm, uint32_t b, uint32_t tid) {
     if (G::WAIT_TMEM > 0 && (int)b < G::WAIT_TMEM) {
-        if constexpr (G::R == 8) {
+        if constexpr (G::R > 2) {
 #pragma unroll
             for (int r = 0; r < 16; r++) {
                 asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(tm + r * 8 + b * 4),
@@ -351,7 +374,8 @@ __device__ __forceinline__ void enc_park(const cpx (&v)[G::COLUMNS][G::R], unsig
             tmem_put8(tm + G::PARK_AT + i0, w);
         } else {
 #pragma unroll
-            for (int i = 0; i < G::K; i++) __stcg(reinterpret_cast<uint32_t *>(park) + (i0 + i) * G::NT + tid, w[i]);
+            for (int i = 0; i < G::K; i += 4)
+                __stcg(reinterpret_cast<uint4 *>(park) + (i0 + i) / 4 * G::NT + tid, make_uint4(w[i], w[i + 1], w[i + 2], w[i + 3]));
         }
     } else {                                              // two pieces, 61 bits on the longer rings
         long long *p = reinterpret_cast<long long *>(park) + i0 * G::NT + tid;
@@ -363,8 +387,8 @@ __device__ __forceinline__ void enc_park(const cpx (&v)[G::COLUMNS][G::R], unsig
     }
 }
 template <class G>
-__device__ __forceinline__ void enc_parked(int64_t (&val)[G::K], const unsigned char *park, uint32_t tm, const FftSplit &f,
-                                           uint32_t of_pair, uint32_t r0, uint32_t tid) {
+__device__ __forceinline__ void enc_parked(int64_t (&val)[G::K], const unsigned char *park, const EncAhead<G> &ahead, uint32_t tm,
+                                           const FftSplit &f, uint32_t of_pair, uint32_t r0, uint32_t tid) {
     const uint32_t i0 = r0 * G::R * 2;
     // the low piece's product: the word itself, or, of a pair, its lower 16 bits (signed) or what they leave
     auto low_of = [&](int w) {
@@ -379,7 +403,7 @@ __device__ __forceinline__ void enc_parked(int64_t (&val)[G::K], const unsigned 
             for (int i = 0; i < G::K; i++) val[i] += low_of((int)w[i]);
         } else {
 #pragma unroll
-            for (int i = 0; i < G::K; i++) val[i] += low_of(__ldcg(reinterpret_cast<const int *>(park) + (i0 + i) * G::NT + tid));
+            for (int i = 0; i < G::K; i++) val[i] += low_of(ahead.low[i]);
         }
     } else if (!G::ALL_NARROW && f.pieces > 1) {
 #pragma unroll
@@ -655,11 +679,16 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
                     for (int r = 0; r < 16; r++) buf[r * NT + tid] = make_double2(x[r].re, x[r].im);
                 }
                 constexpr int K = G::K;
+                EncAhead<G> ahead;
+                if constexpr (G::FAR_AHEAD) ahead.fetch_wait(wait, 0, tid);
                 if (pair ? p == 0 : p + 1 < f.pieces) {
 #pragma unroll(R <= 2 ? 16 : 1)
                     for (uint32_t r0 = 0; r0 < 16; r0 += G::COLUMNS) {
                         cpx v[G::COLUMNS][R];
-                        enc_columns<G>(v, x, buf, wait, tm, tab, r0, tid);
+                        if constexpr (!G::FAR_AHEAD) ahead.fetch_wait(wait, r0, tid);
+                        enc_columns<G>(v, x, buf, ahead, tm, r0, tid);
+                        if (G::FAR_AHEAD && r0 + G::COLUMNS < 16) ahead.fetch_wait(wait, r0 + G::COLUMNS, tid);
+                        enc_between<G>(v, tab, r0, tid);
                         enc_park<G>(v, park, tm, f, r0, tid);
                     }
                     if constexpr (G::PARK_TMEM) tmem_wait_put();
@@ -684,15 +713,26 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
                 };
                 int64_t next[K];
                 terms_of(next, 0);
+                if (G::FAR_AHEAD && f.narrow) ahead.fetch_low(park, 0, tid);
 #pragma unroll(R <= 2 ? 16 : 1)
                 for (uint32_t r0 = 0; r0 < 16; r0 += G::COLUMNS) {
                     int64_t val[K];
 #pragma unroll
                     for (int i = 0; i < K; i++) val[i] = big && comp == 0 ? 0 : next[i];
-                    if (r0 + G::COLUMNS < 16) terms_of(next, r0 + G::COLUMNS);
-                    enc_parked<G>(val, park, tm, f, pair ? p : 0, r0, tid);
+                    if (!G::FAR_AHEAD) {
+                        if (r0 + G::COLUMNS < 16) terms_of(next, r0 + G::COLUMNS);
+                        if (f.narrow) ahead.fetch_low(park, r0, tid);
+                    }
+                    enc_parked<G>(val, park, ahead, tm, f, pair ? p : 0, r0, tid);
                     cpx v[G::COLUMNS][R];
-                    enc_columns<G>(v, x, buf, wait, tm, tab, r0, tid);
+                    if (!G::FAR_AHEAD) ahead.fetch_wait(wait, r0, tid);
+                    enc_columns<G>(v, x, buf, ahead, tm, r0, tid);
+                    if (G::FAR_AHEAD && r0 + G::COLUMNS < 16) {
+                        terms_of(next, r0 + G::COLUMNS);
+                        if (f.narrow) ahead.fetch_low(park, r0 + G::COLUMNS, tid);
+                        ahead.fetch_wait(wait, r0 + G::COLUMNS, tid);
+                    }
+                    enc_between<G>(v, tab, r0, tid);
                     // streaming stores: the finished ciphertext should not push tables and scratch out of L2
 #pragma unroll
                     for (int i = 0; i < K; i++) {
