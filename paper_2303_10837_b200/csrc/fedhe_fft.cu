@@ -34,7 +34,8 @@ struct FftJoin {
     uint64_t minus_q, fix;
     double scale;
     uint32_t shift;
-    __device__ __forceinline__ FftJoin(const FftSplit &f, uint64_t q) : minus_q(0 - q), scale(f.top_scale), shift(f.shift[f.pieces - 1]) {
+    __device__ __forceinline__ FftJoin(const FftSplit &f, uint64_t q) : FftJoin(q, f.top_scale, f.shift[f.pieces - 1]) {}
+    __device__ __forceinline__ FftJoin(uint64_t q, double top_scale, uint32_t top_shift) : minus_q(0 - q), scale(top_scale), shift(top_shift) {
         // the quotient carries 2^17, which keeps it positive
         fix = (q << 17) - ((uint64_t)FFT_ROUND_BITS << shift);
     }
@@ -258,15 +259,28 @@ struct EncRing {
     static constexpr size_t SMEM = (size_t)NB * 16 + (size_t)Tab::WORDS * 16 + (E_IN_SMEM ? N : 0);
 };
 
-// first unit of a ciphertext, of both components, that begins at or after `pos` products
-__host__ __device__ __forceinline__ uint32_t fft_unit_at(const EncWay &w, uint32_t pos) {
-    uint32_t half = pos >= w.products ? 1 : 0, rest = pos - half * w.products, j = 0;
-    while (rest) {
-        const uint32_t p = w.unit[j].products;
-        rest = rest > p ? rest - p : 0;
-        j++;
+// What a thread block needs to know of a product, in shared memory: looked up in the kernel's parameters, by the unit's number, then
+// its limb's, it was a chain of misses of 900 clocks before every block of a transform (N = 16384).
+struct alignas(16) EncJob {
+    uint64_t q;
+    double scale;                // of the limb's quotients
+    uint32_t key[2];
+    uint32_t shift, what;        // the top piece's; limb and EncJob flags
+    static constexpr uint32_t PARKS = 1u << 8, NARROW = 1u << 9, JOINS = 10;      // flags; the limb is below them, `joins` above
+};
+struct EncJobs {
+    EncJob job[2 * HE_MAX_LIMBS];
+    uint8_t start[4 * HE_MAX_LIMBS + 4];
+};
+__device__ __forceinline__ void enc_jobs_load(EncJobs &s, const CtxDev &c, const EncWay &way, uint32_t split) {
+    for (uint32_t i = threadIdx.x; i < way.products; i += FftLay::NT) {
+        const EncProduct &p = way.product[i];
+        const LimbDev &limb = c.limb[p.limb];
+        const FftSplit &f = limb.split[split];
+        s.job[i] = EncJob{limb.q, f.top_scale, {p.key[0], p.key[1]}, f.shift[f.pieces - 1],
+                          p.limb | (p.parks ? EncJob::PARKS : 0u) | (f.narrow ? EncJob::NARROW : 0u) | (uint32_t)p.joins << EncJob::JOINS};
     }
-    return half * w.units + j;
+    for (uint32_t i = threadIdx.x; i <= 2 * way.products; i += FftLay::NT) s.start[i] = way.start[i];
 }
 
 // value i (column, row, real or imaginary part) of a thread's columns from r0: its coefficient less the thread's number
@@ -359,10 +373,10 @@ __device__ __forceinline__ int64_t fft_round(double z) { return fft_round_bits(z
 
 // A low piece's values are parked for the same thread, which will join the top one.
 template <class G>
-__device__ __forceinline__ void enc_park(const cpx (&v)[G::COLUMNS][G::R], unsigned char *park, uint32_t tm, const FftSplit &f,
+__device__ __forceinline__ void enc_park(const cpx (&v)[G::COLUMNS][G::R], unsigned char *park, uint32_t tm, bool narrow,
                                          uint32_t r0, uint32_t tid) {
     const uint32_t i0 = r0 * G::R * 2;
-    if (G::ALL_NARROW || f.narrow) {
+    if (G::ALL_NARROW || narrow) {
         uint32_t w[G::K];
 #pragma unroll
         for (int i = 0; i < G::K; i++) {
@@ -388,14 +402,15 @@ __device__ __forceinline__ void enc_park(const cpx (&v)[G::COLUMNS][G::R], unsig
 }
 template <class G>
 __device__ __forceinline__ void enc_parked(int64_t (&val)[G::K], const unsigned char *park, const EncAhead<G> &ahead, uint32_t tm,
-                                           const FftSplit &f, uint32_t of_pair, uint32_t r0, uint32_t tid) {
+                                           bool narrow, uint32_t joins, uint32_t r0, uint32_t tid) {
     const uint32_t i0 = r0 * G::R * 2;
     // the low piece's product: the word itself, or, of a pair, its lower 16 bits (signed) or what they leave
     auto low_of = [&](int w) {
-        if (of_pair == 0) return w;
-        return of_pair == 1 ? (int)(int16_t)w : (w - (int)(int16_t)w) >> 16;
+        if (joins < 2) return w;
+        return joins == 2 ? (int)(int16_t)w : (w - (int)(int16_t)w) >> 16;
     };
-    if (f.narrow) {
+    if (joins == 0) return;
+    if (G::ALL_NARROW || narrow) {
         if constexpr (G::PARK_TMEM) {
             uint32_t w[8];
             tmem_get8(tm + G::PARK_AT + i0, w);
@@ -405,7 +420,7 @@ __device__ __forceinline__ void enc_parked(int64_t (&val)[G::K], const unsigned 
 #pragma unroll
             for (int i = 0; i < G::K; i++) val[i] += low_of(ahead.low[i]);
         }
-    } else if (!G::ALL_NARROW && f.pieces > 1) {
+    } else {
 #pragma unroll
         for (int i = 0; i < G::K; i++) val[i] += __ldcg(reinterpret_cast<const long long *>(park) + (i0 + i) * G::NT + tid);
     }
@@ -444,10 +459,12 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
     root_t *tab = reinterpret_cast<root_t *>(smem + (size_t)NB * 16);
     int8_t *e1_smem = reinterpret_cast<int8_t *>(tab + G::Tab::WORDS);
     __shared__ GaussTables gt;
+    __shared__ EncJobs jobs;
     __shared__ uint32_t tmem_base;
     __shared__ __align__(8) uint64_t key_bar;
     const uint32_t rank = blockIdx.x % S, cid = blockIdx.x / S, nc = gridDim.x / S;
     gauss_tables_load(gt, c.gauss, threadIdx.x, NT);
+    enc_jobs_load(jobs, c, way, PAIRS);
     for (uint32_t i = threadIdx.x; i < (uint32_t)G::Tab::WORDS; i += NT) tab[i] = c.fft_inv[i];
     if (threadIdx.x == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(&key_bar)) : "memory");
@@ -480,7 +497,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
     const uint32_t whole = T / nc * nc, rem = T - whole;
     const uint32_t parts = rem ? (nc / rem < most_parts ? nc / rem : most_parts) : 1;
     const uint32_t items = whole + rem * parts;           // at least as many as clusters
-    const uint32_t pieces = 2 * way.products;
+    const uint32_t products = way.products, all = 2 * products;
     const bool leader = rank == 0 && threadIdx.x == 0;
     uint32_t next_item = cid;
 #pragma unroll 1
@@ -497,10 +514,10 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
             part = (item - whole) % parts;
             of = parts;
         }
-        const uint32_t first = fft_unit_at(way, pieces * part / of), last = fft_unit_at(way, pieces * (part + 1) / of);
-        const uint32_t unit_end = fft_unit_at(way, pieces * (part * S + rank + 1) / (of * S));
-        uint32_t unit = fft_unit_at(way, pieces * (part * S + rank) / (of * S));
-        const bool c0_too = first < way.units, c1_too = last > way.units;
+        const uint32_t first = jobs.start[all * part / of], last = jobs.start[all * (part + 1) / of];
+        const uint32_t job_end = jobs.start[all * (part * S + rank + 1) / (of * S)];
+        uint32_t job = jobs.start[all * (part * S + rank) / (of * S)];
+        const bool c0_too = first < products, c1_too = last > products;
         const uint32_t t = t0 + tl;
 
         // ---- preparation: u, four columns of one half at a time ----
@@ -590,7 +607,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
             if (far) atomicOr(flags + (it & 1u), 1u);
         }
         meet();
-        if (unit == unit_end) continue;
+        if (job == job_end) continue;
         const bool big = __ldcg(flags + (it & 1u)) != 0;  // a term of c0 needs reducing first
         if constexpr (G::E_IN_SMEM) {
             if (c1_too) {
@@ -614,24 +631,18 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
         auto wait_for_key = [&]() {
             if (!turns.take([&](uint32_t parity) { return key_try(&key_bar, parity); })) atomicOr(c.status, STATUS_COPY);
         };
-        auto key_of = [&](uint32_t u, uint32_t pb) {
-            const uint32_t comp = u >= way.units ? 1 : 0;
-            const EncUnit &e = way.unit[u - comp * way.units];
-            return k.fft_pk + e.fft_key + ((size_t)comp * e.products * R + pb) * NB;
+        auto key_of = [&](uint32_t i, uint32_t b) {
+            const uint32_t comp = i >= products ? 1 : 0;
+            return k.fft_pk + (size_t)(jobs.job[i - comp * products].key[comp] + b) * NB;
         };
         if constexpr (!(G::E_IN_SMEM)) __syncthreads();   // the buffer's last readers are done
-        if (threadIdx.x == 0 && !turns.lost()) key_fetch(buf, key_of(unit, 0), &key_bar);
+        if (threadIdx.x == 0 && !turns.lost()) key_fetch(buf, key_of(job, 0), &key_bar);
 #pragma unroll 1
-        for (; unit < unit_end; unit++) {
-            const uint32_t comp = unit >= way.units ? 1 : 0;
-            const EncUnit &e = way.unit[unit - comp * way.units];
-            const bool pair = PAIRS && e.limb2 != NO_LIMB;
+        for (; job < job_end; job++) {
+            const uint32_t comp = job >= products ? 1 : 0;
+            const EncJob &e = jobs.job[job - comp * products];
 #pragma unroll 1
-            for (uint32_t pb = 0; pb < e.products * R; pb++) {
-                const uint32_t p = pb >> CL, b = pb & (R - 1);
-                const uint32_t j = pair && p == 2 ? e.limb2 : e.limb;
-                const FftSplit &f = c.limb[j].split[PAIRS];
-                const uint64_t q = c.limb[j].q;
+            for (uint32_t b = 0; b < R; b++) {
                 cpx x[16];
                 {
                     const uint32_t tid = fresh_tid();
@@ -659,11 +670,11 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
                     }
                 }
                 // the next key may come as soon as the buffer is read; where a column loop needs the buffer, after it
-                const bool more = pb + 1 < e.products * R || unit + 1 < unit_end;
+                const bool more = b + 1 < R || job + 1 < job_end;
                 auto fetch_next = [&]() {
                     __syncthreads();
                     if (more && threadIdx.x == 0 && !turns.lost())
-                        key_fetch(buf, pb + 1 < e.products * R ? key_of(unit, pb + 1) : key_of(unit + 1, 0), &key_bar);
+                        key_fetch(buf, b + 1 < R ? key_of(job, b + 1) : key_of(job + 1, 0), &key_bar);
                 };
                 fft_inverse<0>(x, buf, tab, fresh_tid(), [&] {
                     if (R <= 2 || b + 1 < R) fetch_next();
@@ -679,9 +690,11 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
                     for (int r = 0; r < 16; r++) buf[r * NT + tid] = make_double2(x[r].re, x[r].im);
                 }
                 constexpr int K = G::K;
+                const uint32_t what = e.what, joins = what >> EncJob::JOINS;
+                const bool narrow = (what & EncJob::NARROW) != 0;
                 EncAhead<G> ahead;
                 if constexpr (G::FAR_AHEAD) ahead.fetch_wait(wait, 0, tid);
-                if (pair ? p == 0 : p + 1 < f.pieces) {
+                if (what & EncJob::PARKS) {
 #pragma unroll(R <= 2 ? 16 : 1)
                     for (uint32_t r0 = 0; r0 < 16; r0 += G::COLUMNS) {
                         cpx v[G::COLUMNS][R];
@@ -689,14 +702,16 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
                         enc_columns<G>(v, x, buf, ahead, tm, r0, tid);
                         if (G::FAR_AHEAD && r0 + G::COLUMNS < 16) ahead.fetch_wait(wait, r0 + G::COLUMNS, tid);
                         enc_between<G>(v, tab, r0, tid);
-                        enc_park<G>(v, park, tm, f, r0, tid);
+                        enc_park<G>(v, park, tm, narrow, r0, tid);
                     }
                     if constexpr (G::PARK_TMEM) tmem_wait_put();
                     if constexpr (R > 2) fetch_next();
                     continue;
                 }
+                const uint32_t j = what & (EncJob::PARKS - 1);
+                const uint64_t q = e.q;
                 uint64_t *out = ct + (((size_t)tl * 2 + comp) * c.L + j) * N + tid;
-                const FftJoin join(f, q);
+                const FftJoin join(q, e.scale, e.shift);
                 // the offsets of a thread's coefficients are multiples of R, so they split off the number of the first
                 const long long *my_terms = term_of(tid);
                 auto terms_of = [&](int64_t (&val)[K], uint32_t r0) {
@@ -713,7 +728,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
                 };
                 int64_t next[K];
                 terms_of(next, 0);
-                if (G::FAR_AHEAD && f.narrow) ahead.fetch_low(park, 0, tid);
+                if (G::FAR_AHEAD && joins && narrow) ahead.fetch_low(park, 0, tid);
 #pragma unroll(R <= 2 ? 16 : 1)
                 for (uint32_t r0 = 0; r0 < 16; r0 += G::COLUMNS) {
                     int64_t val[K];
@@ -721,15 +736,15 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
                     for (int i = 0; i < K; i++) val[i] = big && comp == 0 ? 0 : next[i];
                     if (!G::FAR_AHEAD) {
                         if (r0 + G::COLUMNS < 16) terms_of(next, r0 + G::COLUMNS);
-                        if (f.narrow) ahead.fetch_low(park, r0, tid);
+                        if (joins && narrow) ahead.fetch_low(park, r0, tid);
                     }
-                    enc_parked<G>(val, park, ahead, tm, f, pair ? p : 0, r0, tid);
+                    enc_parked<G>(val, park, ahead, tm, narrow, PAIRS || joins == 0 ? joins : 1, r0, tid);
                     cpx v[G::COLUMNS][R];
                     if (!G::FAR_AHEAD) ahead.fetch_wait(wait, r0, tid);
                     enc_columns<G>(v, x, buf, ahead, tm, r0, tid);
                     if (G::FAR_AHEAD && r0 + G::COLUMNS < 16) {
                         terms_of(next, r0 + G::COLUMNS);
-                        if (f.narrow) ahead.fetch_low(park, r0 + G::COLUMNS, tid);
+                        if (joins && narrow) ahead.fetch_low(park, r0 + G::COLUMNS, tid);
                         ahead.fetch_wait(wait, r0 + G::COLUMNS, tid);
                     }
                     enc_between<G>(v, tab, r0, tid);
@@ -989,10 +1004,25 @@ static bool cut_limbs(CtxDev &c, bool in_pairs, EncWay &w, size_t &words) {
         if (f.pieces > 2 || (f.pieces == 2 && !f.narrow && logN <= 14)) return false;
     }
     w.products = 0;
+    const uint32_t R = 1u << (logN - 13);
     for (uint32_t u = 0; u < w.units; u++) {
-        w.unit[u].fft_key = words;
-        words += 2 * (size_t)w.unit[u].products * (c.N / 2);
-        w.products += w.unit[u].products;
+        EncUnit &e = w.unit[u];
+        e.fft_key = words;
+        for (uint32_t p = 0; p < e.products; p++) {
+            EncProduct &d = w.product[w.products + p];
+            const bool pair = e.limb2 != NO_LIMB;
+            for (uint32_t comp = 0; comp < 2; comp++) d.key[comp] = (uint32_t)(words / FftLay::NB) + (comp * e.products + p) * R;
+            d.limb = (uint16_t)(pair && p == 2 ? e.limb2 : e.limb);
+            d.parks = pair ? p == 0 : p + 1 < e.products;
+            d.joins = (uint8_t)(d.parks || e.products == 1 ? 0 : pair ? p + 1 : 1);
+        }
+        words += 2 * (size_t)e.products * (c.N / 2);
+        w.products += e.products;
+    }
+    uint32_t begin = 0, of_unit = 0;
+    for (uint32_t pos = 0; pos <= 2 * w.products; pos++) {
+        if (pos > begin) begin += w.unit[of_unit++ % w.units].products;
+        w.start[pos] = (uint8_t)begin;
     }
     return true;
 }
@@ -1011,9 +1041,7 @@ bool fft_cut(CtxDev &c, EncWays &e) {
         for (uint32_t of = 1; of < ENC_SHARES; of++) {
             uint32_t most = 0;
             for (uint32_t part = 0; part < of; part++) {
-                uint32_t sum = 0;
-                const uint32_t end = fft_unit_at(w, 2 * w.products * (part + 1) / of);
-                for (uint32_t u = fft_unit_at(w, 2 * w.products * part / of); u < end; u++) sum += w.unit[u % w.units].products;
+                const uint32_t sum = w.start[2 * w.products * (part + 1) / of] - w.start[2 * w.products * part / of];
                 most = sum > most ? sum : most;
             }
             e.most[i][of] = (uint16_t)most;
@@ -1032,14 +1060,15 @@ size_t fft_key_words(const CtxDev &c) {
 // two that take half of it each do run side by side.  This kernel has the same shape without it.
 __global__ void __launch_bounds__(FftLay::NT, 2) enc_shape_kernel() {}
 
-// shared memory that leaves no room for a second thread block on the SM
-constexpr int ENC_ALONE_SMEM = 116 * 1024;
+// shared memory that leaves no room for a second thread block on the SM, and the most that the kernel has besides the dynamic part
+constexpr int ENC_ALONE_SMEM = 116 * 1024, ENC_STATIC_SMEM = 5 * 1024;
+static_assert(sizeof(GaussTables) + sizeof(EncJobs) + 64 <= ENC_STATIC_SMEM, "static shared memory of the encryption");
 
 // How many clusters of 1 .. ENC_MOST blocks the device holds at once, two blocks to an SM and one.
 template <int CL>
 static cudaError_t setup_ring(CtxDev &c, int n_sm) {
     using G = EncRing<CL>;
-    static_assert(G::SMEM + 4096 <= ENC_ALONE_SMEM - 1024, "two thread blocks to an SM");
+    static_assert(G::SMEM + ENC_STATIC_SMEM <= ENC_ALONE_SMEM - 3072, "two thread blocks to an SM");
     cudaError_t e;
     for (uint32_t i = 0; i < c.enc->count; i++)
         if ((e = cudaFuncSetAttribute(pairs_limbs(c, i) ? encrypt_fft_kernel<CL, true> : encrypt_fft_kernel<CL, false>,
@@ -1053,7 +1082,7 @@ static cudaError_t setup_ring(CtxDev &c, int n_sm) {
             cudaLaunchAttribute attr;
             cfg.blockDim = dim3(G::NT, 1, 1);
             cfg.gridDim = dim3(S, 1, 1);
-            cfg.dynamicSmemBytes = alone ? ENC_ALONE_SMEM : G::SMEM + 4096;        // and the static part
+            cfg.dynamicSmemBytes = alone ? ENC_ALONE_SMEM : G::SMEM + ENC_STATIC_SMEM;
             attr.id = cudaLaunchAttributeClusterDimension;
             attr.val.clusterDim.x = S;
             attr.val.clusterDim.y = 1;

@@ -41,10 +41,19 @@ struct EncUnit {
     uint32_t products;
     size_t fft_key;              // first word of its key tables: [2 components][products][n]
 };
+// A product of a unit, in the order in which a thread block works them off: a low piece's is parked, a top one's ends its limb.
+struct EncProduct {
+    uint32_t key[2];             // blocks of 2^12 words before its key tables, for either component
+    uint16_t limb;               // of the low product of a pair: of the first of them
+    uint8_t parks;
+    uint8_t joins;               // what is parked for a top piece: 0 nothing, 1 its low piece's product, 2, 3 that of a pair, lower or upper limb
+};
 // The units of a public-key half.
 struct EncWay {
     uint32_t units, products;    // of all units
     EncUnit unit[HE_MAX_LIMBS];
+    EncProduct product[2 * HE_MAX_LIMBS];
+    uint8_t start[4 * HE_MAX_LIMBS + 1];       // of the products of both components: the first at or after a number that begins a unit
 };
 // Limbs in pairs where that is possible, and, if any are, every limb by itself too: fewer products, or more units to share out.
 constexpr uint32_t ENC_MOST = 8;       // thread blocks of a cluster that encrypts, at most
