@@ -21,7 +21,7 @@ CUDA_SOURCES = ["fedhe_transform.cu", "fedhe_slots.cu", "fedhe_encrypt.cu", "fed
                 "fedhe_mask.cu", "fedhe_api.cu", "fedhe_noalloc.cu"]
 HOST_SOURCES = ["fedhe_host.cpp"]
 HEADERS = ["fedhe_device.cuh", "fedhe_ntt.cuh", "fedhe_fft.cuh", "fedhe_internal.cuh", "fedhe_launch.h", "fedhe_host.h",
-           "fedhe_kernels.cuh", "fedhe_slots.cuh",
+           "fedhe_kernels.cuh", "fedhe_gauss.cuh", "fedhe_slots.cuh",
            os.path.join("..", "..", "include", "fedhe.h")]
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

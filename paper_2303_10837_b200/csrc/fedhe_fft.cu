@@ -251,9 +251,14 @@ struct EncRing {
     static constexpr int COLUMNS = R == 1 ? 4 : R == 2 ? 2 : 1, K = COLUMNS * R * 2;      // columns, values finished together
     // whether what a column needs from L2 is fetched a column ahead: of R = 8 it does not fit the registers
     static constexpr bool FAR_AHEAD = R == 4;
-    // a cluster's: the transform of u, the message and e0, e1, u in two bits each, flags
-    static constexpr size_t UHAT = (size_t)n * 16, TERMS = (size_t)N * 8, E1 = N, UBITS = (size_t)NB * 4,
-                            SHARED = UHAT + TERMS + E1 + UBITS + 128;
+    // a cluster's: the transform of u, the message and e0, flags
+    static constexpr size_t UHAT = (size_t)n * 16, TERMS = (size_t)N * 8, SHARED = UHAT + TERMS + 128;
+    // a ciphertext's samples: e0, e1 (a byte each), u in two bits each, the rows of a column side by side
+    using Row = typename std::conditional<(R <= 4), uint8_t, uint16_t>::type;
+    static constexpr size_t E0 = 0, E1 = N, U = 2 * (size_t)N, SAMPLES = U + 2 * NB * sizeof(Row);
+    // items of 512 stream blocks: of u, of either error
+    static constexpr uint32_t U_COLUMNS = R == 1 ? 2 : 1, U_ITEMS = 2 * NB / 4 / (NT * U_COLUMNS), E_ITEMS = N / 2 / (2 * NT),
+                              ITEMS = U_ITEMS + 2 * E_ITEMS;
     // a thread block's: what waits, joined low pieces
     static constexpr size_t WAIT = (size_t)WAIT_L2 * NB * 16, PARK = ALL_NARROW ? 0 : (size_t)N * 8, OWN = WAIT + PARK;
     static constexpr size_t SMEM = (size_t)NB * 16 + (size_t)Tab::WORDS * 16 + (E_IN_SMEM ? N : 0);
@@ -282,6 +287,9 @@ __device__ __forceinline__ void enc_jobs_load(EncJobs &s, const CtxDev &c, const
     }
     for (uint32_t i = threadIdx.x; i <= 2 * way.products; i += FftLay::NT) s.start[i] = way.start[i];
 }
+
+// What a ciphertext's draws depend on besides its number, and whether the clusters draw for themselves.
+struct EncDraw { uint64_t seed; uint32_t client, t0, inside; };
 
 // value i (column, row, real or imaginary part) of a thread's columns from r0: its coefficient less the thread's number
 template <class G>
@@ -426,13 +434,78 @@ __device__ __forceinline__ void enc_parked(int64_t (&val)[G::K], const unsigned 
     }
 }
 
+// One of the ITEMS of a ciphertext's random draws, by a thread block: first those of e0, then e1, then u.
+template <int CL>
+__device__ __forceinline__ void enc_sample_item(const GaussTables &gt, uint32_t part, uint64_t seed, uint32_t t, uint32_t client,
+                                                unsigned char *samples) {
+    using G = EncRing<CL>;
+    constexpr uint32_t NB = G::NB, NT = G::NT, R = G::R, n = G::n;
+    if (part < 2 * G::E_ITEMS) {
+        const uint32_t second = part >= G::E_ITEMS ? 1 : 0, b = (part - second * G::E_ITEMS) * 2 * NT + threadIdx.x;
+        int2 e[2];
+        gauss_pairs<2>(e, gt, seed, b, NT, t, client, second ? TAG_ENC_E1 : TAG_ENC_E0);
+        char2 *dst = reinterpret_cast<char2 *>(samples + (second ? G::E1 : G::E0));
+#pragma unroll
+        for (int j = 0; j < 2; j++) __stcg(dst + b + j * NT, make_char2((signed char)e[j].x, (signed char)e[j].y));
+    } else {
+        // four columns of one half, all their rows
+#pragma unroll
+        for (uint32_t j = 0; j < G::U_COLUMNS; j++) {
+            const uint32_t w = ((part - 2 * G::E_ITEMS) * G::U_COLUMNS + j) * NT + threadIdx.x;
+            uint32_t f[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (uint32_t a = 0; a < R; a++) {
+                const u32x4 v = stream_block(seed, (w / (NB / 4)) * (n / 4) + a * (NB / 4) + w % (NB / 4), t, client, TAG_ENC_U);
+                f[0] |= (uint32_t)(ternary_from_word(v.x) + 1) << (2 * a);
+                f[1] |= (uint32_t)(ternary_from_word(v.y) + 1) << (2 * a);
+                f[2] |= (uint32_t)(ternary_from_word(v.z) + 1) << (2 * a);
+                f[3] |= (uint32_t)(ternary_from_word(v.w) + 1) << (2 * a);
+            }
+            unsigned char *dst = samples + G::U;
+            if constexpr (R <= 4) __stcg(reinterpret_cast<uint32_t *>(dst) + w, f[0] | f[1] << 8 | f[2] << 16 | f[3] << 24);
+            else __stcg(reinterpret_cast<uint2 *>(dst) + w, make_uint2(f[0] | f[1] << 16, f[2] | f[3] << 16));
+        }
+    }
+}
+
+// Every S-th of `count` items from the first one on, leaving out those of e0 or e1 from `skip` on.  Not inlined: the samplers' registers would
+// cost the kernel that calls it spills.  The tables go where the transforms will work: 3 KB more shared memory to a block would leave the SM
+// 28 KB of L1 instead of 60 (N = 32768, 200 ciphertexts: 784 -> 816 us).
+template <int CL>
+__device__ __noinline__ void enc_sample_items(const void *gauss, GaussTables &gt, uint32_t first, uint32_t S, uint32_t count, uint32_t skip, uint64_t seed,
+                                              uint32_t t, uint32_t client, unsigned char *samples) {
+    __syncthreads();                                      // the buffer's last readers are done
+    gauss_tables_load(gt, gauss, threadIdx.x, FftLay::NT);
+    __syncthreads();
+#pragma unroll 1
+    for (uint32_t i = first; i < count; i += S) enc_sample_item<CL>(gt, i < skip ? i : i + EncRing<CL>::E_ITEMS, seed, t, client, samples);
+}
+
+// The random draws of T ciphertexts from number t0 on, [T][SAMPLES], for the kernel below.  Drawn there, by clusters that have 16
+// warps to an SM and nothing else to do meanwhile, they take 15 % of the time; here the integer multiplies of Philox set it.
+// That kernel may start when every thread block of this one has: it waits for the end of this one where it needs the samples.
+template <int CL>
+__global__ void __launch_bounds__(FftLay::NT)
+enc_sample_kernel(const void *gauss, EncDraw draw, uint32_t T, unsigned char *samples) {
+    using G = EncRing<CL>;
+    __shared__ GaussTables gt;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    gauss_tables_load(gt, gauss, threadIdx.x, G::NT);
+    __syncthreads();
+#pragma unroll 1
+    for (uint32_t i = blockIdx.x; i < T * G::ITEMS; i += gridDim.x) {
+        const uint32_t tl = i / G::ITEMS;
+        enc_sample_item<CL>(gt, i % G::ITEMS, draw.seed, draw.t0 + tl, draw.client, samples + (size_t)tl * G::SAMPLES);
+    }
+}
+
 // A cluster of thread blocks encrypts ciphertexts one after the other: first it prepares one together -- u
-// is drawn and transformed, the slots are encoded, e0 and the message added up, e1 drawn, all in R blocks
+// is transformed, the slots are encoded and e0 added, in R blocks
 // of 2^12 points that its thread blocks share out -- and then each of them works off its own units
 // (component, limb) of it: per piece of the key and block of the transform the product with the key's table
 // and the inverse transform, per piece the stages between blocks and the rounding, then joining, error and
-// message terms, canonical residues.  HBM sees the slots and the ciphertext once, the cluster meets three
-// times per ciphertext.  (With the blocks of every product spread over the cluster it met twice per
+// message terms, canonical residues.  HBM sees the slots and the ciphertext once, the cluster meets twice
+// per ciphertext.  (With the blocks of every product spread over the cluster it met twice per
 // piece, and waiting for one another took 6, 9 and 11 of 19, 22 and 26 thousand clocks per block and piece for R = 2, 4, 8.)
 //
 // Two thread blocks fit on an SM on every ring, so that one's memory phases meet the other's arithmetic.
@@ -450,20 +523,18 @@ __device__ __forceinline__ void enc_parked(int64_t (&val)[G::K], const unsigned 
 // PAIRS: some units are of two limbs (the code for both kinds costs the others 1.5 %).
 template <int CL, bool PAIRS>
 __global__ void __launch_bounds__(FftLay::NT, 2)
-encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ EncWay way, const KeysDev k, const float *sel, unsigned char *work,
-                   uint32_t t0, uint64_t seed, uint32_t client, uint64_t *ct, uint32_t T, uint32_t S, uint32_t most_parts) {
+encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ EncWay way, const KeysDev k, const float *sel,
+                   const EncDraw draw, unsigned char *samples, unsigned char *work, uint64_t *ct, uint32_t T, uint32_t S, uint32_t most_parts) {
     using G = EncRing<CL>;
     constexpr uint32_t N = G::N, n = G::n, NB = G::NB, NT = G::NT, R = G::R;
     extern __shared__ __align__(128) unsigned char smem[];
     double2 *buf = reinterpret_cast<double2 *>(smem);
     root_t *tab = reinterpret_cast<root_t *>(smem + (size_t)NB * 16);
     int8_t *e1_smem = reinterpret_cast<int8_t *>(tab + G::Tab::WORDS);
-    __shared__ GaussTables gt;
     __shared__ EncJobs jobs;
     __shared__ uint32_t tmem_base;
     __shared__ __align__(8) uint64_t key_bar;
     const uint32_t rank = blockIdx.x % S, cid = blockIdx.x / S, nc = gridDim.x / S;
-    gauss_tables_load(gt, c.gauss, threadIdx.x, NT);
     enc_jobs_load(jobs, c, way, PAIRS);
     for (uint32_t i = threadIdx.x; i < (uint32_t)G::Tab::WORDS; i += NT) tab[i] = c.fft_inv[i];
     if (threadIdx.x == 0) {
@@ -480,9 +551,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
     auto term_of = [&](uint32_t coef) {
         return terms + ((coef & (n - 1)) >> CL) + ((coef & (R - 1)) + (coef >= n ? R : 0)) * NB;
     };
-    int8_t *e1 = reinterpret_cast<int8_t *>(terms + N);
-    uint16_t *ubits = reinterpret_cast<uint16_t *>(e1 + N);                     // value + 1 per row of the column: [2 halves][NB]
-    uint32_t *flags = reinterpret_cast<uint32_t *>(ubits + 2 * NB);
+    uint32_t *flags = reinterpret_cast<uint32_t *>(terms + N);
     double2 *wait = reinterpret_cast<double2 *>(own);
     unsigned char *park = own + G::WAIT;
     auto meet = [&]() {                                   // everything the cluster wrote is visible to all of it
@@ -500,6 +569,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
     const uint32_t products = way.products, all = 2 * products;
     const bool leader = rank == 0 && threadIdx.x == 0;
     uint32_t next_item = cid;
+    asm volatile("griddepcontrol.wait;" ::: "memory");    // for samples drawn by the kernel above
 #pragma unroll 1
     for (uint32_t it = 0; next_item < items; it++) {
         const uint32_t item = next_item;
@@ -518,27 +588,19 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
         const uint32_t job_end = jobs.start[all * (part * S + rank + 1) / (of * S)];
         uint32_t job = jobs.start[all * (part * S + rank) / (of * S)];
         const bool c0_too = first < products, c1_too = last > products;
-        const uint32_t t = t0 + tl;
+        unsigned char *drawn = samples + (size_t)tl * G::SAMPLES;
 
-        // ---- preparation: u, four columns of one half at a time ----
-#pragma unroll 1
-        for (uint32_t w = rank * NT + threadIdx.x; w < 2 * NB / 4; w += S * NT) {
-            uint32_t f[4] = {0, 0, 0, 0};
-#pragma unroll
-            for (uint32_t a = 0; a < R; a++) {
-                const uint32_t b = (w / (NB / 4)) * (n / 4) + a * (NB / 4) + w % (NB / 4);
-                const u32x4 v = stream_block(seed, b, t, client, TAG_ENC_U);
-                f[0] |= (uint32_t)(ternary_from_word(v.x) + 1) << (2 * a);
-                f[1] |= (uint32_t)(ternary_from_word(v.y) + 1) << (2 * a);
-                f[2] |= (uint32_t)(ternary_from_word(v.z) + 1) << (2 * a);
-                f[3] |= (uint32_t)(ternary_from_word(v.w) + 1) << (2 * a);
-            }
-            __stcg(reinterpret_cast<uint2 *>(ubits) + w, make_uint2(f[0] | f[1] << 16, f[2] | f[3] << 16));
+        if (draw.inside && first != last) {
+            // clusters that share a ciphertext write the same samples
+            constexpr uint32_t E = G::E_ITEMS;
+            const uint32_t count = G::ITEMS - (c0_too && c1_too ? 0 : E);
+            enc_sample_items<CL>(c.gauss, *reinterpret_cast<GaussTables *>(smem), rank, S, count, c0_too ? (c1_too ? G::ITEMS : E) : 0, draw.seed, draw.t0 + tl, draw.client, drawn);
         }
-        meet();                                           // u is there, and nobody works on the last ciphertext any more
+        meet();                                           // the samples are there, and nobody works on the last ciphertext any more
         next_item = __ldcg(flags + 2 + (it & 1u));
         if (first == last) continue;                      // more parts than units
-        // the transform of u and the encoder's network: 2 R blocks of 2^12 points
+        // ---- preparation: the transform of u and the encoder's network, 2 R blocks of 2^12 points ----
+        int far = 0;
 #pragma unroll 1
         for (uint32_t item = rank; item < 2 * R; item += S) {
             const uint32_t b = item & (R - 1);
@@ -546,7 +608,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
                 cpx x[16];
                 {
                     const OuterPath<CL> outer(c.fft_fwd, b);
-                    const uint16_t *p = ubits + fresh_tid();
+                    const typename G::Row *p = reinterpret_cast<const typename G::Row *>(drawn + G::U) + fresh_tid();     // [2 halves][NB]
                     auto ternary = [](uint32_t f) {       // 0, 1, 2 -> -1.0, 0.0, 1.0
                         return __hiloint2double(f == 1 ? 0 : 0x3ff00000 | (int)((f == 0 ? 1u : 0u) << 31), 0);
                     };
@@ -565,50 +627,29 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
                 for (int r = 0; r < 16; r++) __stcg(dst + r * NT, make_double2(x[r].re, x[r].im));
             } else if (c0_too) {
                 const float *slots = sel + (size_t)tl * n;
-                long long *row = terms + (CL ? bitrev(b, CL ? CL : 1) : 0u) * NB;
+                const uint32_t first_of_row = CL ? bitrev(b, CL ? CL : 1) : 0u;
+                long long *row = terms + first_of_row * NB;
+                const int8_t *e0 = reinterpret_cast<const int8_t *>(drawn + G::E0) + first_of_row;
                 __syncthreads();                          // the buffer's last readers are done
                 if (encode_block_in_place<Lay<FftLay::LB, 4>>(
                         c, [&](uint32_t i) { return encoder_stages<CL>(slots, c.ftw, n, b, i); },
                         reinterpret_cast<uint64_t *>(buf), CL,
-                        [&](uint32_t kk, int64_t re, int64_t im) {
+                        [&](uint32_t kk) { return make_char2(__ldcg(e0 + R * kk), __ldcg(e0 + n + R * kk)); },
+                        [&](uint32_t kk, int64_t re, int64_t im, char2 e) {
+                            re += e.x;
+                            im += e.y;
+                            far |= (re < 0 ? -re : re) >= c.term_limit || (im < 0 ? -im : im) >= c.term_limit;
                             __stcg(row + kk, (long long)re);
                             __stcg(row + R * NB + kk, (long long)im);
                         }))
                     atomicOr(c.status, STATUS_RANGE);
             }
         }
-        meet();
-        // error terms, a pair of neighbours at a time
-#pragma unroll 1
-        for (int comp = c0_too ? 0 : 1; comp < (c1_too ? 2 : 1); comp++) {
-            int far = 0;
-#pragma unroll 1
-            for (uint32_t b = rank * NT + threadIdx.x; b < N / 2; b += S * NT) {
-                if (comp == 0) {
-                    long long *p = term_of(2 * b);
-                    longlong2 m;
-                    if constexpr (CL == 0) m = __ldcg(reinterpret_cast<const longlong2 *>(p));
-                    else m = make_longlong2(__ldcg(p), __ldcg(p + NB));
-                    const int2 e = gauss_pair(gt, seed, b, t, client, TAG_ENC_E0);
-                    m.x += e.x;
-                    m.y += e.y;
-                    far |= (m.x < 0 ? -m.x : m.x) >= c.term_limit || (m.y < 0 ? -m.y : m.y) >= c.term_limit;
-                    if constexpr (CL == 0) {
-                        __stcg(reinterpret_cast<longlong2 *>(p), m);
-                    } else {
-                        __stcg(p, m.x);
-                        __stcg(p + NB, m.y);
-                    }
-                } else {
-                    const int2 e = gauss_pair(gt, seed, b, t, client, TAG_ENC_E1);
-                    __stcg(reinterpret_cast<char2 *>(e1) + b, make_char2((signed char)e.x, (signed char)e.y));
-                }
-            }
-            if (far) atomicOr(flags + (it & 1u), 1u);
-        }
+        if (far) atomicOr(flags + (it & 1u), 1u);         // a term of c0 needs reducing first
         meet();
         if (job == job_end) continue;
-        const bool big = __ldcg(flags + (it & 1u)) != 0;  // a term of c0 needs reducing first
+        const bool big = __ldcg(flags + (it & 1u)) != 0;
+        const int8_t *e1 = reinterpret_cast<const int8_t *>(drawn + G::E1);
         if constexpr (G::E_IN_SMEM) {
             if (c1_too) {
                 for (uint32_t i = threadIdx.x; i < N / 16; i += NT)
@@ -1061,8 +1102,8 @@ size_t fft_key_words(const CtxDev &c) {
 __global__ void __launch_bounds__(FftLay::NT, 2) enc_shape_kernel() {}
 
 // shared memory that leaves no room for a second thread block on the SM, and the most that the kernel has besides the dynamic part
-constexpr int ENC_ALONE_SMEM = 116 * 1024, ENC_STATIC_SMEM = 5 * 1024;
-static_assert(sizeof(GaussTables) + sizeof(EncJobs) + 64 <= ENC_STATIC_SMEM, "static shared memory of the encryption");
+constexpr int ENC_ALONE_SMEM = 116 * 1024, ENC_STATIC_SMEM = 1280;
+static_assert(sizeof(EncJobs) + 64 <= ENC_STATIC_SMEM, "static shared memory of the encryption");
 
 // How many clusters of 1 .. ENC_MOST blocks the device holds at once, two blocks to an SM and one.
 template <int CL>
@@ -1100,6 +1141,7 @@ static cudaError_t setup_this_ring(CtxDev &c, int n_sm) { FEDHE_FOR_RING(c, setu
 cudaError_t fft_setup(CtxDev &c, int n_sm) {
     const cudaError_t e = setup_this_ring(c, n_sm);
     if (e) return e;
+    c.sm_count = (uint32_t)n_sm;
     c.passes_most = passes_most(c);
     return cudaSuccess;
 }
@@ -1204,9 +1246,16 @@ static size_t ring_scratch(const CtxDev &c, size_t T) {
     }
     return most;
 }
+// ciphertexts whose samples are made ahead at once
+constexpr size_t ENC_SAMPLE_BYTES = (size_t)256 << 20;
+template <int CL>
+static size_t ring_samples(size_t T) {
+    const size_t most = ENC_SAMPLE_BYTES / EncRing<CL>::SAMPLES;
+    return T < most ? T : most;
+}
 template <int CL>
 static size_t ring_work(const CtxDev &c, size_t T) {
-    const size_t a = ring_scratch<CL>(c, T), b = encrypt_passes_work_bytes(c, T);
+    const size_t a = ring_scratch<CL>(c, T) + ring_samples<CL>(T) * EncRing<CL>::SAMPLES, b = encrypt_passes_work_bytes(c, T);
     return a > b ? a : b;
 }
 size_t fft_work_bytes(const CtxDev &c, size_t T) {
@@ -1215,28 +1264,54 @@ size_t fft_work_bytes(const CtxDev &c, size_t T) {
 }
 
 template <int CL>
-static cudaError_t launch_encrypt_ring(const CtxDev &c, const KeysDev &k, const float *sel, void *work, uint32_t t0,
+static cudaError_t launch_encrypt_part(const CtxDev &c, const KeysDev &k, const float *sel, unsigned char *work, uint32_t t0,
                                        size_t T, uint64_t seed, uint32_t client, uint64_t *ct, cudaStream_t s) {
     using G = EncRing<CL>;
+    static_assert(G::SAMPLES % 16 == 0, "scratch behind the samples, and e1 in 16-byte words");
     const EncPlan p = enc_plan(c, T);
     if (p.clusters < 1) return cudaErrorLaunchOutOfResources;
+    cudaError_t e;
+    // Few ciphertexts are drawn by their clusters: the launch costs the host more than the clusters take (N = 8192, a round of three
+    // clients with 25 ciphertexts each: 170 us, and 193 us with three more launches).  With enough of them it pays: 100
+    // ciphertexts of N = 8192 69.7 -> 63.5 us, 40 of N = 16384 72.7 -> 66.1, 68 of N = 32768 303 -> 267.
+    EncDraw draw = {seed, client, t0, T * G::N < (size_t)1 << 19};
+    if (!draw.inside) {
+        const size_t items = T * G::ITEMS, fill = (size_t)c.sm_count * 8;
+        enc_sample_kernel<CL><<<(unsigned)(items < fill ? items : fill), G::NT, 0, s>>>(c.gauss, draw, (uint32_t)T, work);
+        if ((e = FEDHE_LAUNCHED())) return e;
+    }
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr;
+    cudaLaunchAttribute attr[2];
     cfg.stream = s;
     cfg.blockDim = dim3(G::NT, 1, 1);
     cfg.gridDim = dim3(p.clusters * p.S, 1, 1);
     cfg.dynamicSmemBytes = p.alone ? ENC_ALONE_SMEM : G::SMEM;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = p.S;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    cudaError_t e;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = p.S;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    // The clusters start beside the last samples if there is one to a ciphertext.  With more, all the clusters that fit have to be there
+    // at once, and those that come first may leave no room for a whole one (200 ciphertexts of N = 32768: 784 -> 800 us).
+    cfg.numAttrs = !draw.inside && T <= p.clusters ? 2 : 1;
     if ((e = cudaLaunchKernelEx(&cfg, pairs_limbs(c, p.way) ? encrypt_fft_kernel<CL, true> : encrypt_fft_kernel<CL, false>, c, c.enc->way[p.way],
-                                k, sel, static_cast<unsigned char *>(work), t0, seed, client, ct, (uint32_t)T, p.S, p.parts)))
+                                k, sel, draw, work, work + T * G::SAMPLES, ct, (uint32_t)T, p.S, p.parts)))
         return e;
     return FEDHE_LAUNCHED();
+}
+template <int CL>
+static cudaError_t launch_encrypt_ring(const CtxDev &c, const KeysDev &k, const float *sel, void *work, uint32_t t0,
+                                       size_t T, uint64_t seed, uint32_t client, uint64_t *ct, cudaStream_t s) {
+    using G = EncRing<CL>;
+    const size_t most = ring_samples<CL>(T);
+    for (size_t t = 0; t < T; t += most) {
+        const cudaError_t e = launch_encrypt_part<CL>(c, k, sel + t * G::n, static_cast<unsigned char *>(work), t0 + (uint32_t)t,
+                                                      T - t < most ? T - t : most, seed, client, ct + t * 2 * c.L * G::N, s);
+        if (e) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_encrypt(const CtxDev &c, const KeysDev &k, const float *sel, void *work, uint32_t t0, size_t T,

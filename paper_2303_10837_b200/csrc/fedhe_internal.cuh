@@ -118,6 +118,7 @@ struct CtxDev {
     uint16_t enc_fit[2][ENC_MOST + 1]; // clusters of a size that the device holds: two blocks to an SM, one
     uint32_t passes_most;              // encryption by passes (N = 2^16): the most ciphertexts that go by them
     const void *gauss;   // GaussTables
+    uint32_t sm_count;
     uint32_t *deal;      // encryption hands out ciphertexts here: next one, thread blocks (clusters) that are done; 0 between calls
     int *status;         // sticky anomaly word
 };

@@ -122,13 +122,13 @@ __device__ __forceinline__ uint32_t stage_swz(uint32_t k) { return k ^ (((k >> 8
 // it enters the block's stages (the slot itself when the block is the whole
 // vector, the output of the earlier stages otherwise); `sm` is a buffer of
 // 2^LF::LOGB cpx values, used first for the exchanges between phases and then
-// to put the rounded integers in order; out(kk, re, im) receives coefficient kk
+// to put the rounded integers in order; out(kk, re, im, extra) receives coefficient kk
 // of the block (kk its bit-reversed position) and its imaginary partner, kk in
-// order over the threads.  The whole vector has 2^(LF::LOGB + A) slots.  Ends with
+// order over the threads, with extra(kk), of which a few are asked for before the first is used.  The whole vector has 2^(LF::LOGB + A) slots.  Ends with
 // a block barrier after which `sm` is free and the block may read what `out` stored.
 // Returns whether a coefficient left the range (the caller raises the status word).
-template <class LF, class In, class Out>
-__device__ __forceinline__ bool encode_block_in_place(const CtxDev &c, const In &in, uint64_t *sm, uint32_t A, const Out &out) {
+template <class LF, class In, class Extra, class Out>
+__device__ __forceinline__ bool encode_block_in_place(const CtxDev &c, const In &in, uint64_t *sm, uint32_t A, const Extra &extra, const Out &out) {
     constexpr uint32_t NB = 1u << LF::LOGB;
     const uint32_t tid = threadIdx.x;
     cpx x[LF::E];
@@ -150,7 +150,18 @@ __device__ __forceinline__ bool encode_block_in_place(const CtxDev &c, const In 
         stage[NB + stage_swz(kk)] = __double2ll_rn(im);
     }
     __syncthreads();
-    for (uint32_t kk = tid; kk < NB; kk += LF::NT) out(kk, stage[stage_swz(kk)], stage[NB + stage_swz(kk)]);
+    constexpr int U = LF::E < 4 ? LF::E : 4;
+#pragma unroll 1
+    for (uint32_t k0 = tid; k0 < NB; k0 += U * LF::NT) {
+        decltype(extra(0u)) e[U];
+#pragma unroll
+        for (int j = 0; j < U; j++) e[j] = extra(k0 + j * LF::NT);
+#pragma unroll
+        for (int j = 0; j < U; j++) {
+            const uint32_t kk = k0 + j * LF::NT;
+            out(kk, stage[stage_swz(kk)], stage[NB + stage_swz(kk)], e[j]);
+        }
+    }
     __syncthreads();
     return bad;
 }
@@ -159,8 +170,8 @@ __device__ __forceinline__ bool encode_block_in_place(const CtxDev &c, const In 
 template <class LF>
 __device__ __forceinline__ bool encode_in_block(const CtxDev &c, const float *slots, uint64_t *sm, int64_t *m_out) {
     return encode_block_in_place<LF>(
-        c, [&](uint32_t i) { return cpx{(double)__ldg(slots + i), 0.0}; }, sm, 0,
-        [&](uint32_t kk, int64_t re, int64_t im) {
+        c, [&](uint32_t i) { return cpx{(double)__ldg(slots + i), 0.0}; }, sm, 0, [](uint32_t) { return 0; },
+        [&](uint32_t kk, int64_t re, int64_t im, int) {
             m_out[kk] = re;
             m_out[kk + (1u << LF::LOGB)] = im;
         });
