@@ -377,7 +377,7 @@ static int build_mask(he_ctx *ctx, const float *score, size_t P, size_t k, const
     // third with ranges | candidates
     cudaMemPool_t pool = mask_pool(ctx->device);
     if (!pool) return HE_ERR_CUDA;
-    const size_t scratch_words = SELECT_ZEROED + 4 * 64 + 2 * SELECT_RUNS + 3 * tiles + tiles * TILE_CANDIDATES;
+    const size_t scratch_words = SELECT_ZEROED + SELECT_BINS + 4 * 64 + 2 * SELECT_RUNS + 4 * tiles + tiles * TILE_CANDIDATES;
     uint32_t *scratch = nullptr;
     if (cudaMallocFromPoolAsync(reinterpret_cast<void **>(&scratch), scratch_words * sizeof(uint32_t), pool, st) != cudaSuccess) {
         cudaGetLastError();
@@ -385,14 +385,16 @@ static int build_mask(he_ctx *ctx, const float *score, size_t P, size_t k, const
     }
     SelectWork w;
     w.hist = scratch;
-    w.done = scratch + 4096;
-    w.state = reinterpret_cast<SelectState *>(scratch + 4100);
-    w.total = scratch + 4102;
-    uint64_t *ranges_dev = reinterpret_cast<uint64_t *>(scratch + SELECT_ZEROED);
+    w.done = scratch + SELECT_HIST;
+    w.state = reinterpret_cast<SelectState *>(w.done + 4);
+    w.total = w.done + 8;
+    w.sampled = scratch + SELECT_ZEROED;
+    uint64_t *ranges_dev = reinterpret_cast<uint64_t *>(w.sampled + SELECT_BINS);
     w.runs = ranges_dev + 2 * 64;
     w.tile_above = reinterpret_cast<uint32_t *>(w.runs + SELECT_RUNS);
     w.tile_cand = w.tile_above + tiles;
-    uint32_t *tile_sel = w.tile_cand + tiles, *total = w.total;
+    w.tile_found = w.tile_cand + tiles;
+    uint32_t *tile_sel = w.tile_found + tiles, *total = w.total;
     w.cand = tile_sel + tiles;
     // The mask owns one allocation: bit mask | per-word prefix counts | index list (its size is
     // known up to the overlap of the forced ranges with the top-k set and with each other).
@@ -404,22 +406,32 @@ static int build_mask(he_ctx *ctx, const float *score, size_t P, size_t k, const
         return HE_ERR_ALLOC;
     }
     uint32_t *wpre = bits + nwords, *idx = wpre + nwords;
+    w.bits = bits;
+    bool by_sample = num_ranges == 0 && select_by_sample(P, k);
     int rc = HE_OK;
     he_mask *m = nullptr;
     do {
 #define MCU(expr) if ((expr) != cudaSuccess) { rc = HE_ERR_CUDA; break; }
-        // Radix select of the k-th largest key, entirely on the device: nothing is read back before the end.
-        MCU(launch_select(score, P, k, w, ctx->sm_count, st));
+        // The selection is entirely on the device: nothing is read back before the end.  A sample may have missed the threshold; then
+        // all is done once more without one.
         if (num_ranges)
             MCU(cudaMemcpyAsync(ranges_dev, ranges_host, 2 * num_ranges * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
-        MCU(launch_mask_mark(score, P, w, ranges_dev, (uint32_t)num_ranges, bits, wpre, idx, tile_sel, st));
-        if (num_ranges) {
-            MCU(launch_scan(tile_sel, tiles, total, st));
-            MCU(launch_mask_write(P, bits, tile_sel, wpre, idx, st));
+        uint32_t ksel = 0, got[2] = {0, 0};
+        cudaError_t e = cudaSuccess;
+        for (;;) {
+            if ((e = launch_select(score, P, k, by_sample, w, ctx->sm_count, st))) break;
+            if ((e = launch_mask_mark(score, P, w, ranges_dev, (uint32_t)num_ranges, wpre, idx, kmax, tile_sel, st))) break;
+            if (num_ranges) {
+                if ((e = launch_scan(tile_sel, tiles, total, st))) break;
+                if ((e = launch_mask_write(P, bits, tile_sel, wpre, idx, st))) break;
+            }
+            if ((e = cudaMemcpyAsync(got, total, sizeof(got), cudaMemcpyDeviceToHost, st))) break;
+            if ((e = cudaStreamSynchronize(st))) break;                      // the one wait of the call
+            ksel = got[0];
+            if (!by_sample || !got[1]) break;
+            by_sample = false;
         }
-        uint32_t ksel = 0;
-        MCU(cudaMemcpyAsync(&ksel, total, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-        MCU(cudaStreamSynchronize(st));                                      // the one wait of the call
+        MCU(e);
         if ((num_ranges == 0 && ksel != k) || ksel > kmax) { rc = HE_ERR_CUDA; break; }     // cannot happen
         m = new (std::nothrow) he_mask();
         if (!m) { rc = HE_ERR_ALLOC; break; }

@@ -111,27 +111,31 @@ int ctx_workspace(he_ctx *ctx, size_t T, void **out);
 
 // mask construction (tiles of MASK_BLOCK consecutive parameters)
 constexpr uint32_t MASK_BLOCK = 1024, TILE_CANDIDATES = 128;
-// progress of the radix selection, in device memory: the key prefix found so far (tau after
-// the last step) and how many keys are still to be covered (after the last step: how many keys
-// equal to tau belong to the mask)
-struct SelectState { uint32_t prefix, need; };
-// work space of a selection; the SELECT_ZEROED words from `hist` are cleared at its start
-constexpr size_t SELECT_ZEROED = 4096 + 4 + 4;
+// progress of the selection, in device memory: the window [base, base + 2^20) of keys that the threshold is looked for in, how much
+// of its place in there is found (all of it after the last step: tau = base + place), and how many keys are still to be covered
+// (after the last step: how many keys equal to tau belong to the mask)
+struct SelectState { uint32_t base, place, need, above; };      // above: keys beyond the window
+// work space of a selection; the words from `hist` to the end of `sampled` are cleared at its start
+constexpr size_t SELECT_HIST = 2048 + 1024 + 1024, SELECT_BINS = 1u << 12, SELECT_ZEROED = SELECT_HIST + 4 + 8;
 constexpr size_t SELECT_RUNS = 2 * 1024;          // thread blocks that a device holds at once, at most
 struct SelectWork {
     uint32_t *hist;              // 2048, 1024, 1024
     uint32_t *done;              // [4] thread blocks that finished a pass
     SelectState *state;
-    uint32_t *total;             // selected parameters (without forced ranges)
-    uint32_t *tile_above, *tile_cand, *cand;     // per tile; [tiles][TILE_CANDIDATES]
+    uint32_t *total;             // selected parameters (without forced ranges), then whether the threshold was outside the window
+    uint32_t *sampled;           // [SELECT_BINS] keys of the sample by their upper bits
+    uint32_t *tile_above, *tile_cand, *tile_found, *cand;     // per tile; [tiles][TILE_CANDIDATES]
     uint64_t *runs;              // [SELECT_RUNS] counts before a run of tiles
     uint32_t run;                // tiles of a run (set by launch_select)
+    uint32_t *bits;              // the mask's: the keys beyond the window are marked by the pass that looks for candidates
 };
-cudaError_t launch_select(const float *score, size_t P, size_t k, SelectWork &w, int n_sm, cudaStream_t s);
+// whether a sample may choose the window (without forced ranges); it can miss, and total[1] is not 0 then
+bool select_by_sample(size_t P, size_t k);
+cudaError_t launch_select(const float *score, size_t P, size_t k, bool by_sample, SelectWork &w, int n_sm, cudaStream_t s);
 // in-place exclusive scan of a[0..count); the grand total goes to *total
 cudaError_t launch_scan(uint32_t *a, size_t count, uint32_t *total, cudaStream_t s);
 cudaError_t launch_mask_mark(const float *score, size_t P, const SelectWork &w, const uint64_t *ranges, uint32_t nranges,
-                             uint32_t *bits, uint32_t *wpre, uint32_t *idx, uint32_t *tile_sel, cudaStream_t s);
+                             uint32_t *wpre, uint32_t *idx, size_t room, uint32_t *tile_sel, cudaStream_t s);      // idx holds `room`
 cudaError_t launch_mask_write(size_t P, const uint32_t *bits, const uint32_t *blk_sel_prefix,
                               uint32_t *wpre, uint32_t *idx, cudaStream_t s);
 

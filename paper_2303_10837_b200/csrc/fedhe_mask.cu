@@ -43,15 +43,15 @@ __device__ __forceinline__ T block_exclusive_scan(T v, T *warp_sums, T &total) {
     return res;
 }
 
-// ---- radix selection of the k-th largest key: digits of 11, 10 and 10 bits (a key has 31) ----
+// ---- selection of the k-th largest key ----
 //
-// Three passes over the scores: the histogram of the first digit; the histogram of the second among the
-// keys that have the first (the candidates, a few per cent of real scores), which are also gathered by tiles;
-// and, when the threshold tau is known, the marking.  What lies between works on the candidates.  The
-// last thread block of a pass to finish does the one-block step that follows it: picking the digit, or
-// the scan over the tiles.  (With three histogram passes, a counting pass and one-block kernels between them
-// the selection of 2.56 M out of 25.6 M took 341 us; the first pass was bound by conflicts of its shared-memory
-// atomics, because neighbouring scores share an exponent.)
+// A window of 2^20 keys that holds the threshold, from a sample of the scores or from the histogram of the keys' first digit
+// (11 of their 31 bits); one pass over the scores that counts and marks the keys beyond the window and
+// gathers those within (the candidates, a few per cent of real scores) by tiles; then two digits of ten bits and the marking on the
+// candidates.  The last thread block of a pass to finish does the one-block step that follows it: picking the digit, or
+// the scan over the tiles.  For 2.56 M out of 25.6 M scores the call took 341 us by three histogram passes, a counting pass
+// and one-block kernels between them (conflicts of shared-memory atomics, because neighbouring scores share an exponent), 165 us
+// with the histogram of the first digit over all scores (27 us) and the scores read again for the marking (33 us).
 
 // true in all threads of the block that finishes last; what the others wrote is visible to it
 __device__ __forceinline__ bool last_block(uint32_t *done) {
@@ -64,12 +64,12 @@ __device__ __forceinline__ bool last_block(uint32_t *done) {
     return is_last != 0;
 }
 
-// Walks the digits of a histogram from the largest down until `need` keys are covered, appends the
-// digit found to the prefix and takes the keys above it off `need`.  By a block of 1024 threads.
-template <int BITS>
-__device__ __forceinline__ void radix_pick(const uint32_t *hist, uint32_t prefix, uint32_t need, SelectState *state) {
+// Walks the digits of a histogram from the largest down until `need` keys are covered: found(digit, keys above it, its keys), by
+// one thread, if there are as many.  By a block of NT threads.
+template <int BITS, uint32_t NT = 1024, class Found>
+__device__ __forceinline__ void radix_pick(const uint32_t *hist, uint32_t need, const Found &found) {
     __shared__ uint32_t warp_sums[33];
-    constexpr uint32_t bins = 1u << BITS, per = bins / 1024u;        // thread t: digits from bins - 1 - per t down
+    constexpr uint32_t bins = 1u << BITS, per = bins / NT;           // thread t: digits from bins - 1 - per t down
     uint32_t h[per], mine = 0u;
 #pragma unroll
     for (uint32_t j = 0; j < per; j++) {
@@ -82,10 +82,7 @@ __device__ __forceinline__ void radix_pick(const uint32_t *hist, uint32_t prefix
     for (uint32_t j = 0; j < per; j++) {
         const uint32_t pos = threadIdx.x * per + j;
         // the digit where the running count first reaches `need`
-        if (above < need && above + h[j] >= need) {
-            state->prefix = (prefix << BITS) | (bins - 1u - pos);
-            state->need = need - above;
-        }
+        if (above < need && above + h[j] >= need) found(bins - 1u - pos, above, h[j]);
         above += h[j];
     }
 }
@@ -145,12 +142,50 @@ key_histogram_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
     if (odd) atomicAdd(w.hist + 2 * threadIdx.x + 1, odd);
     if (last_block(w.done)) {
         if (k == 0) {
-            if (threadIdx.x == 0) *w.state = SelectState{0xffffffffu, 0u};       // no key reaches the threshold
+            if (threadIdx.x == 0) w.state->base = 0x80000000u;                   // no key reaches the window
         } else {
-            radix_pick<11>(w.hist, 0u, k, w.state);
+            radix_pick<11>(w.hist, k, [&](uint32_t digit, uint32_t, uint32_t) { w.state->base = digit << 20; });
         }
     }
 }
+
+// The window from a sample: a score at a pseudo-random place of every SAMPLE-th part of them, in a histogram of the keys'
+// upper 12 bits of 31; the last block puts the window around the place of the sample's share of k, between the ends of its bin.  A
+// block counts in shared memory: sampled keys share some hundred bins, and as atomics in L2 they took 58 us.
+constexpr uint32_t SAMPLE_BLOCKS = 128, SAMPLE_LOADS = 1, SAMPLE = SAMPLE_BLOCKS * SAMPLE_LOADS * 1024;
+static_assert(SELECT_BINS == 1u << 12, "bins of 2^19 keys");
+
+__global__ void __launch_bounds__(1024, 1) key_sample_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
+    __shared__ __align__(16) uint32_t sh[SELECT_BINS];
+    const size_t step = P / SAMPLE;
+    float v[SAMPLE_LOADS];
+#pragma unroll
+    for (uint32_t j = 0; j < SAMPLE_LOADS; j++) {
+        const uint32_t i = (blockIdx.x * SAMPLE_LOADS + j) * 1024u + threadIdx.x;
+        v[j] = __ldg(score + i * step + (uint32_t)(((uint64_t)(i * 2654435761u) * step) >> 32));
+    }
+    for (uint32_t b = threadIdx.x; b < SELECT_BINS / 4; b += 1024u) reinterpret_cast<uint4 *>(sh)[b] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+#pragma unroll
+    for (uint32_t j = 0; j < SAMPLE_LOADS; j++) atomicAdd(sh + (score_key(v[j]) >> 19), 1u);
+    __syncthreads();
+    for (uint32_t b = threadIdx.x; b < SELECT_BINS; b += 1024u)
+        if (sh[b]) atomicAdd(w.sampled + b, sh[b]);
+    if (!last_block(w.done)) return;
+    const uint32_t need = (uint32_t)((double)k / (double)P * SAMPLE + 0.5);
+    const uint32_t rank = need ? need : 1u;
+    radix_pick<12>(w.sampled, rank, [&](uint32_t bin, uint32_t above, uint32_t count) {
+        const uint32_t down = (uint32_t)(((float)(rank - above) - 0.5f) / (float)count * (float)(1u << 19));
+        const uint32_t middle = ((bin + 1u) << 19) - down;
+        w.state->base = middle > 1u << 19 ? middle - (1u << 19) : 0u;
+    });
+}
+
+// The standard deviation of a sample's share of k is sqrt(p (1 - p) / SAMPLE), and the window reaches 3 to 6 % to either side of the
+// threshold, where p changes by that times 1.3 for real scores (products of two normal variables) and p = 0.1, and 3 and more in their
+// tail: 5 and 3 standard deviations for p = 0.1 and 1 / 256.  A selection that misses costs another one, so fewer scores beyond the threshold,
+// or in all, go by the histogram of all: at 2.5 M scores that is as quick (88 us and 90).
+bool select_by_sample(size_t P, size_t k) { return P >= (size_t)1 << 22 && k >= P / 256 && P - k >= P / 256; }
 
 // f(first word, words' keys) for LOADS words of a tile at a time, by a warp: lane l the l-th parameter of each word.
 // Beyond the end keys are 0, and f is told how many parameters are left (LOADS * 32 or less).
@@ -175,108 +210,189 @@ __device__ __forceinline__ void for_tile(const float *score, size_t P, size_t fi
     }
 }
 
-// Second digit.  A warp takes a tile of MASK_BLOCK scores, counts the keys above the first digit and
-// gathers the lower 20 bits of those that have it; a tile with more than TILE_CANDIDATES of them is read again instead.
-__global__ void __launch_bounds__(1024, 2)
-key_candidates_kernel(const float *score, size_t P, SelectWork w) {
-    __shared__ uint32_t sh[1024];
-    sh[threadIdx.x] = 0;
+// The pass over the scores.  A warp takes a tile of MASK_BLOCK of them, marks and counts the keys beyond the window and gathers those
+// within, lane by lane: the place in the tile and 20 bits of the key, less the window's base.  A tile with more than TILE_CANDIDATES of
+// them is read again instead.  It is bound by its instructions, so the scores' bit patterns themselves are compared (a key is 0 where
+// they are not those of a number from 0 to infinity, and only a window at 0 holds such keys), and a lane only notes its candidates in a word,
+// and reads them again at the tile's end (gathering them word by word took 52 us for 25.6 M scores).
+__device__ __forceinline__ uint32_t window_place(uint32_t key, uint32_t base) { return key - base; }        // below 2^20 within
+constexpr int CAND_THREADS = 512;
+__global__ void __launch_bounds__(CAND_THREADS, 3)
+key_candidates_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
+    __shared__ uint32_t sh[1024], beyond;
+    for (uint32_t b = threadIdx.x; b < 1024u; b += CAND_THREADS) sh[b] = 0;
+    if (threadIdx.x == 0) beyond = 0;
     __syncthreads();
-    const uint32_t prefix = w.state->prefix, need = w.state->need;
+    const uint32_t base = w.state->base, infinity = 0x7f800000u;
+    // bit patterns beyond the window and within: from `last` + 1 and from `base`, so many
+    const uint32_t last = base + 0xfffffu, many = infinity > last ? infinity - last : 0u;
+    const uint32_t within = base > infinity ? 0u : infinity - base < 0xfffffu ? infinity - base + 1u : 1u << 20;
     const uint32_t lane = threadIdx.x & 31u;
-    const size_t tiles = (P + MASK_BLOCK - 1) / MASK_BLOCK;
-    for (size_t tile = (size_t)blockIdx.x * 32u + (threadIdx.x >> 5); tile < tiles; tile += (size_t)gridDim.x * 32u) {
-        const size_t first = tile * MASK_BLOCK;
-        uint32_t above = 0, found = 0;
+    const size_t tiles = (P + MASK_BLOCK - 1) / MASK_BLOCK, whole = P / MASK_BLOCK, stride = (size_t)gridDim.x * (CAND_THREADS / 32);
+    size_t tile = (size_t)blockIdx.x * (CAND_THREADS / 32) + (threadIdx.x >> 5);
+    uint32_t all_above = 0;
+    const float *p = score + tile * MASK_BLOCK + lane;
+    // the next words are on their way while these are looked at
+    float next[LOADS];
+    if (tile < whole) {
+#pragma unroll
+        for (int j = 0; j < LOADS; j++) next[j] = __ldg(p + j * 32);
+    }
+#pragma unroll 1
+    for (; tile < tiles; tile += stride, p += stride * MASK_BLOCK) {
+        uint32_t my_bits = 0, mine = 0;                             // word `lane` of the marks; bit i: the lane's key in word i is a candidate
+        static_assert(MASK_BLOCK == 1024, "a word of the tile for every lane");
+        if (tile < whole && base) {
+#pragma unroll 1
+            for (uint32_t w0 = 0; w0 < 32; w0 += LOADS) {
+                uint32_t who[LOADS], some = 0;
+#pragma unroll
+                for (int j = 0; j < LOADS; j++) {
+                    const uint32_t raw = __float_as_uint(next[j]);
+                    who[j] = __ballot_sync(0xffffffffu, raw - last - 1u < many);
+                    if (window_place(raw, base) < within) some |= 1u << j;
+                }
+                mine |= some << w0;
+                const bool same = w0 + LOADS < 32;
+                const float *q = same ? p + (w0 + LOADS) * 32 : p + stride * MASK_BLOCK;
+                if (same || tile + stride < whole) {
+#pragma unroll
+                    for (int j = 0; j < LOADS; j++) next[j] = __ldg(q + j * 32);
+                }
+                // the word of the lane's number among these
+                static_assert(LOADS == 8, "three bits pick it");
+                const uint32_t a = lane & 1u ? who[1] : who[0], b = lane & 1u ? who[3] : who[2], c = lane & 1u ? who[5] : who[4],
+                               d = lane & 1u ? who[7] : who[6], e = lane & 2u ? b : a, f = lane & 2u ? d : c;
+                if ((lane & ~7u) == w0) my_bits = lane & 4u ? f : e;
+            }
+        } else {
+            // the last tile, and a window at 0
+            const uint32_t left = tile < whole ? MASK_BLOCK : (uint32_t)(P - tile * MASK_BLOCK);
+#pragma unroll 1
+            for (uint32_t word = 0; word < 32; word++) {
+                const bool there = word * 32 + lane < left;
+                const uint32_t key = there ? score_key(__ldg(p + word * 32)) : 0u;
+                const uint32_t who = __ballot_sync(0xffffffffu, key > last);
+                if (lane == word) my_bits = who;
+                if (there && window_place(key, base) < 1u << 20) mine |= 1u << word;
+            }
+            if (tile + stride < whole) {
+#pragma unroll
+                for (int j = 0; j < LOADS; j++) next[j] = __ldg(p + stride * MASK_BLOCK + j * 32);
+            }
+        }
+        uint32_t at = __popc(mine);
+        const uint32_t n = at;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t o = __shfl_up_sync(0xffffffffu, at, d);
+            if (lane >= (uint32_t)d) at += o;
+        }
+        const uint32_t found = __shfl_sync(0xffffffffu, at, 31);
+        at -= n;
         uint32_t *cand = w.cand + tile * TILE_CANDIDATES;
-        for_tile(score, P, first, [&](uint32_t w0, const uint32_t (&key)[LOADS], uint32_t left) {
-            // a bit for every candidate among the lane's keys; the few there are get their places together
-            uint32_t mine = 0;
+        while (mine) {
+            constexpr int A = 4;
+            uint32_t word[A];
+            float v[A];
 #pragma unroll
-            for (int j = 0; j < LOADS; j++) {
-                const uint32_t top = key[j] >> 20;
-                if (top > prefix) above++;
-                if (top == prefix) mine |= 1u << j;
+            for (int i = 0; i < A; i++) {
+                word[i] = mine ? __ffs((int)mine) - 1 : 32;
+                mine &= mine - 1u;                                  // 0 stays 0
+                v[i] = word[i] < 32 ? __ldg(p + word[i] * 32) : 0.0f;
             }
-            if (left < LOADS * 32u) {                              // keys beyond the end are 0 and not above any digit
-                const uint32_t words = left > lane ? (left - lane + 31u) / 32u : 0u;
-                mine &= (1u << words) - 1u;
-            }
-            const uint32_t n = __popc(mine);
-            uint32_t at = n;
 #pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const uint32_t o = __shfl_up_sync(0xffffffffu, at, d);
-                if (lane >= (uint32_t)d) at += o;
-            }
-            const uint32_t all = __shfl_sync(0xffffffffu, at, 31);
-            at += found - n;
-            found += all;
-            while (mine) {
-                const uint32_t j = __ffs((int)mine) - 1;
-                mine &= mine - 1u;
-                const uint32_t low = score_key(__ldg(score + first + (w0 + j) * 32u + lane)) & 0xfffffu;
-                if (at < TILE_CANDIDATES) cand[at] = low;
+            for (int i = 0; i < A; i++) {
+                if (word[i] == 32) break;
+                const uint32_t low = window_place(score_key(v[i]), base);
+                if (at < TILE_CANDIDATES) cand[at] = low << 10 | (word[i] * 32u + lane);
                 at++;
-                atomicAdd(sh + (low >> 10), 1u);
+                atomicAdd(sh + (low >> 10 & 1023u), 1u);
             }
-        });
-        above = __reduce_add_sync(0xffffffffu, above);
+        }
+        if (tile < whole || lane * 32u < P - tile * MASK_BLOCK) w.bits[tile * (MASK_BLOCK / 32) + lane] = my_bits;
+        const uint32_t above = __reduce_add_sync(0xffffffffu, __popc(my_bits));
+        all_above += above;
         if (lane == 0) {
             w.tile_above[tile] = above;
             w.tile_cand[tile] = found;
+            w.tile_found[tile] = found;
         }
     }
+    if (lane == 0 && all_above) atomicAdd(&beyond, all_above);
     __syncthreads();
-    if (sh[threadIdx.x]) atomicAdd(w.hist + 2048 + threadIdx.x, sh[threadIdx.x]);
-    if (last_block(w.done + 1)) radix_pick<10>(w.hist + 2048, prefix, need, w.state);
+    for (uint32_t b = threadIdx.x; b < 1024u; b += CAND_THREADS)
+        if (sh[b]) atomicAdd(w.hist + 2048 + b, sh[b]);
+    if (threadIdx.x == 0 && beyond) atomicAdd(&w.state->above, beyond);
+    if (!last_block(w.done + 1)) return;
+    const uint32_t too_many = __ldcg(&w.state->above);
+    if (threadIdx.x == 0) w.total[1] = k ? 1u : 0u;                    // until the threshold is found
+    __syncthreads();
+    if (k > too_many)
+        radix_pick<10, CAND_THREADS>(w.hist + 2048, k - too_many, [&](uint32_t digit, uint32_t over, uint32_t) {
+            w.state->place = digit;
+            w.state->need = k - too_many - over;
+            w.total[1] = 0u;
+        });
 }
 
-// f(in, lower 20 bits) for the candidates of a tile, by a whole warp: f may use warp operations
+// f(in, lower 20 bits and place in the tile) for the candidates of a tile, by a whole warp: f may use warp operations
 template <class F>
-__device__ __forceinline__ void for_candidates(const float *score, size_t P, const SelectWork &w, size_t tile, uint32_t first_digit, F f) {
-    const uint32_t lane = threadIdx.x & 31u, found = w.tile_cand[tile];
+__device__ __forceinline__ void for_candidates(const float *score, size_t P, const SelectWork &w, size_t tile, uint32_t base, F f) {
+    const uint32_t lane = threadIdx.x & 31u, found = w.tile_found[tile];
+    const uint32_t *cand = w.cand + tile * TILE_CANDIDATES + lane;
+    uint32_t c = *cand;                                             // rarely more than 32: these come with their number
     if (found <= TILE_CANDIDATES) {
         for (uint32_t i = 0; i < found; i += 32) {
             const bool in = i + lane < found;
-            f(in, in ? w.cand[tile * TILE_CANDIDATES + i + lane] : 0u);
+            f(in, in ? c : 0u);
+            if (i + 32 < found) c = cand[i + 32];
         }
     } else {
-        for_tile(score, P, tile * MASK_BLOCK, [&](uint32_t, const uint32_t (&key)[LOADS], uint32_t left) {
+        for_tile(score, P, tile * MASK_BLOCK, [&](uint32_t w0, const uint32_t (&key)[LOADS], uint32_t left) {
 #pragma unroll
-            for (int j = 0; j < LOADS; j++) f(j * 32u + lane < left && (key[j] >> 20) == first_digit, key[j] & 0xfffffu);
+            for (int j = 0; j < LOADS; j++) {
+                const uint32_t low = window_place(key[j], base);
+                f(j * 32u + lane < left && low < 1u << 20, low << 10 | ((w0 + j) * 32u + lane));
+            }
         });
     }
 }
 
-// third digit, over the candidates
+// second digit of ten bits, over the candidates
 __global__ void __launch_bounds__(1024, 2) key_last_digit_kernel(const float *score, size_t P, SelectWork w) {
     __shared__ uint32_t sh[1024];
     sh[threadIdx.x] = 0;
     __syncthreads();
-    const uint32_t prefix = w.state->prefix, need = w.state->need;
+    if (w.total[1]) return;                               // not in the window
+    const uint32_t base = w.state->base, digit = w.state->place, need = w.state->need;
     const size_t tiles = (P + MASK_BLOCK - 1) / MASK_BLOCK;
     for (size_t tile = (size_t)blockIdx.x * 32u + (threadIdx.x >> 5); tile < tiles; tile += (size_t)gridDim.x * 32u)
-        for_candidates(score, P, w, tile, prefix >> 10, [&](bool in, uint32_t low) {
-            if (in && (low >> 10) == (prefix & 1023u)) atomicAdd(sh + (low & 1023u), 1u);
+        for_candidates(score, P, w, tile, base, [&](bool in, uint32_t c) {
+            if (in && c >> 20 == digit) atomicAdd(sh + (c >> 10 & 1023u), 1u);
         });
     __syncthreads();
     if (sh[threadIdx.x]) atomicAdd(w.hist + 3072 + threadIdx.x, sh[threadIdx.x]);
-    if (last_block(w.done + 2)) radix_pick<10>(w.hist + 3072, prefix, need, w.state);
+    if (last_block(w.done + 2) && need)
+        radix_pick<10>(w.hist + 3072, need, [&](uint32_t low, uint32_t over, uint32_t) {
+            w.state->place = digit << 10 | low;
+            w.state->need = need - over;
+        });
 }
 
 // Keys above and equal to tau: a block takes a run of tiles, and leaves for each the counts before it within the run
 // (equal keys in the upper half); the last block does the same for the runs.
 __global__ void __launch_bounds__(1024, 2) tile_counts_kernel(const float *score, size_t P, SelectWork w) {
     __shared__ uint64_t warp_sums[33];
-    const uint32_t tau = w.state->prefix, need = w.state->need, lane = threadIdx.x & 31u;
+    if (w.total[1]) return;                               // not in the window
+    const uint32_t base = w.state->base, place = w.state->place, need = w.state->need, lane = threadIdx.x & 31u;
     const size_t tiles = (P + MASK_BLOCK - 1) / MASK_BLOCK;
     const size_t begin = (size_t)blockIdx.x * w.run, end = begin + w.run < tiles ? begin + w.run : tiles;
     for (size_t tile = begin + (threadIdx.x >> 5); tile < end; tile += 32u) {
         uint32_t gt = 0, eq = 0;
-        for_candidates(score, P, w, tile, tau >> 20, [&](bool in, uint32_t low) {
-            gt += in && low > (tau & 0xfffffu) ? 1u : 0u;
-            eq += in && low == (tau & 0xfffffu) ? 1u : 0u;
+        for_candidates(score, P, w, tile, base, [&](bool in, uint32_t c) {
+            gt += in && c >> 10 > place ? 1u : 0u;
+            eq += in && c >> 10 == place ? 1u : 0u;
         });
         gt = __reduce_add_sync(0xffffffffu, gt);
         eq = __reduce_add_sync(0xffffffffu, eq);
@@ -311,22 +427,29 @@ __global__ void __launch_bounds__(1024, 2) tile_counts_kernel(const float *score
     if (threadIdx.x == 0) *w.total = (uint32_t)before + (eq_all < need ? eq_all : need);
 }
 
-cudaError_t launch_select(const float *score, size_t P, size_t k, SelectWork &w, int n_sm, cudaStream_t s) {
+cudaError_t launch_select(const float *score, size_t P, size_t k, bool by_sample, SelectWork &w, int n_sm, cudaStream_t s) {
     cudaError_t e;
-    if ((e = cudaMemsetAsync(w.hist, 0, SELECT_ZEROED * sizeof(uint32_t), s))) return e;
+    if ((e = cudaMemsetAsync(w.hist, 0, (SELECT_ZEROED + (by_sample ? SELECT_BINS : 0)) * sizeof(uint32_t), s))) return e;
+    if (by_sample) {
+        key_sample_kernel<<<SAMPLE_BLOCKS, 1024, 0, s>>>(score, P, w, (uint32_t)k);
+        if ((e = FEDHE_LAUNCHED())) return e;
+    }
     if ((e = cudaFuncSetAttribute(key_histogram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HIST_SMEM))) return e;
     // One thread block of the first pass to an SM, unless its counters could overflow; two keys to a thread are enough (with
     // sixteen, 100 k scores left a thread fourteen loads one after the other: 10 us more).
     const unsigned want = blocks_for(P, 1024 * 2), least = blocks_for(P, (unsigned)HIST_KEYS);
     unsigned g1 = want < (unsigned)n_sm ? want : (unsigned)n_sm;
     if (g1 < least) g1 = least;
-    key_histogram_kernel<<<g1, 1024, HIST_SMEM, s>>>(score, P, w, (uint32_t)k);
-    if ((e = FEDHE_LAUNCHED())) return e;
+    if (!by_sample) {
+        key_histogram_kernel<<<g1, 1024, HIST_SMEM, s>>>(score, P, w, (uint32_t)k);
+        if ((e = FEDHE_LAUNCHED())) return e;
+    }
     auto grid = [&](unsigned per_block) {
         const unsigned blocks = blocks_for(P, per_block), resident = n_sm < 1024 ? 2u * (unsigned)n_sm : (unsigned)SELECT_RUNS;
         return blocks < resident ? blocks : resident;
     };
-    key_candidates_kernel<<<grid(32 * MASK_BLOCK), 1024, 0, s>>>(score, P, w);
+    const unsigned cand_blocks = blocks_for(P, CAND_THREADS / 32 * MASK_BLOCK), cand_fit = 3u * (unsigned)n_sm;
+    key_candidates_kernel<<<cand_blocks < cand_fit ? cand_blocks : cand_fit, CAND_THREADS, 0, s>>>(score, P, w, (uint32_t)k);
     if ((e = FEDHE_LAUNCHED())) return e;
     key_last_digit_kernel<<<grid(32 * MASK_BLOCK), 1024, 0, s>>>(score, P, w);
     if ((e = FEDHE_LAUNCHED())) return e;
@@ -362,63 +485,88 @@ cudaError_t launch_scan(uint32_t *a, size_t count, uint32_t *total, cudaStream_t
 }
 
 // Membership: key > tau, or key == tau and fewer than `need` equal keys at lower indices, or (RANGES)
-// inside a forced index range.  A warp takes a tile, a lane the parameter of its number in every word of
-// the bit mask.  Without ranges the positions are known, and the prefix counts and the index list are written too.
+// inside a forced index range.  A warp takes a tile, lane l ends up with word l of its bits.
+
+// from the bits of the keys beyond the window and the candidates
+__device__ __forceinline__ uint32_t tile_bits(const float *score, size_t P, const SelectWork &w, size_t tile, uint32_t eq_before, uint32_t *words) {
+    const uint32_t place = w.state->place, need = w.state->need, found = w.tile_found[tile];
+    const uint32_t lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
+    const uint32_t *cand = w.cand + tile * TILE_CANDIDATES;
+    words[lane] = tile * MASK_BLOCK + lane * 32u < P ? w.bits[tile * (MASK_BLOCK / 32) + lane] : 0u;
+    __syncwarp();
+    for_candidates(score, P, w, tile, w.state->base, [&](bool in, uint32_t c) {
+        const bool eq = in && c >> 10 == place;
+        uint32_t rank = eq_before;                                  // of an equal key among all of them
+        if (found > TILE_CANDIDATES) {                              // in order
+            const uint32_t eqs = __ballot_sync(0xffffffffu, eq);
+            rank += __popc(eqs & below);
+            eq_before += __popc(eqs);
+        } else if (eq) {
+            for (uint32_t i = 0; i < found; i++) rank += cand[i] >> 10 == place && cand[i] < c ? 1u : 0u;
+        }
+        if ((in && c >> 10 > place) || (eq && rank < need)) atomicOr(words + (c >> 5 & 31u), 1u << (c & 31u));
+    });
+    __syncwarp();
+    return words[lane];
+}
 template <bool RANGES>
 __global__ void __launch_bounds__(256)
-mask_mark_kernel(const float *score, size_t P, SelectWork w, const uint64_t *ranges, uint32_t nranges, uint32_t *bits,
-                 uint32_t *wpre, uint32_t *idx, uint32_t *tile_sel) {
-    const uint32_t tau = w.state->prefix, need = w.state->need;
-    const uint32_t lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
+mask_mark_kernel(const float *score, size_t P, SelectWork w, const uint64_t *ranges, uint32_t nranges,
+                 uint32_t *wpre, uint32_t *idx, uint32_t room, uint32_t *tile_sel) {
+    __shared__ uint32_t words[8][32];
+    if (w.total[1]) return;
+    const uint32_t need = w.state->need;
+    const uint32_t lane = threadIdx.x & 31u;
     const size_t tile = (size_t)blockIdx.x * 8u + (threadIdx.x >> 5), first = tile * MASK_BLOCK;
     if (first >= P) return;
     const uint64_t run = w.runs[tile / w.run];
-    uint32_t eq_before = w.tile_cand[tile] + (uint32_t)(run >> 32);
-    // selected before the tile: the keys above tau and the first `need` of the equal ones
-    uint32_t at = RANGES ? 0u : w.tile_above[tile] + (uint32_t)run + (eq_before < need ? eq_before : need);
-    // lane l keeps the bits and the prefix count of word l of the tile, which are stored together
-    uint32_t my_bits = 0, my_pre = 0;
-    static_assert(MASK_BLOCK == 1024, "a word of the tile for every lane");
-    for_tile(score, P, first, [&](uint32_t w0, const uint32_t (&key)[LOADS], uint32_t left) {
-        bool equal = false;
-#pragma unroll
-        for (int j = 0; j < LOADS; j++) equal = equal || key[j] == tau;
-        // keys equal to tau are rare (among real scores), and keys beyond the end are 0
-        const bool some = __any_sync(0xffffffffu, equal);
-#pragma unroll
-        for (int j = 0; j < LOADS; j++) {
-            const uint32_t i = (uint32_t)first + (w0 + j) * 32u + lane;        // parameters are fewer than 2^32
-            bool sel = key[j] > tau;
-            if (some || RANGES) {
-                const bool in = j * 32u + lane < left, eq = in && key[j] == tau;
-                const uint32_t eqs = __ballot_sync(0xffffffffu, eq);
-                sel = sel || (eq && eq_before + __popc(eqs & below) < need);
-                eq_before += __popc(eqs);
-                if (RANGES && in && !sel)
-                    for (uint32_t r = 0; r < nranges; r++)
-                        if (i >= ranges[2 * r] && i < ranges[2 * r + 1]) sel = true;
-            }
-            const uint32_t who = __ballot_sync(0xffffffffu, sel);
-            if (lane == w0 + j) {
-                my_bits = who;
-                my_pre = at;
-            }
-            if (!RANGES && sel) idx[at + __popc(who & below)] = i;
-            at += __popc(who);
+    const uint32_t eq_before = w.tile_cand[tile] + (uint32_t)(run >> 32);
+    uint32_t bits = tile_bits(score, P, w, tile, eq_before, words[threadIdx.x >> 5]);
+    const size_t word = first + lane * 32u;
+    if (RANGES) {
+        for (uint32_t r = 0; r < nranges; r++) {
+            // the part of the range in this word
+            const uint64_t lo = ranges[2 * r] > word ? ranges[2 * r] : word, end = word + 32u, hi = ranges[2 * r + 1] < end ? ranges[2 * r + 1] : end;
+            if (lo < hi) bits |= (uint32_t)(((1ull << (hi - lo)) - 1ull) << (lo - word));
         }
-    });
-    if (first + lane * 32u < P) {
-        bits[(first >> 5) + lane] = my_bits;
-        if (!RANGES) wpre[(first >> 5) + lane] = my_pre;
     }
-    if (RANGES && lane == 0) tile_sel[tile] = at;
+    if (word < P) w.bits[word >> 5] = bits;
+    // positions: what is selected before the tile (the keys above tau and the first `need` of the equal ones), and in the lanes below
+    uint32_t at = __popc(bits);
+    const uint32_t mine = at;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xffffffffu, at, d);
+        if (lane >= (uint32_t)d) at += o;
+    }
+    if (RANGES) {
+        if (lane == 31) tile_sel[tile] = at;
+        return;
+    }
+    at += w.tile_above[tile] + (uint32_t)run + (eq_before < need ? eq_before : need) - mine;
+    if (word < P) wpre[word >> 5] = at;
+    // few bits: every lane its own word's; many: all lanes a word's, which are neighbours in the list
+    if (__reduce_max_sync(0xffffffffu, mine) <= 12) {
+        while (bits) {
+            if (at < room) idx[at] = (uint32_t)word + (uint32_t)(__ffs((int)bits) - 1);
+            at++;
+            bits &= bits - 1u;
+        }
+    } else {
+        const uint32_t below = (1u << lane) - 1u;
+#pragma unroll 8
+        for (uint32_t l = 0; l < 32; l++) {
+            const uint32_t who = __shfl_sync(0xffffffffu, bits, l), to = __shfl_sync(0xffffffffu, at, l) + __popc(who & below);
+            if ((who >> lane & 1u) && to < room) idx[to] = (uint32_t)first + l * 32u + lane;
+        }
+    }
 }
 
 cudaError_t launch_mask_mark(const float *score, size_t P, const SelectWork &w, const uint64_t *ranges, uint32_t nranges,
-                             uint32_t *bits, uint32_t *wpre, uint32_t *idx, uint32_t *tile_sel, cudaStream_t s) {
+                             uint32_t *wpre, uint32_t *idx, size_t room, uint32_t *tile_sel, cudaStream_t s) {
     const unsigned grid = blocks_for(P, 8 * MASK_BLOCK);
-    if (nranges) mask_mark_kernel<true><<<grid, 256, 0, s>>>(score, P, w, ranges, nranges, bits, wpre, idx, tile_sel);
-    else mask_mark_kernel<false><<<grid, 256, 0, s>>>(score, P, w, ranges, nranges, bits, wpre, idx, tile_sel);
+    if (nranges) mask_mark_kernel<true><<<grid, 256, 0, s>>>(score, P, w, ranges, nranges, wpre, idx, (uint32_t)room, tile_sel);
+    else mask_mark_kernel<false><<<grid, 256, 0, s>>>(score, P, w, ranges, nranges, wpre, idx, (uint32_t)room, tile_sel);
     return FEDHE_LAUNCHED();
 }
 

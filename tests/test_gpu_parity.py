@@ -524,6 +524,35 @@ def test_select_mask_tiles_and_candidates(he, P, spread):
         assert mask.k == k and np.array_equal(got, oracle.select_mask(score, k)), k
 
 
+@pytest.mark.parametrize("kind", ["products", "two clusters", "few values", "one value"])
+def test_select_mask_by_a_sample(he, kind):
+    """From 2^22 scores on a sample says where the threshold is looked for: scores as they come, thresholds at the edge of a
+    gap that the sample can only guess (the selection is made again then), and ties that fill the window."""
+    g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
+    rng = np.random.default_rng(91)
+    P = (1 << 22) + 1013
+    if kind == "products":
+        score = np.abs(rng.standard_normal(P, dtype=np.float32)) * np.abs(rng.standard_normal(P, dtype=np.float32))
+        score[:2] = [np.nan, -1.0]
+        ks = [P // 256, P // 256 + 1, P // 10, P // 2, P - P // 256, P - P // 256 + 1]
+    elif kind == "two clusters":
+        high = rng.random(P) < 0.3
+        score = np.where(high, 2.0, 1.0).astype(np.float32) * (1 + 0.01 * rng.random(P, dtype=np.float32))
+        c = int(high.sum())
+        ks = [c - 1, c, c + 1]
+    elif kind == "few values":
+        score = rng.integers(0, 5, P).astype(np.float32)
+        ks = [P // 7, int((score == 4).sum()), P // 2]
+    else:
+        score = np.full(P, 0.25, np.float32)
+        ks = [P // 3]
+    d = dev_f32(score)
+    for k in ks:
+        mask = he.he_select_mask(g, d, k)
+        got = he.he_mask_indices(mask).cpu().numpy().view(np.uint32)
+        assert mask.k == k and np.array_equal(got, oracle.select_mask(score, k)), k
+
+
 def test_mask_with_forced_ranges(he):
     """Top-k plus whole index ranges (first and last layers)."""
     g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
