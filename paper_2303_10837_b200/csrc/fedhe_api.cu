@@ -570,34 +570,38 @@ static int weighted_aggregate(he_ctx *ctx, const uint64_t *const *cts_host, cons
     const uint32_t L = d.L;
     // weights as constant polynomials at scale q_{L-1}: W_i = rint(alpha_i * q_{L-1})
     const double ql = (double)d.limb[L - 1].q;
-    std::vector<unsigned char> host(C * (sizeof(void *) + L * sizeof(tw_t)));
-    const uint64_t **ptrs = reinterpret_cast<const uint64_t **>(host.data());
-    tw_t *wt = reinterpret_cast<tw_t *>(host.data() + C * sizeof(void *));
+    SumTable tab;
+    const size_t words = (size_t)C * (1 + 2 * L);
+    std::vector<uint64_t> large(words <= SumTable::WORDS ? 0 : words);
+    uint64_t *host = large.empty() ? tab.words : large.data(), *wt = host + C;
     for (int i = 0; i < C; i++) {
         if (T && (!cts_host[i] || !aligned16(cts_host[i]))) return HE_ERR_INVALID_ARG;
         const double a = alpha_host[i];
         if (!(a >= 0.0) || !(a <= 1.0)) return HE_ERR_INVALID_ARG;
         const double prod = a * ql;
         const uint64_t W = (uint64_t)rint(prod);
-        ptrs[i] = cts_host[i];
+        host[i] = reinterpret_cast<uintptr_t>(cts_host[i]);
         for (uint32_t j = 0; j < L; j++) {
             const HostTw w = host_shoup(W % d.limb[j].q, d.limb[j].q);
-            wt[i * L + j] = tw_t{w.w, w.wp};
+            wt[2 * (i * L + j)] = w.w;
+            wt[2 * (i * L + j) + 1] = w.wp;
         }
     }
     if (T == 0) return HE_OK;
     cudaStream_t st = as_stream(stream);
-    CU(cudaMemcpyAsync(ctx->tab, host.data(), host.size(), cudaMemcpyHostToDevice, st));
-    const uint64_t *const *dptrs = static_cast<const uint64_t *const *>(ctx->tab);
-    const tw_t *dw = reinterpret_cast<const tw_t *>(static_cast<unsigned char *>(ctx->tab) + C * sizeof(void *));
+    tab.far = nullptr;
+    if (!large.empty()) {
+        CU(cudaMemcpyAsync(ctx->tab, host, words * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
+        tab.far = static_cast<const uint64_t *>(ctx->tab);
+    }
     if (mode == AGG_NTT) {
         int rc = ensure(&ctx->ws, &ctx->ws_bytes, 2 * T * (size_t)L * d.N * sizeof(uint64_t));
         if (rc != HE_OK) return rc;
-        CU(launch_aggregate_ntt(d, dptrs, dw, C, T, static_cast<uint64_t *>(ctx->ws), agg_dev, ctx->sm_count, st));
+        CU(launch_aggregate_ntt(d, tab, C, T, static_cast<uint64_t *>(ctx->ws), agg_dev, ctx->sm_count, st));
     } else if (mode == AGG_PARTIAL) {
-        CU(launch_aggregate_partial(d, dptrs, dw, C, T, agg_dev, ctx->sm_count, st));
+        CU(launch_aggregate_partial(d, tab, C, T, agg_dev, ctx->sm_count, st));
     } else {
-        CU(launch_aggregate(d, dptrs, dw, C, T, agg_dev, ctx->sm_count, st));
+        CU(launch_aggregate(d, tab, C, T, agg_dev, ctx->sm_count, st));
     }
     return HE_OK;
 }
@@ -652,24 +656,26 @@ int he_plain_aggregate(he_ctx *ctx, const float *const *rests_host, const double
     if (C > HE_MAX_CLIENTS) return HE_ERR_SIZE;
     if (len == 0) return HE_OK;
     if (!out_dev) return HE_ERR_INVALID_ARG;
-    std::vector<unsigned char> host(C * (sizeof(void *) + sizeof(double)));
-    const float **ptrs = reinterpret_cast<const float **>(host.data());
-    double *al = reinterpret_cast<double *>(host.data() + C * sizeof(void *));
+    SumTable tab;
+    const size_t words = 2 * (size_t)C;
+    std::vector<uint64_t> large(words <= SumTable::WORDS ? 0 : words);
+    uint64_t *host = large.empty() ? tab.words : large.data();
     bool aligned = true;
     for (int i = 0; i < C; i++) {
         if (!rests_host[i]) return HE_ERR_INVALID_ARG;
-        ptrs[i] = rests_host[i];
-        al[i] = alpha_host[i];
+        host[i] = reinterpret_cast<uintptr_t>(rests_host[i]);
+        memcpy(host + C + i, alpha_host + i, sizeof(double));
         aligned = aligned && aligned16(rests_host[i]);
     }
     cudaStream_t st = as_stream(stream);
-    // second half of the table buffer, so that it does not collide with a
-    // ciphertext aggregation queued just before
-    unsigned char *base = static_cast<unsigned char *>(ctx->tab) + HE_MAX_CLIENTS * (sizeof(void *) + HE_MAX_LIMBS * sizeof(tw_t));
-    CU(cudaMemcpyAsync(base, host.data(), host.size(), cudaMemcpyHostToDevice, st));
-    CU(launch_plain_aggregate(reinterpret_cast<const float *const *>(base),
-                              reinterpret_cast<const double *>(base + C * sizeof(void *)), C, len, out_dev, aligned,
-                              st));
+    tab.far = nullptr;
+    if (!large.empty()) {
+        // second half of the table buffer, so that it does not collide with a ciphertext aggregation queued just before
+        uint64_t *base = static_cast<uint64_t *>(ctx->tab) + HE_MAX_CLIENTS * (1 + 2 * HE_MAX_LIMBS);
+        CU(cudaMemcpyAsync(base, host, words * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
+        tab.far = base;
+    }
+    CU(launch_plain_aggregate(tab, C, len, out_dev, aligned, st));
     return HE_OK;
 }
 

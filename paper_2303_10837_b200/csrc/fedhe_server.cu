@@ -150,24 +150,28 @@ __device__ __forceinline__ void weighted_sum_limb(const LimbDev &lb, const uint6
     if (lb.fwd_d) weighted_sum_pair_f64(sp, sw, C, L, j, off, lb.qd, lb.qi, ax, ay);
     else weighted_sum_pair(sp, sw, C, L, j, off, lb, ax, ay);
 }
+__device__ __forceinline__ uint64_t table_word(const SumTable &tab, int i) { return tab.far ? __ldg(tab.far + i) : tab.words[i]; }
+// pointers and weights to shared memory
 template <bool SPLIT>
-__device__ __forceinline__ staged_t<SPLIT> staged_weight(const LimbDev &lb, const tw_t *w) {
-    const uint64_t v = __ldg(&w->w);
-    if constexpr (SPLIT) return lb.fwd_d ? f64_bits(f64_from_u64(v)) : (v & LOW30) | (v >> 30) << 32;
-    else return tw_t{v, __ldg(&w->wp)};
+__device__ __forceinline__ void stage_table(const CtxDev &c, const SumTable &tab, int C, staged_t<SPLIT> *sw, const uint64_t **sp) {
+    const int L = (int)c.L;
+    for (int e = threadIdx.x; e < C * L; e += blockDim.x) {
+        const uint64_t v = table_word(tab, C + 2 * e);
+        if constexpr (SPLIT) sw[e] = c.limb[e % L].fwd_d ? f64_bits(f64_from_u64(v)) : (v & LOW30) | (v >> 30) << 32;
+        else sw[e] = tw_t{v, table_word(tab, C + 2 * e + 1)};
+    }
+    for (int e = threadIdx.x; e < C; e += blockDim.x) sp[e] = reinterpret_cast<const uint64_t *>(table_word(tab, e));
+    __syncthreads();
 }
 
 template <bool SPLIT>
 __global__ void __launch_bounds__(256)
-aggregate_rescale_kernel(const __grid_constant__ CtxDev c, const uint64_t *const *ptrs, const tw_t *wtab,
-                         int C, uint64_t *out, size_t total) {
+aggregate_rescale_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ SumTable tab, int C, uint64_t *out, size_t total) {
     extern __shared__ __align__(16) unsigned char agg_sm[];
     const uint32_t L = c.L;
     auto *sw = reinterpret_cast<staged_t<SPLIT> *>(agg_sm);                         // [C][L]
     const uint64_t **sp = reinterpret_cast<const uint64_t **>(sw + (size_t)C * L);  // [C]
-    for (int e = threadIdx.x; e < C * (int)L; e += blockDim.x) sw[e] = staged_weight<SPLIT>(c.limb[e % (int)L], wtab + e);
-    for (int e = threadIdx.x; e < C; e += blockDim.x) sp[e] = ptrs[e];
-    __syncthreads();
+    stage_table<SPLIT>(c, tab, C, sw, sp);
     const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= total) return;
     const uint32_t pairs = c.N >> 1;
@@ -222,13 +226,13 @@ static cudaError_t launch_sum(K kernel, size_t smem, size_t total, cudaStream_t 
     return FEDHE_LAUNCHED();
 }
 
-cudaError_t launch_aggregate(const CtxDev &c, const uint64_t *const *ptrs, const tw_t *wtab, int C,
+cudaError_t launch_aggregate(const CtxDev &c, const SumTable &tab, int C,
                              size_t T, uint64_t *out, int n_sm, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
     const size_t total = T * 2 * (c.N >> 1);
     const bool split = split_pays(c, C, total, n_sm, true);
     return launch_sum(split ? aggregate_rescale_kernel<true> : aggregate_rescale_kernel<false>, sum_smem(c, C, split), total, s,
-                      c, ptrs, wtab, C, out, total);
+                      c, tab, C, out, total);
 }
 
 // ---------------------------------------------------------------------------
@@ -244,15 +248,13 @@ cudaError_t launch_aggregate(const CtxDev &c, const uint64_t *const *ptrs, const
 // limbs go to `out` ([T][2][L][N]): the partial sum of a subset of the clients
 template <bool SPLIT>
 __global__ void __launch_bounds__(256)
-aggregate_sum_kernel(const __grid_constant__ CtxDev c, const uint64_t *const *ptrs, const tw_t *wtab, int C,
+aggregate_sum_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ SumTable tab, int C,
                      uint64_t *out, uint64_t *last, size_t total) {
     extern __shared__ __align__(16) unsigned char agg_sm[];
     const uint32_t L = c.L;
     auto *sw = reinterpret_cast<staged_t<SPLIT> *>(agg_sm);
     const uint64_t **sp = reinterpret_cast<const uint64_t **>(sw + (size_t)C * L);
-    for (int e = threadIdx.x; e < C * (int)L; e += blockDim.x) sw[e] = staged_weight<SPLIT>(c.limb[e % (int)L], wtab + e);
-    for (int e = threadIdx.x; e < C; e += blockDim.x) sp[e] = ptrs[e];
-    __syncthreads();
+    stage_table<SPLIT>(c, tab, C, sw, sp);
     const size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= total) return;
     const uint32_t pairs = c.N >> 1;
@@ -311,18 +313,18 @@ rescale_partial_sum_kernel(const __grid_constant__ CtxDev c, const uint64_t *con
     }
 }
 
-static cudaError_t launch_limb_sums(const CtxDev &c, const uint64_t *const *ptrs, const tw_t *wtab, int C, uint64_t *out,
+static cudaError_t launch_limb_sums(const CtxDev &c, const SumTable &tab, int C, uint64_t *out,
                                     uint64_t *last, size_t pairs, int n_sm, cudaStream_t s) {
     const bool split = split_pays(c, C, pairs, n_sm, false);
-    return launch_sum(split ? aggregate_sum_kernel<true> : aggregate_sum_kernel<false>, sum_smem(c, C, split), pairs, s, c, ptrs, wtab,
+    return launch_sum(split ? aggregate_sum_kernel<true> : aggregate_sum_kernel<false>, sum_smem(c, C, split), pairs, s, c, tab,
                       C, out, last, pairs);
 }
 
-cudaError_t launch_aggregate_partial(const CtxDev &c, const uint64_t *const *ptrs, const tw_t *wtab, int C,
+cudaError_t launch_aggregate_partial(const CtxDev &c, const SumTable &tab, int C,
                                      size_t T, uint64_t *out, int n_sm, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
     const size_t pairs = T * 2 * (c.N >> 1);
-    return launch_limb_sums(c, ptrs, wtab, C, out, nullptr, pairs, n_sm, s);
+    return launch_limb_sums(c, tab, C, out, nullptr, pairs, n_sm, s);
 }
 
 cudaError_t launch_rescale_partial_sum(const CtxDev &c, const uint64_t *const *parts, int P, size_t T,
@@ -362,13 +364,13 @@ aggregate_finish_kernel(const __grid_constant__ CtxDev c, const uint64_t *rem, u
 }
 
 // scratch: [T][2][N] + [T][2][L-1][N] words
-cudaError_t launch_aggregate_ntt(const CtxDev &c, const uint64_t *const *ptrs, const tw_t *wtab, int C,
+cudaError_t launch_aggregate_ntt(const CtxDev &c, const SumTable &tab, int C,
                                  size_t T, uint64_t *scratch, uint64_t *out, int n_sm, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
     uint64_t *last = scratch, *rem = scratch + 2 * T * c.N;
     cudaError_t e;
     const size_t pairs = T * 2 * (c.N >> 1);
-    if ((e = launch_limb_sums(c, ptrs, wtab, C, out, last, pairs, n_sm, s))) return e;
+    if ((e = launch_limb_sums(c, tab, C, out, last, pairs, n_sm, s))) return e;
     if ((e = launch_ntt(c, false, last, 2 * T, c.N, c.L - 1, 1, s))) return e;
     if (c.L > 1) {
         const size_t n_last = 2 * T * c.N, n_out = n_last * (c.L - 1);
@@ -386,15 +388,17 @@ cudaError_t launch_aggregate_ntt(const CtxDev &c, const uint64_t *const *ptrs, c
 // load per client, two 16-byte stores) when every pointer allows it, and the
 // loads of several clients are in flight at once.
 __global__ void __launch_bounds__(256)
-plain_aggregate_kernel(const float *const *ptrs, const double *alpha, int C, size_t len, double *out, bool vec) {
+plain_aggregate_kernel(const __grid_constant__ SumTable tab, int C, size_t len, double *out, bool vec) {
+    auto rest = [&](int cl) { return reinterpret_cast<const float *>(table_word(tab, cl)); };
+    auto weight = [&](int cl) { return f64_from_bits(table_word(tab, C + cl)); };
     const size_t g = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
     if (g >= len) return;
     double a[4] = {0.0, 0.0, 0.0, 0.0};
     if (vec && g + 4 <= len) {
 #pragma unroll 5
         for (int cl = 0; cl < C; cl++) {
-            const float4 v = __ldg(reinterpret_cast<const float4 *>(ptrs[cl] + g));
-            const double al = alpha[cl];
+            const float4 v = __ldg(reinterpret_cast<const float4 *>(rest(cl) + g));
+            const double al = weight(cl);
             a[0] = __dadd_rn(a[0], __dmul_rn(al, (double)v.x));
             a[1] = __dadd_rn(a[1], __dmul_rn(al, (double)v.y));
             a[2] = __dadd_rn(a[2], __dmul_rn(al, (double)v.z));
@@ -406,18 +410,18 @@ plain_aggregate_kernel(const float *const *ptrs, const double *alpha, int C, siz
     }
     const uint32_t cnt = len - g < 4 ? (uint32_t)(len - g) : 4u;
     for (int cl = 0; cl < C; cl++) {
-        const double al = alpha[cl];
-        for (uint32_t j = 0; j < cnt; j++) a[j] = __dadd_rn(a[j], __dmul_rn(al, (double)__ldg(ptrs[cl] + g + j)));
+        const double al = weight(cl);
+        for (uint32_t j = 0; j < cnt; j++) a[j] = __dadd_rn(a[j], __dmul_rn(al, (double)__ldg(rest(cl) + g + j)));
     }
     for (uint32_t j = 0; j < cnt; j++) out[g + j] = a[j];
 }
 
 // aligned16: every client's pointer is 16-byte aligned
-cudaError_t launch_plain_aggregate(const float *const *ptrs, const double *alpha, int C, size_t len,
+cudaError_t launch_plain_aggregate(const SumTable &tab, int C, size_t len,
                                    double *out, bool aligned16, cudaStream_t s) {
     if (len == 0) return cudaSuccess;
     const bool vec = aligned16 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
-    plain_aggregate_kernel<<<blocks_for((len + 3) / 4, 256), 256, 0, s>>>(ptrs, alpha, C, len, out, vec);
+    plain_aggregate_kernel<<<blocks_for((len + 3) / 4, 256), 256, 0, s>>>(tab, C, len, out, vec);
     return FEDHE_LAUNCHED();
 }
 

@@ -590,6 +590,21 @@ def test_pack_unpack_plain_aggregate_bit_exact(he):
 
 # --------------------------------------------------------------------------- whole rounds
 
+@pytest.mark.parametrize("C", [1, 64, 65, 256])
+def test_plain_aggregate_of_many_clients(he, C):
+    """Pointers and weights in the kernel's parameters (up to 64 clients) and in device memory."""
+    g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
+    rng = np.random.default_rng(C)
+    rests = [rng.standard_normal(1003, dtype=np.float32) for _ in range(C)]
+    alpha = rng.random(C)
+    alpha /= alpha.sum()
+    want = np.zeros(1003)
+    for a, r in zip(alpha, rests):
+        want = want + a * r.astype(np.float64)
+    got = he.he_plain_aggregate(g, [dev_f32(r) for r in rests], alpha.tolist()).cpu().numpy()
+    assert np.array_equal(got, want)
+
+
 def run_round_gpu(he, g, keys, mask, xs, alpha, w):
     cts, rests = [], []
     for i, x in enumerate(xs):
