@@ -110,6 +110,10 @@ def _check(code: int, where: str) -> None:
 
 
 def _stream() -> int:
+    """The current stream's handle.  The raw query makes no stream object: 0.2 us instead of 3.2, of 14 us that a short call
+    (packing or encrypting a ciphertext) takes the host."""
+    if torch.cuda.is_initialized():
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return torch.cuda.current_stream().cuda_stream
 
 
