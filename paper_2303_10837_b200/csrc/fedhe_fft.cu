@@ -513,12 +513,14 @@ enc_sample_kernel(const void *gauss, EncDraw draw, uint32_t T, unsigned char *sa
 // longer than the mean).  Of the `rem` ciphertexts after the last whole round each is cut in `parts`: clusters that
 // all prepare it and share its units.
 //
-// What bounds it is latency: registers leave 16 warps to an SM, the fp64 pipe is 31 to 35 % busy, the load and store
-// path half, and on N = 2^15 part of the 98 MB of scratch misses L2.  Measured, against modular transforms of every limb:
-//   N = 2^13, L = 3, 1 ciphertext       67.7 us -> 30.7 us
-//   N = 2^14, L = 4, 313 ciphertexts    0.69 ms -> 0.32 ms
-//   N = 2^14, L = 4, 1429 ciphertexts   2.82 ms -> 1.38 ms (1.1 TB/s of ciphertext)
-//   N = 2^15, L = 6, 6714 ciphertexts   40.2 ms -> 26.8 ms (0.8 TB/s)
+// What bounds it: in the transforms shared memory (3360 of 3500 clocks a block of 2^12 points and SM: two exchanges of 1024, the key's table in and
+// out 1024, twiddles 288), between them latency at the 16 warps that registers leave; the fp64 pipe is 30 to 35 % busy.  Measured, against
+// modular transforms of every limb; with the draws of u and the errors by the clusters; and with these from the kernel above and what a
+// product needs to know in shared memory:
+//   N = 2^13, L = 3, 1 ciphertext       67.7 us -> 30.7 us -> 24.9 us
+//   N = 2^14, L = 4, 313 ciphertexts    0.69 ms -> 0.32 ms -> 0.30 ms
+//   N = 2^14, L = 4, 1429 ciphertexts   2.82 ms -> 1.38 ms -> 1.27 ms (1.2 TB/s of ciphertext)
+//   N = 2^15, L = 6, 672 ciphertexts              2.69 ms -> 2.33 ms (0.9 TB/s)
 //
 // PAIRS: some units are of two limbs (the code for both kinds costs the others 1.5 %).
 template <int CL, bool PAIRS>
@@ -1186,7 +1188,7 @@ static uint32_t enc_sure_fit(const CtxDev &c, uint32_t alone, uint32_t S) {
 
 // What a plan takes, in us: a round is fixed + by_size / S + product * (block transforms of the busiest block's products),
 // fitted to 10,000 measurements of all plans for up to 200 ciphertexts of 2 to 12 limbs of 45 and 60 bits (nine of ten within
-// 10 %), for two blocks to an SM and for one.
+// 10 %), for two blocks to an SM and for one, when the clusters drew for themselves; with the draws made before, all plans take about a tenth less.
 struct EncCost { double fixed, by_size, product; };
 static const EncCost ENC_COST[4][2] = {{{27.3, 12.7, 7.7}, {33.1, 2.2, 4.9}},
                                        {{27.4, 40.1, 9.1}, {43.5, 13.7, 5.7}},

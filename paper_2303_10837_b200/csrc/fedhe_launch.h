@@ -29,8 +29,8 @@ cudaError_t launch_decode(const CtxDev &c, const int64_t *d, size_t T, double2 *
                           cudaStream_t s);
 
 // Encode + encrypt ciphertexts t0 .. t0+T-1 (sel and ct point at the first of
-// them).  `work` is scratch of fft_work_bytes() bytes: what the resident thread
-// blocks keep in L2, or, by passes, what those need.
+// them).  `work` is scratch of fft_work_bytes() bytes: the random draws (for 256 MiB
+// of them at a time) and what the resident thread blocks keep in L2, or, by passes, what those need.
 size_t fft_work_bytes(const CtxDev &c, size_t T);
 cudaError_t launch_encrypt(const CtxDev &c, const KeysDev &k, const float *sel, void *work, uint32_t t0, size_t T,
                            uint64_t seed, uint32_t client, uint64_t *ct, cudaStream_t s);
