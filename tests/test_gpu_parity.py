@@ -590,6 +590,24 @@ def test_pack_unpack_plain_aggregate_bit_exact(he):
 
 # --------------------------------------------------------------------------- whole rounds
 
+@pytest.mark.parametrize("N,primes,T", [
+    (8192, si.PRIMES_N8192, 63), (8192, si.PRIMES_N8192, 64), (8192, si.PRIMES_N8192, 10_930), (16384, si.PRIMES_N16384, 33),
+    (16384, si.PRIMES_N16384, 200), (32768, si.PRIMES_N32768, 17), (32768, si.PRIMES_N32768, 90), (65536, si.PRIMES_SWEEP[:2], 9)])
+def test_samples_drawn_ahead_are_those_drawn_by_the_clusters(he, N, primes, T):
+    """From 2^19 coefficients on a kernel of its own draws u and the errors (for 256 MiB of them at a time), and with no more
+    ciphertexts than clusters the encryption starts beside it; fewer ciphertexts are drawn by their clusters."""
+    g, _ = contexts(he, N, primes, 40)
+    keys = he.he_keygen(g, 77)
+    n, few = N // 2, 7
+    x = torch.randn(T * n, generator=torch.Generator(device="cuda").manual_seed(T), device="cuda").mul_(0.01)
+    ct = he.he_encrypt(g, keys, x, 5, 3)
+    part = torch.empty((few, 2, len(primes), N), dtype=torch.int64, device="cuda")
+    for first in sorted({0, max(0, T // 2 - few), max(0, T - 9 - few), T - few}):
+        he.he_encrypt_range(g, keys, x[first * n:(first + few) * n].contiguous(), first, few, 5, 3, part)
+        assert torch.equal(ct[first:first + few], part), first
+    assert he.he_ctx_status(g) == he.HE_OK
+
+
 @pytest.mark.parametrize("C", [1, 64, 65, 256])
 def test_plain_aggregate_of_many_clients(he, C):
     """Pointers and weights in the kernel's parameters (up to 64 clients) and in device memory."""
