@@ -608,6 +608,29 @@ def test_samples_drawn_ahead_are_those_drawn_by_the_clusters(he, N, primes, T):
     assert he.he_ctx_status(g) == he.HE_OK
 
 
+@pytest.mark.parametrize("T", [9, 70])
+def test_encryption_and_sum_in_a_graph(he, T):
+    """A captured encryption (its draws by the clusters, and by a kernel that it starts beside) and weighted sum give the same again."""
+    g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
+    keys = he.he_keygen(g, 78)
+    x = torch.randn(T * 4096, generator=torch.Generator(device="cuda").manual_seed(T), device="cuda").mul_(0.01)
+    he.he_ctx_reserve(g, T * 4096)
+    want = he.he_encrypt(g, keys, x, 6, 1)
+    want_sum = he.he_weighted_aggregate(g, [want, want], [0.25, 0.5])
+    ct, total = torch.zeros_like(want), torch.zeros_like(want_sum)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        he.he_encrypt(g, keys, x, 6, 1, out=ct)
+        he.he_weighted_aggregate(g, [ct, ct], [0.25, 0.5], out=total)
+    for _ in range(2):
+        ct.zero_()
+        total.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(ct, want) and torch.equal(total, want_sum)
+
+
 @pytest.mark.parametrize("C", [1, 64, 65, 256])
 def test_plain_aggregate_of_many_clients(he, C):
     """Pointers and weights in the kernel's parameters (up to 64 clients) and in device memory."""
