@@ -65,7 +65,7 @@ UNIT = "params/s"
 # the slots, and one inverse per product of u with a piece of the public key.
 # DRAM bytes (read + write) per ciphertext of the encrypt kernel, by (N, L), from an ncu capture of
 # the profile_case.py encrypt case (traffic grows in proportion to the number of ciphertexts).
-ENCRYPT_DRAM_BYTES_PER_CT = {(8192, 3): 110.983168e6 / 296, (16384, 4): 332.172544e6 / 296, (32768, 6): 999.883776e6 / 142}
+ENCRYPT_DRAM_BYTES_PER_CT = {(8192, 3): 109.837312e6 / 296, (16384, 4): 325.827072e6 / 296, (32768, 6): 965.808128e6 / 142}
 SLOTS_PER_SM_CLK = 64.0
 WIDE_COST = 2.5
 INT_SLOTS_PER_BUTTERFLY = 6 * WIDE_COST + 4
@@ -521,6 +521,8 @@ def measure(job, w, steps, warmup, with_cpu_baseline):
     alg_bytes = (4.0 + 32.0 * w.L) * n * per_launch          # read the slots, write the ciphertext
     if not transform and launches_per_encrypt == 1:
         kname = "encrypt_fft_kernel"
+    elif not transform and launches_per_encrypt == 2:
+        kname = "enc_sample_kernel and encrypt_fft_kernel, timed as one call"
     elif w.N <= 16384:
         kname = "encrypt_fused2_kernel" if w.N == 16384 else "encrypt_fused_kernel"
     else:

@@ -631,9 +631,9 @@ def test_encryption_and_sum_in_a_graph(he, T):
         assert torch.equal(ct, want) and torch.equal(total, want_sum)
 
 
-@pytest.mark.parametrize("C", [1, 64, 65, 256])
+@pytest.mark.parametrize("C", [1, 24, 25, 256])
 def test_plain_aggregate_of_many_clients(he, C):
-    """Pointers and weights in the kernel's parameters (up to 64 clients) and in device memory."""
+    """Pointers and weights in the kernel's parameters (up to 24 clients) and in device memory."""
     g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
     rng = np.random.default_rng(C)
     rests = [rng.standard_normal(1003, dtype=np.float32) for _ in range(C)]
