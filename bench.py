@@ -430,7 +430,7 @@ def measure(job, w, steps, warmup, with_cpu_baseline):
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     reps = 5
     encode_ms = 0.0
-    if launches_per_encrypt > 1 and Tr:
+    if transform and launches_per_encrypt > 1 and Tr:     # the coefficient format's other kernel draws the samples
         he.he_encode(g, sel0)
         e0.record()
         for _ in range(reps):
