@@ -24,6 +24,11 @@
  *     pointer that is not is refused with HE_ERR_INVALID_ARG before anything is
  *     launched.  float, double, int64 and index buffers need only their
  *     natural alignment (the kernels fall back to narrower accesses).
+ *   - Host arrays of pointers, weights and ranges are read before the call
+ *     returns, also when `stream` is being captured: a graph holds what they
+ *     said at the capture.  The calls that are asynchronous can be captured once
+ *     the context's work buffers are large enough (he_ctx_reserve, or the same
+ *     call before); a graph must not outlive a call that makes them larger.
  *   - The library cannot see how large a caller's buffer is: every size below
  *     is a requirement on the caller (the Python binding checks them).
  *   - `stream` is a cudaStream_t passed as void* (NULL = default stream).

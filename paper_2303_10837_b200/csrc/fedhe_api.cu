@@ -559,6 +559,16 @@ int he_encrypt(he_ctx *ctx, const he_keys *keys, const float *sel_dev, size_t k,
     return he_encrypt_range(ctx, keys, sel_dev, 0, he_num_ct(ctx, k), seed, client_id, ct_dev, stream);
 }
 
+// A table of the host in device memory.  The host's ends with the call: the copy has read it by then, but a captured one would read it again at
+// every replay of the graph, so a stream that is being captured gets it as parameters of kernels.
+static cudaError_t put_table(void *dst, const void *host, size_t words, cudaStream_t st) {
+    cudaStreamCaptureStatus capture;
+    const cudaError_t e = cudaStreamIsCapturing(st, &capture);
+    if (e) return e;
+    if (capture != cudaStreamCaptureStatusNone) return launch_table(host, words, static_cast<uint64_t *>(dst), st);
+    return cudaMemcpyAsync(dst, host, words * sizeof(uint64_t), cudaMemcpyHostToDevice, st);
+}
+
 enum AggMode { AGG_RESCALE, AGG_NTT, AGG_PARTIAL };
 
 static int weighted_aggregate(he_ctx *ctx, const uint64_t *const *cts_host, const double *alpha_host, int C,
@@ -591,7 +601,7 @@ static int weighted_aggregate(he_ctx *ctx, const uint64_t *const *cts_host, cons
     cudaStream_t st = as_stream(stream);
     tab.far = nullptr;
     if (!large.empty()) {
-        CU(cudaMemcpyAsync(ctx->tab, host, words * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
+        CU(put_table(ctx->tab, host, words, st));
         tab.far = static_cast<const uint64_t *>(ctx->tab);
     }
     if (mode == AGG_NTT) {
@@ -629,7 +639,7 @@ static int rescale_partial(he_ctx *ctx, const uint64_t *const *parts_host, int P
     for (int p = 0; p < P; p++)
         if (!parts_host[p] || !aligned16(parts_host[p])) return HE_ERR_INVALID_ARG;
     cudaStream_t st = as_stream(stream);
-    CU(cudaMemcpyAsync(ctx->tab, parts_host, P * sizeof(void *), cudaMemcpyHostToDevice, st));
+    CU(put_table(ctx->tab, parts_host, (size_t)P, st));
     CU(launch_rescale_partial_sum(ctx->dev, static_cast<const uint64_t *const *>(ctx->tab), P, T, agg_dev, st));
     return HE_OK;
 }
@@ -672,7 +682,7 @@ int he_plain_aggregate(he_ctx *ctx, const float *const *rests_host, const double
     if (!large.empty()) {
         // second half of the table buffer, so that it does not collide with a ciphertext aggregation queued just before
         uint64_t *base = static_cast<uint64_t *>(ctx->tab) + HE_MAX_CLIENTS * (1 + 2 * HE_MAX_LIMBS);
-        CU(cudaMemcpyAsync(base, host, words * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
+        CU(put_table(base, host, words, st));
         tab.far = base;
     }
     CU(launch_plain_aggregate(tab, C, len, out_dev, aligned, st));

@@ -76,6 +76,8 @@ struct SumTable {
     const uint64_t *far;                  // in device memory; null: here
     uint64_t words[WORDS];
 };
+// `words` words of the host to device memory, as parameters of kernels that write them
+cudaError_t launch_table(const void *host, size_t words, uint64_t *dst, cudaStream_t s);
 cudaError_t launch_aggregate(const CtxDev &c, const SumTable &tab, int C,
                              size_t T, uint64_t *out, int n_sm, cudaStream_t s);
 // transform-domain ciphertexts in and out; scratch: uint64 [T][2][L][N]

@@ -1,6 +1,8 @@
 // Server-side kernels: weighted ciphertext sum with rescale, plaintext remainder (part 4 of the kernels).
 #include "fedhe_kernels.cuh"
 
+#include <cstring>
+
 namespace fedhe {
 
 // ===========================================================================
@@ -150,6 +152,24 @@ __device__ __forceinline__ void weighted_sum_limb(const LimbDev &lb, const uint6
     if (lb.fwd_d) weighted_sum_pair_f64(sp, sw, C, L, j, off, lb.qd, lb.qi, ax, ay);
     else weighted_sum_pair(sp, sw, C, L, j, off, lb, ax, ay);
 }
+// what fits the 4 KB of a kernel's parameters beside the rest
+struct TablePart { uint64_t words[480]; };
+__global__ void __launch_bounds__(256) table_kernel(const __grid_constant__ TablePart part, uint32_t count, uint64_t *dst) {
+    for (uint32_t i = threadIdx.x; i < count; i += blockDim.x) dst[i] = part.words[i];
+}
+cudaError_t launch_table(const void *host, size_t words, uint64_t *dst, cudaStream_t s) {
+    constexpr size_t MOST = sizeof(TablePart) / sizeof(uint64_t);
+    for (size_t at = 0; at < words; at += MOST) {
+        TablePart part;
+        const size_t count = words - at < MOST ? words - at : MOST;
+        memcpy(part.words, static_cast<const uint64_t *>(host) + at, count * sizeof(uint64_t));
+        table_kernel<<<1, 256, 0, s>>>(part, (uint32_t)count, dst + at);
+        const cudaError_t e = FEDHE_LAUNCHED();
+        if (e) return e;
+    }
+    return cudaSuccess;
+}
+
 __device__ __forceinline__ uint64_t table_word(const SumTable &tab, int i) { return tab.far ? __ldg(tab.far + i) : tab.words[i]; }
 // pointers and weights to shared memory
 template <bool SPLIT>
