@@ -227,6 +227,8 @@ key_candidates_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
     // bit patterns beyond the window and within: from `last` + 1 and from `base`, so many
     const uint32_t last = base + 0xfffffu, many = infinity > last ? infinity - last : 0u;
     const uint32_t within = base > infinity ? 0u : infinity - base < 0xfffffu ? infinity - base + 1u : 1u << 20;
+    // in a window at 0, where a key of 0 has many bit patterns, is all that is not beyond it
+    const uint32_t in_from = base ? base : last + 1u, in_many = base ? within : many, turned = base ? 0u : 0xffffffffu;
     const uint32_t lane = threadIdx.x & 31u;
     const size_t tiles = (P + MASK_BLOCK - 1) / MASK_BLOCK, whole = P / MASK_BLOCK, stride = (size_t)gridDim.x * (CAND_THREADS / 32);
     size_t tile = (size_t)blockIdx.x * (CAND_THREADS / 32) + (threadIdx.x >> 5);
@@ -242,7 +244,7 @@ key_candidates_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
     for (; tile < tiles; tile += stride, p += stride * MASK_BLOCK) {
         uint32_t my_bits = 0, mine = 0;                             // word `lane` of the marks; bit i: the lane's key in word i is a candidate
         static_assert(MASK_BLOCK == 1024, "a word of the tile for every lane");
-        if (tile < whole && base) {
+        if (tile < whole) {
 #pragma unroll 1
             for (uint32_t w0 = 0; w0 < 32; w0 += LOADS) {
                 uint32_t who[LOADS], some = 0;
@@ -250,7 +252,7 @@ key_candidates_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
                 for (int j = 0; j < LOADS; j++) {
                     const uint32_t raw = __float_as_uint(next[j]);
                     who[j] = __ballot_sync(0xffffffffu, raw - last - 1u < many);
-                    if (window_place(raw, base) < within) some |= 1u << j;
+                    if (raw - in_from < in_many) some |= 1u << j;
                 }
                 mine |= some << w0;
                 const bool same = w0 + LOADS < 32;
@@ -265,9 +267,9 @@ key_candidates_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
                                d = lane & 1u ? who[7] : who[6], e = lane & 2u ? b : a, f = lane & 2u ? d : c;
                 if ((lane & ~7u) == w0) my_bits = lane & 4u ? f : e;
             }
+            mine ^= turned;
         } else {
-            // the last tile, and a window at 0
-            const uint32_t left = tile < whole ? MASK_BLOCK : (uint32_t)(P - tile * MASK_BLOCK);
+            const uint32_t left = (uint32_t)(P - tile * MASK_BLOCK);        // the last tile
 #pragma unroll 1
             for (uint32_t word = 0; word < 32; word++) {
                 const bool there = word * 32 + lane < left;
@@ -275,10 +277,6 @@ key_candidates_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
                 const uint32_t who = __ballot_sync(0xffffffffu, key > last);
                 if (lane == word) my_bits = who;
                 if (there && window_place(key, base) < 1u << 20) mine |= 1u << word;
-            }
-            if (tile + stride < whole) {
-#pragma unroll
-                for (int j = 0; j < LOADS; j++) next[j] = __ldg(p + stride * MASK_BLOCK + j * 32);
             }
         }
         uint32_t at = __popc(mine);
@@ -336,18 +334,26 @@ key_candidates_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
         });
 }
 
-// f(in, lower 20 bits and place in the tile) for the candidates of a tile, by a whole warp: f may use warp operations
+// f(in, lower 20 bits and place in the tile) for the listed candidates of a tile, by a whole warp: the lane's every 32nd, of which the
+// first is there already (rarely more than 32: these come with their number)
+template <class F>
+__device__ __forceinline__ void for_listed(const uint32_t *cand, uint32_t c, uint32_t found, F f) {
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint32_t i = 0; i < found; i += 32) {
+        const bool in = i + lane < found;
+        f(in, in ? c : 0u);
+        if (i + 32 < found) c = cand[i + 32];
+    }
+}
+
+// the same for all candidates, of which there may be too many for the list
 template <class F>
 __device__ __forceinline__ void for_candidates(const float *score, size_t P, const SelectWork &w, size_t tile, uint32_t base, F f) {
     const uint32_t lane = threadIdx.x & 31u, found = w.tile_found[tile];
     const uint32_t *cand = w.cand + tile * TILE_CANDIDATES + lane;
-    uint32_t c = *cand;                                             // rarely more than 32: these come with their number
+    const uint32_t c0 = *cand;
     if (found <= TILE_CANDIDATES) {
-        for (uint32_t i = 0; i < found; i += 32) {
-            const bool in = i + lane < found;
-            f(in, in ? c : 0u);
-            if (i + 32 < found) c = cand[i + 32];
-        }
+        for_listed(cand, c0, found, f);
     } else {
         for_tile(score, P, tile * MASK_BLOCK, [&](uint32_t w0, const uint32_t (&key)[LOADS], uint32_t left) {
 #pragma unroll
@@ -487,33 +493,60 @@ cudaError_t launch_scan(uint32_t *a, size_t count, uint32_t *total, cudaStream_t
 // Membership: key > tau, or key == tau and fewer than `need` equal keys at lower indices, or (RANGES)
 // inside a forced index range.  A warp takes a tile, lane l ends up with word l of its bits.
 
-// from the bits of the keys beyond the window and the candidates
+// From the bits of the keys beyond the window and the candidates: these set their bits one by one where they are listed, and by words where
+// the tile is read again (its 32 keys of a word would take turns at it: 25.6 M equal scores, half of them wanted: 235 us a selection, and 191).
+// words: the warp's own [2][32].
 __device__ __forceinline__ uint32_t tile_bits(const float *score, size_t P, const SelectWork &w, size_t tile, uint32_t eq_before, uint32_t *words) {
-    const uint32_t place = w.state->place, need = w.state->need, found = w.tile_found[tile];
-    const uint32_t lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
-    const uint32_t *cand = w.cand + tile * TILE_CANDIDATES;
-    words[lane] = tile * MASK_BLOCK + lane * 32u < P ? w.bits[tile * (MASK_BLOCK / 32) + lane] : 0u;
-    __syncwarp();
-    for_candidates(score, P, w, tile, w.state->base, [&](bool in, uint32_t c) {
-        const bool eq = in && c >> 10 == place;
-        uint32_t rank = eq_before;                                  // of an equal key among all of them
-        if (found > TILE_CANDIDATES) {                              // in order
-            const uint32_t eqs = __ballot_sync(0xffffffffu, eq);
-            rank += __popc(eqs & below);
-            eq_before += __popc(eqs);
-        } else if (eq) {
-            for (uint32_t i = 0; i < found; i++) rank += cand[i] >> 10 == place && cand[i] < c ? 1u : 0u;
+    const uint32_t base = w.state->base, place = w.state->place, need = w.state->need, found = w.tile_found[tile], lane = threadIdx.x & 31u;
+    const uint32_t *cand = w.cand + tile * TILE_CANDIDATES + lane;
+    const uint32_t c0 = *cand;
+    uint32_t bits = tile * MASK_BLOCK + lane * 32u < P ? w.bits[tile * (MASK_BLOCK / 32) + lane] : 0u, equal = 0;
+    if (found <= TILE_CANDIDATES) {
+        words[lane] = bits;
+        words[32 + lane] = 0;
+        __syncwarp();
+        for_listed(cand, c0, found, [&](bool in, uint32_t c) {
+            const uint32_t at = c >> 10;
+            if (in && at >= place) atomicOr(words + (at == place ? 32 : 0) + (c >> 5 & 31u), 1u << (c & 31u));
+        });
+        __syncwarp();
+        bits = words[lane];
+        equal = words[32 + lane];
+    } else {
+        for_tile(score, P, tile * MASK_BLOCK, [&](uint32_t w0, const uint32_t (&key)[LOADS], uint32_t left) {
+#pragma unroll
+            for (int j = 0; j < LOADS; j++) {
+                const uint32_t at = window_place(key[j], base);
+                const bool in = j * 32u + lane < left && at < 1u << 20;
+                const uint32_t gt = __ballot_sync(0xffffffffu, in && at > place), eq = __ballot_sync(0xffffffffu, in && at == place);
+                if (lane == w0 + j) {
+                    bits |= gt;
+                    equal = eq;
+                }
+            }
+        });
+    }
+    if (__any_sync(0xffffffffu, equal != 0)) {
+        // the first `need` of all equal keys
+        uint32_t before = __popc(equal);
+        const uint32_t mine = before;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t o = __shfl_up_sync(0xffffffffu, before, d);
+            if (lane >= (uint32_t)d) before += o;
         }
-        if ((in && c >> 10 > place) || (eq && rank < need)) atomicOr(words + (c >> 5 & 31u), 1u << (c & 31u));
-    });
-    __syncwarp();
-    return words[lane];
+        before += eq_before - mine;
+        const uint32_t room = need > before ? need - before : 0u;
+        for (uint32_t over = mine > room ? mine - room : 0u; over; over--) equal &= ~(0x80000000u >> __clz((int)equal));
+        bits |= equal;
+    }
+    return bits;
 }
 template <bool RANGES>
 __global__ void __launch_bounds__(256)
 mask_mark_kernel(const float *score, size_t P, SelectWork w, const uint64_t *ranges, uint32_t nranges,
                  uint32_t *wpre, uint32_t *idx, uint32_t room, uint32_t *tile_sel) {
-    __shared__ uint32_t words[8][32];
+    __shared__ uint32_t words[8][64];
     if (w.total[1]) return;
     const uint32_t need = w.state->need;
     const uint32_t lane = threadIdx.x & 31u;

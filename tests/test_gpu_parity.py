@@ -553,6 +553,26 @@ def test_select_mask_by_a_sample(he, kind):
         assert mask.k == k and np.array_equal(got, oracle.select_mask(score, k)), k
 
 
+@pytest.mark.parametrize("P", [1024, 5 * 1024 + 77, (1 << 22) + 1024])
+def test_select_mask_of_tied_scores(he, P):
+    """Tiles of more candidates than are listed, marked by words, and a window at 0, where negative scores and NaN are: thresholds among
+    the zeros, among equal scores and between them, on whole tiles and a part of one."""
+    g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
+    rng = np.random.default_rng(P)
+    kind = rng.random(P)
+    score = np.where(kind < 0.5, -rng.random(P), 0.25 * rng.integers(1, 4, P)).astype(np.float32)
+    score[kind > 0.99] = 0.5 * rng.random(int((kind > 0.99).sum()))
+    score[rng.integers(0, P, 9)] = [np.nan, -np.nan, np.inf, 0.0, -0.0, 1e-40, 1.5e-38, -np.inf, 2.0]
+    d = dev_f32(score)
+    for k in sorted({1, P // 9, P // 3, P // 2, int(0.7 * P), P - 1, P}):
+        got = he.he_mask_indices(he.he_select_mask(g, d, k)).cpu().numpy().view(np.uint32)
+        assert np.array_equal(got, oracle.select_mask(score, k)), k
+        mask = he.he_select_mask_ranges(g, d, k, [(3, 40), (P - 70, P - 2)])
+        got = he.he_mask_indices(mask).cpu().numpy().view(np.uint32)
+        want = np.union1d(oracle.select_mask(score, k), np.r_[3:40, P - 70:P - 2])
+        assert np.array_equal(got, want), k
+
+
 def test_mask_with_forced_ranges(he):
     """Top-k plus whole index ranges (first and last layers)."""
     g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
