@@ -386,8 +386,8 @@ static int build_mask(he_ctx *ctx, const float *score, size_t P, size_t k, const
     SelectWork w;
     w.hist = scratch;
     w.done = scratch + SELECT_HIST;
-    w.state = reinterpret_cast<SelectState *>(w.done + 4);
-    w.total = w.done + 8;
+    w.state = reinterpret_cast<SelectState *>(w.done + 8);
+    w.total = w.done + 14;
     w.sampled = scratch + SELECT_ZEROED;
     uint64_t *ranges_dev = reinterpret_cast<uint64_t *>(w.sampled + SELECT_BINS);
     w.runs = ranges_dev + 2 * 64;

@@ -121,16 +121,17 @@ int ctx_workspace(he_ctx *ctx, size_t T, void **out);
 
 // mask construction (tiles of MASK_BLOCK consecutive parameters)
 constexpr uint32_t MASK_BLOCK = 1024, TILE_CANDIDATES = 128;
-// progress of the selection, in device memory: the window [base, base + 2^20) of keys that the threshold is looked for in, how much
+// progress of the selection, in device memory: the window [base, base + 2^(20 + shift)) of keys that the threshold is looked for in, how much
 // of its place in there is found (all of it after the last step: tau = base + place), and how many keys are still to be covered
 // (after the last step: how many keys equal to tau belong to the mask)
-struct SelectState { uint32_t base, place, need, above; };      // above: keys beyond the window
+struct SelectState { uint32_t base, shift, place, need, above; };      // above: keys beyond the window
+constexpr uint32_t WINDOW_OPEN = 3;               // shift: the sample could not say
 // work space of a selection; the words from `hist` to the end of `sampled` are cleared at its start
-constexpr size_t SELECT_HIST = 2048 + 1024 + 1024, SELECT_BINS = 1u << 12, SELECT_ZEROED = SELECT_HIST + 4 + 8;
+constexpr size_t SELECT_LAST = 4096, SELECT_HIST = 2048 + 1024 + SELECT_LAST, SELECT_BINS = 1u << 12, SELECT_ZEROED = SELECT_HIST + 8 + 8;
 constexpr size_t SELECT_RUNS = 2 * 1024;          // thread blocks that a device holds at once, at most
 struct SelectWork {
-    uint32_t *hist;              // 2048, 1024, 1024
-    uint32_t *done;              // [4] thread blocks that finished a pass
+    uint32_t *hist;              // 2048, 1024, SELECT_LAST
+    uint32_t *done;              // [5] thread blocks that finished a pass
     SelectState *state;
     uint32_t *total;             // selected parameters (without forced ranges), then whether the threshold was outside the window
     uint32_t *sampled;           // [SELECT_BINS] keys of the sample by their upper bits

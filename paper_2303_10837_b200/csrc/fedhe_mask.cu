@@ -64,10 +64,9 @@ __device__ __forceinline__ bool last_block(uint32_t *done) {
     return is_last != 0;
 }
 
-// Walks the digits of a histogram from the largest down until `need` keys are covered: found(digit, keys above it, its keys), by
-// one thread, if there are as many.  By a block of NT threads.
-template <int BITS, uint32_t NT = 1024, class Found>
-__device__ __forceinline__ void radix_pick(const uint32_t *hist, uint32_t need, const Found &found) {
+// Calls see(digit, keys above it, its keys) for every digit of a histogram, by one thread each.  By a block of NT threads.
+template <int BITS, uint32_t NT = 1024, class See>
+__device__ __forceinline__ void radix_walk(const uint32_t *hist, const See &see) {
     __shared__ uint32_t warp_sums[33];
     constexpr uint32_t bins = 1u << BITS, per = bins / NT;           // thread t: digits from bins - 1 - per t down
     uint32_t h[per], mine = 0u;
@@ -81,10 +80,16 @@ __device__ __forceinline__ void radix_pick(const uint32_t *hist, uint32_t need, 
 #pragma unroll
     for (uint32_t j = 0; j < per; j++) {
         const uint32_t pos = threadIdx.x * per + j;
-        // the digit where the running count first reaches `need`
-        if (above < need && above + h[j] >= need) found(bins - 1u - pos, above, h[j]);
+        see(bins - 1u - pos, above, h[j]);
         above += h[j];
     }
+}
+// found(digit, keys above it) for the digit where the count from the largest down first reaches `need`, if there are as many
+template <int BITS, uint32_t NT = 1024, class Found>
+__device__ __forceinline__ void radix_pick(const uint32_t *hist, uint32_t need, const Found &found) {
+    radix_walk<BITS, NT>(hist, [&](uint32_t digit, uint32_t above, uint32_t count) {
+        if (above < need && above + count >= need) found(digit, above);
+    });
 }
 
 // First digit.  Every lane counts in a column of its own, so the lanes of a warp never meet in a word or a bank: two
@@ -144,19 +149,22 @@ key_histogram_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
         if (k == 0) {
             if (threadIdx.x == 0) w.state->base = 0x80000000u;                   // no key reaches the window
         } else {
-            radix_pick<11>(w.hist, k, [&](uint32_t digit, uint32_t, uint32_t) { w.state->base = digit << 20; });
+            radix_pick<11>(w.hist, k, [&](uint32_t digit, uint32_t) { w.state->base = digit << 20; });
         }
     }
 }
 
 // The window from a sample: a score at a pseudo-random place of every SAMPLE-th part of them, in a histogram of the keys'
-// upper 12 bits of 31; the last block puts the window around the place of the sample's share of k, between the ends of its bin.  A
-// block counts in shared memory: sampled keys share some hundred bins, and as atomics in L2 they took 58 us.
-constexpr uint32_t SAMPLE_BLOCKS = 128, SAMPLE_LOADS = 1, SAMPLE = SAMPLE_BLOCKS * SAMPLE_LOADS * 1024;
+// upper 12 bits of 31.  The threshold is surely between the bins of two places in the sample (SampleRanks); the last block puts a window of 2^20,
+// 2^21 or 2^22 keys around these, or leaves it to the histogram of all keys.  A block counts in shared memory: sampled keys share some
+// hundred bins, and as atomics in L2 they took 58 us.
+constexpr uint32_t SAMPLE_BLOCKS = 128, SAMPLE_LOADS = 2, SAMPLE = SAMPLE_BLOCKS * SAMPLE_LOADS * 1024;
 static_assert(SELECT_BINS == 1u << 12, "bins of 2^19 keys");
+struct SampleRanks { uint32_t first, last; };
 
-__global__ void __launch_bounds__(1024, 1) key_sample_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
+__global__ void __launch_bounds__(1024, 1) key_sample_kernel(const float *score, size_t P, SelectWork w, SampleRanks r) {
     __shared__ __align__(16) uint32_t sh[SELECT_BINS];
+    __shared__ uint32_t upper, lower;
     const size_t step = P / SAMPLE;
     float v[SAMPLE_LOADS];
 #pragma unroll
@@ -171,21 +179,31 @@ __global__ void __launch_bounds__(1024, 1) key_sample_kernel(const float *score,
     __syncthreads();
     for (uint32_t b = threadIdx.x; b < SELECT_BINS; b += 1024u)
         if (sh[b]) atomicAdd(w.sampled + b, sh[b]);
-    if (!last_block(w.done)) return;
-    const uint32_t need = (uint32_t)((double)k / (double)P * SAMPLE + 0.5);
-    const uint32_t rank = need ? need : 1u;
-    radix_pick<12>(w.sampled, rank, [&](uint32_t bin, uint32_t above, uint32_t count) {
-        const uint32_t down = (uint32_t)(((float)(rank - above) - 0.5f) / (float)count * (float)(1u << 19));
-        const uint32_t middle = ((bin + 1u) << 19) - down;
-        w.state->base = middle > 1u << 19 ? middle - (1u << 19) : 0u;
+    if (!last_block(w.done + 4)) return;
+    radix_walk<12>(w.sampled, [&](uint32_t bin, uint32_t above, uint32_t count) {
+        if (above < r.first && above + count >= r.first) upper = bin;
+        if (above < r.last && above + count >= r.last) lower = bin;
     });
+    __syncthreads();
+    if (threadIdx.x) return;
+    const uint32_t bins = upper - lower + 1u, shift = bins <= 2u ? 0u : bins <= 4u ? 1u : bins <= 8u ? 2u : WINDOW_OPEN;
+    w.state->shift = shift;
+    if (shift == WINDOW_OPEN) return;
+    const uint32_t under = ((2u << shift) - bins) << 18, from = lower << 19;       // what is left over goes to both sides
+    w.state->base = from > under ? from - under : 0u;
 }
 
-// The standard deviation of a sample's share of k is sqrt(p (1 - p) / SAMPLE), and the window reaches 3 to 6 % to either side of the
-// threshold, where p changes by that times 1.3 for real scores (products of two normal variables) and p = 0.1, and 3 and more in their
-// tail: 5 and 3 standard deviations for p = 0.1 and 1 / 256.  A selection that misses costs another one, so fewer scores beyond the threshold,
-// or in all, go by the histogram of all: at 2.5 M scores that is as quick (88 us and 90).
+// The standard deviation of a sample's share of k is sqrt(p (1 - p) / SAMPLE): 0.6, 1.9 and 3.1 % of p = 0.1, 0.01 and 1 / 256.  Four of them to either
+// side move the threshold by 2, 3 and 5 % for scores that are products of two normal variables, and by 12 % for log-normal ones whose logarithm
+// has a standard deviation of 3 and p = 0.005; the windows are at least 6, 12 and 25 % wide.  Scores in a wider spread go by the histogram
+// (155 us; 140 without the sample).  With one window of 2^20 keys around the place that 131,072 samples guessed, log-normal scores missed it in up to
+// half of all selections, and a miss costs the whole selection again (25.6 M scores, 1 in 200 of them: 181 us instead of 100).  Fewer scores beyond the
+// threshold, or in all, go by the histogram of all: at 2.5 M scores that is as quick (88 us and 90).
 bool select_by_sample(size_t P, size_t k) { return P >= (size_t)1 << 22 && k >= P / 256 && P - k >= P / 256; }
+static SampleRanks sample_ranks(size_t P, size_t k) {
+    const double p = (double)k / (double)P, mean = p * SAMPLE, off = 4.0 * sqrt(mean * (1.0 - p));
+    return SampleRanks{(uint32_t)(mean - off), (uint32_t)(mean + off) + 2u};         // within 1 .. SAMPLE: k and P - k are P / 256 at least
+}
 
 // f(first word, words' keys) for LOADS words of a tile at a time, by a warp: lane l the l-th parameter of each word.
 // Beyond the end keys are 0, and f is told how many parameters are left (LOADS * 32 or less).
@@ -211,22 +229,26 @@ __device__ __forceinline__ void for_tile(const float *score, size_t P, size_t fi
 }
 
 // The pass over the scores.  A warp takes a tile of MASK_BLOCK of them, marks and counts the keys beyond the window and gathers those
-// within, lane by lane: the place in the tile and 20 bits of the key, less the window's base.  A tile with more than TILE_CANDIDATES of
+// within, lane by lane: the place in the tile and the key less the window's base, 22 bits.  A tile with more than TILE_CANDIDATES of
 // them is read again instead.  It is bound by its instructions, so the scores' bit patterns themselves are compared (a key is 0 where
 // they are not those of a number from 0 to infinity, and only a window at 0 holds such keys), and a lane only notes its candidates in a word,
 // and reads them again at the tile's end (gathering them word by word took 52 us for 25.6 M scores).
-__device__ __forceinline__ uint32_t window_place(uint32_t key, uint32_t base) { return key - base; }        // below 2^20 within
+__device__ __forceinline__ uint32_t window_place(uint32_t key, uint32_t base) { return key - base; }        // below the number of its keys within
 constexpr int CAND_THREADS = 512;
 __global__ void __launch_bounds__(CAND_THREADS, 3)
 key_candidates_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
     __shared__ uint32_t sh[1024], beyond;
+    if (w.state->shift == WINDOW_OPEN) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) w.total[1] = 1u;
+        return;
+    }
     for (uint32_t b = threadIdx.x; b < 1024u; b += CAND_THREADS) sh[b] = 0;
     if (threadIdx.x == 0) beyond = 0;
     __syncthreads();
-    const uint32_t base = w.state->base, infinity = 0x7f800000u;
+    const uint32_t base = w.state->base, shift = w.state->shift, keys = 1u << (20 + shift), infinity = 0x7f800000u;
     // bit patterns beyond the window and within: from `last` + 1 and from `base`, so many
-    const uint32_t last = base + 0xfffffu, many = infinity > last ? infinity - last : 0u;
-    const uint32_t within = base > infinity ? 0u : infinity - base < 0xfffffu ? infinity - base + 1u : 1u << 20;
+    const uint32_t last = base + keys - 1u, many = infinity > last ? infinity - last : 0u;
+    const uint32_t within = base > infinity ? 0u : infinity - base < keys - 1u ? infinity - base + 1u : keys;
     // in a window at 0, where a key of 0 has many bit patterns, is all that is not beyond it
     const uint32_t in_from = base ? base : last + 1u, in_many = base ? within : many, turned = base ? 0u : 0xffffffffu;
     const uint32_t lane = threadIdx.x & 31u;
@@ -276,7 +298,7 @@ key_candidates_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
                 const uint32_t key = there ? score_key(__ldg(p + word * 32)) : 0u;
                 const uint32_t who = __ballot_sync(0xffffffffu, key > last);
                 if (lane == word) my_bits = who;
-                if (there && window_place(key, base) < 1u << 20) mine |= 1u << word;
+                if (there && window_place(key, base) < keys) mine |= 1u << word;
             }
         }
         uint32_t at = __popc(mine);
@@ -305,7 +327,7 @@ key_candidates_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
                 const uint32_t low = window_place(score_key(v[i]), base);
                 if (at < TILE_CANDIDATES) cand[at] = low << 10 | (word[i] * 32u + lane);
                 at++;
-                atomicAdd(sh + (low >> 10 & 1023u), 1u);
+                atomicAdd(sh + (low >> (10 + shift) & 1023u), 1u);
             }
         }
         if (tile < whole || lane * 32u < P - tile * MASK_BLOCK) w.bits[tile * (MASK_BLOCK / 32) + lane] = my_bits;
@@ -327,14 +349,14 @@ key_candidates_kernel(const float *score, size_t P, SelectWork w, uint32_t k) {
     if (threadIdx.x == 0) w.total[1] = k ? 1u : 0u;                    // until the threshold is found
     __syncthreads();
     if (k > too_many)
-        radix_pick<10, CAND_THREADS>(w.hist + 2048, k - too_many, [&](uint32_t digit, uint32_t over, uint32_t) {
+        radix_pick<10, CAND_THREADS>(w.hist + 2048, k - too_many, [&](uint32_t digit, uint32_t over) {
             w.state->place = digit;
             w.state->need = k - too_many - over;
             w.total[1] = 0u;
         });
 }
 
-// f(in, lower 20 bits and place in the tile) for the listed candidates of a tile, by a whole warp: the lane's every 32nd, of which the
+// f(in, place in the window and, below it, in the tile) for the listed candidates of a tile, by a whole warp: the lane's every 32nd, of which the
 // first is there already (rarely more than 32: these come with their number)
 template <class F>
 __device__ __forceinline__ void for_listed(const uint32_t *cand, uint32_t c, uint32_t found, F f) {
@@ -348,7 +370,7 @@ __device__ __forceinline__ void for_listed(const uint32_t *cand, uint32_t c, uin
 
 // the same for all candidates, of which there may be too many for the list
 template <class F>
-__device__ __forceinline__ void for_candidates(const float *score, size_t P, const SelectWork &w, size_t tile, uint32_t base, F f) {
+__device__ __forceinline__ void for_candidates(const float *score, size_t P, const SelectWork &w, size_t tile, uint32_t base, uint32_t keys, F f) {
     const uint32_t lane = threadIdx.x & 31u, found = w.tile_found[tile];
     const uint32_t *cand = w.cand + tile * TILE_CANDIDATES + lane;
     const uint32_t c0 = *cand;
@@ -359,29 +381,30 @@ __device__ __forceinline__ void for_candidates(const float *score, size_t P, con
 #pragma unroll
             for (int j = 0; j < LOADS; j++) {
                 const uint32_t low = window_place(key[j], base);
-                f(j * 32u + lane < left && low < 1u << 20, low << 10 | ((w0 + j) * 32u + lane));
+                f(j * 32u + lane < left && low < keys, low << 10 | ((w0 + j) * 32u + lane));
             }
         });
     }
 }
 
-// second digit of ten bits, over the candidates
+// the second digit, of the 10 to 12 bits that are left, over the candidates
 __global__ void __launch_bounds__(1024, 2) key_last_digit_kernel(const float *score, size_t P, SelectWork w) {
-    __shared__ uint32_t sh[1024];
-    sh[threadIdx.x] = 0;
-    __syncthreads();
+    __shared__ uint32_t sh[SELECT_LAST];
     if (w.total[1]) return;                               // not in the window
-    const uint32_t base = w.state->base, digit = w.state->place, need = w.state->need;
+    const uint32_t base = w.state->base, shift = w.state->shift, digit = w.state->place, need = w.state->need, digits = 1024u << shift;
+    for (uint32_t b = threadIdx.x; b < digits; b += 1024u) sh[b] = 0;
+    __syncthreads();
     const size_t tiles = (P + MASK_BLOCK - 1) / MASK_BLOCK;
     for (size_t tile = (size_t)blockIdx.x * 32u + (threadIdx.x >> 5); tile < tiles; tile += (size_t)gridDim.x * 32u)
-        for_candidates(score, P, w, tile, base, [&](bool in, uint32_t c) {
-            if (in && c >> 20 == digit) atomicAdd(sh + (c >> 10 & 1023u), 1u);
+        for_candidates(score, P, w, tile, base, 1u << (20 + shift), [&](bool in, uint32_t c) {
+            if (in && c >> (20 + shift) == digit) atomicAdd(sh + (c >> 10 & (digits - 1u)), 1u);
         });
     __syncthreads();
-    if (sh[threadIdx.x]) atomicAdd(w.hist + 3072 + threadIdx.x, sh[threadIdx.x]);
+    for (uint32_t b = threadIdx.x; b < digits; b += 1024u)
+        if (sh[b]) atomicAdd(w.hist + 3072 + b, sh[b]);
     if (last_block(w.done + 2) && need)
-        radix_pick<10>(w.hist + 3072, need, [&](uint32_t low, uint32_t over, uint32_t) {
-            w.state->place = digit << 10 | low;
+        radix_pick<12>(w.hist + 3072, need, [&](uint32_t low, uint32_t over) {
+            w.state->place = digit << (10 + shift) | low;
             w.state->need = need - over;
         });
 }
@@ -391,12 +414,12 @@ __global__ void __launch_bounds__(1024, 2) key_last_digit_kernel(const float *sc
 __global__ void __launch_bounds__(1024, 2) tile_counts_kernel(const float *score, size_t P, SelectWork w) {
     __shared__ uint64_t warp_sums[33];
     if (w.total[1]) return;                               // not in the window
-    const uint32_t base = w.state->base, place = w.state->place, need = w.state->need, lane = threadIdx.x & 31u;
+    const uint32_t base = w.state->base, keys = 1u << (20 + w.state->shift), place = w.state->place, need = w.state->need, lane = threadIdx.x & 31u;
     const size_t tiles = (P + MASK_BLOCK - 1) / MASK_BLOCK;
     const size_t begin = (size_t)blockIdx.x * w.run, end = begin + w.run < tiles ? begin + w.run : tiles;
     for (size_t tile = begin + (threadIdx.x >> 5); tile < end; tile += 32u) {
         uint32_t gt = 0, eq = 0;
-        for_candidates(score, P, w, tile, base, [&](bool in, uint32_t c) {
+        for_candidates(score, P, w, tile, base, keys, [&](bool in, uint32_t c) {
             gt += in && c >> 10 > place ? 1u : 0u;
             eq += in && c >> 10 == place ? 1u : 0u;
         });
@@ -437,7 +460,7 @@ cudaError_t launch_select(const float *score, size_t P, size_t k, bool by_sample
     cudaError_t e;
     if ((e = cudaMemsetAsync(w.hist, 0, (SELECT_ZEROED + (by_sample ? SELECT_BINS : 0)) * sizeof(uint32_t), s))) return e;
     if (by_sample) {
-        key_sample_kernel<<<SAMPLE_BLOCKS, 1024, 0, s>>>(score, P, w, (uint32_t)k);
+        key_sample_kernel<<<SAMPLE_BLOCKS, 1024, 0, s>>>(score, P, w, sample_ranks(P, k));
         if ((e = FEDHE_LAUNCHED())) return e;
     }
     if ((e = cudaFuncSetAttribute(key_histogram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)HIST_SMEM))) return e;
@@ -497,7 +520,8 @@ cudaError_t launch_scan(uint32_t *a, size_t count, uint32_t *total, cudaStream_t
 // the tile is read again (its 32 keys of a word would take turns at it: 25.6 M equal scores, half of them wanted: 235 us a selection, and 191).
 // words: the warp's own [2][32].
 __device__ __forceinline__ uint32_t tile_bits(const float *score, size_t P, const SelectWork &w, size_t tile, uint32_t eq_before, uint32_t *words) {
-    const uint32_t base = w.state->base, place = w.state->place, need = w.state->need, found = w.tile_found[tile], lane = threadIdx.x & 31u;
+    const uint32_t base = w.state->base, keys = 1u << (20 + w.state->shift), place = w.state->place, need = w.state->need,
+                   found = w.tile_found[tile], lane = threadIdx.x & 31u;
     const uint32_t *cand = w.cand + tile * TILE_CANDIDATES + lane;
     const uint32_t c0 = *cand;
     uint32_t bits = tile * MASK_BLOCK + lane * 32u < P ? w.bits[tile * (MASK_BLOCK / 32) + lane] : 0u, equal = 0;
@@ -517,7 +541,7 @@ __device__ __forceinline__ uint32_t tile_bits(const float *score, size_t P, cons
 #pragma unroll
             for (int j = 0; j < LOADS; j++) {
                 const uint32_t at = window_place(key[j], base);
-                const bool in = j * 32u + lane < left && at < 1u << 20;
+                const bool in = j * 32u + lane < left && at < keys;
                 const uint32_t gt = __ballot_sync(0xffffffffu, in && at > place), eq = __ballot_sync(0xffffffffu, in && at == place);
                 if (lane == w0 + j) {
                     bits |= gt;

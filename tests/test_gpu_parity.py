@@ -527,7 +527,7 @@ def test_select_mask_tiles_and_candidates(he, P, spread):
 @pytest.mark.parametrize("kind", ["products", "two clusters", "few values", "one value"])
 def test_select_mask_by_a_sample(he, kind):
     """From 2^22 scores on a sample says where the threshold is looked for: scores as they come, thresholds at the edge of a
-    gap that the sample can only guess (the selection is made again then), and ties that fill the window."""
+    gap that no sample can tell (the histogram of all scores does then), and ties that fill the window."""
     g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
     rng = np.random.default_rng(91)
     P = (1 << 22) + 1013
@@ -551,6 +551,39 @@ def test_select_mask_by_a_sample(he, kind):
         mask = he.he_select_mask(g, d, k)
         got = he.he_mask_indices(mask).cpu().numpy().view(np.uint32)
         assert mask.k == k and np.array_equal(got, oracle.select_mask(score, k)), k
+
+
+@pytest.mark.parametrize("spread,parts,launches", [(1.0, [0.3, 0.005], 5), (3.0, [0.9, 0.1, 0.01, 0.005], 5), (4.0, [0.1, 0.02], 5), (20.0, [0.005], 10)])
+def test_select_mask_of_log_normal_scores(he, spread, parts, launches):
+    """The window is as wide as the sample's doubt: no selection is made twice (more launches) but where the widest is too narrow."""
+    g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
+    P = (1 << 22) + 77
+    for seed in range(5):
+        score = np.exp(spread * np.random.default_rng(seed).standard_normal(P)).astype(np.float32)
+        d = dev_f32(score)
+        for part in parts:
+            k = int(part * P)
+            before = he.he_launch_count()
+            mask = he.he_select_mask(g, d, k)
+            assert he.he_launch_count() - before == launches, (seed, part)
+            assert np.array_equal(he.he_mask_indices(mask).cpu().numpy().view(np.uint32), oracle.select_mask(score, k)), (seed, part)
+
+
+@pytest.mark.parametrize("wrong", [0.0, 1.0, 100.0])
+def test_select_mask_with_a_sample_that_misleads(he, wrong):
+    """All sampled scores are alike and no others are: the threshold is not in the window, and the selection is made again."""
+    g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
+    P, sample = (1 << 22) + 4099, 1 << 18
+    i = np.arange(sample, dtype=np.uint64)
+    step = np.uint64(P // sample)
+    at = i * step + (((i * np.uint64(2654435761)) & np.uint64(0xffffffff)) * step >> np.uint64(32))
+    score = (10.0 + np.random.default_rng(5).random(P, dtype=np.float32)).astype(np.float32)
+    score[at] = wrong
+    k = P // 2
+    before = he.he_launch_count()
+    mask = he.he_select_mask(g, dev_f32(score), k)
+    assert he.he_launch_count() - before == 10
+    assert np.array_equal(he.he_mask_indices(mask).cpu().numpy().view(np.uint32), oracle.select_mask(score, k))
 
 
 @pytest.mark.parametrize("P", [1024, 5 * 1024 + 77, (1 << 22) + 1024])
