@@ -199,6 +199,7 @@ int he_ctx_create(const he_params *p, he_ctx **out) {
         rc = upload(ctx, reinterpret_cast<const double2 *>(ftw.data()), ftw.size() / 2, &d.ftw);
         if (!fft_cut(d, ctx->enc)) { rc = HE_ERR_PARAMS; break; }     // no prime that host_check_params() lets pass
         d.enc = &ctx->enc;
+        if (rc == HE_OK) rc = upload(ctx, ctx->enc.jobs, 2, &d.enc_jobs);
         host_fft_tables(d.N, roots, fwd, inv, slot_of);
         if (rc == HE_OK) rc = upload(ctx, reinterpret_cast<const root_t *>(fwd.data()), fwd.size() / 2, &d.fft_fwd);
         if (rc == HE_OK) rc = upload(ctx, reinterpret_cast<const root_t *>(inv.data()), inv.size() / 2, &d.fft_inv);

@@ -264,28 +264,13 @@ struct EncRing {
     static constexpr size_t SMEM = (size_t)NB * 16 + (size_t)Tab::WORDS * 16 + (E_IN_SMEM ? N : 0);
 };
 
-// What a thread block needs to know of a product, in shared memory: looked up in the kernel's parameters, by the unit's number, then
-// its limb's, it was a chain of misses of 900 clocks before every block of a transform (N = 16384).
-struct alignas(16) EncJob {
-    uint64_t q;
-    double scale;                // of the limb's quotients
-    uint32_t key[2];
-    uint32_t shift, what;        // the top piece's; limb and EncJob flags
-    static constexpr uint32_t PARKS = 1u << 8, NARROW = 1u << 9, JOINS = 10;      // flags; the limb is below them, `joins` above
-};
-struct EncJobs {
-    EncJob job[2 * HE_MAX_LIMBS];
-    uint8_t start[4 * HE_MAX_LIMBS + 4];
-};
-__device__ __forceinline__ void enc_jobs_load(EncJobs &s, const CtxDev &c, const EncWay &way, uint32_t split) {
-    for (uint32_t i = threadIdx.x; i < way.products; i += FftLay::NT) {
-        const EncProduct &p = way.product[i];
-        const LimbDev &limb = c.limb[p.limb];
-        const FftSplit &f = limb.split[split];
-        s.job[i] = EncJob{limb.q, f.top_scale, {p.key[0], p.key[1]}, f.shift[f.pieces - 1],
-                          p.limb | (p.parks ? EncJob::PARKS : 0u) | (f.narrow ? EncJob::NARROW : 0u) | (uint32_t)p.joins << EncJob::JOINS};
-    }
-    for (uint32_t i = threadIdx.x; i <= 2 * way.products; i += FftLay::NT) s.start[i] = way.start[i];
+// What a thread block needs to know of the products, in shared memory: looked up in the kernel's parameters, by the unit's number, then
+// its limb's, it was a chain of misses of 900 clocks before every block of a transform (N = 16384).  Put together from the parameters at the
+// start of the kernel it was these misses again, for every product one behind the other (one ciphertext of N = 8192, 8 limbs of
+// 60 bits: 24.7 us, 22.3 before that and 22.6 now; 888 of 8 limbs of 45 bits: 645, 650 to 700, 628); one load brings the finished table.
+__device__ __forceinline__ void enc_jobs_load(EncJobs &s, const EncJobs *made) {
+    static_assert(sizeof(EncJobs) / 16 <= FftLay::NT, "a load for every thread");
+    if (threadIdx.x < sizeof(EncJobs) / 16) reinterpret_cast<uint4 *>(&s)[threadIdx.x] = __ldg(reinterpret_cast<const uint4 *>(made) + threadIdx.x);
 }
 
 // What a ciphertext's draws depend on besides its number, and whether the clusters draw for themselves.
@@ -522,10 +507,11 @@ enc_sample_kernel(const void *gauss, EncDraw draw, uint32_t T, unsigned char *sa
 //   N = 2^14, L = 4, 1429 ciphertexts   2.82 ms -> 1.38 ms -> 1.27 ms (1.2 TB/s of ciphertext)
 //   N = 2^15, L = 6, 672 ciphertexts              2.69 ms -> 2.33 ms (0.9 TB/s)
 //
+struct EncTable { const EncJobs *jobs; uint32_t products; };
 // PAIRS: some units are of two limbs (the code for both kinds costs the others 1.5 %).
 template <int CL, bool PAIRS>
 __global__ void __launch_bounds__(FftLay::NT, 2)
-encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ EncWay way, const KeysDev k, const float *sel,
+encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ EncTable made, const KeysDev k, const float *sel,
                    const EncDraw draw, unsigned char *samples, unsigned char *work, uint64_t *ct, uint32_t T, uint32_t S, uint32_t most_parts) {
     using G = EncRing<CL>;
     constexpr uint32_t N = G::N, n = G::n, NB = G::NB, NT = G::NT, R = G::R;
@@ -537,7 +523,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
     __shared__ uint32_t tmem_base;
     __shared__ __align__(8) uint64_t key_bar;
     const uint32_t rank = blockIdx.x % S, cid = blockIdx.x / S, nc = gridDim.x / S;
-    enc_jobs_load(jobs, c, way, PAIRS);
+    enc_jobs_load(jobs, made.jobs);
     for (uint32_t i = threadIdx.x; i < (uint32_t)G::Tab::WORDS; i += NT) tab[i] = c.fft_inv[i];
     if (threadIdx.x == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(&key_bar)) : "memory");
@@ -568,7 +554,7 @@ encrypt_fft_kernel(const __grid_constant__ CtxDev c, const __grid_constant__ Enc
     const uint32_t whole = T / nc * nc, rem = T - whole;
     const uint32_t parts = rem ? (nc / rem < most_parts ? nc / rem : most_parts) : 1;
     const uint32_t items = whole + rem * parts;           // at least as many as clusters
-    const uint32_t products = way.products, all = 2 * products;
+    const uint32_t products = made.products, all = 2 * products;
     const bool leader = rank == 0 && threadIdx.x == 0;
     uint32_t next_item = cid;
     asm volatile("griddepcontrol.wait;" ::: "memory");    // for samples drawn by the kernel above
@@ -1018,7 +1004,7 @@ static void cut_residues(uint64_t q, int most, int narrow_bits, FftSplit &f) {
 // to fit 32 bits (a coefficient is below N 2^(width - 1)), or else as high as the top one may be wide, where it
 // fits all the same (exponent 95: under 2^-136).
 // False for a prime that the kernels are not made for: more than two pieces, or, for N <= 2^14, a wide low one.
-static bool cut_limbs(CtxDev &c, bool in_pairs, EncWay &w, size_t &words) {
+static bool cut_limbs(CtxDev &c, bool in_pairs, EncWay &w, EncJobs &jobs, size_t &words) {
     const int logN = (int)c.logN, sure = fft_sure_bits(logN), wide = fft_wide_bits(logN), narrow = fft_random_bits(logN, 32, FFT_NARROW_EXPONENT);
     uint32_t waiting = NO_LIMB;                        // unit of a limb that could share its low product
     w.units = 0;
@@ -1052,12 +1038,15 @@ static bool cut_limbs(CtxDev &c, bool in_pairs, EncWay &w, size_t &words) {
         EncUnit &e = w.unit[u];
         e.fft_key = words;
         for (uint32_t p = 0; p < e.products; p++) {
-            EncProduct &d = w.product[w.products + p];
-            const bool pair = e.limb2 != NO_LIMB;
+            const bool pair = e.limb2 != NO_LIMB, parks = pair ? p == 0 : p + 1 < e.products;
+            const uint32_t j = pair && p == 2 ? e.limb2 : e.limb, joins = parks || e.products == 1 ? 0 : pair ? p + 1 : 1;
+            const FftSplit &f = c.limb[j].split[in_pairs];
+            EncJob &d = jobs.job[w.products + p];
+            d.q = c.limb[j].q;
+            d.scale = f.top_scale;
             for (uint32_t comp = 0; comp < 2; comp++) d.key[comp] = (uint32_t)(words / FftLay::NB) + (comp * e.products + p) * R;
-            d.limb = (uint16_t)(pair && p == 2 ? e.limb2 : e.limb);
-            d.parks = pair ? p == 0 : p + 1 < e.products;
-            d.joins = (uint8_t)(d.parks || e.products == 1 ? 0 : pair ? p + 1 : 1);
+            d.shift = f.shift[f.pieces - 1];
+            d.what = j | (parks ? EncJob::PARKS : 0u) | (f.narrow ? EncJob::NARROW : 0u) | joins << EncJob::JOINS;
         }
         words += 2 * (size_t)e.products * (c.N / 2);
         w.products += e.products;
@@ -1065,7 +1054,7 @@ static bool cut_limbs(CtxDev &c, bool in_pairs, EncWay &w, size_t &words) {
     uint32_t begin = 0, of_unit = 0;
     for (uint32_t pos = 0; pos <= 2 * w.products; pos++) {
         if (pos > begin) begin += w.unit[of_unit++ % w.units].products;
-        w.start[pos] = (uint8_t)begin;
+        jobs.start[pos] = (uint8_t)begin;
     }
     return true;
 }
@@ -1075,16 +1064,17 @@ bool fft_cut(CtxDev &c, EncWays &e) {
     for (uint32_t j = 0; j < c.L; j++)
         if ((int64_t)(c.limb[j].q / 4) < c.term_limit) c.term_limit = (int64_t)(c.limb[j].q / 4);
     size_t words = 0;
-    if (!cut_limbs(c, true, e.way[0], words)) return false;
+    if (!cut_limbs(c, true, e.way[0], e.jobs[0], words)) return false;
     e.count = e.way[0].units < c.L ? 2 : 1;
     if (e.count == 1) words = 0;
-    if (!cut_limbs(c, false, e.way[e.count - 1], words)) return false;
+    if (!cut_limbs(c, false, e.way[e.count - 1], e.jobs[e.count - 1], words)) return false;
     for (uint32_t i = 0; i < e.count; i++) {
         const EncWay &w = e.way[i];
         for (uint32_t of = 1; of < ENC_SHARES; of++) {
             uint32_t most = 0;
             for (uint32_t part = 0; part < of; part++) {
-                const uint32_t sum = w.start[2 * w.products * (part + 1) / of] - w.start[2 * w.products * part / of];
+                const uint8_t *start = e.jobs[i].start;
+                const uint32_t sum = start[2 * w.products * (part + 1) / of] - start[2 * w.products * part / of];
                 most = sum > most ? sum : most;
             }
             e.most[i][of] = (uint16_t)most;
@@ -1298,8 +1288,8 @@ static cudaError_t launch_encrypt_part(const CtxDev &c, const KeysDev &k, const 
     // The clusters start beside the last samples if there is one to a ciphertext.  With more, all the clusters that fit have to be there
     // at once, and those that come first may leave no room for a whole one (200 ciphertexts of N = 32768: 784 -> 800 us).
     cfg.numAttrs = !draw.inside && T <= p.clusters ? 2 : 1;
-    if ((e = cudaLaunchKernelEx(&cfg, pairs_limbs(c, p.way) ? encrypt_fft_kernel<CL, true> : encrypt_fft_kernel<CL, false>, c, c.enc->way[p.way],
-                                k, sel, draw, work, work + T * G::SAMPLES, ct, (uint32_t)T, p.S, p.parts)))
+    if ((e = cudaLaunchKernelEx(&cfg, pairs_limbs(c, p.way) ? encrypt_fft_kernel<CL, true> : encrypt_fft_kernel<CL, false>, c, EncTable{c.enc_jobs + p.way,
+                                c.enc->way[p.way].products}, k, sel, draw, work, work + T * G::SAMPLES, ct, (uint32_t)T, p.S, p.parts)))
         return e;
     return FEDHE_LAUNCHED();
 }

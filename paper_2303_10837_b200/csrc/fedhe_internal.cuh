@@ -41,18 +41,23 @@ struct EncUnit {
     uint32_t products;
     size_t fft_key;              // first word of its key tables: [2 components][products][n]
 };
-// A product of a unit, in the order in which a thread block works them off: a low piece's is parked, a top one's ends its limb.
-struct EncProduct {
-    uint32_t key[2];             // blocks of 2^12 words before its key tables, for either component
-    uint16_t limb;               // of the low product of a pair: of the first of them
-    uint8_t parks;
-    uint8_t joins;               // what is parked for a top piece: 0 nothing, 1 its low piece's product, 2, 3 that of a pair, lower or upper limb
-};
 // The units of a public-key half.
 struct EncWay {
     uint32_t units, products;    // of all units
     EncUnit unit[HE_MAX_LIMBS];
-    EncProduct product[2 * HE_MAX_LIMBS];
+};
+// Its products, in the order in which a thread block works them off: a low piece's is parked, a top one's ends its limb.
+struct alignas(16) EncJob {
+    uint64_t q;
+    double scale;                // of the limb's quotients
+    uint32_t key[2];             // blocks of 2^12 words before the key tables, for either component
+    uint32_t shift;              // the top piece's
+    uint32_t what;               // limb (of the low product of a pair: of the first of them), flags, and above them what is parked for
+                                 // a top piece: 0 nothing, 1 its low piece's product, 2, 3 that of a pair, lower or upper limb
+    static constexpr uint32_t PARKS = 1u << 8, NARROW = 1u << 9, JOINS = 10;
+};
+struct alignas(16) EncJobs {
+    EncJob job[2 * HE_MAX_LIMBS];
     uint8_t start[4 * HE_MAX_LIMBS + 1];       // of the products of both components: the first at or after a number that begins a unit
 };
 // Limbs in pairs where that is possible, and, if any are, every limb by itself too: fewer products, or more units to share out.
@@ -61,6 +66,7 @@ constexpr uint32_t ENC_SHARES = 2 * HE_MAX_LIMBS + ENC_MOST;
 struct EncWays {
     uint32_t count;
     EncWay way[2];
+    EncJobs jobs[2];
     uint16_t most[2][ENC_SHARES];      // of the products of a ciphertext shared out to so many blocks, the most that one has
 };
 
@@ -114,6 +120,7 @@ struct CtxDev {
     const uint32_t *slot_of;           // slot of every value that the forward transform leaves
     FftSplit dec_split;                // of c1 on limb 0, for any c1
     const EncWays *enc;                // host memory (the context's): kernels get the way they take by value
+    const EncJobs *enc_jobs;           // of either way, in device memory
     int64_t term_limit;                // a quarter of the smallest prime
     uint16_t enc_fit[2][ENC_MOST + 1]; // clusters of a size that the device holds: two blocks to an SM, one
     uint32_t passes_most;              // encryption by passes (N = 2^16): the most ciphertexts that go by them
