@@ -3,6 +3,8 @@ takes plain pointers and cannot know a buffer's extent, and a short buffer on th
 an out-of-bounds access, not an error.  No GPU is needed: the size checks come before the check
 that a tensor lives on the device, so host tensors of the wrong size must raise HeError and host
 tensors of the right size must get as far as the device check (TypeError)."""
+import importlib.util
+
 import pytest
 import torch
 
@@ -100,3 +102,19 @@ def test_unpack_pack_and_transform_sizes(ctx):
     refused(lambda: he.he_round_host(ctx, keys(ctx), None, [torch.zeros(10)], [0.5, 0.5], 1,
                                      torch.zeros(10, dtype=torch.float64)))
     reaches_device_check(lambda: he.he_unpack(ctx, mask, z, rest, 100, out=torch.zeros(100, dtype=torch.float64)))
+
+
+@pytest.mark.parametrize("absent", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_stream_without_the_private_names(absent):
+    """A torch without the raw query that the binding prefers still gives the current stream, by the public call."""
+    import types
+    private = {"_cuda_getCurrentRawStream": lambda device: -1, "_cuda_getDevice": lambda: 0}
+    del private[absent]
+    with pytest.MonkeyPatch.context() as m:
+        m.setattr(torch, "_C", types.SimpleNamespace(**private))
+        spec = importlib.util.spec_from_file_location("binding_alone", he.__file__)
+        alone = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(alone)
+        m.setattr(torch.cuda, "is_initialized", lambda: True)
+        m.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=77))
+        assert alone._stream() == 77
