@@ -519,6 +519,7 @@ cudaError_t launch_encrypt_ntt(const CtxDev &c, const KeysDev &k, const float *s
 //   two 60-bit limbs: 10, 24, 40, 92, 600 ciphertexts   143 214, 216 224, 341 333, 653 546, 3961 2870
 //   eight: 3, 5, 18, 40   180 177, 214 173, 452 478, 986 642;      four of 45 bits: 10, 31, 40, 92, 600   147 185, 298 298, 394 439, 761 824, 4608 4919
 //   twelve of 45 bits: 3, 10, 31, 92, 300   165 179, 300 407, 718 732, 1949 2141, 6166 6578
+// (by transforms that have got 4 to 9 % faster since, with two 60-bit limbs 24 and 600 ciphertexts take 197 and 2770 now; the passes are as they were).
 // The passes by the line through these (up to 20 % low short of a whole wave of their thread blocks, hence 4 to 7 % in their favour),
 // the transforms by the cost of their plan.
 bool encrypt_by_passes(const CtxDev &c, size_t T) {

@@ -256,7 +256,7 @@ struct EncRing {
     // a ciphertext's samples: e0, e1 (a byte each), u in two bits each, the rows of a column side by side
     using Row = typename std::conditional<(R <= 4), uint8_t, uint16_t>::type;
     static constexpr size_t E0 = 0, E1 = N, U = 2 * (size_t)N, SAMPLES = U + 2 * NB * sizeof(Row);
-    // items of 512 stream blocks: of u, of either error
+    // items of u (four neighbouring columns of a half to a thread, all their rows: 512, 512, 1024, 2048 stream blocks), of either error (512)
     static constexpr uint32_t U_COLUMNS = R == 1 ? 2 : 1, U_ITEMS = 2 * NB / 4 / (NT * U_COLUMNS), E_ITEMS = N / 2 / (2 * NT),
                               ITEMS = U_ITEMS + 2 * E_ITEMS;
     // a thread block's: what waits, joined low pieces
@@ -1178,7 +1178,9 @@ static uint32_t enc_sure_fit(const CtxDev &c, uint32_t alone, uint32_t S) {
 
 // What a plan takes, in us: a round is fixed + by_size / S + product * (block transforms of the busiest block's products),
 // fitted to 10,000 measurements of all plans for up to 200 ciphertexts of 2 to 12 limbs of 45 and 60 bits (nine of ten within
-// 10 %), for two blocks to an SM and for one, when the clusters drew for themselves; with the draws made before, all plans take about a tenth less.
+// 10 %), for two blocks to an SM and for one, when the clusters drew for themselves.  Not fitted again since: plans
+// take 9 to 13 % less now at N = 16384 (4 limbs, 1 to 60 ciphertexts) and 32768 (6 limbs), 4 to 9 % at 65536 (2 limbs, 24 to 600), and where
+// an estimate is compared with another path's (encrypt_by_passes) it is too high by that.
 struct EncCost { double fixed, by_size, product; };
 static const EncCost ENC_COST[4][2] = {{{27.3, 12.7, 7.7}, {33.1, 2.2, 4.9}},
                                        {{27.4, 40.1, 9.1}, {43.5, 13.7, 5.7}},

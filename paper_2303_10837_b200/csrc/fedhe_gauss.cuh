@@ -44,8 +44,8 @@ HD int gauss_from_u64(uint64_t r) {
 // the entry the number of thresholds certainly not above r, below it 2^24 less the next 24 bits of the one threshold that shares
 // the entry's range.  Adding the next 24 bits of r carries into the top byte when r is not below that threshold, so a
 // sample costs one 4-byte load, an addition and a shift.  Not decided are ranges with more than one threshold
-// (1 sample in 30,000) and sums whose low 24 bits are close to a carry, where bits that are not in the word count: behind
-// the second byte it has 16 bits and not 24, so up to 255 may be missing (1 in 30,000).  With the bytes 00
+// (1 sample in 32,768) and sums whose low 24 bits are close to a carry, where bits that are not in the word count: behind
+// the second byte it has 16 bits and not 24, so up to 255 may be missing (1 in 65,536).  With the bytes 00
 // and ff undecided (1 sample in 128) two calls of five had a lane that needed the whole block.
 struct alignas(16) GaussTables {
     uint32_t entry[3 * 256];         // by the top byte; by the second byte behind 00; by the second byte behind ff

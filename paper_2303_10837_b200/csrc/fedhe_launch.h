@@ -69,10 +69,11 @@ cudaError_t launch_encrypt_ntt(const CtxDev &c, const KeysDev &k, const float *s
 
 // What a weighted sum needs to know of C clients: their C pointers, then what they are weighed by ([C][L] tw_t for ciphertexts, [C]
 // doubles for the remainder).  A small table goes with the kernel's parameters: a copy to the device from memory that is not pinned
-// costs the call 2 us on the host and makes the kernel wait for it (a whole round of three clients with 25 ciphertexts of N = 8192
-// each: 167.8 -> 165.9 us).  A larger one is copied: threads that read different words of the parameters take turns (64 clients, 200 words: 121.2 us, 122.0).
+// costs the call 2 us on the host and makes the kernel wait for it (25 ciphertexts of N = 8192, three limbs, copied and not: 3 clients, 21 words,
+// 14.5 and 12.4 us; 9, 63 words, 26.8 and 24.8; 18, 126 words, 43.9 and 42.9).  A larger one is copied: threads that read different words of the
+// parameters take turns, and what is gained is lost again (32 clients, 224 words, 66.6 and 66.5; 64, 448 words, 120.4 and 121.9).
 struct SumTable {
-    static constexpr size_t WORDS = 48;
+    static constexpr size_t WORDS = 128;
     const uint64_t *far;                  // in device memory; null: here
     uint64_t words[WORDS];
 };

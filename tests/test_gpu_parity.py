@@ -692,9 +692,9 @@ def test_encryption_and_sum_in_a_graph(he, T):
         assert torch.equal(ct, want) and torch.equal(total, want_sum)
 
 
-@pytest.mark.parametrize("C", [7, 25, 69, 256])
+@pytest.mark.parametrize("C", [7, 18, 19, 64, 69, 256])
 def test_sums_of_many_clients_in_a_graph(he, C):
-    """A graph must not read the host's tables again, which end with the call: from 49 words (7 clients here, 25 for the remainder) on
+    """A graph must not read the host's tables again, which end with the call: from 129 words (19 clients here, 65 for the remainder) on
     a captured sum brings them by kernels, 480 words each, before its own.  Replayed only if their number says so."""
     g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
     rng = np.random.default_rng(C)
@@ -705,13 +705,13 @@ def test_sums_of_many_clients_in_a_graph(he, C):
     cts, rests = [cts[i % 3] for i in range(C)], [rests[i % 3] for i in range(C)]
     parts = [he.he_weighted_partial(g, cts[i::2], alpha[i::2]) for i in range(2)]
     added = parts[0] + parts[1]
-    kernels = -(-7 * C // 480)
+    kernels = -(-7 * C // 480) if C > 18 else 0
     calls = [(lambda out: he.he_weighted_aggregate(g, cts, alpha, out=out), kernels),
              (lambda out: he.he_weighted_partial(g, cts, alpha, out=out), kernels),
              (lambda out: he.he_weighted_aggregate_ntt(g, cts, alpha, out=out), kernels),
              (lambda out: he.he_rescale_partial_sum(g, added, 2, out=out), 1),
              (lambda out: he.he_rescale_partial_parts(g, parts, out=out), 1),
-             (lambda out: he.he_plain_aggregate(g, rests, alpha), -(-2 * C // 480) if C > 24 else 0)]
+             (lambda out: he.he_plain_aggregate(g, rests, alpha), -(-2 * C // 480) if C > 64 else 0)]
     for call, more in calls:
         before = he.he_launch_count()
         want = call(None)
@@ -732,9 +732,9 @@ def test_sums_of_many_clients_in_a_graph(he, C):
             assert torch.equal(got, want)
 
 
-@pytest.mark.parametrize("C", [1, 24, 25, 256])
+@pytest.mark.parametrize("C", [1, 24, 25, 64, 65, 256])
 def test_plain_aggregate_of_many_clients(he, C):
-    """Pointers and weights in the kernel's parameters (up to 24 clients) and in device memory."""
+    """Pointers and weights in the kernel's parameters (up to 64 clients) and in device memory."""
     g, _ = contexts(he, 8192, si.PRIMES_N8192, 40)
     rng = np.random.default_rng(C)
     rests = [rng.standard_normal(1003, dtype=np.float32) for _ in range(C)]
