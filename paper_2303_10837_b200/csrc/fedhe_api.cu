@@ -992,7 +992,7 @@ static int round_host_queued(he_ctx *ctx, const he_keys *keys, const he_mask *ma
 
     // Equal ranges, as many as make the call shortest by this account (us): a client's part of a range comes up
     // at 55 GB/s (the link of the machine that this was measured on); its ciphertexts take `first` (N = 2^13 .. 2^16) and, each,
-    // `product` for every product of a public-key half and two more; a range costs range_us besides; after the last upload
+    // `product` for every product of a public-key half and two more (measured when the clusters drew for themselves; 4 to 13 % high since); a range costs range_us besides; after the last upload
     // come one client's ciphertexts, and the range's download.  (With ranges of 2^20 parameters, 12 clients and 3 M
     // parameters at N = 2^15 spent 5.0 instead of 3.5 ms on short encryptions; with the cost of a ciphertext by the ring alone, 10
     // clients and 3 M parameters, half of them masked, at N = 2^13 with twelve 60-bit primes 9.6 instead of 7.0 ms.)

@@ -499,10 +499,10 @@ enc_sample_kernel(const void *gauss, EncDraw draw, uint32_t T, unsigned char *sa
 // all prepare it and share its units.
 //
 // What bounds it: in the transforms shared memory (3360 of 3500 clocks a block of 2^12 points and SM: two exchanges of 1024, the key's table in and
-// out 1024, twiddles 288), between them latency at the 16 warps that registers leave; the fp64 pipe is 30 to 35 % busy.  Measured, against
+// out 1024, twiddles 288), between them latency at the 16 warps that registers leave; the fp64 pipe is 36 to 41 % busy.  Measured, against
 // modular transforms of every limb; with the draws of u and the errors by the clusters; and with these from the kernel above and what a
 // product needs to know in shared memory:
-//   N = 2^13, L = 3, 1 ciphertext       67.7 us -> 30.7 us -> 24.9 us
+//   N = 2^13, L = 3, 1 ciphertext       67.7 us -> 30.7 us -> 23.5 us
 //   N = 2^14, L = 4, 313 ciphertexts    0.69 ms -> 0.32 ms -> 0.30 ms
 //   N = 2^14, L = 4, 1429 ciphertexts   2.82 ms -> 1.38 ms -> 1.27 ms (1.2 TB/s of ciphertext)
 //   N = 2^15, L = 6, 672 ciphertexts              2.69 ms -> 2.33 ms (0.9 TB/s)

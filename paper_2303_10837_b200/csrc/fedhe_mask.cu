@@ -45,10 +45,10 @@ __device__ __forceinline__ T block_exclusive_scan(T v, T *warp_sums, T &total) {
 
 // ---- selection of the k-th largest key ----
 //
-// A window of 2^20 keys that holds the threshold, from a sample of the scores or from the histogram of the keys' first digit
-// (11 of their 31 bits); one pass over the scores that counts and marks the keys beyond the window and
-// gathers those within (the candidates, a few per cent of real scores) by tiles; then two digits of ten bits and the marking on the
-// candidates.  The last thread block of a pass to finish does the one-block step that follows it: picking the digit, or
+// A window of keys that holds the threshold, 2^20 to 2^22 of them by a sample of the scores or 2^20 by the histogram of the keys' first
+// digit (11 of their 31 bits); one pass over the scores that counts and marks the keys beyond the window and
+// gathers those within (the candidates, a few per cent of real scores) by tiles; then a digit of ten bits, one of the 10 to 12 that are left
+// and the marking on the candidates.  The last thread block of a pass to finish does the one-block step that follows it: picking the digit, or
 // the scan over the tiles.  For 2.56 M out of 25.6 M scores the call took 341 us by three histogram passes, a counting pass
 // and one-block kernels between them (conflicts of shared-memory atomics, because neighbouring scores share an exponent), 165 us
 // with the histogram of the first digit over all scores (27 us) and the scores read again for the marking (33 us).
